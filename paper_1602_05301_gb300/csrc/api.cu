@@ -316,6 +316,19 @@ extern "C" qbx_status qbx_tree_build(qbx_handle* h, const qbx_tree_desc* d) {
   h->stats[2] = h->n_tgt;
   h->stats[3] = h->n_qbx_tgt;
   if (d->mode == QBX_DIRECT) {
+    std::vector<char> used((size_t)h->n_ctr, 0);
+    for (int64_t t = 0; t < h->n_tgt; ++t) {
+      if (assoc[t] < 0) continue;
+      used[assoc[t]] = 1;
+      // a two-sided target also reads its node's interior centre
+      if (h->has_avg && !on_side.empty() && on_node[t] >= 0 && on_side[t] == 0)
+        used[assoc[t] + h->n_nodes] = 1;
+    }
+    std::vector<int32_t> ul;
+    for (int64_t c = 0; c < h->n_ctr; ++c)
+      if (used[c]) ul.push_back((int32_t)c);
+    h->n_used_ctr = (int64_t)ul.size();
+    QBX_TRY(copy_in(h->used_ctr, ul.data(), ul.size()));
     h->stats[12] = h->n_src * h->n_ctr;
     h->stats[13] = h->n_src * h->n_direct_tgt;
   }
@@ -379,10 +392,10 @@ extern "C" qbx_status qbx_layer_potential_eval(qbx_handle* h, double cS_re, doub
     QBX_TRY(fmm_eval(h, has_S, has_D, o, precision, alpha_out != nullptr, s));
   } else {
     stage_begin(h, QBX_STAGE_P2QBXL, s);
-    QBX_TRY(launch_p2qbxl_direct(h, has_S, has_D, precision, s));
+    QBX_TRY(launch_p2qbxl_direct(h, has_S, has_D, alpha_out != nullptr, s));
     stage_end(h, QBX_STAGE_P2QBXL, s);
     stage_begin(h, QBX_STAGE_P2P, s);
-    QBX_TRY(launch_p2p_direct(h, has_S, has_D, o, precision, s));
+    QBX_TRY(launch_p2p_direct(h, has_S, has_D, o, s));
     stage_end(h, QBX_STAGE_P2P, s);
   }
   stage_begin(h, QBX_STAGE_QBXL2P, s);

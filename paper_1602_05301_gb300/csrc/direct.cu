@@ -11,11 +11,9 @@
 #include <cstdio>
 
 #include "qbx_internal.h"
-#include "special.cuh"
+#include "p2qbxl_pair.cuh"
 
 namespace {
-
-constexpr int kTile = 128;
 
 // q_j = (i/4) w_j cS sigmaS_j,  d_j = (i/4) w_j cD sigmaD_j
 __global__ void strengths_kernel(int64_t n, const double* __restrict__ w, cd cS,
@@ -28,145 +26,85 @@ __global__ void strengths_kernel(int64_t n, const double* __restrict__ w, cd cS,
   d[j] = sD ? cmul(i4, cmul(cD, sD[j])) : mk(0.0, 0.0);
 }
 
-// One thread per centre; sources streamed through shared memory.
-// With W_m = H_m(k r) e^{i m th} (th = arg(s - c)) and the complex normal
-// nu = n_x + i n_y, the double-layer kernel of order m is
-//   n . grad_s W_m = (k/2) (nu W_{m-1} - conj(nu) W_{m+1}),
-// from (d_x +- i d_y) [Z_m(kr) e^{i m th}] = -+ k Z_{m+-1}(kr) e^{i(m+-1) th}
-// (DLMF 10.6.2 in polar form). W_{-m} = (-1)^m H_m conj(e^{i m th}).
-template <int PM, bool HS, bool HD>
-__global__ void __launch_bounds__(kTile) p2qbxl_direct_kernel(
-    int64_t n_ctr, const double* __restrict__ ctr_xy, int64_t n_src,
+// alpha at the centres list[0..n) (every centre when list is NULL), SW warps per
+// centre and one centre per block: the lanes deal the sources round-robin, each
+// keeps 2p+1 partial coefficients (p2qbxl_pair), a reduce-scatter of shuffles
+// adds the lanes and, for SW > 1, the warps' sums are added in warp order
+// through shared memory (deterministic). FP64-pipe-bound; what matters besides
+// the instruction count is that every SM has a few warps: a thread per centre
+// (the form before) put the 1024 centres of a circle on 8 of the 152 SMs.
+// One-warp blocks even the load over the SMs to within one centre.
+template <int PM, bool HS, bool HD, int SW>
+__global__ void __launch_bounds__(32 * SW) p2qbxl_direct_kernel(
+    const int32_t* __restrict__ list, const double* __restrict__ ctr_xy, int64_t n_src,
     const double* __restrict__ src_xy, const double* __restrict__ src_nrm,
     const cd* __restrict__ qs, const cd* __restrict__ ds, double k, int p,
     cd* __restrict__ alpha) {
-  __shared__ double2 s_xy[kTile];
-  __shared__ double2 s_nu[kTile];
-  __shared__ cd s_q[kTile];
-  __shared__ cd s_d[kTile];
-  const int64_t c = blockIdx.x * (int64_t)kTile + threadIdx.x;
-  const bool active = c < n_ctr;
-  const double cx = active ? ctr_xy[2 * c] : 0.0;
-  const double cy = active ? ctr_xy[2 * c + 1] : 0.0;
-  const double hk = 0.5 * k;
-  cd acc[2 * PM + 1];
+  constexpr int NC = 2 * PM + 2;
+  const int64_t c = list ? (int64_t)list[blockIdx.x] : (int64_t)blockIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const double cx = ctr_xy[2 * c], cy = ctr_xy[2 * c + 1];
+  const double ik = 1.0 / k, hk = 0.5 * k;
+  cd acc[NC];
 #pragma unroll
-  for (int i = 0; i <= 2 * PM; ++i) acc[i] = mk(0.0, 0.0);
-
-  for (int64_t base = 0; base < n_src; base += kTile) {
-    const int64_t j = base + threadIdx.x;
-    if (j < n_src) {
-      s_xy[threadIdx.x] = make_double2(src_xy[2 * j], src_xy[2 * j + 1]);
-      if (HD) {
-        s_nu[threadIdx.x] = make_double2(src_nrm[2 * j], src_nrm[2 * j + 1]);
-        s_d[threadIdx.x] = ds[j];
-      }
-      if (HS) s_q[threadIdx.x] = qs[j];
+  for (int i = 0; i < NC; ++i) acc[i] = mk(0.0, 0.0);
+  for (int64_t j = threadIdx.x; j < n_src; j += 32 * SW) {
+    const cd z = mk(0.0, 0.0);
+    p2qbxl_pair<PM, HS, HD>(acc, src_xy[2 * j] - cx, src_xy[2 * j + 1] - cy, HS ? qs[j] : z,
+                            HD ? cscale(ds[j], hk) : z, HD ? src_nrm[2 * j] : 0.0,
+                            HD ? src_nrm[2 * j + 1] : 0.0, k, ik, p);
+  }
+  cd x32, x33;
+  warp_reduce_scatter<NC>(acc, lane, x32, x33);
+  cd v = acc[0];
+  if (SW > 1) {
+    __shared__ cd part[SW][34];
+    part[w][lane] = v;
+    if (lane == 0) {
+      part[w][32] = x32;
+      part[w][33] = x33;
     }
     __syncthreads();
-    const int cnt = (int)min((int64_t)kTile, n_src - base);
-    if (active) {
-      for (int jj = 0; jj < cnt; ++jj) {
-        const double dx = s_xy[jj].x - cx, dy = s_xy[jj].y - cy;
-        const double r = sqrt(dx * dx + dy * dy);
-        if (r == 0.0) continue;  // a source on a centre has no expansion (Condition 1)
-        const double ir = 1.0 / r, x = k * r, ix2 = 2.0 / x;
-        const cd e1 = mk(dx * ir, dy * ir);
-        cd h0, h1;
-        hankel01(x, h0, h1);
-        cd q = HS ? s_q[jj] : mk(0.0, 0.0);
-        cd dk = HD ? cscale(s_d[jj], hk) : mk(0.0, 0.0);
-        cd nu = HD ? mk(s_nu[jj].x, s_nu[jj].y) : mk(0.0, 0.0);
-        cd nub = cconj(nu);
-        // m = 0
-        cd w1 = cmul(h1, e1);              // W_1
-        cd wm1 = cscale(cmul(h1, cconj(e1)), -1.0);  // W_{-1} = -H_1 conj(e1)
-        if (HS) cfma(acc[PM], q, h0);
-        if (HD) cfma(acc[PM], dk, csub(cmul(nu, wm1), cmul(nub, w1)));
-        // running values: H_{m-1}, H_m, e^{i(m-1)th}, e^{i m th}
-        cd hprev = h0, hcur = h1, eprev = mk(1.0, 0.0), ecur = e1;
-        double sgn = -1.0;  // (-1)^m for m = 1
-#pragma unroll
-        for (int m = 1; m <= PM; ++m) {
-          if (m > p) break;
-          cd hnext = csub(cscale(hcur, (double)m * ix2), hprev);  // H_{m+1}
-          cd enext = cmul(ecur, e1);
-          cd w_m = cmul(hcur, ecur);
-          cd w_p = cmul(hnext, enext);
-          cd w_pm = cmul(hprev, eprev);
-          // negative orders: W_{-m} = (-1)^m H_m conj(e_m)
-          cd v_m = cscale(cmul(hcur, cconj(ecur)), sgn);
-          cd v_p = cscale(cmul(hnext, cconj(enext)), -sgn);   // W_{-(m+1)}
-          cd v_pm = cscale(cmul(hprev, cconj(eprev)), -sgn);  // W_{-(m-1)}
-          if (HS) {
-            cfma(acc[PM + m], q, w_m);
-            cfma(acc[PM - m], q, v_m);
-          }
-          if (HD) {
-            cfma(acc[PM + m], dk, csub(cmul(nu, w_pm), cmul(nub, w_p)));
-            cfma(acc[PM - m], dk, csub(cmul(nu, v_p), cmul(nub, v_pm)));
-          }
-          hprev = hcur;
-          hcur = hnext;
-          eprev = ecur;
-          ecur = enext;
-          sgn = -sgn;
-        }
-      }
+    if (w > 0) return;
+    x32 = part[0][32];
+    x33 = part[0][33];
+    for (int u = 1; u < SW; ++u) {
+      v = cadd(v, part[u][lane]);
+      x32 = cadd(x32, part[u][32]);
+      x33 = cadd(x33, part[u][33]);
     }
-    __syncthreads();
   }
-  if (active) {
-    const int P = 2 * p + 1;
-#pragma unroll
-    for (int l = -PM; l <= PM; ++l)
-      if (l >= -p && l <= p) alpha[c * P + (l + p)] = acc[PM + l];
-  }
+  cd* dst = alpha + c * (2 * p + 1) + p;
+  pair_coefficients<PM>(v, x32, x33, lane, p, [&](int l, cd a) { dst[l] = a; });
 }
 
-// Smooth quadrature: u(t) = sum_j q_j H_0(k r) + d_j k H_1(k r) n_j.(t - s_j)/r
+// Smooth quadrature: u(t) = sum_j q_j H_0(k r) + d_j k H_1(k r) n_j.(t - s_j)/r.
+// A warp per target, the lanes over the sources, a shuffle tree; one-warp blocks
+// for the same reason as above.
 template <bool HS, bool HD>
-__global__ void __launch_bounds__(kTile) p2p_direct_kernel(
-    int64_t n_list, const int32_t* __restrict__ list, const double* __restrict__ tgt_xy,
-    int64_t n_src, const double* __restrict__ src_xy, const double* __restrict__ src_nrm,
+__global__ void __launch_bounds__(32) p2p_direct_kernel(
+    const int32_t* __restrict__ list, const double* __restrict__ tgt_xy, int64_t n_src,
+    const double* __restrict__ src_xy, const double* __restrict__ src_nrm,
     const cd* __restrict__ qs, const cd* __restrict__ ds, double k, cd* __restrict__ out) {
-  __shared__ double2 s_xy[kTile];
-  __shared__ double2 s_n[kTile];
-  __shared__ cd s_q[kTile];
-  __shared__ cd s_d[kTile];
-  const int64_t i = blockIdx.x * (int64_t)kTile + threadIdx.x;
-  const bool active = i < n_list;
-  const int64_t t = active ? list[i] : 0;
-  const double tx = active ? tgt_xy[2 * t] : 0.0;
-  const double ty = active ? tgt_xy[2 * t + 1] : 0.0;
+  const int64_t t = list[blockIdx.x];
+  const double tx = tgt_xy[2 * t], ty = tgt_xy[2 * t + 1], ik = 1.0 / k;
   cd acc = mk(0.0, 0.0);
-  for (int64_t base = 0; base < n_src; base += kTile) {
-    const int64_t j = base + threadIdx.x;
-    if (j < n_src) {
-      s_xy[threadIdx.x] = make_double2(src_xy[2 * j], src_xy[2 * j + 1]);
-      if (HS) s_q[threadIdx.x] = qs[j];
-      if (HD) {
-        s_n[threadIdx.x] = make_double2(src_nrm[2 * j], src_nrm[2 * j + 1]);
-        s_d[threadIdx.x] = ds[j];
-      }
-    }
-    __syncthreads();
-    const int cnt = (int)min((int64_t)kTile, n_src - base);
-    if (active) {
-      for (int jj = 0; jj < cnt; ++jj) {
-        const double dx = tx - s_xy[jj].x, dy = ty - s_xy[jj].y;
-        const double r = sqrt(dx * dx + dy * dy);
-        if (r == 0.0) continue;
-        const double x = k * r;
-        cd h0, h1;
-        hankel01_any<false, HS, HD>(x, 1.0 / x, h0, h1);
-        if (HS) cfma(acc, s_q[jj], h0);
-        if (HD) cfma(acc, s_d[jj], cscale(h1, k * (s_n[jj].x * dx + s_n[jj].y * dy) / r));
-      }
-    }
-    __syncthreads();
+  for (int64_t j = threadIdx.x; j < n_src; j += 32) {
+    const double dx = tx - src_xy[2 * j], dy = ty - src_xy[2 * j + 1];
+    const double r2 = dx * dx + dy * dy;
+    if (r2 == 0.0) continue;
+    const double ir = rsqrt(r2), x = k * (r2 * ir);
+    cd h0, h1;
+    hankel01_any<false, HS, HD>(x, ik * ir, h0, h1);
+    if (HS) cfma(acc, qs[j], h0);
+    if (HD) cfma(acc, ds[j], cscale(h1, k * (src_nrm[2 * j] * dx + src_nrm[2 * j + 1] * dy) * ir));
   }
-  if (active) out[t] = acc;
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+  }
+  if (threadIdx.x == 0) out[t] = acc;
 }
 
 // u(t) = sum_{|l| <= p} alpha_l(c) J_l(k rho) e^{-i l theta}, (rho, theta) the
@@ -292,21 +230,43 @@ __global__ void place_centres_kernel(int64_t n, int q, int sides, const double* 
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
-template <int PM>
-void p2qbxl_dispatch_flags(qbx_handle* h, bool S, bool D, cudaStream_t s) {
-  dim3 g(nblk(h->n_ctr, kTile));
-  if (S && D)
-    p2qbxl_direct_kernel<PM, true, true><<<g, kTile, 0, s>>>(
-        h->n_ctr, h->ctr_xy.ptr, h->n_src, h->src_xy.ptr, h->src_nrm.ptr, h->q_str.ptr,
-        h->d_str.ptr, h->k, h->p, h->alpha.ptr);
-  else if (S)
-    p2qbxl_direct_kernel<PM, true, false><<<g, kTile, 0, s>>>(
-        h->n_ctr, h->ctr_xy.ptr, h->n_src, h->src_xy.ptr, h->src_nrm.ptr, h->q_str.ptr,
-        h->d_str.ptr, h->k, h->p, h->alpha.ptr);
+// Warps per centre: one while the centres alone give every SM kWarpsPerSm warps
+// (enough to keep the FP64 pipe busy), else four, as long as that leaves every
+// lane a source.
+constexpr int64_t kWarpsPerSm = 6;
+
+template <int PM, bool HS, bool HD>
+void p2qbxl_direct_launch(int64_t n, const int32_t* list, const double* cxy, int64_t n_src,
+                          const double* sxy, const double* snrm, const cd* q, const cd* d,
+                          double k, int p, cd* alpha, cudaStream_t s) {
+  if (n >= 152 * kWarpsPerSm || n_src < 128)
+    p2qbxl_direct_kernel<PM, HS, HD, 1><<<(unsigned)n, 32, 0, s>>>(list, cxy, n_src, sxy, snrm, q,
+                                                                   d, k, p, alpha);
   else
-    p2qbxl_direct_kernel<PM, false, true><<<g, kTile, 0, s>>>(
-        h->n_ctr, h->ctr_xy.ptr, h->n_src, h->src_xy.ptr, h->src_nrm.ptr, h->q_str.ptr,
-        h->d_str.ptr, h->k, h->p, h->alpha.ptr);
+    p2qbxl_direct_kernel<PM, HS, HD, 4><<<(unsigned)n, 128, 0, s>>>(list, cxy, n_src, sxy, snrm, q,
+                                                                    d, k, p, alpha);
+}
+
+// alpha at n centres (list, or 0..n-1 when it is NULL) from every source
+template <int PM>
+void p2qbxl_direct_flags(int64_t n, const int32_t* list, const double* cxy, int64_t n_src,
+                         const double* sxy, const double* snrm, const cd* q, const cd* d, bool S,
+                         bool D, double k, int p, cd* alpha, cudaStream_t s) {
+  if (S && D)
+    p2qbxl_direct_launch<PM, true, true>(n, list, cxy, n_src, sxy, snrm, q, d, k, p, alpha, s);
+  else if (S)
+    p2qbxl_direct_launch<PM, true, false>(n, list, cxy, n_src, sxy, snrm, q, d, k, p, alpha, s);
+  else
+    p2qbxl_direct_launch<PM, false, true>(n, list, cxy, n_src, sxy, snrm, q, d, k, p, alpha, s);
+}
+
+void p2qbxl_direct(int64_t n, const int32_t* list, const double* cxy, int64_t n_src,
+                   const double* sxy, const double* snrm, const cd* q, const cd* d, bool S, bool D,
+                   double k, int p, cd* alpha, cudaStream_t s) {
+  if (p <= 4) p2qbxl_direct_flags<4>(n, list, cxy, n_src, sxy, snrm, q, d, S, D, k, p, alpha, s);
+  else if (p <= 8) p2qbxl_direct_flags<8>(n, list, cxy, n_src, sxy, snrm, q, d, S, D, k, p, alpha, s);
+  else if (p <= 12) p2qbxl_direct_flags<12>(n, list, cxy, n_src, sxy, snrm, q, d, S, D, k, p, alpha, s);
+  else p2qbxl_direct_flags<16>(n, list, cxy, n_src, sxy, snrm, q, d, S, D, k, p, alpha, s);
 }
 
 }  // namespace
@@ -321,44 +281,36 @@ qbx_status launch_strengths(qbx_handle* h, cd cS, const cd* sigS, cd cD, const c
   return QBX_OK;
 }
 
-qbx_status launch_p2qbxl_direct(qbx_handle* h, bool S, bool D, int precision, cudaStream_t s) {
-  (void)precision;
+qbx_status launch_p2qbxl_direct(qbx_handle* h, bool S, bool D, bool all_centres, cudaStream_t s) {
   if (h->n_ctr == 0) return QBX_OK;
   if (!S && !D) {
     QBX_CUDA_TRY(cudaMemsetAsync(h->alpha.ptr, 0, h->alpha.n * sizeof(cd), s));
     return QBX_OK;
   }
-  if (h->p <= 4) p2qbxl_dispatch_flags<4>(h, S, D, s);
-  else if (h->p <= 8) p2qbxl_dispatch_flags<8>(h, S, D, s);
-  else if (h->p <= 12) p2qbxl_dispatch_flags<12>(h, S, D, s);
-  else p2qbxl_dispatch_flags<16>(h, S, D, s);
+  // every centre when the caller reads the coefficients, else those that some
+  // target is associated with (the only ones QBXL2P reads), as in FMM mode
+  const int64_t n = all_centres ? h->n_ctr : h->n_used_ctr;
+  if (n == 0) return QBX_OK;
+  p2qbxl_direct(n, all_centres ? nullptr : h->used_ctr.ptr, h->ctr_xy.ptr, h->n_src,
+                h->src_xy.ptr, h->src_nrm.ptr, h->q_str.ptr, h->d_str.ptr, S, D, h->k, h->p,
+                h->alpha.ptr, s);
   QBX_CUDA_TRY(cudaGetLastError());
   h->launches += 1;
   return QBX_OK;
 }
 
-qbx_status launch_p2p_direct(qbx_handle* h, bool S, bool D, cd* out, int precision,
-                             cudaStream_t s) {
-  (void)precision;
+qbx_status launch_p2p_direct(qbx_handle* h, bool S, bool D, cd* out, cudaStream_t s) {
   const int64_t n = h->n_direct_tgt;
   if (n == 0) return QBX_OK;
-  dim3 g(nblk(n, kTile));
-  if (S && D)
-    p2p_direct_kernel<true, true><<<g, kTile, 0, s>>>(n, h->direct_tgt_list.ptr, h->tgt_xy.ptr,
-                                                      h->n_src, h->src_xy.ptr, h->src_nrm.ptr,
-                                                      h->q_str.ptr, h->d_str.ptr, h->k, out);
-  else if (S)
-    p2p_direct_kernel<true, false><<<g, kTile, 0, s>>>(n, h->direct_tgt_list.ptr, h->tgt_xy.ptr,
-                                                       h->n_src, h->src_xy.ptr, h->src_nrm.ptr,
-                                                       h->q_str.ptr, h->d_str.ptr, h->k, out);
-  else if (D)
-    p2p_direct_kernel<false, true><<<g, kTile, 0, s>>>(n, h->direct_tgt_list.ptr, h->tgt_xy.ptr,
-                                                       h->n_src, h->src_xy.ptr, h->src_nrm.ptr,
-                                                       h->q_str.ptr, h->d_str.ptr, h->k, out);
-  else
-    p2p_direct_kernel<false, false><<<g, kTile, 0, s>>>(n, h->direct_tgt_list.ptr, h->tgt_xy.ptr,
-                                                        h->n_src, h->src_xy.ptr, h->src_nrm.ptr,
-                                                        h->q_str.ptr, h->d_str.ptr, h->k, out);
+#define P2P_DIRECT_LAUNCH(HS, HD)                                                              \
+  p2p_direct_kernel<HS, HD><<<(unsigned)n, 32, 0, s>>>(                                        \
+      h->direct_tgt_list.ptr, h->tgt_xy.ptr, h->n_src, h->src_xy.ptr, h->src_nrm.ptr,          \
+      h->q_str.ptr, h->d_str.ptr, h->k, out)
+  if (S && D) P2P_DIRECT_LAUNCH(true, true);
+  else if (S) P2P_DIRECT_LAUNCH(true, false);
+  else if (D) P2P_DIRECT_LAUNCH(false, true);
+  else P2P_DIRECT_LAUNCH(false, false);
+#undef P2P_DIRECT_LAUNCH
   QBX_CUDA_TRY(cudaGetLastError());
   h->launches += 1;
   return QBX_OK;
@@ -470,28 +422,6 @@ bool on_device(const void* p, int dev) {
   return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == dev;
 }
 
-template <int PM>
-void noalloc_launch(int64_t n_src, const double* sxy, const double* snrm, const cd* q,
-                    const cd* d, bool S, bool D, double k, int64_t n_ctr, const double* cxy,
-                    int p, cd* alpha, int64_t n_tgt, const double* txy, const int32_t* tc,
-                    cd* out, cudaStream_t s) {
-  if (n_ctr > 0) {
-    dim3 g(nblk(n_ctr, kTile));
-    if (S && D)
-      p2qbxl_direct_kernel<PM, true, true><<<g, kTile, 0, s>>>(n_ctr, cxy, n_src, sxy, snrm, q,
-                                                               d, k, p, alpha);
-    else if (S)
-      p2qbxl_direct_kernel<PM, true, false><<<g, kTile, 0, s>>>(n_ctr, cxy, n_src, sxy, snrm, q,
-                                                                d, k, p, alpha);
-    else
-      p2qbxl_direct_kernel<PM, false, true><<<g, kTile, 0, s>>>(n_ctr, cxy, n_src, sxy, snrm, q,
-                                                                d, k, p, alpha);
-  }
-  if (n_tgt > 0)
-    qbxl2p_each_kernel<PM><<<nblk(n_tgt, 128), 128, 0, s>>>(n_tgt, txy, tc, n_ctr, cxy, alpha, k,
-                                                            p, out);
-}
-
 }  // namespace
 
 extern "C" qbx_status qbx_direct_qbx_eval_noalloc(
@@ -559,22 +489,21 @@ extern "C" qbx_status qbx_direct_qbx_eval_noalloc(
     strengths_kernel<<<nblk(n_src, 256), 256, 0, s>>>(
         n_src, src_weight, mk(cS_re, cS_im), (const cd*)sigma_S, mk(cD_re, cD_im),
         (const cd*)sigma_D, q, d);
-  const bool S = sigma_S != nullptr, D = sigma_D != nullptr;
-  const cd* cq = q;
-  const cd* cdd = d;
-  cd* o = (cd*)out;
-  if (p <= 4)
-    noalloc_launch<4>(n_src, src_xy, src_normal_xy, cq, cdd, S, D, k, n_ctr, ctr_xy, p, alpha,
-                      n_tgt, tgt_xy, tgt_centre, o, s);
-  else if (p <= 8)
-    noalloc_launch<8>(n_src, src_xy, src_normal_xy, cq, cdd, S, D, k, n_ctr, ctr_xy, p, alpha,
-                      n_tgt, tgt_xy, tgt_centre, o, s);
-  else if (p <= 12)
-    noalloc_launch<12>(n_src, src_xy, src_normal_xy, cq, cdd, S, D, k, n_ctr, ctr_xy, p, alpha,
-                       n_tgt, tgt_xy, tgt_centre, o, s);
-  else
-    noalloc_launch<16>(n_src, src_xy, src_normal_xy, cq, cdd, S, D, k, n_ctr, ctr_xy, p, alpha,
-                       n_tgt, tgt_xy, tgt_centre, o, s);
+  if (n_ctr > 0)
+    p2qbxl_direct(n_ctr, nullptr, ctr_xy, n_src, src_xy, src_normal_xy, q, d, sigma_S != nullptr,
+                  sigma_D != nullptr, k, p, alpha, s);
+  if (n_tgt > 0) {
+    const unsigned g = nblk(n_tgt, 128);
+    cd* o = (cd*)out;
+    if (p <= 4)
+      qbxl2p_each_kernel<4><<<g, 128, 0, s>>>(n_tgt, tgt_xy, tgt_centre, n_ctr, ctr_xy, alpha, k, p, o);
+    else if (p <= 8)
+      qbxl2p_each_kernel<8><<<g, 128, 0, s>>>(n_tgt, tgt_xy, tgt_centre, n_ctr, ctr_xy, alpha, k, p, o);
+    else if (p <= 12)
+      qbxl2p_each_kernel<12><<<g, 128, 0, s>>>(n_tgt, tgt_xy, tgt_centre, n_ctr, ctr_xy, alpha, k, p, o);
+    else
+      qbxl2p_each_kernel<16><<<g, 128, 0, s>>>(n_tgt, tgt_xy, tgt_centre, n_ctr, ctr_xy, alpha, k, p, o);
+  }
   QBX_CUDA_TRY(cudaGetLastError());
   return QBX_OK;
 }

@@ -27,7 +27,7 @@
 #include <set>
 #include <vector>
 
-#include "special.cuh"
+#include "p2qbxl_pair.cuh"
 #include "tree.cuh"
 
 namespace {
@@ -861,77 +861,6 @@ __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
 }
 
 
-// One source's contribution to the QBX coefficients of a centre (P2QBXL):
-// alpha_l += q W_l + d (k/2) (nu W_{l-1} - conj(nu) W_{l+1}),  W_l = H_l(k r) e^{i l th},
-// (r, th) the polar coordinates of source - centre; upward Hankel recurrence.
-template <int PM, bool HS, bool HD>
-__device__ __forceinline__ void p2qbxl_pair(cd (&acc)[2 * PM + 1], double dx, double dy, cd q,
-                                            cd A, cd B, double k, double ik, int p) {
-  // A = d (k/2) nu, B = d (k/2) conj(nu): alpha_l += q W_l + A W_{l-1} - B W_{l+1}.
-  // W_m and W_{-m} are kept in sliding windows so each is formed once. One
-  // reciprocal square root gives r, 1/r and 1/x (ik = 1/k): no division.
-  const double r2 = dx * dx + dy * dy;
-  if (r2 == 0.0) return;
-  const double ir = rsqrt(r2), rr = r2 * ir, x = k * rr, ix = ik * ir, ix2 = 2.0 * ix;
-  const cd e1 = mk(dx * ir, dy * ir);
-  cd h0, h1;
-  hankel01(x, ix, h0, h1);
-  const cd w1 = cmul(h1, e1);
-  const cd wm1 = cscale(cmul(h1, cconj(e1)), -1.0);
-  if (HS) cfma(acc[PM], q, h0);
-  if (HD) {
-    cfma(acc[PM], A, wm1);
-    cfma(acc[PM], mk(-B.x, -B.y), w1);
-  }
-  cd hprev = h0, hcur = h1, ecur = e1;
-  cd wp_prev = h0, wp_cur = w1;   // W_{m-1}, W_m
-  cd wn_prev = h0, wn_cur = wm1;  // W_{-(m-1)}, W_{-m}
-  const cd mB = mk(-B.x, -B.y);
-  // H_{m+1} = (2m/x) H_m - H_{m-1} (two FMAs per component; 2m/x = dm ix2 with
-  // dm counted exactly); W_{m+1} = H_{m+1} e^{i(m+1)th} and
-  // W_{-(m+1)} = (-1)^{m+1} H_{m+1} e^{-i(m+1)th} from the same four products
-  double dm = 0.0;
-  auto step = [&](int m, cd& hnext, cd& enext, cd& wp, cd& wn) {
-    dm += 1.0;
-    const double cm = dm * ix2;
-    hnext = mk(fma(cm, hcur.x, -hprev.x), fma(cm, hcur.y, -hprev.y));
-    enext = cmul(ecur, e1);
-    const double rr_ = hnext.x * enext.x, ii_ = hnext.y * enext.y;
-    const double ri_ = hnext.x * enext.y, ir_ = hnext.y * enext.x;
-    wp = mk(rr_ - ii_, ri_ + ir_);
-    wn = (m & 1) ? mk(rr_ + ii_, ir_ - ri_) : mk(-(rr_ + ii_), ri_ - ir_);
-  };
-#pragma unroll
-  for (int m = 1; m <= PM; ++m) {
-    if (m > p) break;
-    if (HS) {
-      cfma(acc[PM + m], q, wp_cur);
-      cfma(acc[PM - m], q, wn_cur);
-    }
-    if (HD) {
-      cd hnext, enext, wp_next, wn_next;
-      step(m, hnext, enext, wp_next, wn_next);
-      cfma(acc[PM + m], A, wp_prev);
-      cfma(acc[PM + m], mB, wp_next);
-      cfma(acc[PM - m], A, wn_next);
-      cfma(acc[PM - m], mB, wn_prev);
-      hprev = hcur;
-      hcur = hnext;
-      ecur = enext;
-      wp_prev = wp_cur;
-      wp_cur = wp_next;
-      wn_prev = wn_cur;
-      wn_cur = wn_next;
-    } else if (m < p) {
-      cd hnext, enext;
-      step(m, hnext, enext, wp_cur, wn_cur);
-      hprev = hcur;
-      hcur = hnext;
-      ecur = enext;
-    }
-  }
-}
-
 // M2QBXL: alpha_l += (-1)^l sum_n mh_n Wh_{n+l} s^{|n| - |n+l|},  Wh_m = s^|m| W_m(z - m_c),
 // for the (centre, W-list box) pairs whose box is far enough from the centre's
 // disk for the multipole series to converge on it ((R_c + r_z) <= kW |z - m_c|;
@@ -1699,11 +1628,45 @@ qbx_status configure_kernels() {
 // ---------------------------------------------------------------- P2QBXL, one warp per centre
 // Lanes stride over the concatenated sources of the centre's U-list boxes (so
 // the load is balanced to within one source), each lane keeps partial
-// coefficients, and a reduce-scatter of shuffles adds them: after it, lane L
-// holds coefficient indices K L .. K L + K - 1 of the 32 K padded ones
-// (K = 1 for p <= 15, 2 for p = 16). Padding indices hold zeros.
+// coefficients (p2qbxl_pair), and a reduce-scatter of shuffles adds them.
+template <int PM, bool HS, bool HD>
+__global__ void __launch_bounds__(kThreads) p2qbxl_warp_kernel(Fmm F, const int* __restrict__ cleaf,
+                                                               const int* __restrict__ wdoff,
+                                                               const int* __restrict__ wdbox,
+                                                               const int* __restrict__ clist,
+                                                               int n_ctr, cd* __restrict__ alpha) {
+  constexpr int NC = 2 * PM + 2;
+  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // position in clist
+  const int lane = threadIdx.x & 31;
+  if (w >= n_ctr) return;  // whole warps leave together
+  const int i = clist[w];  // sorted centre
+  const int b = cleaf[i];
+  const double k = F.k, ik = F.ik, hk = 0.5 * k;
+  const int p = F.p;
+  const double2 c = F.cxy[i];
+  cd acc[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) acc[j] = mk(0.0, 0.0);
+  auto one = [&](int j) {
+    const double2 y = F.sxy[j];
+    const double2 nv = HD ? F.snrm[j] : make_double2(0.0, 0.0);
+    const cd z = mk(0.0, 0.0);
+    p2qbxl_pair<PM, HS, HD>(acc, y.x - c.x, y.y - c.y, HS ? F.qs[j] : z,
+                            HD ? cscale(F.ds[j], hk) : z, nv.x, nv.y, k, ik, p);
+  };
+  // U-list boxes of the leaf, then the W-list boxes summed directly for this centre
+  const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], wdoff[i],
+                        wdoff[i + 1] - wdoff[i], wdbox};
+  deal_sources(sc, lane, one);
+  cd x32, x33;
+  warp_reduce_scatter<NC>(acc, lane, x32, x33);
+  cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
+  pair_coefficients<PM>(acc[0], x32, x33, lane, p,
+                        [&](int l, cd a) { dst[l] = cadd(dst[l], a); });
+}
+
 template <int NC>
-__device__ __forceinline__ void warp_reduce_scatter(cd (&acc)[NC], int lane) {
+__device__ __forceinline__ void warp_reduce_scatter_idx(cd (&acc)[NC], int lane) {
   constexpr int NP = 32 * ((NC + 31) / 32);
 #pragma unroll
   for (int h = NP / 2, off = 16; off >= 1; h >>= 1, off >>= 1) {
@@ -1718,48 +1681,6 @@ __device__ __forceinline__ void warp_reduce_scatter(cd (&acc)[NC], int lane) {
       keep.y += __shfl_xor_sync(0xffffffffu, send.y, off);
       if (i < NC) acc[i] = keep;
     }
-  }
-}
-
-template <int PM, bool HS, bool HD>
-__global__ void __launch_bounds__(kThreads) p2qbxl_warp_kernel(Fmm F, const int* __restrict__ cleaf,
-                                                               const int* __restrict__ wdoff,
-                                                               const int* __restrict__ wdbox,
-                                                               const int* __restrict__ clist,
-                                                               int n_ctr, cd* __restrict__ alpha) {
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // position in clist  // sorted centre
-  const int lane = threadIdx.x & 31;
-  if (w >= n_ctr) return;  // whole warps leave together
-  const int i = clist[w];  // sorted centre
-  const int b = cleaf[i];
-  const double k = F.k, ik = 1.0 / k;
-  const int p = F.p, P = 2 * p + 1;
-  const double2 c = F.cxy[i];
-  cd acc[2 * PM + 1];
-#pragma unroll
-  for (int j = 0; j <= 2 * PM; ++j) acc[j] = mk(0.0, 0.0);
-  auto one = [&](int j) {
-    const double2 y = F.sxy[j];
-    cd A = mk(0.0, 0.0), B = mk(0.0, 0.0);
-    if (HD) {
-      const cd dk = cscale(F.ds[j], 0.5 * k);
-      const cd nu = mk(F.snrm[j].x, F.snrm[j].y);
-      A = cmul(dk, nu);
-      B = cmul(dk, cconj(nu));
-    }
-    p2qbxl_pair<PM, HS, HD>(acc, y.x - c.x, y.y - c.y, HS ? F.qs[j] : mk(0.0, 0.0), A, B, k, ik, p);
-  };
-  // U-list boxes of the leaf, then the W-list boxes summed directly for this centre
-  const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], wdoff[i],
-                        wdoff[i + 1] - wdoff[i], wdbox};
-  deal_sources(sc, lane, one);
-  warp_reduce_scatter<2 * PM + 1>(acc, lane);
-  constexpr int K = (2 * PM + 1 + 31) / 32;
-  cd* dst = alpha + (size_t)F.cid[i] * P;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    const int lo = K * lane + j - PM;
-    if (lo >= -p && lo <= p) dst[lo + p] = cadd(dst[lo + p], acc[j]);
   }
 }
 
@@ -1804,7 +1725,7 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
 #pragma unroll
   for (int j = 0; j <= 2 * PM; ++j)
     acc[j] = mk((double)S[j].x - (double)C[j].x, (double)S[j].y - (double)C[j].y);
-  warp_reduce_scatter<2 * PM + 1>(acc, lane);
+  warp_reduce_scatter_idx<2 * PM + 1>(acc, lane);
   constexpr int K = (2 * PM + 1 + 31) / 32;
   cd* dst = alpha + (size_t)F.cid[i] * P;
 #pragma unroll

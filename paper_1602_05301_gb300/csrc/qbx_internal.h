@@ -104,6 +104,9 @@ struct qbx_handle {
   DevBuf<double> tgt_xy;
   DevBuf<int32_t> assoc;                    // [n_tgt] centre or -1
   DevBuf<int32_t> qbx_tgt_list, direct_tgt_list;
+  // direct mode: the centres some target is associated with, ascending
+  int64_t n_used_ctr = 0;
+  DevBuf<int32_t> used_ctr;
   // on-surface targets that ask for the on-surface value (side 0): the mean of
   // the two one-sided QBX limits, from the node's exterior centre (assoc) and
   // its interior centre (assoc + n_nodes)
@@ -130,10 +133,9 @@ struct qbx_handle {
 // direct.cu
 qbx_status launch_strengths(qbx_handle* h, cd cS, const cd* sigS, cd cD, const cd* sigD,
                             cudaStream_t s);
-qbx_status launch_p2qbxl_direct(qbx_handle* h, bool has_S, bool has_D, int precision,
+qbx_status launch_p2qbxl_direct(qbx_handle* h, bool has_S, bool has_D, bool all_centres,
                                 cudaStream_t s);
-qbx_status launch_p2p_direct(qbx_handle* h, bool has_S, bool has_D, cd* out, int precision,
-                             cudaStream_t s);
+qbx_status launch_p2p_direct(qbx_handle* h, bool has_S, bool has_D, cd* out, cudaStream_t s);
 qbx_status launch_qbxl2p(qbx_handle* h, cd* out, cudaStream_t s);
 qbx_status launch_associate_direct(qbx_handle* h, const int64_t* on_node, const int8_t* on_side,
                                    double eps, cudaStream_t s);
