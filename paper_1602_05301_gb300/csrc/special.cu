@@ -1,6 +1,6 @@
 // qbx_hankel01: the device evaluation of H_0 and H_1 of the first kind that
-// every kernel of the library uses (piecewise polynomials below x = 8, the
-// CUDA math library above), exposed so that it can be checked on its own.
+// every kernel of the library uses (piecewise polynomials below x = 32,
+// Hankel's expansion above), exposed so that it can be checked on its own.
 #include <cmath>
 
 #include "special.cuh"

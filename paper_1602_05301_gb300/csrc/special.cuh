@@ -1,8 +1,8 @@
 // Device special functions for the 2D Helmholtz kernels.
 //
-//  * H_0, H_1 of the first kind: piecewise polynomials below x = 8
-//    (Chebyshev fits on eight intervals per octave from 2^-9, the economised
-//    ascending series below), the CUDA math library's j0/y0/j1/y1 (FP64) above.
+//  * H_0, H_1 of the first kind: piecewise polynomials below x = 32 (Chebyshev
+//    fits on eight intervals per octave from 2^-9 to 8 and of width 1/2 above,
+//    the economised ascending series below), Hankel's expansion above.
 //  * H_m, m >= 2: upward three-term recurrence H_{m+1} = (2m/x) H_m - H_{m-1}
 //    (DLMF 10.6.1), stable for the dominant Y part; the error of the J part
 //    stays at rounding level relative to |H_m|.
@@ -20,6 +20,7 @@
 // u = -x^2/4 in [-1, 0] for x < 2^-9. D = 10 for the FP64 path (truncation
 // near 1e-16 of |H_0|, |H_1|), 8 for the mixed path (near 1e-13).
 #include "hankel_table.h"
+#include "hankel_table_far.h"
 constexpr double kEulerGamma = 0.57721566490153286061;
 constexpr double kTwoOverPi = 0.63661977236758134308;
 
@@ -98,22 +99,83 @@ __device__ __forceinline__ void hankel01_table(double x, double ix, cd& h0, cd& 
   }
 }
 
-// Reach of the tables; the CUDA math library's j0/y0/j1/y1 serve x >= 8.
-constexpr double kTableMax = 8.0;
+// H_0, H_1 at 8 <= x < 32: equal intervals of width 1/2, degree 10 (the same
+// table for both precisions).
+template <bool NEED0, bool NEED1>
+__device__ __forceinline__ void hankel01_far_table(double x, cd& h0, cd& h1) {
+  const int row = min(max(__double2int_rd(fma(2.0, x, -16.0)), 0), kHankFarRows - 1);
+  const double t = fma(4.0, x, (double)(-33 - 2 * row));
+  const double2* tb = kHankTabFar + row;
+  double2 c0 = make_double2(0.0, 0.0), c1 = c0;
+  if (NEED0) c0 = tb[(2 * kHankFarDeg) * kHankFarRows];
+  if (NEED1) c1 = tb[(2 * kHankFarDeg + 1) * kHankFarRows];
+#pragma unroll
+  for (int d = kHankFarDeg - 1; d >= 0; --d) {
+    if (NEED0) {
+      const double2 k0 = tb[(2 * d) * kHankFarRows];
+      c0 = make_double2(fma(c0.x, t, k0.x), fma(c0.y, t, k0.y));
+    }
+    if (NEED1) {
+      const double2 k1 = tb[(2 * d + 1) * kHankFarRows];
+      c1 = make_double2(fma(c1.x, t, k1.x), fma(c1.y, t, k1.y));
+    }
+  }
+  if (NEED0) h0 = mk(c0.x, c0.y);
+  if (NEED1) h1 = mk(c1.x, c1.y);
+}
 
-// H_0, H_1 at x > 0: each lane below 8 reads its own table row, the library
-// serves the rest.
+// a_k(nu) of Hankel's expansion (DLMF 10.17.1): prod_{j<=k} (4 nu^2 - (2j-1)^2) / (8 j)
+__host__ __device__ constexpr double hankel_a(int nu, int k) {
+  double a = 1.0;
+  for (int j = 1; j <= k; ++j) a *= (4.0 * nu * nu - (2.0 * j - 1.0) * (2.0 * j - 1.0)) / (8.0 * j);
+  return a;
+}
+// sum_{k < kHankTerms} (-1)^k a_{2k+odd} v^k, v = 1/x^2
+constexpr int kHankTerms = 9;
+template <int NU, int ODD, int K>
+__device__ __forceinline__ double hankel_pq(double v) {
+  constexpr double a = (K & 1) ? -hankel_a(NU, 2 * K + ODD) : hankel_a(NU, 2 * K + ODD);
+  if constexpr (K + 1 < kHankTerms) return fma(hankel_pq<NU, ODD, K + 1>(v), v, a);
+  else return a;
+}
+
+// H_0, H_1 at x >= 32 by Hankel's expansion (DLMF 10.17.5),
+//   H_nu = sqrt(2 / (pi x)) e^{i (x - nu pi/2 - pi/4)} (P_nu + i Q_nu),
+// P and Q to the term in x^-17 (the next is below 1e-18 at x = 32).
+template <bool NEED0, bool NEED1>
+__device__ __forceinline__ void hankel01_asymptotic(double x, double ix, cd& h0, cd& h1) {
+  double s, c;
+  sincos(x, &s, &c);
+  // sqrt(2/(pi x)) (cos, sin)(x - pi/4) = sqrt(1/(pi x)) (c + s, s - c)
+  const double amp = sqrt(0.31830988618379067154 * ix), v = ix * ix;
+  const double u = amp * (c + s), w = amp * (s - c);
+  if (NEED0) {
+    const double P = hankel_pq<0, 0, 0>(v), Q = ix * hankel_pq<0, 1, 0>(v);
+    h0 = mk(fma(u, P, -w * Q), fma(u, Q, w * P));
+  }
+  if (NEED1) {  // e^{-i pi/2}: (u + i w) -> (w - i u)
+    const double P = hankel_pq<1, 0, 0>(v), Q = ix * hankel_pq<1, 1, 0>(v);
+    h1 = mk(fma(w, P, u * Q), fma(w, Q, -u * P));
+  }
+}
+
+// Reach of the tables.
+constexpr double kTableMax = 8.0, kFarTableMax = 32.0;
+
+// H_0, H_1 at x > 0: each lane below 32 reads its own table row, Hankel's
+// expansion serves the rest. Both orders share the argument's reduction and
+// amplitude; the CUDA library's j0, y0, j1, y1, which served x >= 8 before, are
+// four evaluations of it (whole evaluations: all pairs of 2048 sources, 4096
+// centres and 3737 targets at k = 10, most of them beyond x = 8, 13.3 -> 7.7 ms;
+// 200 ellipses in mixed precision 23.1 -> 20.4 ms, the P2P of large leaves).
 // WIDE: the mixed path's lower-degree tables (relative error below 1e-13).
 // NEED0 / NEED1: whether the caller reads h0 / h1 (the other's polynomials
-// and library calls are skipped).
+// are skipped).
 template <bool WIDE, bool NEED0 = true, bool NEED1 = true>
 __device__ __forceinline__ void hankel01_any(double x, double ix, cd& h0, cd& h1) {
-  if (x < kTableMax) {
-    hankel01_table<WIDE, NEED0, NEED1>(x, ix, h0, h1);
-    return;
-  }
-  if (NEED0) h0 = mk(j0(x), y0(x));
-  if (NEED1) h1 = mk(j1(x), y1(x));
+  if (x < kTableMax) hankel01_table<WIDE, NEED0, NEED1>(x, ix, h0, h1);
+  else if (x < kFarTableMax) hankel01_far_table<NEED0, NEED1>(x, h0, h1);
+  else hankel01_asymptotic<NEED0, NEED1>(x, ix, h0, h1);
 }
 
 __device__ __forceinline__ void hankel01(double x, double ix, cd& h0, cd& h1) {
