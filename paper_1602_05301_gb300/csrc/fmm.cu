@@ -27,6 +27,7 @@
 #include <set>
 #include <vector>
 
+#include "ff.cuh"
 #include "p2qbxl_pair.cuh"
 #include "tree.cuh"
 
@@ -76,6 +77,7 @@ struct Fmm {
   const cd* ds;
   const float2* q32;     // FP32 charges (mixed path)
   const float4* ab32;    // FP32 dipole factors (A, B) (mixed path)
+  const float4* dn32;    // FP32 (d k/2, nu) (mixed path)
   const double2* cxy;
   const double* crad;    // sorted centre radii
   const int* cid;
@@ -240,7 +242,8 @@ __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
                                         const cd* __restrict__ q, const cd* __restrict__ d,
                                         const double2* __restrict__ snrm, double k,
                                         cd* __restrict__ qs, cd* __restrict__ ds,
-                                        float2* __restrict__ q32, float4* __restrict__ ab32) {
+                                        float2* __restrict__ q32, float4* __restrict__ ab32,
+                                        float4* __restrict__ dn32) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const cd qi = q[perm[i]], di = d[perm[i]];
@@ -252,6 +255,7 @@ __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
     const cd A = cmul(dk, nu), B = cmul(dk, cconj(nu));
     q32[i] = make_float2((float)qi.x, (float)qi.y);
     ab32[i] = make_float4((float)A.x, (float)A.y, (float)B.x, (float)B.y);
+    dn32[i] = make_float4((float)dk.x, (float)dk.y, (float)nu.x, (float)nu.y);
   }
 }
 
@@ -987,11 +991,13 @@ __global__ void m2qbxl_sum_kernel(int n, int P, const int* __restrict__ cpo,
 }
 
 // ---------------------------------------------------------------- mixed precision P2QBXL
-// H_0, H_1 and the Hankel recurrence stay FP64; the terms sigma^|l| W_l
-// (sigma = 2^s near rho = k r_c, which keeps them of moderate size) are
+// H_0, H_1 and the Hankel recurrence in float-float (ff.cuh); the terms are
 // rounded to FP32, multiplied by the FP32 strengths and added with Kahan
-// compensation into ah_l = alpha_l sigma^|l|; alpha_l = ah_l sigma^-|l| is
-// formed in FP64 at the end.
+// compensation; the lanes' sums are added and unscaled in FP64 at the end.
+// With the recurrence in FP64 the kernel was bound by the FP64 pipe (82 % of
+// its rate, 95 FP64 instructions per pair); now two FP64 subtractions per pair
+// are left and FP32 issue bounds it: 104 459 centres of 200 ellipses, p = 16, 5.83
+// -> 3.45 ms; 32 curves as a batch, p = 12, both layers, 14.0 -> 10.0 ms in all.
 __device__ __forceinline__ void kahan2(float2& s, float2& c, float2 v) {
   float y = v.x - c.x, t = s.x + y;
   c.x = (t - s.x) - y;
@@ -1007,84 +1013,127 @@ __device__ __forceinline__ float2 fmul(float2 a, float2 b) {
 __device__ __forceinline__ float2 fsub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 f2(cd a) { return make_float2(f32_from_f64(a.x), f32_from_f64(a.y)); }
 
+// Lengths in the float-float kernels are in units of 2^-sh (sh = floor(log2 k)), so
+// that the wavenumber is kk in [1, 2) and every quantity of order x = k r: off =
+// 896 - sh is ff_from_f64's offset.
+struct FfUnits {
+  int off;
+  ff kk, ik2;  // kk and 2 / kk
+  __device__ __forceinline__ explicit FfUnits(double k) {
+    const int sh = ilogb(k);
+    const double q = k * pow2d(-sh);
+    off = 896 - sh;
+    kk = ff_round(q);
+    ik2 = ff_round(2.0 / q);
+  }
+};
+
+// (x, y) = a displacement in those units; x = k r, ir = 1 / r and the direction
+// e^{i th} in FP32. False at r = 0.
+struct FfPolar {
+  ff x, y, ir, z;  // z = k r
+  float c, s;
+  __device__ __forceinline__ bool set(double dx, double dy, const FfUnits& U) {
+    x = ff_from_f64(dx, U.off);
+    y = ff_from_f64(dy, U.off);
+    const ff xx = ff_mul_raw(x, x), yy = ff_mul_raw(y, y);
+    const ff d2 = ff_add(xx, yy);
+    if (d2.h == 0.f) return false;
+    ir = ff_rsqrt(d2);
+    z = ff_mul(ff_mul_raw(d2, ir), U.kk);
+    const float irf = ff_f32(ir);
+    c = ff_f32(x) * irf;
+    s = ff_f32(y) * irf;
+    return true;
+  }
+};
+
+// a = ah + al with ah on 17 bits, so that m ah is exact for 0 <= m < 128
+__device__ __forceinline__ ff split17(ff a) {
+  const ff n = fast_two_sum(a.h, a.l);
+  const float h = __uint_as_float(__float_as_uint(n.h) & 0xFFFFFF80u);
+  return mkff(h, __fadd_rn(__fsub_rn(n.h, h), n.l));
+}
+
+// One source's contribution to the scaled sums of a centre, in the split of
+// p2qbxl_pair: sigma^{m+1} A_m and sigma^{m+1} B_m, sigma = 2^s close to k r_c,
+// which keeps every term of moderate size. The Hankel recurrence runs in
+// float-float on Ht_m = sigma^m H_m,
+//   P_m = (2 m sigma / x) Ht_m = sigma^{m+1} K_m,  Z_m = sigma^2 Ht_{m-1},
+//   Ht_{m+1} = P_m - Z_m,  sigma^{m+1} E_m = 2 Z_m - P_m,
+// everything after it (rounded to FP32) in FP32 with Kahan sums, as before.
+// q: sigma times the charge; dn: (d k/2, nu).
 template <int PM, bool HS, bool HD>
-__device__ __forceinline__ void p2qbxl_pair_mixed(float2 (&S)[2 * PM + 1], float2 (&C)[2 * PM + 1],
-                                                  double dx, double dy, float2 q, float2 A,
-                                                  float2 B, double k, double ik, int s, float fr,
-                                                  float fi, int p) {
-  // one reciprocal square root gives r, 1/r and 1/x (ik = 1/k): no division
-  const double d2 = dx * dx + dy * dy;
-  if ((__double2hiint(d2) | __double2loint(d2)) == 0) return;  // d2 == 0 (integer test)
-  const double irr = rsqrt(d2), rr = d2 * irr, x = k * rr, ix = ik * irr;
-  cd h0, h1;
-  hankel01_wide(x, ix, h0, h1);
-  // The FP64 recurrence runs on H_m itself, H_{m+1} = (2m/x) H_m - H_{m-1}
-  // (two FMAs per order); the terms are sigma^|l| W_l with sigma = 2^s close
-  // to rho = k r_c (fr = sigma, fi = 1/sigma), so H_m sigma^m is formed by an
-  // exponent offset while H_m is rounded to FP32, which keeps the terms of
-  // moderate size.
-  const double c2 = 2.0 * ix;
-  cd hprev = h0, hcur = h1;
-  // angular factors e^{i m th} in FP32 (unit modulus; rounding grows like m eps_32),
-  // from the FP32 roundings of dx, dy and 1/r
-  const float irf = f32_from_f64(irr);
-  const float2 e1f = make_float2(f32_from_f64(dx) * irf, f32_from_f64(dy) * irf);
-  float2 ecur = e1f;
-  // W^s_m = sigma^|m| W_m for m = -1, 0, 1, the products in FP32 as for every
-  // other order
-  const float2 h1s = make_float2(f32_from_f64_sh(h1.x, s), f32_from_f64_sh(h1.y, s));
-  const float2 t1 = fmul(h1s, make_float2(e1f.x, -e1f.y));
-  float2 wm1 = make_float2(-t1.x, -t1.y);  // W^s_{-1}
-  float2 w0 = f2(h0);
-  float2 w1 = fmul(h1s, e1f);
-  // l = 0: q W_0 + A W_{-1} - B W_1, with W_{-1} = W^s_{-1} / sigma, W_1 = W^s_1 / sigma
+__device__ __forceinline__ void p2qbxl_pair_mixed(float2 (&S)[2 * PM + 2], float2 (&C)[2 * PM + 2],
+                                                  double dx, double dy, float2 q, float4 dn,
+                                                  const FfUnits& U, ff c2s, float sg, float sg2,
+                                                  int p) {
+  FfPolar D;
+  if (!D.set(dx, dy, U)) return;
+  ffh hp, hc;
+  hankel01_ff_any<3>(D.z, hp, hc);
+  hc.x = ff_scale(hc.x, sg);
+  hc.y = ff_scale(hc.y, sg);
+  const ff c2 = split17(ff_mul_raw(c2s, D.ir));  // 2 sigma / x
+  float cpsi = 0.f, spsi = 0.f;
+  const float2 dk = make_float2(dn.x, dn.y);
   {
     float2 v = make_float2(0.f, 0.f);
-    if (HS) v = fmul(q, w0);
+    if (HS) v = fmul(q, make_float2(ff_f32(hp.x), ff_f32(hp.y)));
     if (HD) {
-      const float2 t = fsub(fmul(A, wm1), fmul(B, w1));
-      v = make_float2(v.x + fi * t.x, v.y + fi * t.y);
+      cpsi = fmaf(D.c, dn.z, D.s * dn.w);
+      spsi = fmaf(D.s, dn.z, -D.c * dn.w);
+      const float2 u = fmul(dk, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
+      const float t = -2.f * cpsi;  // E_0 = -2 H_1, K_0 = 0
+      v = make_float2(fmaf(u.x, t, v.x), fmaf(u.y, t, v.y));
     }
-    kahan2(S[PM], C[PM], v);
+    kahan2(S[0], C[0], v);
   }
-  float2 wp_prev = w0, wp_cur = w1;   // W^s_{m-1}, W^s_m (positive side)
-  float2 wn_prev = w0, wn_cur = wm1;  // W^s_{-(m-1)}, W^s_{-m}
-  double cm = 0.0;                    // 2m/x, kept by addition
+  float c = D.c, sn = D.s;
+  float ac = cpsi * c, as = cpsi * sn, bc = spsi * c, bs = spsi * sn;
+  auto turn = [&](float& u, float& v) {
+    const float t = fmaf(u, D.c, -v * D.s);
+    v = fmaf(u, D.s, v * D.c);
+    u = t;
+  };
 #pragma unroll
   for (int m = 1; m <= PM; ++m) {
     if (m > p) break;
-    cm += c2;
-    const cd hnext = mk(fma(cm, hcur.x, -hprev.x), fma(cm, hcur.y, -hprev.y));
-    const float2 enext = fmul(ecur, e1f);
-    const int sh = (m + 1) * s;
-    const float2 hn32 = make_float2(f32_from_f64_sh(hnext.x, sh), f32_from_f64_sh(hnext.y, sh));
-    const float2 wp_next = fmul(hn32, enext);                                // W^s_{m+1}
-    const float2 wq = fmul(hn32, make_float2(enext.x, -enext.y));
-    // W^s_{-(m+1)} = (-1)^{m+1} conj-angle term
-    const float2 wn_next = (m & 1) ? wq : make_float2(-wq.x, -wq.y);
-    // sigma^m W_{m-1} = sigma W^s_{m-1},  sigma^m W_{m+1} = W^s_{m+1} / sigma (same for -m)
-    float2 vp = make_float2(0.f, 0.f), vn = make_float2(0.f, 0.f);
-    if (HS) {
-      vp = fmul(q, wp_cur);
-      vn = fmul(q, wn_cur);
+    if (m > 1) {
+      if (HS) {
+        turn(c, sn);
+        if (HD) {
+          ac = cpsi * c;
+          as = cpsi * sn;
+          bc = spsi * c;
+          bs = spsi * sn;
+        }
+      } else {
+        turn(ac, as);
+        turn(bc, bs);
+      }
     }
+    const ff cm = mkff((float)m * c2.h, (float)m * c2.l);
+    const ff Px = ff_mul_raw(cm, hc.x), Py = ff_mul_raw(cm, hc.y);
+    const ff Zx = ff_scale(hp.x, sg2), Zy = ff_scale(hp.y, sg2);
+    float2 va = make_float2(0.f, 0.f), vb = va;
     if (HD) {
-      const float2 ap = fmul(A, wp_prev), bp = fmul(B, wp_next);
-      vp.x += fr * ap.x - fi * bp.x;
-      vp.y += fr * ap.y - fi * bp.y;
-      const float2 an = fmul(A, wn_next), bn = fmul(B, wn_prev);
-      vn.x += fi * an.x - fr * bn.x;
-      vn.y += fi * an.y - fr * bn.y;
+      const float px = ff_f32(Px), py = ff_f32(Py);
+      const float ex = fmaf(2.f, ff_f32(Zx), -px), ey = fmaf(2.f, ff_f32(Zy), -py);
+      va = fmul(dk, make_float2(fmaf(ex, ac, px * bs), fmaf(ey, ac, py * bs)));
+      vb = fmul(dk, make_float2(fmaf(ex, as, -px * bc), fmaf(ey, as, -py * bc)));
     }
-    kahan2(S[PM + m], C[PM + m], vp);
-    kahan2(S[PM - m], C[PM - m], vn);
-    hprev = hcur;
-    hcur = hnext;
-    ecur = enext;
-    wp_prev = wp_cur;
-    wp_cur = wp_next;
-    wn_prev = wn_cur;
-    wn_cur = wn_next;
+    if (HS) {
+      const float2 t = fmul(q, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
+      va = make_float2(fmaf(t.x, c, va.x), fmaf(t.y, c, va.y));
+      vb = make_float2(fmaf(t.x, sn, vb.x), fmaf(t.y, sn, vb.y));
+    }
+    kahan2(S[2 * m], C[2 * m], va);
+    kahan2(S[2 * m + 1], C[2 * m + 1], vb);
+    const ff nx = ff_sub_raw(Px, Zx), ny = ff_sub_raw(Py, Zy);
+    hp = hc;
+    hc.x = nx;
+    hc.y = ny;
   }
 }
 
@@ -1665,77 +1714,54 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_kernel(Fmm F, const int*
                         [&](int l, cd a) { dst[l] = cadd(dst[l], a); });
 }
 
-template <int NC>
-__device__ __forceinline__ void warp_reduce_scatter_idx(cd (&acc)[NC], int lane) {
-  constexpr int NP = 32 * ((NC + 31) / 32);
-#pragma unroll
-  for (int h = NP / 2, off = 16; off >= 1; h >>= 1, off >>= 1) {
-    const bool upper = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const cd lo = i < NC ? acc[i] : mk(0.0, 0.0);
-      const cd hi = i + h < NC ? acc[i + h] : mk(0.0, 0.0);
-      const cd send = upper ? lo : hi;
-      cd keep = upper ? hi : lo;
-      keep.x += __shfl_xor_sync(0xffffffffu, send.x, off);
-      keep.y += __shfl_xor_sync(0xffffffffu, send.y, off);
-      if (i < NC) acc[i] = keep;
-    }
-  }
-}
-
 template <int PM, bool HS, bool HD>
 __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, const int* __restrict__ cleaf,
                                                                      const int* __restrict__ wdoff,
                                                                      const int* __restrict__ wdbox,
                                                                      const int* __restrict__ clist,
                                                                      int n_ctr, cd* __restrict__ alpha) {
+  constexpr int NC = 2 * PM + 2;
   const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // position in clist
   const int lane = threadIdx.x & 31;
   if (w >= n_ctr) return;
   const int i = clist[w];
   const int b = cleaf[i];
-  const double k = F.k, ik = 1.0 / k;
-  const int p = F.p, P = 2 * p + 1;
+  const double k = F.k;
+  const int p = F.p;
   const double2 c = F.cxy[i];
-  // sigma = 2^s within a factor sqrt 2 of rho = k r_c: the power that scales
-  // the lane sums (ah_l = alpha_l sigma^|l|)
+  // sigma = 2^s within a factor sqrt 2 of k r_c
   const int s = ilogb(k * F.crad[i] * 1.4142135623730951);
-  const float fr = pow2f(s), fi = pow2f(-s);
-  float2 S[2 * PM + 1], C[2 * PM + 1];
+  const float sg = pow2f(s), sg2 = pow2f(2 * s);
+  const FfUnits U(k);
+  const ff c2s = ff_scale(U.ik2, sg);
+  float2 S[NC], C[NC];
 #pragma unroll
-  for (int j = 0; j <= 2 * PM; ++j) S[j] = C[j] = make_float2(0.f, 0.f);
+  for (int j = 0; j < NC; ++j) S[j] = C[j] = make_float2(0.f, 0.f);
   auto one = [&](int j) {
     const double2 y = F.sxy[j];
-    float2 A = make_float2(0.f, 0.f), B = make_float2(0.f, 0.f);
-    if (HD) {  // A = d (k/2) nu, B = d (k/2) conj(nu), formed once per source
-      const float4 ab = F.ab32[j];
-      A = make_float2(ab.x, ab.y);
-      B = make_float2(ab.z, ab.w);
+    float2 q = make_float2(0.f, 0.f);
+    if (HS) {
+      q = F.q32[j];
+      q = make_float2(q.x * sg, q.y * sg);
     }
-    p2qbxl_pair_mixed<PM, HS, HD>(S, C, y.x - c.x, y.y - c.y,
-                                  HS ? F.q32[j] : make_float2(0.f, 0.f), A, B, k, ik, s, fr, fi,
-                                  p);
+    p2qbxl_pair_mixed<PM, HS, HD>(S, C, y.x - c.x, y.y - c.y, q,
+                                  HD ? F.dn32[j] : make_float4(0.f, 0.f, 0.f, 0.f), U, c2s, sg,
+                                  sg2, p);
   };
   const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], wdoff[i],
                         wdoff[i + 1] - wdoff[i], wdbox};
   deal_sources(sc, lane, one);
   // lane partial sums (compensation removed) in FP64, then the warp sum
-  cd acc[2 * PM + 1];
+  cd acc[NC];
 #pragma unroll
-  for (int j = 0; j <= 2 * PM; ++j)
+  for (int j = 0; j < NC; ++j)
     acc[j] = mk((double)S[j].x - (double)C[j].x, (double)S[j].y - (double)C[j].y);
-  warp_reduce_scatter_idx<2 * PM + 1>(acc, lane);
-  constexpr int K = (2 * PM + 1 + 31) / 32;
-  cd* dst = alpha + (size_t)F.cid[i] * P;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    const int lo = K * lane + j - PM;
-    if (lo >= -p && lo <= p) {
-      const double ip = pow2d(-s * abs(lo));  // sigma^-|lo|: ah_l = alpha_l sigma^|l|
-      dst[lo + p] = cadd(dst[lo + p], cscale(acc[j], ip));
-    }
-  }
+  cd x32, x33;
+  warp_reduce_scatter<NC>(acc, lane, x32, x33);
+  cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
+  pair_coefficients<PM>(acc[0], x32, x33, lane, p, [&](int l, cd a) {
+    dst[l] = cadd(dst[l], cscale(a, pow2d(-s * (abs(l) + 1))));  // the sums carry sigma^{|l|+1}
+  });
 }
 
 }  // namespace
@@ -1860,6 +1886,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
   QBX_CUDA_TRY(f->ds.alloc(std::max<int64_t>(1, h->n_src)));
   QBX_CUDA_TRY(f->q32.alloc(std::max<int64_t>(1, h->n_src)));
   QBX_CUDA_TRY(f->ab32.alloc(std::max<int64_t>(1, h->n_src)));
+  QBX_CUDA_TRY(f->dn32.alloc(std::max<int64_t>(1, h->n_src)));
   // leaves holding sources (P2M)
   QBX_CUDA_TRY(cudaDeviceSynchronize());
   // stats
@@ -2192,7 +2219,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.woff = f->W.off.ptr; F.widx = f->W.idx.ptr;
   F.xoff = f->X.off.ptr; F.xidx = f->X.idx.ptr;
   F.sxy = f->s_xy.ptr; F.snrm = f->s_nrm.ptr; F.qs = f->qs.ptr; F.ds = f->ds.ptr;
-  F.q32 = f->q32.ptr; F.ab32 = f->ab32.ptr;
+  F.q32 = f->q32.ptr; F.ab32 = f->ab32.ptr; F.dn32 = f->dn32.ptr;
   F.cxy = f->c_xy.ptr; F.crad = f->c_r.ptr; F.cid = f->perm[PT_CTR].ptr;
   F.txy = f->t_xy.ptr; F.tid = f->perm[PT_TGT].ptr; F.tassoc = f->t_assoc.ptr;
   F.lpb = f->lpb.ptr; F.eoff = f->eoff.ptr;
@@ -2354,7 +2381,8 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   if (h->n_src > 0) {
     gather_strengths_kernel<<<nblk(h->n_src, 256), 256, 0, s>>>(
         h->n_src, f->perm[PT_SRC].ptr, h->q_str.ptr, h->d_str.ptr, f->s_nrm.ptr, h->k,
-        f->qs.ptr, f->ds.ptr, mixed ? f->q32.ptr : nullptr, mixed ? f->ab32.ptr : nullptr);
+        f->qs.ptr, f->ds.ptr, mixed ? f->q32.ptr : nullptr, mixed ? f->ab32.ptr : nullptr,
+        f->dn32.ptr);
     QBX_KCHECK("gather_strengths", s);
     h->launches += 1;
   }
