@@ -96,6 +96,7 @@ struct Fmm {
   cd* mpole;
   cd* local;
   cd* lpq;               // [n_coef] leaf cos/sin coefficients of L2P (see unscale_leaf_locals_kernel)
+  const int* ffs;        // [n_levels] power-of-two scale exponent of the float-float kernels
   const double* conv;    // [n_levels][pbmax + 1] s^j / sig_j (mixed path)
   const double* lsig;    // [n_levels][pbmax + 1] log sig_j
   const double* isig;    // [n_levels][pbmax + 2] 1 / sig_min(j, pb) (mixed P2M)
@@ -677,11 +678,13 @@ __global__ void __launch_bounds__(kThreads) l2p_kernel(Fmm F, const int* __restr
   *dst = cadd(*dst, cscale(acc, 1.0 / norm));
 }
 
-// M2P: one thread per (direct target, W-list box of its leaf) pair, in
-// target order; writes the pair's value to partial[pair]. m2p_sum_kernel adds
+// M2P: one thread per (direct target, W-list box of its leaf) pair, ordered by
+// (leaf, box, target) so that the lanes of a warp read one box's coefficients;
+// the value goes to the pair's slot in target order, and m2p_sum_kernel adds
 // each target's pairs in order.
 __global__ void __launch_bounds__(kThreads) m2p_pair_kernel(Fmm F, const int* __restrict__ pt,
-                                                            const int* __restrict__ pbx, int n,
+                                                            const int* __restrict__ pbx,
+                                                            const int* __restrict__ slot, int n,
                                                             cd* __restrict__ partial) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -716,7 +719,7 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_kernel(Fmm F, const int* __
     hm1 = hm;
     hm = hn;
   }
-  partial[t] = sum;
+  partial[slot[t]] = sum;
 }
 
 // out[target] += sum of its M2P pairs, in pair order (targets wtgt[0..n)).
@@ -1344,84 +1347,106 @@ __global__ void __launch_bounds__(32) l2qbxl_mixed_kernel(Fmm F, const int* __re
 }
 
 // ---------------------------------------------------------------- M2P in mixed precision
-// The FP32 multipoles that M2P reads. On levels where the unscaled Hankel
-// recurrence stays in range (scaled[l] == 0): mu'_n = a_n 2^-t_|n|, a_n = mh_n
-// s^|n| the true coefficient and t_m = round(log2 sig_m), so that mu' is of
-// order one; otherwise the sigma-normalised mu_n = mh_n conv_|n| (conv = s^j /
-// sig_j).
+// The FP32 multipoles that M2P reads, at entry eoff[b] + b of a float2 array
+// (2 pb + 2 entries per box). On float-float levels (ffs[l] = s)
+// box b holds float4 (P_m, Q_m), m = 0..pb, of the term of order m
+//   a_m H_m e^{i m th} + a_{-m} H_{-m} e^{-i m th} = H_m (P_m cos m th + Q_m sin m th),
+//   P_m = a_m + (-1)^m a_{-m},  Q_m = i (a_m - (-1)^m a_{-m}),  P_0 = a_0,
+// times 2^{-s m} (a_n = mh_n s_l^|n| the true coefficient); on the other levels
+// the sigma-normalised mu_n = mh_n conv_|n| (conv = s^j / sig_j), n = -pb..pb.
 __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
     Fmm F, const int* __restrict__ boxes, const double* __restrict__ conv,
-    const int* __restrict__ tpow, const int* __restrict__ scaled, float2* __restrict__ mu) {
+    float2* __restrict__ mu) {
   const int b = boxes[blockIdx.x];
   const int l = F.level[b];
   const int pb = F.lpb[l];
-  const double* cv = conv + (size_t)l * (F.pbmax + 1);
+  const int s = F.ffs[l];
+  const cd* a = F.mpole + F.eoff[b] + pb;
+  float2* dst = mu + F.eoff[b] + b;
+  if (s == kNoFf) {
+    const double* cv = conv + (size_t)l * (F.pbmax + 1);
+    for (int n = (int)threadIdx.x - pb; n <= pb; n += kThreads) {
+      const double f = cv[abs(n)];
+      dst[n + pb] = make_float2((float)(a[n].x * f), (float)(a[n].y * f));
+    }
+    return;
+  }
   const double* pwl = pw_row(F, l);
-  const int* tl = tpow + (size_t)l * (F.pbmax + 2);
-  const bool sc = scaled[l] != 0;
-  const cd* a = F.mpole + F.eoff[b];
-  float2* dst = mu + F.eoff[b];
-  for (int n = threadIdx.x; n <= 2 * pb; n += kThreads) {
-    const int m = abs(n - pb);
-    const double f = sc ? cv[m] : pwl[m] * pow2d(-tl[m]);
-    dst[n] = make_float2((float)(a[n].x * f), (float)(a[n].y * f));
+  for (int m = threadIdx.x; m <= pb; m += kThreads) {
+    const double f = pwl[m] * pow2d(-s * m);
+    cd g = m > 0 ? a[-m] : mk(0.0, 0.0);
+    if (m & 1) g = mk(-g.x, -g.y);
+    const cd P = cadd(a[m], g), d = csub(a[m], g);
+    reinterpret_cast<float4*>(dst)[m] =
+        make_float4((float)(P.x * f), (float)(P.y * f), m ? (float)(-d.y * f) : 0.f,
+                    m ? (float)(d.x * f) : 0.f);
   }
 }
 
-// M2P with the Hankel recurrence in FP64 and the rest in FP32: the multipole
-// sum_m a_m H_m(kr) e^{imth}, each term formed as an FP32 product of order-one
-// factors:
-//  * unscaled levels: H_{m+1} = (2m/x) H_m - H_{m-1} (two FMAs per order), H_m
-//    rounded to FP32 with the exponent offset t_m (H_m 2^t_m, t_m = round(log2
-//    sig_m)) against mu'_m = a_m 2^-t_m;
-//  * levels where H_pb could leave the FP64 range: G_m = sig_m H_m by
+// M2P: a thread per (direct target, W-list box) pair, pairs ordered by (leaf,
+// box, target) so that the lanes of a warp read the same box's coefficients;
+// slot[t] is the pair's place in target order, where m2p_sum_kernel adds.
+//  * float-float levels: Ht_m = 2^{s m} H_m(k r) by the float-float recurrence
+//      Ht_{m+1} = (2 m 2^s / x) Ht_m - 4^s Ht_{m-1};
+//  * levels whose orders do not fit FP32's range that way (hundreds of orders
+//    over boxes of many wavelengths): G_m = sig_m H_m in FP64 by
 //      G_{m+1} = (2m/x)(sig_{m+1}/sig_m) G_m - (sig_{m+1}/sig_{m-1}) G_{m-1}
 //    (rec[l][m] = (2m sig_{m+1}/sig_m, sig_{m+1}/sig_{m-1}), rec[l][0].x =
 //    sig_1) against mu_m = a_m / sig_m.
-// Angular factors, products and the compensated (Kahan) sum are FP32;
-// H_{-m} = (-1)^m H_m.
+// Angular factors, products and the compensated (Kahan) sum are FP32. With the
+// recurrence in FP64 on every level the kernel ran at 87 % of the FP64 pipe (4.8 M
+// pairs of 200 ellipses: 2.11 -> 0.76 ms).
 __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
-    Fmm F, const int* __restrict__ pt, const int* __restrict__ pbx, int n,
-    const float2* __restrict__ mu, const double2* __restrict__ rec, const int* __restrict__ tpow,
-    const int* __restrict__ scaled, cd* __restrict__ partial) {
+    Fmm F, const int* __restrict__ pt, const int* __restrict__ pbx, const int* __restrict__ slot,
+    int n, const float2* __restrict__ mu, const double2* __restrict__ rec,
+    cd* __restrict__ partial) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const int i = pt[t], c = pbx[t];
   const int lc = F.level[c];
   const int pb = F.lpb[lc];
-  const float2* a = mu + F.eoff[c] + pb;  // a[m], |m| <= pb
+  const int s = F.ffs[lc];
   const double2 mc = F.centre[c];
   const double dx = F.txy[i].x - mc.x, dy = F.txy[i].y - mc.y;
-  const double d2 = dx * dx + dy * dy;
-  const double irr = rsqrt(d2), rr = d2 * irr, x = F.k * rr, ix = irr * F.ik;
-  cd h0, h1;
-  hankel01_wide(x, ix, h0, h1);
-  const float irf = f32_from_f64(irr);
-  const float2 e1 = make_float2(f32_from_f64(dx) * irf, f32_from_f64(dy) * irf);
-  float2 ee = e1;
-  float2 S = fmul(a[0], f2(h0)), C = make_float2(0.f, 0.f);
-  if (!scaled[lc]) {
-    const int* tl = tpow + (size_t)lc * (F.pbmax + 2);
-    const double c2 = 2.0 * ix;
-    double cm = 0.0;  // 2m/x
-    cd hprev = h0, hcur = h1;
+  float2 S, C = make_float2(0.f, 0.f);
+  if (s != kNoFf) {
+    const float4* a = reinterpret_cast<const float4*>(mu + F.eoff[c] + c);
+    const FfUnits U(F.k);
+    FfPolar D;
+    D.set(dx, dy, U);
+    ffh hp, hc;
+    hankel01_ff_any<3>(D.z, hp, hc);
+    const float sg = pow2f(s), sg2 = pow2f(2 * s);
+    hc.x = ff_scale(hc.x, sg);
+    hc.y = ff_scale(hc.y, sg);
+    const ff c2 = split17(ff_mul_raw(ff_scale(U.ik2, sg), D.ir));  // 2 2^s / x
+    S = fmul(make_float2(a[0].x, a[0].y), make_float2(ff_f32(hp.x), ff_f32(hp.y)));
+    float co = D.c, si = D.s, fm = 1.f;
     for (int m = 1; m <= pb; ++m) {
-      const int sh = tl[m];
-      const float2 g = make_float2(f32_from_f64_sh(hcur.x, sh), f32_from_f64_sh(hcur.y, sh));
-      const float2 wp = fmul(g, ee);                                // H_m 2^t e^{im th}
-      float2 wn = fmul(g, make_float2(ee.x, -ee.y));                // H_m 2^t e^{-im th}
-      if (m & 1) wn = make_float2(-wn.x, -wn.y);                    // (-1)^m
-      const float2 vp = fmul(a[m], wp), vn = fmul(a[-m], wn);
-      kahan2(S, C, make_float2(vp.x + vn.x, vp.y + vn.y));
-      if (m < pb) {
-        cm += c2;
-        const cd hn = mk(fma(cm, hcur.x, -hprev.x), fma(cm, hcur.y, -hprev.y));
-        hprev = hcur;
-        hcur = hn;
-        ee = fmul(ee, e1);
-      }
+      const float4 pq = a[m];
+      const float2 v = make_float2(fmaf(pq.x, co, pq.z * si), fmaf(pq.y, co, pq.w * si));
+      kahan2(S, C, fmul(v, make_float2(ff_f32(hc.x), ff_f32(hc.y))));
+      const ff cm = mkff(fm * c2.h, fm * c2.l);
+      fm += 1.f;
+      const ff nx = ff_sub_raw(ff_mul_raw(cm, hc.x), ff_scale(hp.x, sg2));
+      const ff ny = ff_sub_raw(ff_mul_raw(cm, hc.y), ff_scale(hp.y, sg2));
+      hp = hc;
+      hc.x = nx;
+      hc.y = ny;
+      const float u = fmaf(co, D.c, -si * D.s);
+      si = fmaf(co, D.s, si * D.c);
+      co = u;
     }
   } else {
+    const float2* a = mu + F.eoff[c] + c + pb;  // a[m], |m| <= pb
+    const double d2 = dx * dx + dy * dy;
+    const double irr = rsqrt(d2), rr = d2 * irr, x = F.k * rr, ix = irr * F.ik;
+    cd h0, h1;
+    hankel01_wide(x, ix, h0, h1);
+    const float irf = f32_from_f64(irr);
+    const float2 e1 = make_float2(f32_from_f64(dx) * irf, f32_from_f64(dy) * irf);
+    float2 ee = e1;
+    S = fmul(a[0], f2(h0));
     const double2* R = rec + (size_t)lc * (F.pbmax + 2);
     cd gprev = h0, gcur = cscale(h1, R[0].x);
     for (int m = 1; m <= pb; ++m) {
@@ -1440,7 +1465,7 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
       }
     }
   }
-  partial[t] = mk((double)S.x - (double)C.x, (double)S.y - (double)C.y);
+  partial[slot[t]] = mk((double)S.x - (double)C.x, (double)S.y - (double)C.y);
 }
 
 // ---------------------------------------------------------------- P2M in mixed precision
@@ -1947,15 +1972,28 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
         QBX_CUDA_TRY(cudaMemcpy(d.ptr, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice));
       return QBX_OK;
     };
-    // M2P work items: (target, W box) pairs in wtgt order, CSR by position
-    std::vector<int> mt, mbx, moff(wt.size() + 1, 0);
+    // M2P work items: the (target, W box) pairs by (leaf, box, target), so that
+    // neighbouring threads share a box; slot: the pair's place in target order
+    // (CSR by wtgt position), where its value is stored for the ordered sum
+    std::vector<int> mt, mbx, mslot, moff(wt.size() + 1, 0);
     for (size_t t = 0; t < wt.size(); ++t) {
       const int b = tl[wt[t]];
-      for (int e = woff[b]; e < woff[b + 1]; ++e) {
-        mt.push_back(wt[t]);
-        mbx.push_back(widx[e]);
-      }
-      moff[t + 1] = (int)mt.size();
+      moff[t + 1] = moff[t] + woff[b + 1] - woff[b];
+    }
+    mt.reserve(moff.back());
+    mbx.reserve(moff.back());
+    mslot.reserve(moff.back());
+    for (size_t t0 = 0; t0 < wt.size();) {
+      const int b = tl[wt[t0]];
+      size_t t1 = t0;
+      while (t1 < wt.size() && tl[wt[t1]] == b) ++t1;
+      for (int e = woff[b]; e < woff[b + 1]; ++e)
+        for (size_t t = t0; t < t1; ++t) {
+          mt.push_back(wt[t]);
+          mbx.push_back(widx[e]);
+          mslot.push_back(moff[t] + e - woff[b]);
+        }
+      t0 = t1;
     }
     TRY(up(f->tleaf, tl));
     TRY(up(f->dtgt, dt));
@@ -1963,6 +2001,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
     TRY(up(f->wtgt, wt));
     TRY(up(f->m2p_tgt, mt));
     TRY(up(f->m2p_box, mbx));
+    TRY(up(f->m2p_slot, mslot));
     TRY(up(f->m2p_off, moff));
     QBX_CUDA_TRY(f->m2p_part.alloc(std::max<size_t>(1, mt.size())));
     {  // the boxes M2P reads, and FP32 room for their normalised multipoles
@@ -1971,7 +2010,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
       wb.erase(std::unique(wb.begin(), wb.end()), wb.end());
       TRY(up(f->m2p_wbox, wb));
       f->n_m2p_wbox = (int)wb.size();
-      QBX_CUDA_TRY(f->m2p_mu.alloc(wb.empty() ? 1 : std::max<int64_t>(1, f->n_coef)));
+      QBX_CUDA_TRY(f->m2p_mu.alloc(wb.empty() ? 2 : f->n_coef + f->n_boxes));
     }
     f->n_dtgt = (int)dt.size();
     f->n_utgt = (int)ut.size();
@@ -2226,6 +2265,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.scale = f->scale.ptr; F.pw = f->pw.ptr; F.ipw = f->ipw.ptr;
   F.t_m2l = f->t_m2l.ptr; F.t_m2m = f->t_m2m.ptr; F.t_l2l = f->t_l2l.ptr;
   F.mpole = f->mpole.ptr; F.local = f->local.ptr; F.lpq = f->lpq.ptr;
+  F.ffs = f->ff_s.ptr;
   F.conv = f->conv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.sigr = f->sigr.ptr;
   F.k = h->k; F.ik = 1.0 / h->k; F.side = f->side; F.pbmax = f->pb_max; F.p = h->p; F.n_levels = f->n_levels;
   F.has_S = S ? 1 : 0; F.has_D = D ? 1 : 0;
@@ -2503,15 +2543,15 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   if (f->n_wtgt > 0 && f->n_m2p_pairs > 0) {
     if (mixed) {
       mpole_f32_list_kernel<<<f->n_m2p_wbox, kThreads, 0, s2>>>(
-          F, f->m2p_wbox.ptr, f->conv.ptr, f->m2p_t.ptr, f->m2p_scaled.ptr, f->m2p_mu.ptr);
+          F, f->m2p_wbox.ptr, f->conv.ptr, f->m2p_mu.ptr);
       QBX_KCHECK("m2p_mu", s2);
       m2p_pair_mixed_kernel<<<nblk(f->n_m2p_pairs, kThreads), kThreads, 0, s2>>>(
-          F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->n_m2p_pairs, f->m2p_mu.ptr, f->m2p_rec.ptr,
-          f->m2p_t.ptr, f->m2p_scaled.ptr, f->m2p_part.ptr);
+          F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->m2p_slot.ptr, f->n_m2p_pairs, f->m2p_mu.ptr,
+          f->m2p_rec.ptr, f->m2p_part.ptr);
       h->launches += 1;
     } else {
       m2p_pair_kernel<<<nblk(f->n_m2p_pairs, kThreads), kThreads, 0, s2>>>(
-          F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->n_m2p_pairs, f->m2p_part.ptr);
+          F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->m2p_slot.ptr, f->n_m2p_pairs, f->m2p_part.ptr);
     }
     QBX_KCHECK("m2p", s2);
     m2p_sum_kernel<<<nblk(f->n_wtgt, kThreads), kThreads, 0, s2>>>(

@@ -69,17 +69,6 @@ __global__ void m2p_rec_kernel(int n_levels, int pbmax, const int* __restrict__ 
   }
 }
 
-// t[l][m] = round(log2 sig_m) of level l: the power of two that M2P moves from
-// the multipole to the Hankel value (exponent offsets, no arithmetic)
-__global__ void m2p_t_kernel(int n_levels, int pbmax, const int* __restrict__ lpb,
-                             const double* __restrict__ lsig, int* __restrict__ t) {
-  const int l = blockIdx.x;
-  if (l >= n_levels) return;
-  const double* sg = lsig + (size_t)l * (pbmax + 1);
-  for (int m = threadIdx.x; m <= pbmax + 1; m += blockDim.x)
-    t[(size_t)l * (pbmax + 2) + m] = m <= lpb[l] ? (int)lrint(sg[m] * 1.4426950408889634) : 0;
-}
-
 // r[l][m] = (sig_{m-1} / sig_m, sig_{m+1} / sig_m) of level l, 1 where the
 // neighbour order is outside 0..pb (the mixed P2M's dipole terms)
 __global__ void sig_ratio_kernel(int n_levels, int pbmax, const int* __restrict__ lpb,
@@ -775,6 +764,27 @@ qbx_status configure_mixed_kernels(int smem_optin) {
   return QBX_OK;
 }
 
+// The exponent s for which 2^{s m} H_m(x) and 2^{-s m} J_m(y), m <= pb, stay in
+// FP32's range at the arguments that boxes of k side = x0 meet: a W-list box's
+// targets and a local expansion's sources lie 1.5 sides or more from the centre
+// (x >= 1.4 x0), its own points within 0.71 sides (y <= 0.71 x0). H_m grows like
+// (2 m / (e x))^m, so s puts the turn of (2 m 2^s / (e x))^m at 0.6 pb: it falls
+// to 2^{-0.32 pb} before and rises to 2^{0.44 pb} at pb. Refused (FP64 kernels)
+// when the largest |2^{s m} H_m| exceeds 2^60, or an order reaches 128 (the
+// recurrence's exact products m c hold 7 bits of m).
+static int float_float_scale(double x0, int pb) {
+  if (pb < 1 || pb > 126) return kNoFf;
+  const double xl = 1.4 * x0;
+  const int s = (int)std::lrint(std::min(0.0, std::log2(xl * 1.3591409142295226 / (0.6 * pb))));
+  if (s < -50) return kNoFf;
+  double top = 0.0;
+  for (int m = 1; m <= pb; ++m)  // |H_m(x)| <~ (m-1)!/pi (2/x)^m for m > x, of order one below
+    if (m > xl)
+      top = std::max(top, s * m + (std::lgamma((double)m) - 1.1447298858494002 +
+                                   m * std::log(2.0 / xl)) / 0.69314718055994531);
+  return top > 60.0 ? kNoFf : s;
+}
+
 qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
   const int pbm = f->pb_max;
   QBX_CUDA_TRY(f->lsig.alloc((size_t)f->n_levels * (pbm + 1)));
@@ -789,21 +799,12 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
   QBX_CUDA_TRY(f->sigr.alloc((size_t)f->n_levels * (pbm + 2)));
   sig_ratio_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->lsig.ptr, f->sigr.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
-  QBX_CUDA_TRY(f->m2p_t.alloc((size_t)f->n_levels * (pbm + 2)));
-  m2p_t_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->lsig.ptr, f->m2p_t.ptr);
-  QBX_CUDA_TRY(cudaGetLastError());
-  {  // levels where H_pb(x) could leave the FP64 range: x = k |t - m_c| >= 1.5 k
-     // side for a W-list box (taken as 0.5 k side), |H_m(x)| <~ (m-1)! (2/x)^m
-    std::vector<int> scaled(f->n_levels, 0);
-    for (int l = 0; l < f->n_levels; ++l) {
-      const int pb = f->h_pb[l];
-      if (pb < 1) continue;
-      const double x_lo = 0.5 * h->k * f->side / (double)(1LL << std::min(l, 62));
-      const double ln_h = std::lgamma((double)pb) + pb * std::log(2.0 / x_lo);
-      scaled[l] = ln_h > 650.0 ? 1 : 0;
-    }
-    QBX_CUDA_TRY(f->m2p_scaled.alloc(f->n_levels));
-    QBX_CUDA_TRY(cudaMemcpy(f->m2p_scaled.ptr, scaled.data(), f->n_levels * sizeof(int),
+  {
+    std::vector<int> ffs(f->n_levels, kNoFf);
+    for (int l = 2; l < f->n_levels; ++l)
+      ffs[l] = float_float_scale(h->k * f->side / std::ldexp(1.0, l), f->h_pb[l]);
+    QBX_CUDA_TRY(f->ff_s.alloc(f->n_levels));
+    QBX_CUDA_TRY(cudaMemcpy(f->ff_s.ptr, ffs.data(), f->n_levels * sizeof(int),
                             cudaMemcpyHostToDevice));
   }
   // matrices for the levels that have V lists

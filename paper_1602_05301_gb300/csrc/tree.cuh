@@ -45,6 +45,9 @@ struct TcLevelOp {
   DevBuf<int> fexp, xexp, src, rowsrc, rowdst, prow;
 };
 
+// No power-of-two scaling of a level fits FP32 (see float_float_scale).
+constexpr int kNoFf = -100000;
+
 struct FmmPlan {
   // concurrency of the near-field stages (see fmm_eval)
   cudaStream_t near_stream = nullptr;
@@ -114,16 +117,19 @@ struct FmmPlan {
   DevBuf<int> tleaf;                    // [n_targets] leaf of each sorted target
   DevBuf<int> dtgt, utgt, wtgt;         // direct targets (sorted indices): all, with
   int n_dtgt = 0, n_utgt = 0, n_wtgt = 0;  // U-list sources, with a W list
-  DevBuf<int> m2p_tgt, m2p_box, m2p_off;   // M2P (target, W box) pairs, CSR by wtgt position
+  // M2P (target, W box) pairs by (leaf, box, target), their places in target
+  // order, and the CSR of that order by wtgt position
+  DevBuf<int> m2p_tgt, m2p_box, m2p_slot, m2p_off;
   DevBuf<cd> m2p_part;                   // [pairs] partial values
   int n_m2p_pairs = 0;
   DevBuf<int> m2p_wbox;                  // boxes M2P reads (mixed path converts them)
   int n_m2p_wbox = 0;
-  DevBuf<float2> m2p_mu;                 // [n_coef] their sigma-normalised FP32 multipoles
+  DevBuf<float2> m2p_mu;                 // [n_coef + n_boxes] their FP32 multipoles
   DevBuf<double2> m2p_rec;               // [n_levels][pbmax + 2] sigma-scaled Hankel recurrence
-  DevBuf<int> m2p_t;                     // [n_levels][pbmax + 2] round(log2 sig_m)
   DevBuf<double2> sigr;                  // [n_levels][pbmax + 2] (sig_{m-1}/sig_m, sig_{m+1}/sig_m)
-  DevBuf<int> m2p_scaled;                // [n_levels] 1: the unscaled recurrence could overflow
+  // [n_levels] s of the scaling 2^{s m} H_m, 2^{-s m} J_m that keeps orders up to
+  // the level's in FP32's range (float-float kernels), or kNoFf
+  DevBuf<int> ff_s;
   // Centre sets: [0] every centre, [1] the centres some target uses. Each
   // lists sorted centre indices (clist) and its M2QBXL work items, the
   // (sorted centre, W-list box) pairs grouped by list position (CSR wp_off).
