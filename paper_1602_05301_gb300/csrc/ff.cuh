@@ -164,3 +164,45 @@ __device__ __forceinline__ void hankel01_ff_any(ff x, ffh& h0, ffh& h1) {
   if (NEED0) { h0.x = ff_round(h[0]); h0.y = ff_round(h[1]); }
   if (NEED1) { h1.x = ff_round(h[2]); h1.y = ff_round(h[3]); }
 }
+
+// Lengths in the float-float kernels are in units of 2^-sh (sh = floor(log2 k)), so
+// that the wavenumber is kk in [1, 2) and every quantity of order x = k r: off =
+// 896 - sh is ff_from_f64's offset.
+struct FfUnits {
+  int off;
+  ff kk, ik2;  // kk and 2 / kk
+  __device__ __forceinline__ explicit FfUnits(double k) {
+    const int sh = ilogb(k);
+    const double q = k * pow2d(-sh);
+    off = 896 - sh;
+    kk = ff_round(q);
+    ik2 = ff_round(2.0 / q);
+  }
+};
+
+// (x, y) = a displacement in those units; x = k r, ir = 1 / r and the direction
+// e^{i th} in FP32. False at r = 0.
+struct FfPolar {
+  ff x, y, ir, z;  // z = k r
+  float c, s;
+  __device__ __forceinline__ bool set(double dx, double dy, const FfUnits& U) {
+    x = ff_from_f64(dx, U.off);
+    y = ff_from_f64(dy, U.off);
+    const ff xx = ff_mul_raw(x, x), yy = ff_mul_raw(y, y);
+    const ff d2 = ff_add(xx, yy);
+    if (d2.h == 0.f) return false;
+    ir = ff_rsqrt(d2);
+    z = ff_mul(ff_mul_raw(d2, ir), U.kk);
+    const float irf = ff_f32(ir);
+    c = ff_f32(x) * irf;
+    s = ff_f32(y) * irf;
+    return true;
+  }
+};
+
+// a = ah + al with ah on 17 bits, so that m ah is exact for 0 <= m < 128
+__device__ __forceinline__ ff split17(ff a) {
+  const ff n = fast_two_sum(a.h, a.l);
+  const float h = __uint_as_float(__float_as_uint(n.h) & 0xFFFFFF80u);
+  return mkff(h, __fadd_rn(__fsub_rn(n.h, h), n.l));
+}

@@ -78,6 +78,7 @@ struct Fmm {
   const float2* q32;     // FP32 charges (mixed path)
   const float4* ab32;    // FP32 dipole factors (A, B) (mixed path)
   const float4* dn32;    // FP32 (d k/2, nu) (mixed path)
+  const float4 *qf, *df, *nf;  // float-float charges, d k and normals (mixed P2P)
   const double2* cxy;
   const double* crad;    // sorted centre radii
   const int* cid;
@@ -244,7 +245,8 @@ __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
                                         const double2* __restrict__ snrm, double k,
                                         cd* __restrict__ qs, cd* __restrict__ ds,
                                         float2* __restrict__ q32, float4* __restrict__ ab32,
-                                        float4* __restrict__ dn32) {
+                                        float4* __restrict__ dn32, float4* __restrict__ qf,
+                                        float4* __restrict__ df, float4* __restrict__ nf) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const cd qi = q[perm[i]], di = d[perm[i]];
@@ -257,6 +259,13 @@ __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
     q32[i] = make_float2((float)qi.x, (float)qi.y);
     ab32[i] = make_float4((float)A.x, (float)A.y, (float)B.x, (float)B.y);
     dn32[i] = make_float4((float)dk.x, (float)dk.y, (float)nu.x, (float)nu.y);
+    auto two = [](cd v) {
+      const ff a = ff_round(v.x), b = ff_round(v.y);
+      return make_float4(a.h, a.l, b.h, b.l);
+    };
+    qf[i] = two(qi);
+    df[i] = two(cscale(di, k));
+    nf[i] = two(nu);
   }
 }
 
@@ -735,10 +744,8 @@ __global__ void m2p_sum_kernel(int n, const int* __restrict__ wtgt, const int* _
 }
 
 // P2P over the U list: one warp per direct target whose leaf's U list holds
-// sources; lanes deal the sources round-robin, a shuffle tree adds them. WIDE:
-// the mixed path's Hankel tables (relative error below 1e-13 instead of 1e-15;
-// the sum stays FP64).
-template <bool HS, bool HD, bool WIDE>
+// sources; lanes deal the sources round-robin, a shuffle tree adds them.
+template <bool HS, bool HD>
 __global__ void __launch_bounds__(kThreads) p2p_warp_kernel(Fmm F, const int* __restrict__ utgt,
                                                             const int* __restrict__ tleaf, int n,
                                                             cd* __restrict__ out) {
@@ -747,7 +754,7 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_kernel(Fmm F, const int* __
   if (t >= n) return;
   const int i = utgt[t];
   const int b = tleaf[i];
-  const double k = F.k, ik = 1.0 / k;
+  const double k = F.k, ik = F.ik;
   const double tx = F.txy[i].x, ty = F.txy[i].y;
   cd acc = mk(0.0, 0.0);
   const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], 0, 0, nullptr};
@@ -757,7 +764,7 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_kernel(Fmm F, const int* __
     if (r2 == 0.0) return;
     const double ir = rsqrt(r2), x = k * r2 * ir;
     cd h0, h1;
-    hankel01_any<WIDE, HS, HD>(x, ik * ir, h0, h1);
+    hankel01_any<false, HS, HD>(x, ik * ir, h0, h1);
     if (HS) cfma(acc, F.qs[j], h0);
     if (HD) {
       const double2 nv = F.snrm[j];
@@ -1015,48 +1022,6 @@ __device__ __forceinline__ float2 fmul(float2 a, float2 b) {
 }
 __device__ __forceinline__ float2 fsub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 f2(cd a) { return make_float2(f32_from_f64(a.x), f32_from_f64(a.y)); }
-
-// Lengths in the float-float kernels are in units of 2^-sh (sh = floor(log2 k)), so
-// that the wavenumber is kk in [1, 2) and every quantity of order x = k r: off =
-// 896 - sh is ff_from_f64's offset.
-struct FfUnits {
-  int off;
-  ff kk, ik2;  // kk and 2 / kk
-  __device__ __forceinline__ explicit FfUnits(double k) {
-    const int sh = ilogb(k);
-    const double q = k * pow2d(-sh);
-    off = 896 - sh;
-    kk = ff_round(q);
-    ik2 = ff_round(2.0 / q);
-  }
-};
-
-// (x, y) = a displacement in those units; x = k r, ir = 1 / r and the direction
-// e^{i th} in FP32. False at r = 0.
-struct FfPolar {
-  ff x, y, ir, z;  // z = k r
-  float c, s;
-  __device__ __forceinline__ bool set(double dx, double dy, const FfUnits& U) {
-    x = ff_from_f64(dx, U.off);
-    y = ff_from_f64(dy, U.off);
-    const ff xx = ff_mul_raw(x, x), yy = ff_mul_raw(y, y);
-    const ff d2 = ff_add(xx, yy);
-    if (d2.h == 0.f) return false;
-    ir = ff_rsqrt(d2);
-    z = ff_mul(ff_mul_raw(d2, ir), U.kk);
-    const float irf = ff_f32(ir);
-    c = ff_f32(x) * irf;
-    s = ff_f32(y) * irf;
-    return true;
-  }
-};
-
-// a = ah + al with ah on 17 bits, so that m ah is exact for 0 <= m < 128
-__device__ __forceinline__ ff split17(ff a) {
-  const ff n = fast_two_sum(a.h, a.l);
-  const float h = __uint_as_float(__float_as_uint(n.h) & 0xFFFFFF80u);
-  return mkff(h, __fadd_rn(__fsub_rn(n.h, h), n.l));
-}
 
 // One source's contribution to the scaled sums of a centre, in the split of
 // p2qbxl_pair: sigma^{m+1} A_m and sigma^{m+1} B_m, sigma = 2^s close to k r_c,
@@ -1343,6 +1308,62 @@ __global__ void __launch_bounds__(32) l2qbxl_mixed_kernel(Fmm F, const int* __re
     const double sc = pow2d(emax);
     cd* dst = alpha + (size_t)F.cid[i] * P + p + so;
     *dst = cadd(*dst, mk(((double)S.x - (double)C.x) * sc, ((double)S.y - (double)C.y) * sc));
+  }
+}
+
+// ---------------------------------------------------------------- P2P in mixed precision
+// p2p_warp_kernel with everything but the two coordinate differences in
+// float-float (strengths, normals, tables to degree-6 second parts, the lanes'
+// sums; the warp's sum is FP64): about 300 FP32 instructions per source and
+// layer in place of 45 on the FP64 pipe, which bound it (82 % of its rate): 11 M
+// pairs of 200 ellipses 1.22 -> 0.29 ms, the starfish grid 0.19 -> 0.05 ms.
+struct FfSum {
+  ff x, y;
+  __device__ __forceinline__ FfSum() : x(mkff(0.f, 0.f)), y(mkff(0.f, 0.f)) {}
+  // += a b, complex a given as (re h, re l, im h, im l)
+  __device__ __forceinline__ void fma(float4 a, ff bx, ff by) {
+    const ff ax = mkff(a.x, a.y), ay = mkff(a.z, a.w);
+    x = ff_add(x, ff_sub_raw(ff_mul_raw(ax, bx), ff_mul_raw(ay, by)));
+    y = ff_add(y, ff_sub_raw(ff_mul_raw(ax, by), ff_mul_raw(mkff(-ay.h, -ay.l), bx)));
+  }
+};
+
+template <bool HS, bool HD>
+__global__ void __launch_bounds__(kThreads) p2p_warp_mixed_kernel(Fmm F, const int* __restrict__ utgt,
+                                                                  const int* __restrict__ tleaf,
+                                                                  int n, cd* __restrict__ out) {
+  const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (t >= n) return;
+  const int i = utgt[t];
+  const int b = tleaf[i];
+  const double2 tp = F.txy[i];
+  const FfUnits U(F.k);
+  FfSum acc;
+  const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], 0, 0, nullptr};
+  deal_sources(sc, lane, [&](int j) {
+    const double2 y = F.sxy[j];
+    FfPolar D;
+    if (!D.set(tp.x - y.x, tp.y - y.y, U)) return;
+    ffh h0, h1;
+    hankel01_ff_any<kHankLoFf, HS, HD>(D.z, h0, h1);
+    if (HS) acc.fma(F.qf[j], h0.x, h0.y);
+    if (HD) {
+      const float4 nv = F.nf[j];  // n . (t - y) / r
+      const ff f = ff_mul(ff_add(ff_mul_raw(mkff(nv.x, nv.y), D.x),
+                                 ff_mul_raw(mkff(nv.z, nv.w), D.y)), D.ir);
+      acc.fma(F.df[j], ff_mul_raw(h1.x, f), ff_mul_raw(h1.y, f));
+    }
+  });
+  cd sum = mk(ff_f64(acc.x), ff_f64(acc.y));
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    sum.x += __shfl_xor_sync(0xffffffffu, sum.x, off);
+    sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
+  }
+  if (lane == 0) {
+    cd* dst = out + F.tid[i];
+    *dst = cadd(*dst, sum);
   }
 }
 
@@ -1911,7 +1932,8 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
   QBX_CUDA_TRY(f->ds.alloc(std::max<int64_t>(1, h->n_src)));
   QBX_CUDA_TRY(f->q32.alloc(std::max<int64_t>(1, h->n_src)));
   QBX_CUDA_TRY(f->ab32.alloc(std::max<int64_t>(1, h->n_src)));
-  QBX_CUDA_TRY(f->dn32.alloc(std::max<int64_t>(1, h->n_src)));
+  for (DevBuf<float4>* v : {&f->dn32, &f->qf, &f->df, &f->nf})
+    QBX_CUDA_TRY(v->alloc(std::max<int64_t>(1, h->n_src)));
   // leaves holding sources (P2M)
   QBX_CUDA_TRY(cudaDeviceSynchronize());
   // stats
@@ -2259,6 +2281,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.xoff = f->X.off.ptr; F.xidx = f->X.idx.ptr;
   F.sxy = f->s_xy.ptr; F.snrm = f->s_nrm.ptr; F.qs = f->qs.ptr; F.ds = f->ds.ptr;
   F.q32 = f->q32.ptr; F.ab32 = f->ab32.ptr; F.dn32 = f->dn32.ptr;
+  F.qf = f->qf.ptr; F.df = f->df.ptr; F.nf = f->nf.ptr;
   F.cxy = f->c_xy.ptr; F.crad = f->c_r.ptr; F.cid = f->perm[PT_CTR].ptr;
   F.txy = f->t_xy.ptr; F.tid = f->perm[PT_TGT].ptr; F.tassoc = f->t_assoc.ptr;
   F.lpb = f->lpb.ptr; F.eoff = f->eoff.ptr;
@@ -2422,7 +2445,7 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     gather_strengths_kernel<<<nblk(h->n_src, 256), 256, 0, s>>>(
         h->n_src, f->perm[PT_SRC].ptr, h->q_str.ptr, h->d_str.ptr, f->s_nrm.ptr, h->k,
         f->qs.ptr, f->ds.ptr, mixed ? f->q32.ptr : nullptr, mixed ? f->ab32.ptr : nullptr,
-        f->dn32.ptr);
+        f->dn32.ptr, f->qf.ptr, f->df.ptr, f->nf.ptr);
     QBX_KCHECK("gather_strengths", s);
     h->launches += 1;
   }
@@ -2474,11 +2497,11 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
 #define P2P_LAUNCH(A, B)                                                                      \
     do {                                                                                       \
       if (mixed)                                                                               \
-        p2p_warp_kernel<A, B, true><<<gw, kThreads, 0, s2>>>(F, f->utgt.ptr, f->tleaf.ptr,     \
+        p2p_warp_mixed_kernel<A, B><<<gw, kThreads, 0, s2>>>(F, f->utgt.ptr, f->tleaf.ptr,     \
                                                              f->n_utgt, out);                  \
       else                                                                                     \
-        p2p_warp_kernel<A, B, false><<<gw, kThreads, 0, s2>>>(F, f->utgt.ptr, f->tleaf.ptr,    \
-                                                              f->n_utgt, out);                 \
+        p2p_warp_kernel<A, B><<<gw, kThreads, 0, s2>>>(F, f->utgt.ptr, f->tleaf.ptr,           \
+                                                       f->n_utgt, out);                        \
     } while (0)
     if (S && D) P2P_LAUNCH(true, true);
     else if (S) P2P_LAUNCH(true, false);

@@ -157,7 +157,7 @@ struct FmmPlan {
   DevBuf<cd> qs, ds;                    // sorted strengths
   DevBuf<float2> q32;                   // their FP32 charges and dipole factors (mixed path)
   DevBuf<float4> ab32;
-  DevBuf<float4> dn32;
+  DevBuf<float4> dn32, qf, df, nf;      // FP32 (d k/2, nu); float-float charges, d k, normals
   DevBuf<int> err;                      // device error flags
   // mixed precision (sigma-normalised FP32 M2L)
   DevBuf<double> lsig, conv;            // [n_levels][pb_max+1] log sig_j, s^j / sig_j
