@@ -599,13 +599,7 @@ __device__ __forceinline__ void deal_sources(const SourceCursor& sc, int lane, F
 // backward recurrence yields f_m for descending m, and Clenshaw's recurrences
 // for the cosine and sine sums run in the same loop (two FMAs per real
 // component and order, no complex products).
-__global__ void __launch_bounds__(kThreads) l2p_kernel(Fmm F, const int* __restrict__ dtgt,
-                                                       const int* __restrict__ tleaf, int n,
-                                                       cd* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const int i = dtgt[t];
-  const int b = tleaf[i];
+__device__ __forceinline__ cd l2p_value(const Fmm& F, int i, int b) {
   const int pb = F.lpb[F.level[b]];
   const cd* g = F.local + F.eoff[b];
   const double2 m = F.centre[b];
@@ -683,9 +677,19 @@ __global__ void __launch_bounds__(kThreads) l2p_kernel(Fmm F, const int* __restr
     acc = mk(fma(-c, u2.x, u1.x) + e1.y * v1.x, fma(-c, u2.y, u1.y) + e1.y * v1.y);
     norm = fn + 2.0 * sum;
   }
-  cd* dst = out + F.tid[i];
-  *dst = cadd(*dst, cscale(acc, 1.0 / norm));
+  return cscale(acc, 1.0 / norm);
 }
+
+__global__ void __launch_bounds__(kThreads) l2p_kernel(Fmm F, const int* __restrict__ dtgt,
+                                                       const int* __restrict__ tleaf, int n,
+                                                       cd* __restrict__ out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int i = dtgt[t];
+  cd* dst = out + F.tid[i];
+  *dst = cadd(*dst, l2p_value(F, i, tleaf[i]));
+}
+
 
 // M2P: one thread per (direct target, W-list box of its leaf) pair, ordered by
 // (leaf, box, target) so that the lanes of a warp read one box's coefficients;
@@ -850,27 +854,41 @@ __global__ void __launch_bounds__(32) l2qbxl_kernel(Fmm F, const int* __restrict
 //     = J_m(k r) [P_m cos(m th) + Q_m sin(m th)],
 //   P_m = gamma_m + s_m gamma_{-m},  Q_m = i (s_m gamma_{-m} - gamma_m),  P_0 = gamma_0,
 // stored as lpq[eoff + m] = P_m (m = 0..pb), lpq[eoff + pb + m] = Q_m (m = 1..pb).
+// With ff32 set (mixed path), leaves on float-float levels (ffs[l] = s) get
+// 2^{s m} P_m and 2^{s m} Q_m as float4 (re h, re l, im h, im l) in the same
+// places, for l2p_mixed_kernel.
 __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
-                                                                       const int* __restrict__ leaves) {
+                                                                       const int* __restrict__ leaves,
+                                                                       bool ff32) {
   const int b = leaves[blockIdx.x];
   const int l = F.level[b];
   const int pb = F.lpb[l];
   const double* ipp = ipw_row(F, l);
   cd* lp = F.local + F.eoff[b];
   cd* pq = F.lpq + F.eoff[b];
+  const int s = ff32 ? F.ffs[l] : kNoFf;
+  auto put = [&](int at, int m, cd v) {
+    if (s == kNoFf) {
+      pq[at] = v;
+      return;
+    }
+    const double f = pow2d(s * m);
+    const ff x = ff_round(v.x * f), y = ff_round(v.y * f);
+    reinterpret_cast<float4*>(pq)[at] = make_float4(x.h, x.l, y.h, y.l);
+  };
   for (int m = threadIdx.x; m <= pb; m += kThreads) {
     const cd gp = cscale(lp[pb + m], ipp[m]);
     lp[pb + m] = gp;
     if (m == 0) {
-      pq[0] = gp;
+      put(0, 0, gp);
       continue;
     }
     const cd gn = cscale(lp[pb - m], ipp[m]);
     lp[pb - m] = gn;
     const cd sg = (m & 1) ? mk(-gn.x, -gn.y) : gn;
-    pq[m] = cadd(gp, sg);
+    put(m, m, cadd(gp, sg));
     const cd d = csub(sg, gp);
-    pq[pb + m] = mk(-d.y, d.x);
+    put(pb + m, m, mk(-d.y, d.x));
   }
 }
 
@@ -1365,6 +1383,107 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_mixed_kernel(Fmm F, const i
     cd* dst = out + F.tid[i];
     *dst = cadd(*dst, sum);
   }
+}
+
+// ---------------------------------------------------------------- L2P in mixed precision
+// l2p_kernel's Miller and Clenshaw recurrences in float-float, on 2^{-s m} J_m
+// and the coefficients scaled by 2^{s m} (s = ffs of the level):
+//   f_{n-1} = (2 n 2^s / x) f_n - 4^s f_{n+1},  norm = f_0 + 2 4^s (f_2 + 4^s (f_4 + ...)),
+// everything kept rescaled by 2^-60 when |f| passes 2^20 (with the coefficients
+// below 2^60 no product leaves FP32's range). About 110 FP32 instructions per
+// order instead of 11 on the FP64 pipe, which bound it (86 % of its rate): 0.9 M
+// targets of 200 ellipses 1.75 -> 0.32 ms.
+// Levels without a scale and targets within x = 1e-8 of the centre take the
+// FP64 form, out of line.
+static __device__ __noinline__ void l2p_value_outside(const Fmm& F, int i, int b, cd* v) {
+  *v = l2p_value(F, i, b);
+}
+
+__global__ void __launch_bounds__(kThreads) l2p_mixed_kernel(Fmm F, const int* __restrict__ dtgt,
+                                                             const int* __restrict__ tleaf, int n,
+                                                             cd* __restrict__ out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int i = dtgt[t];
+  const int b = tleaf[i];
+  const int l = F.level[b];
+  const int pb = F.lpb[l], s = F.ffs[l];
+  cd* dst = out + F.tid[i];
+  const double2 mc = F.centre[b], tp = F.txy[i];
+  const FfUnits U(F.k);
+  FfPolar D;
+  const bool in = s != kNoFf && D.set(tp.x - mc.x, tp.y - mc.y, U) && D.z.h >= 1e-8f;
+  if (!in) {
+    cd v;
+    l2p_value_outside(F, i, b, &v);
+    *dst = cadd(*dst, v);
+    return;
+  }
+  const float4* pq = reinterpret_cast<const float4*>(F.lpq + F.eoff[b]);
+  const float sg2 = pow2f(2 * s);
+  ff c2 = ff_mul_raw(ff_scale(U.ik2, pow2f(s)), D.ir);  // 2 2^s / x
+  c2 = fast_two_sum(c2.h, c2.l);
+  const ff co = ff_mul(D.x, D.ir), si = ff_mul(D.y, D.ir);
+  const ff co2 = ff_scale(co, 2.f);
+  const int N = miller_start_f32(pb, D.z.h);
+  ff f1 = mkff(0.f, 0.f), f0 = mkff(0x1p-40f, 0.f), sum = f1;
+  float fn = (float)N;
+  auto step = [&]() {
+    const float ch = __fmul_rn(fn, c2.h);
+    const ff cn = mkff(ch, __fmaf_rn(fn, c2.l, __fmaf_rn(fn, c2.h, -ch)));
+    const ff f = ff_sub_raw(ff_mul_raw(cn, f0), ff_scale(f1, sg2));
+    f1 = f0;
+    f0 = fast_two_sum(f.h, f.l);
+    fn -= 1.f;
+  };
+  auto even = [&]() { sum = ff_add(f0, ff_scale(sum, sg2)); };
+  constexpr float kBig = 0x1p20f, kDown = 0x1p-60f;
+  int nn = N;
+  for (; nn >= pb + 2; --nn) {  // orders above pb: the recurrence alone
+    if ((nn & 1) == 0) even();
+    step();
+    if (fabsf(f0.h) >= kBig) {
+      f0 = ff_scale(f0, kDown);
+      f1 = ff_scale(f1, kDown);
+      sum = ff_scale(sum, kDown);
+    }
+  }
+  // one Clenshaw step of a real component: f c + 2 cos(th) b1 - b2
+  auto clenshaw = [&](ff c, ff& b1, ff& b2) {
+    const ff p = ff_mul_raw(f0, c), q = ff_mul_raw(co2, b1);
+    const ff u = two_sum(q.h, -b2.h), v = two_sum(u.h, p.h);
+    const float lo = __fadd_rn(__fadd_rn(u.l, v.l), __fadd_rn(p.l, __fsub_rn(q.l, b2.l)));
+    b2 = b1;
+    b1 = fast_two_sum(v.h, lo);
+  };
+  const ff z = mkff(0.f, 0.f);
+  ff ux1 = z, ux2 = z, uy1 = z, uy2 = z, vx1 = z, vx2 = z, vy1 = z, vy2 = z;
+  for (; nn >= 1; --nn) {
+    if ((nn & 1) == 0) even();
+    step();
+    const int mm = nn - 1;  // f0 = f_mm
+    const float4 P = pq[mm];
+    clenshaw(mkff(P.x, P.y), ux1, ux2);
+    clenshaw(mkff(P.z, P.w), uy1, uy2);
+    if (mm >= 1) {
+      const float4 Q = pq[pb + mm];
+      clenshaw(mkff(Q.x, Q.y), vx1, vx2);
+      clenshaw(mkff(Q.z, Q.w), vy1, vy2);
+    }
+    if (fabsf(f0.h) >= kBig) {
+      ff* const kept[] = {&f0, &f1, &sum, &ux1, &ux2, &uy1, &uy2, &vx1, &vx2, &vy1, &vy2};
+#pragma unroll
+      for (ff* v : kept) *v = ff_scale(*v, kDown);
+    }
+  }
+  const ff norm = ff_add(f0, ff_scale(sum, 2.f * sg2));
+  // u_0 - cos(th) u_1 + sin(th) v_1, over norm
+  auto finish = [&](ff u1, ff u2, ff v1) {
+    return ff_add(ff_add(u1, ff_mul(mkff(-co.h, -co.l), u2)), ff_mul(si, v1));
+  };
+  const double in64 = 1.0 / ff_f64(norm);
+  const ff ax = finish(ux1, ux2, vx1), ay = finish(uy1, uy2, vy1);
+  *dst = cadd(*dst, mk(ff_f64(ax) * in64, ff_f64(ay) * in64));
 }
 
 // ---------------------------------------------------------------- M2P in mixed precision
@@ -2616,7 +2735,7 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     }
   }
   if (f->n_leaves > 0) {
-    unscale_leaf_locals_kernel<<<f->n_leaves, kThreads, 0, s>>>(F, f->leaves.ptr);
+    unscale_leaf_locals_kernel<<<f->n_leaves, kThreads, 0, s>>>(F, f->leaves.ptr, mixed);
     QBX_KCHECK("unscale_leaf_locals", s);
     h->launches += 1;
   }
@@ -2626,7 +2745,12 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   TRY(wait(s, f->ev_out));
   if (f->n_dtgt > 0) {
     stage_begin(h, QBX_STAGE_L2P, s);
-    l2p_kernel<<<nblk(f->n_dtgt, kThreads), kThreads, 0, s>>>(F, f->dtgt.ptr, f->tleaf.ptr, f->n_dtgt, out);
+    if (mixed)
+      l2p_mixed_kernel<<<nblk(f->n_dtgt, kThreads), kThreads, 0, s>>>(F, f->dtgt.ptr, f->tleaf.ptr,
+                                                                      f->n_dtgt, out);
+    else
+      l2p_kernel<<<nblk(f->n_dtgt, kThreads), kThreads, 0, s>>>(F, f->dtgt.ptr, f->tleaf.ptr,
+                                                                f->n_dtgt, out);
     QBX_KCHECK("l2p", s);
     stage_end(h, QBX_STAGE_L2P, s);
     h->launches += 1;

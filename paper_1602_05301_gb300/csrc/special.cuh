@@ -285,6 +285,14 @@ __device__ __forceinline__ int miller_start(int pmax, double x) {
   return (n + 1) & ~1;  // even
 }
 
+// The same from FP32's x, for the float-float recurrences.
+__device__ __forceinline__ int miller_start_f32(int pmax, float x) {
+  const int m = pmax > (int)x ? pmax : (int)x;
+  const int n = 2.0f * x <= (float)m ? m + 2 + (int)ceilf(20.0f / acoshf((float)m / x))
+                                     : m + 12 + (int)ceilf(2.0f * sqrtf(40.0f * x));
+  return (n + 1) & ~1;  // even
+}
+
 // J_0..J_{PM} (entries above p are not used by callers; they are computed anyway).
 template <int PM>
 __device__ __forceinline__ void bessel_j_array(double x, double (&J)[PM + 1]) {
