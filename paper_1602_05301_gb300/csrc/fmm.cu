@@ -101,6 +101,7 @@ struct Fmm {
   const double* conv;    // [n_levels][pbmax + 1] s^j / sig_j (mixed path)
   const double* lsig;    // [n_levels][pbmax + 1] log sig_j
   const double* isig;    // [n_levels][pbmax + 2] 1 / sig_min(j, pb) (mixed P2M)
+  const float2* isf;     // the same times 2^{ffs j}, float-float
   const double2* sigr;   // [n_levels][pbmax + 2] (sig_{j-1} / sig_j, sig_{j+1} / sig_j)
   double k, ik, side;    // wavenumber, 1 / k, root box side
   int pbmax, p, n_levels, has_S, has_D;
@@ -1609,73 +1610,123 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
 }
 
 // ---------------------------------------------------------------- P2M in mixed precision
-// The item structure of p2m_item_kernel with the sums in FP32: the rows
-// R_t = conj(V_t) / sig_|t| (the FP64 Miller recurrence, FP32 from the
-// normalisation on; stored in the first half of each 16-byte row slot) and,
-// over the item's sources with Kahan compensation,
+// The item structure of p2m_item_kernel with rows and sums in FP32:
+// R_t = conj(V_t) / sig_|t| and, over the item's sources with Kahan compensation,
 //   mu_n = sum_j [q_j R_n + A_j R_{n-1} sig_|n-1| / sig_|n| - B_j R_{n+1} sig_|n+1| / sig_|n|],
 // A = d (k/2) conj(nu), B = d (k/2) nu; mu_n = a_n / sig_|n|, of order one.
 // p2m_sum_mixed_kernel adds a leaf's segments in FP64 and forms mh_n = mu_n /
 // conv_|n| (conv = s^j / sig_j).
-__device__ __forceinline__ void p2m_fill_row_mixed(const Fmm& F, int i, double2 m, int l, int pb,
-                                                   cd* row, cd& sq, cd& sa, cd& sb) {
-  const double dx = F.sxy[i].x - m.x, dy = F.sxy[i].y - m.y;
-  const double d2 = dx * dx + dy * dy;
-  const bool at_centre = (__double2hiint(d2) | __double2loint(d2)) == 0;
-  const double ir = at_centre ? 0.0 : rsqrt(d2);
-  const double norm = miller_row(F.k * (d2 * ir), pb + 1, (double*)row, 2);
-  // R_j = J_j / sig_j e^{-i j th} = row_j / (norm sig_j) e^{-i j th}: row_j / sig_j
-  // in FP64 (one product), the factor 2^-e of norm = mn 2^e as an exponent offset
-  // in the FP32 rounding, 1 / mn and the angular factor in FP32
+// Row of source i for a box of level l with centre m: row[t] = R_t, |t| <= pb + 1
+// (row points at t = 0). On float-float levels the Miller recurrence of
+// l2p_mixed_kernel on 2^{-s j} J_j (its values kept in the row while it runs),
+// normalised and brought to J_j / sig_j by isf[j] = 2^{s j} / sig_j; elsewhere in
+// FP64, one product per order, the normalisation as an exponent offset and an
+// FP32 factor. The angular factors e^{-i j th} are FP32 products between
+// float-float anchors every eighth order. (One warp fills an item's rows while the
+// others wait, so the FP64 recurrence's rate set the kernel's: 2^20 sources in 200
+// ellipses 1.25 -> 0.84 ms.)
+__device__ __forceinline__ void p2m_fill_row_mixed(const Fmm& F, const FfUnits& U, int i, double2 m,
+                                                   int l, int pb, float2* row) {
+  const double2 y = F.sxy[i];
+  FfPolar D;
+  const bool off = D.set(y.x - m.x, y.y - m.y, U);
+  const int s = F.ffs[l];
+  const bool in = s != kNoFf && off && D.z.h >= 1e-8f;
+  ff inv = mkff(0.f, 0.f);
+  int en = 0;
+  float imn = 0.f;
+  if (in) {
+    const float sg2 = pow2f(2 * s);
+    ff c2 = ff_mul_raw(ff_scale(U.ik2, pow2f(s)), D.ir);  // 2 2^s / x
+    c2 = fast_two_sum(c2.h, c2.l);
+    const int M = pb + 1, N = miller_start_f32(M, D.z.h);  // N > M + 1
+    ff f1 = mkff(0.f, 0.f), f0 = mkff(0x1p-40f, 0.f), sum = f1;
+    float fn = (float)N;
+    for (int nn = N; nn >= 1; --nn) {
+      if ((nn & 1) == 0) sum = ff_add(f0, ff_scale(sum, sg2));
+      const float ch = __fmul_rn(fn, c2.h);
+      const ff cn = mkff(ch, __fmaf_rn(fn, c2.l, __fmaf_rn(fn, c2.h, -ch)));
+      const ff f = ff_sub_raw(ff_mul_raw(cn, f0), ff_scale(f1, sg2));
+      f1 = f0;
+      f0 = fast_two_sum(f.h, f.l);
+      fn -= 1.f;
+      if (nn - 1 <= M) row[nn - 1] = make_float2(f0.h, f0.l);
+      if (fabsf(f0.h) >= 0x1p20f) {
+        constexpr float d = 0x1p-60f;
+        f0 = ff_scale(f0, d);
+        f1 = ff_scale(f1, d);
+        sum = ff_scale(sum, d);
+        for (int u = nn - 1; u <= M; ++u) row[u] = make_float2(row[u].x * d, row[u].y * d);
+      }
+    }
+    const ff norm = ff_add(f0, ff_scale(sum, 2.f * sg2));
+    const float r = 1.0f / norm.h;  // 1 / norm by one Newton step
+    inv = mkff(r, __fmul_rn(r, __fmaf_rn(-norm.l, r, __fmaf_rn(-norm.h, r, 1.0f))));
+  } else {
+    const double dx = y.x - m.x, dy = y.y - m.y;
+    const double d2 = dx * dx + dy * dy;
+    const double norm = miller_row(F.k * (off ? d2 * rsqrt(d2) : 0.0), pb + 1, (double*)row, 1);
+    en = (int)((__double2hiint(norm) >> 20) & 0x7FF) - 1023;
+    imn = 1.0f / f32_from_f64_sh(norm, -en);
+  }
   const double* isg = F.isig + (size_t)l * (F.pbmax + 2);
-  const int en = (int)((__double2hiint(norm) >> 20) & 0x7FF) - 1023;
-  const float imn = 1.0f / f32_from_f64_sh(norm, -en);
-  // e^{-i j th}: FP64 anchors every eighth order (e^{-8 i th} by three
-  // squarings), FP32 products in between
-  const cd em = at_centre ? mk(1.0, 0.0) : mk(dx * ir, -dy * ir);
-  cd e8 = cmul(em, em);
-  e8 = cmul(e8, e8);
-  e8 = cmul(e8, e8);
-  const float2 emf = f2(em);
-  cd E = mk(1.0, 0.0);
+  const float2* isf = F.isf + (size_t)l * (F.pbmax + 2);
+  const ff c1 = off ? ff_mul(D.x, D.ir) : mkff(1.f, 0.f);
+  const ff s1 = off ? ff_mul(D.y, D.ir) : mkff(0.f, 0.f);
+  auto turn = [](ff& a, ff& b, ff c, ff d) {  // (a + i b) *= c + i d
+    const ff t = ff_sub_raw(ff_mul_raw(a, c), ff_mul_raw(b, d));
+    const ff u = ff_add(ff_mul_raw(a, d), ff_mul_raw(b, c));
+    a = fast_two_sum(t.h, t.l);
+    b = u;
+  };
+  ff c8 = c1, s8 = mkff(-s1.h, -s1.l);  // e^{-8 i th} by three squarings
+#pragma unroll
+  for (int u = 0; u < 3; ++u) turn(c8, s8, c8, s8);
+  const float2 emf = make_float2(ff_f32(c1), -ff_f32(s1));
+  ff ex = mkff(1.f, 0.f), ey = mkff(0.f, 0.f);
   float2 ef = make_float2(1.f, 0.f);
   for (int j = 0; j <= pb + 1; ++j) {
     if ((j & 7) == 0) {
-      ef = f2(E);
-      E = cmul(E, e8);
+      ef = make_float2(ff_f32(ex), ff_f32(ey));
+      turn(ex, ey, c8, s8);
     } else {
       ef = fmul(ef, emf);
     }
-    const float v = f32_from_f64_sh(row[j].x * isg[j], -en) * imn;
+    float v;
+    if (in) {
+      const float2 f = row[j], g = isf[j];
+      v = ff_f32(ff_mul_raw(ff_mul_raw(mkff(f.x, f.y), mkff(g.x, g.y)), inv));
+    } else {
+      v = f32_from_f64_sh(reinterpret_cast<const double*>(row)[j] * isg[j], -en) * imn;
+    }
     const float2 c = make_float2(ef.x * v, ef.y * v);  // R_j
-    reinterpret_cast<float2*>(row + j)[0] = c;
-    if (j > 0) reinterpret_cast<float2*>(row - j)[0] = (j & 1) ? make_float2(-c.x, c.y)
-                                                                : make_float2(c.x, -c.y);
+    row[j] = c;
+    if (j > 0) row[-j] = (j & 1) ? make_float2(-c.x, c.y) : make_float2(c.x, -c.y);
   }
-  const float4 ab = F.ab32[i];
-  reinterpret_cast<float2*>(&sq)[0] = F.q32[i];
-  reinterpret_cast<float2*>(&sa)[0] = make_float2(ab.z, ab.w);  // d (k/2) conj(nu)
-  reinterpret_cast<float2*>(&sb)[0] = make_float2(ab.x, ab.y);  // d (k/2) nu
 }
 
+// Rows and strengths of an item in shared memory: FP32, half the FP64 form's.
 __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
     Fmm F, const int4* __restrict__ items, const int* __restrict__ seg_leaf,
     const int2* __restrict__ seg_row, const long long* __restrict__ seg_poff,
     const int* __restrict__ src, const int* __restrict__ src_leaf, cd* __restrict__ partial,
-    unsigned sm_bytes) {
-  extern __shared__ cd smem[];
+    int chunk) {
+  extern __shared__ __align__(16) float2 fsmem[];
   const int4 it = items[blockIdx.x];
   const int l = F.level[seg_leaf[it.x]];
   const int pb = F.lpb[l], Q = 2 * pb + 1, RW = 2 * pb + 3;
-  const int chunk = rows_chunk(pb, sm_bytes);  // >= it.w
-  cd* rows = smem;                        // [chunk][RW]
-  cd* sq = rows + chunk * RW;             // [chunk]
-  cd* sa = sq + chunk;                    // [chunk]
-  cd* sb = sa + chunk;                    // [chunk]
+  float2* rows = fsmem;                   // [chunk][RW], it.w <= chunk
+  float2* sq = rows + chunk * RW;         // [chunk]
+  float2* sa = sq + chunk;                // [chunk]
+  float2* sb = sa + chunk;                // [chunk]
   if ((int)threadIdx.x < it.w) {
-    const int j = threadIdx.x;
-    p2m_fill_row_mixed(F, src[it.z + j], F.centre[src_leaf[it.z + j]], l, pb,
-                       rows + j * RW + (pb + 1), sq[j], sa[j], sb[j]);
+    const int j = threadIdx.x, i = src[it.z + j];
+    const FfUnits U(F.k);
+    p2m_fill_row_mixed(F, U, i, F.centre[src_leaf[it.z + j]], l, pb, rows + j * RW + (pb + 1));
+    const float4 ab = F.ab32[i];
+    sq[j] = F.q32[i];
+    sa[j] = make_float2(ab.z, ab.w);  // d (k/2) conj(nu)
+    sb[j] = make_float2(ab.x, ab.y);  // d (k/2) nu
   }
   __syncthreads();
   const double2* sr = F.sigr + (size_t)l * (F.pbmax + 2);
@@ -1684,11 +1735,11 @@ __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
     const int2 rg = seg_row[it.x + u];
     float2 Sq = make_float2(0.f, 0.f), Cq = Sq, Sa = Sq, Ca = Sq, Sb = Sq, Cb = Sq;
     for (int j = rg.x; j < rg.x + rg.y; ++j) {
-      const float2* r = reinterpret_cast<const float2*>(rows + j * RW + (pb + 1));
-      if (F.has_S) kahan2(Sq, Cq, fmul(reinterpret_cast<const float2*>(sq + j)[0], r[2 * n]));
+      const float2* r = rows + j * RW + (pb + 1) + n;
+      if (F.has_S) kahan2(Sq, Cq, fmul(sq[j], r[0]));
       if (F.has_D) {
-        kahan2(Sa, Ca, fmul(reinterpret_cast<const float2*>(sa + j)[0], r[2 * (n - 1)]));
-        kahan2(Sb, Cb, fmul(reinterpret_cast<const float2*>(sb + j)[0], r[2 * (n + 1)]));
+        kahan2(Sa, Ca, fmul(sa[j], r[-1]));
+        kahan2(Sb, Cb, fmul(sb[j], r[1]));
       }
     }
     // sig_|n-1| / sig_|n| and sig_|n+1| / sig_|n| (1 beyond order pb)
@@ -2266,6 +2317,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
     for (int b : src_leaves) pbs = std::max(pbs, f->h_pb[blev[b]]);
     f->p2m_sm = rows_launch_smem(pbs);
     const int chunk = rows_chunk(pbs, f->p2m_sm);  // the least capacity over the leaf levels
+    f->p2m_chunk = chunk;
     std::vector<int> sleaf, psrc, psleaf, lseg(src_leaves.size() + 1, 0);
     std::vector<int2> srow;
     std::vector<long long> spoff;
@@ -2408,7 +2460,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.t_m2l = f->t_m2l.ptr; F.t_m2m = f->t_m2m.ptr; F.t_l2l = f->t_l2l.ptr;
   F.mpole = f->mpole.ptr; F.local = f->local.ptr; F.lpq = f->lpq.ptr;
   F.ffs = f->ff_s.ptr;
-  F.conv = f->conv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.sigr = f->sigr.ptr;
+  F.conv = f->conv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.isf = f->isf.ptr; F.sigr = f->sigr.ptr;
   F.k = h->k; F.ik = 1.0 / h->k; F.side = f->side; F.pbmax = f->pb_max; F.p = h->p; F.n_levels = f->n_levels;
   F.has_S = S ? 1 : 0; F.has_D = D ? 1 : 0;
   return F;
@@ -2634,9 +2686,9 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   stage_begin(h, QBX_STAGE_P2M, s);
   if ((S || D) && f->n_p2m_items > 0) {
     if (mixed) {
-      p2m_item_mixed_kernel<<<f->n_p2m_items, kThreads, f->p2m_sm, s>>>(
+      p2m_item_mixed_kernel<<<f->n_p2m_items, kThreads, f->p2m_sm / 2, s>>>(
           F, f->p2m_items.ptr, f->p2m_segleaf.ptr, f->p2m_segrow.ptr, f->p2m_segpoff.ptr,
-          f->p2m_src.ptr, f->p2m_srcleaf.ptr, f->p2m_part.ptr, (unsigned)f->p2m_sm);
+          f->p2m_src.ptr, f->p2m_srcleaf.ptr, f->p2m_part.ptr, f->p2m_chunk);
       QBX_KCHECK("p2m", s);
       p2m_sum_mixed_kernel<<<f->n_src_leaves, kThreads, 0, s>>>(
           F, f->src_leaves.ptr, f->p2m_lseg.ptr, f->p2m_segpoff.ptr, f->p2m_part.ptr);

@@ -104,6 +104,24 @@ __global__ void m2l_f32_matrix_kernel(int l, int pb, int pbmax, const cd* __rest
   }
 }
 
+// isf[l][j] = 2^{s j} isig[l][j] as a pair of FP32, s = ffs[l] (0 on levels without)
+__global__ void isig_ff_kernel(int n_levels, int pbmax, const int* __restrict__ lpb,
+                               const int* __restrict__ ffs, const double* __restrict__ isig,
+                               float2* __restrict__ isf) {
+  const int l = blockIdx.x;
+  if (l >= n_levels) return;
+  const int s = ffs[l];
+  for (int j = threadIdx.x; j < pbmax + 2; j += blockDim.x) {
+    float2 v = make_float2(0.f, 0.f);
+    if (s != kNoFf && j <= lpb[l] + 1) {
+      const double x = ldexp(isig[(size_t)l * (pbmax + 2) + j], s * j);
+      v.x = (float)x;
+      v.y = (float)(x - (double)v.x);
+    }
+    isf[(size_t)l * (pbmax + 2) + j] = v;
+  }
+}
+
 __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
   const float y = v - c;
   const float t = s + y;
@@ -806,6 +824,10 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     QBX_CUDA_TRY(f->ff_s.alloc(f->n_levels));
     QBX_CUDA_TRY(cudaMemcpy(f->ff_s.ptr, ffs.data(), f->n_levels * sizeof(int),
                             cudaMemcpyHostToDevice));
+    QBX_CUDA_TRY(f->isf.alloc((size_t)f->n_levels * (pbm + 2)));
+    isig_ff_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->ff_s.ptr, f->isig.ptr,
+                                         f->isf.ptr);
+    QBX_CUDA_TRY(cudaGetLastError());
   }
   // matrices for the levels that have V lists
   std::vector<long long> off(f->n_levels, 0);

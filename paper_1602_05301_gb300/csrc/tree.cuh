@@ -109,6 +109,7 @@ struct FmmPlan {
   DevBuf<cd> p2m_part;
   int n_p2m_items = 0;
   size_t p2m_sm = 0;
+  int p2m_chunk = 0;                    // most sources of an item
   // xbox and vbox are ordered by level; [n_levels + 1] offsets
   std::vector<int> xbox_off, vbox_off;
   int q_leaf = 1, q_w = 1;              // largest Q_l among leaves / W-list boxes
@@ -162,6 +163,7 @@ struct FmmPlan {
   // mixed precision (sigma-normalised FP32 M2L)
   DevBuf<double> lsig, conv;            // [n_levels][pb_max+1] log sig_j, s^j / sig_j
   DevBuf<double> isig;                  // [n_levels][pb_max+2] 1 / sig_min(j, pb) (mixed P2M)
+  DevBuf<float2> isf;                   // the same times 2^{s j} (s = ff_s), float-float
   DevBuf<float2> tm_f32;                // per level l >= 2: [49][Q_l][Q_l] M2L matrices
   std::vector<long long> h_tm_off;      // [n_levels] offset of level l's matrices
   // M2L as batched GEMMs: V entries grouped by (level, offset class) into
