@@ -122,6 +122,44 @@ __global__ void isig_ff_kernel(int n_levels, int pbmax, const int* __restrict__ 
   }
 }
 
+// Packed pairs of FP32 values (fma.rn.f32x2 and its kin, sm_100 and later): one
+// issue slot for two FMAs, each rounded as the scalar instruction rounds it. The
+// tile GEMMs were bound by issue (64 % of the slots, the FMA pipe at 53 %): M2L of
+// 200 ellipses 4.03 -> 3.37 ms, M2M 0.83 -> 0.70 ms.
+typedef unsigned long long f32p;
+__device__ __forceinline__ f32p pk(float a, float b) {
+  f32p r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpk(f32p v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32p fma2(f32p a, f32p b, f32p c) {
+  f32p r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32p mul2(f32p a, f32p b) {
+  f32p r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32p add2(f32p a, f32p b) {
+  f32p r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32p sub2(f32p a, f32p b) { return fma2(b, pk(-1.f, -1.f), a); }
+__device__ __forceinline__ void kahan_add2(f32p& s, f32p& c, f32p v) {
+  const f32p y = sub2(v, c);
+  const f32p t = add2(s, y);
+  c = sub2(sub2(t, s), y);
+  s = t;
+}
+
 __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
   const float y = v - c;
   const float t = s + y;
@@ -146,67 +184,80 @@ constexpr int kGemmBlock = 8;
 constexpr int kNarrowRows = 4;
 constexpr int kWideLevel = kGemmRows * 2 * 152;
 
-// Staged rows: x[n * stage_stride(R) + r]. Two float2 of padding per n keep
-// the row pairs 16-byte aligned and spread the staging stores over the banks.
+// Staged rows: order n of the row pair (r, r + 1), r even, is the float4 (re r,
+// re r+1, im r, im r+1) at x + n * stage_stride(R) + r, so that each half is an
+// operand of the packed FMAs. Two float2 of padding per n keep the row pairs
+// 16-byte aligned and spread the staging stores over the banks.
 __host__ __device__ constexpr int stage_stride(int R) { return R + 2; }
+__device__ __forceinline__ void stage_put(float2* x, size_t n, int r, int RS, float2 v) {
+  float* f = reinterpret_cast<float*>(x + n * RS + (r & ~1)) + (r & 1);
+  f[0] = v.x;
+  f[2] = v.y;
+}
 
-// One block of nj (1 <= nj <= kGemmBlock) terms of a tile product column:
-// (tr, ti)[r] = sum_{j < nj} tb[j] * x[j * RS + r], started from the first term.
+// Sums of R rows, row pairs packed: value s, Kahan compensation c (the sum is s - c).
 template <int R>
-__device__ __forceinline__ void gemm_block(const float2 (&tb)[kGemmBlock], int nj,
-                                           const float2* __restrict__ x, float (&tr)[R],
-                                           float (&ti)[R]) {
+struct RowSums {
+  f32p sr[R / 2], si[R / 2], cr[R / 2], ci[R / 2];
+  __device__ __forceinline__ RowSums() {
+#pragma unroll
+    for (int r = 0; r < R / 2; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0ull;
+  }
+  __device__ __forceinline__ float sum_r(int r) const { return part(sr[r / 2], r); }
+  __device__ __forceinline__ float sum_i(int r) const { return part(si[r / 2], r); }
+  __device__ __forceinline__ float comp_r(int r) const { return part(cr[r / 2], r); }
+  __device__ __forceinline__ float comp_i(int r) const { return part(ci[r / 2], r); }
+  __device__ static __forceinline__ float part(f32p v, int r) {
+    const float2 u = unpk(v);
+    return (r & 1) ? u.y : u.x;
+  }
+};
+
+// One block of nj (1 <= nj <= kGemmBlock) terms of a tile product column,
+// sum_{j < nj} tb[j] * x[j], started from the first term and added to S with
+// Kahan compensation.
+template <int R>
+__device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], int nj,
+                                               const float2* __restrict__ x, RowSums<R>& S) {
   static_assert(R % 2 == 0, "rows are read in pairs");
   constexpr int RS = stage_stride(R);
+  f32p tr[R / 2], ti[R / 2];
 #pragma unroll
   for (int j = 0; j < kGemmBlock; ++j) {
     if (j < nj) {
-      const float2 t = tb[j];
-      const float4* m = reinterpret_cast<const float4*>(x + j * RS);
+      const f32p tx = pk(tb[j].x, tb[j].x), ty = pk(tb[j].y, tb[j].y);
+      const f32p my = pk(-tb[j].y, -tb[j].y);
+      const ulonglong2* m = reinterpret_cast<const ulonglong2*>(x + j * RS);
 #pragma unroll
-      for (int r2 = 0; r2 < R / 2; ++r2) {
-        const float4 v = m[r2];  // rows 2 r2 (x, y) and 2 r2 + 1 (z, w)
+      for (int r = 0; r < R / 2; ++r) {
+        const ulonglong2 v = m[r];  // (re, re), (im, im) of rows 2r, 2r + 1
         if (j == 0) {
-          tr[2 * r2] = fmaf(t.x, v.x, -t.y * v.y);
-          ti[2 * r2] = fmaf(t.x, v.y, t.y * v.x);
-          tr[2 * r2 + 1] = fmaf(t.x, v.z, -t.y * v.w);
-          ti[2 * r2 + 1] = fmaf(t.x, v.w, t.y * v.z);
+          tr[r] = fma2(tx, v.x, mul2(my, v.y));
+          ti[r] = fma2(tx, v.y, mul2(ty, v.x));
         } else {
-          tr[2 * r2] = fmaf(t.x, v.x, fmaf(-t.y, v.y, tr[2 * r2]));
-          ti[2 * r2] = fmaf(t.x, v.y, fmaf(t.y, v.x, ti[2 * r2]));
-          tr[2 * r2 + 1] = fmaf(t.x, v.z, fmaf(-t.y, v.w, tr[2 * r2 + 1]));
-          ti[2 * r2 + 1] = fmaf(t.x, v.w, fmaf(t.y, v.z, ti[2 * r2 + 1]));
+          tr[r] = fma2(tx, v.x, fma2(my, v.y, tr[r]));
+          ti[r] = fma2(tx, v.y, fma2(ty, v.x, ti[r]));
         }
       }
     }
   }
-}
-
-template <int R>
-__device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], int nj,
-                                               const float2* __restrict__ x, float (&sr)[R],
-                                               float (&si)[R], float (&cr)[R], float (&ci)[R]) {
-  float tr[R], ti[R];
-  gemm_block<R>(tb, nj, x, tr, ti);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    kahan_add(sr[r], cr[r], tr[r]);
-    kahan_add(si[r], ci[r], ti[r]);
+  for (int r = 0; r < R / 2; ++r) {
+    kahan_add2(S.sr[r], S.cr[r], tr[r]);
+    kahan_add2(S.si[r], S.ci[r], ti[r]);
   }
 }
 
 // One output column lo of a tile product: for every row r < R,
-// (sr, si)[r] += sum_{n < N} M[n * ld + lo] * x[n * RS + r], with x in
-// shared memory (16-byte aligned, RS = stage_stride(R)). Plain FP32 FMAs over
-// blocks of kGemmBlock terms (whose matrix entries are loaded one block ahead,
-// into two alternating register sets), the blocks added with Kahan
-// compensation (cr, ci). Threads with act == false read column 0 and their
-// sums are not used.
+// S[r] += sum_{n < N} M[n * ld + lo] * x[n][r], with x in shared memory (16-byte
+// aligned, stage_put's layout). Packed FP32 FMAs over blocks of kGemmBlock terms
+// (whose matrix entries are loaded one block ahead, into two alternating
+// register sets), the blocks added with Kahan compensation. Threads with
+// act == false read column 0 and their sums are not used.
 template <int R = kGemmRows>
 __device__ __forceinline__ void tile_gemm_column(const float2* __restrict__ M, size_t ld, int N,
                                                  const float2* __restrict__ x, int lo, bool act,
-                                                 float (&sr)[R], float (&si)[R], float (&cr)[R],
-                                                 float (&ci)[R]) {
+                                                 RowSums<R>& S) {
   constexpr int RS = stage_stride(R);
   const float2* Mc = M + (act ? lo : 0);
   const int nfull = N - N % kGemmBlock;
@@ -221,20 +272,20 @@ __device__ __forceinline__ void tile_gemm_column(const float2* __restrict__ M, s
 #pragma unroll
       for (int j = 0; j < kGemmBlock; ++j) bb[j] = Mc[(size_t)(n1 + j) * ld];
     }
-    gemm_block_add<R>(ba, kGemmBlock, x + n0 * RS, sr, si, cr, ci);
+    gemm_block_add<R>(ba, kGemmBlock, x + n0 * RS, S);
     if (n1 >= nfull) break;
     if (n1 + kGemmBlock < nfull) {
 #pragma unroll
       for (int j = 0; j < kGemmBlock; ++j) ba[j] = Mc[(size_t)(n1 + kGemmBlock + j) * ld];
     }
-    gemm_block_add<R>(bb, kGemmBlock, x + n1 * RS, sr, si, cr, ci);
+    gemm_block_add<R>(bb, kGemmBlock, x + n1 * RS, S);
   }
   if (nfull < N) {  // the last, partial block
     const int nj = N - nfull;
 #pragma unroll
     for (int j = 0; j < kGemmBlock; ++j)
       ba[j] = j < nj ? Mc[(size_t)(nfull + j) * ld] : make_float2(0.f, 0.f);
-    gemm_block_add<R>(ba, nj, x + nfull * RS, sr, si, cr, ci);
+    gemm_block_add<R>(ba, nj, x + nfull * RS, S);
   }
 }
 
@@ -283,9 +334,7 @@ __global__ void __launch_bounds__(kT, 4) m2l_f32_gemm_kernel(
   // costs its warp the same however few lanes are active
   const bool warp_act = I.z + (int)(threadIdx.x & ~31u) < Q;
   const float2* M = tm + goff[I.w];
-  float sr[kGemmRows], si[kGemmRows], cr[kGemmRows], ci[kGemmRows];
-#pragma unroll
-  for (int r = 0; r < kGemmRows; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0.f;
+  RowSums<kGemmRows> S;
   for (int n0 = 0; n0 < Q; n0 += kChunkK) {
     const int nk = min(kChunkK, Q - n0);
     __syncthreads();
@@ -293,15 +342,17 @@ __global__ void __launch_bounds__(kT, 4) m2l_f32_gemm_kernel(
       const int r = 2 * (idx / nk), n = idx % nk;  // coalesced reads along each source row
       const float2 a = r < nr ? mu32[row_off[row0 + r] + n0 + n] : make_float2(0.f, 0.f);
       const float2 b = r + 1 < nr ? mu32[row_off[row0 + r + 1] + n0 + n] : make_float2(0.f, 0.f);
-      *reinterpret_cast<float4*>(mu + n * RS + r) = make_float4(a.x, a.y, b.x, b.y);
+      *reinterpret_cast<float4*>(mu + n * RS + r) = make_float4(a.x, b.x, a.y, b.y);
     }
     __syncthreads();
-    if (warp_act) tile_gemm_column(M + (size_t)n0 * Q, Q, nk, mu, lo, act, sr, si, cr, ci);
+    if (warp_act) tile_gemm_column(M + (size_t)n0 * Q, Q, nk, mu, lo, act, S);
   }
   if (act) {
 #pragma unroll
     for (int r = 0; r < kGemmRows; ++r)
-      if (r < nr) Y[yoff[row0 + r] + lo] = make_float2(sr[r] - cr[r], si[r] - ci[r]);
+      if (r < nr)
+        Y[yoff[row0 + r] + lo] =
+            make_float2(S.sum_r(r) - S.comp_r(r), S.sum_i(r) - S.comp_i(r));
   }
 }
 
@@ -493,7 +544,7 @@ __global__ void __launch_bounds__(kT) l2l_f32_kernel(
       const double f = 1.0 / cvp[abs(n - pp)];
       v = make_float2((float)(g.x * f), (float)(g.y * f));
     }
-    lam[n * stage_stride(R) + r] = v;
+    stage_put(lam, n, r, stage_stride(R), v);
   }
   __syncthreads();
   {
@@ -502,10 +553,8 @@ __global__ void __launch_bounds__(kT) l2l_f32_kernel(
     {
       const int so = (int)blockIdx.z * kT + threadIdx.x;  // output chunk blockIdx.z
       const bool act = so < Qc;
-      float sr[R], si[R], cr[R], ci[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0.f;
-      tile_gemm_column<R>(M, Qc, Qp, lam, so, act, sr, si, cr, ci);
+      RowSums<R> S;
+      tile_gemm_column<R>(M, Qc, Qp, lam, so, act, S);
       if (act) {
         const double f = cvc[abs(so - pc)];
 #pragma unroll
@@ -514,8 +563,8 @@ __global__ void __launch_bounds__(kT) l2l_f32_kernel(
           const int d = child[4 * parents[p0 + r] + c];
           if (d < 0) continue;
           cd* dl = local + eoff[d] + so;
-          dl->x += ((double)sr[r] - (double)cr[r]) * f;
-          dl->y += ((double)si[r] - (double)ci[r]) * f;
+          dl->x += ((double)S.sum_r(r) - (double)S.comp_r(r)) * f;
+          dl->y += ((double)S.sum_i(r) - (double)S.comp_i(r)) * f;
         }
       }
     }
@@ -580,9 +629,7 @@ __global__ void __launch_bounds__(kT) m2m_f32_kernel(
   {
     const int so = (int)blockIdx.y * kT + threadIdx.x;  // output chunk blockIdx.y
     const bool act = so < Qp;
-    float sr[R], si[R], cr[R], ci[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0.f;
+    RowSums<R> S;
     for (int c = 0; c < 4; ++c) {
       __syncthreads();
       for (int idx = threadIdx.x; idx < Qc * R; idx += kT) {
@@ -594,10 +641,10 @@ __global__ void __launch_bounds__(kT) m2m_f32_kernel(
           const double f = cvc[abs(n - pc)];
           v = make_float2((float)(a.x * f), (float)(a.y * f));
         }
-        mus[n * stage_stride(R) + r] = v;
+        stage_put(mus, n, r, stage_stride(R), v);
       }
       __syncthreads();
-      tile_gemm_column<R>(Tmm + (size_t)c * Qc * Qp, Qp, Qc, mus, so, act, sr, si, cr, ci);
+      tile_gemm_column<R>(Tmm + (size_t)c * Qc * Qp, Qp, Qc, mus, so, act, S);
     }
     if (act) {
       const double f = 1.0 / cvp[abs(so - pp)];
@@ -605,8 +652,8 @@ __global__ void __launch_bounds__(kT) m2m_f32_kernel(
       for (int r = 0; r < R; ++r) {
         if (r >= nr) break;
         cd* dst = mpole + poff[r] + so;
-        dst->x = ((double)sr[r] - (double)cr[r]) * f;
-        dst->y = ((double)si[r] - (double)ci[r]) * f;
+        dst->x = ((double)S.sum_r(r) - (double)S.comp_r(r)) * f;
+        dst->y = ((double)S.sum_i(r) - (double)S.comp_i(r)) * f;
       }
     }
   }
@@ -622,13 +669,13 @@ __global__ void __launch_bounds__(kT) m2m_f32_kernel(
 constexpr int kSplitCols = 32, kSplitWarps = kT / 32;
 
 template <int R>
-__device__ __forceinline__ void split_reduce(float (&sr)[R], float (&si)[R], float (&cr)[R],
-                                             float (&ci)[R], float2* red, int warp, int lane,
+__device__ __forceinline__ void split_reduce(const RowSums<R>& S, float2* red, int warp, int lane,
                                              double (&outr)[R], double (&outi)[R]) {
   // red: [kSplitWarps][R][32]
 #pragma unroll
   for (int r = 0; r < R; ++r)
-    red[(warp * R + r) * 32 + lane] = make_float2(sr[r] - cr[r], si[r] - ci[r]);
+    red[(warp * R + r) * 32 + lane] =
+        make_float2(S.sum_r(r) - S.comp_r(r), S.sum_i(r) - S.comp_i(r));
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -679,19 +726,17 @@ __global__ void __launch_bounds__(kT) m2m_f32_split_kernel(
       const double f = cvc[abs(n - pc)];
       v = make_float2((float)(a.x * f), (float)(a.y * f));
     }
-    mus4[((size_t)c * Qc + n) * RS + r] = v;
+    stage_put(mus4, (size_t)c * Qc + n, r, RS, v);
   }
   __syncthreads();
   const int so = (int)blockIdx.y * kSplitCols + lane;
   const bool act = so < Qp;
-  float sr[R], si[R], cr[R], ci[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0.f;
+  RowSums<R> S;
   tile_gemm_column<R>(Tmm + (size_t)warp * Qc * Qp, Qp, Qc, mus4 + (size_t)warp * Qc * RS, so,
-                      act, sr, si, cr, ci);
+                      act, S);
   __syncthreads();  // the staged rows are dead: the reduction reuses the space
   double outr[R], outi[R];
-  split_reduce<R>(sr, si, cr, ci, mus4, warp, lane, outr, outi);
+  split_reduce<R>(S, mus4, warp, lane, outr, outi);
   if (warp == 0 && act) {
     const double f = 1.0 / cvp[abs(so - pp)];
 #pragma unroll
@@ -724,7 +769,7 @@ __global__ void __launch_bounds__(kT) l2l_f32_split_kernel(
       const double f = 1.0 / cvp[abs(n - pp)];
       v = make_float2((float)(g.x * f), (float)(g.y * f));
     }
-    lam2[n * RS + r] = v;
+    stage_put(lam2, n, r, RS, v);
   }
   __syncthreads();
   const int c = blockIdx.y;
@@ -733,15 +778,13 @@ __global__ void __launch_bounds__(kT) l2l_f32_split_kernel(
   // warp w: parent orders [n0, n1)
   const int per = (Qp + kSplitWarps - 1) / kSplitWarps;
   const int n0 = min(Qp, warp * per), n1 = min(Qp, n0 + per);
-  float sr[R], si[R], cr[R], ci[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0.f;
+  RowSums<R> S;
   if (n1 > n0)
     tile_gemm_column<R>(Tl + (size_t)c * Qp * Qc + (size_t)n0 * Qc, Qc, n1 - n0, lam2 + n0 * RS,
-                        so, act, sr, si, cr, ci);
+                        so, act, S);
   __syncthreads();
   double outr[R], outi[R];
-  split_reduce<R>(sr, si, cr, ci, lam2, warp, lane, outr, outi);
+  split_reduce<R>(S, lam2, warp, lane, outr, outi);
   if (warp == 0 && act) {
     const double f = cvc[abs(so - pc)];
 #pragma unroll
