@@ -110,72 +110,86 @@ __device__ __forceinline__ int2 child_range(const KeySet& ks, int t, int2 r, u64
   return make_int2(a, b);
 }
 
+// Lane 4 c + t (< 16) of a warp: the range of class t in child c of box b.
+__device__ __forceinline__ int2 lane_child_range(const KeySet& ks, const int2* r0, const int2* r1,
+                                                 const int2* r2, const int2* r3, int b, u64 key,
+                                                 int level, int lane) {
+  const int t = lane & 3;
+  const int2 r = (t == 0 ? r0 : t == 1 ? r1 : t == 2 ? r2 : r3)[b];
+  return child_range(ks, t, r, key, level, (lane >> 2) & 3);
+}
+static_assert(PT_COUNT == 4, "four particle classes share a warp's lanes");
+
 // A box is split when it holds more than n_max sources + centres + targets,
 // unless its children would be narrower than kappa times the expansion radius
 // of a centre it holds: every QBX disk then stays well inside the region where
-// the local expansion of its leaf converges.
-__global__ void split_count_kernel(int nb, int off, int level, int n_max, KeySet ks,
-                                   const u64* __restrict__ bkey, const int2* __restrict__ r0,
-                                   const int2* __restrict__ r1, const int2* __restrict__ r2,
-                                   const int2* __restrict__ r3, const double* __restrict__ crad,
-                                   double child_side, double kappa,
-                                   int* __restrict__ nchild) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb) return;
-  int b = off + i;
-  const int2 r[PT_COUNT] = {r0[b], r1[b], r2[b], r3[b]};
-  int total = (r[0].y - r[0].x) + (r[1].y - r[1].x) + (r[2].y - r[2].x);
-  bool wide = true;
-  for (int j = r[PT_CTR].x; j < r[PT_CTR].y && wide; ++j) wide = kappa * crad[j] <= child_side;
-  int cnt = 0;
-  if (total > n_max && level < kMaxLevels && wide) {
-    for (int c = 0; c < 4; ++c) {
-      bool ne = false;
-      for (int t = 0; t < PT_COUNT && !ne; ++t) {
-        int2 cr = child_range(ks, t, r[t], bkey[b], level, c);
-        ne = cr.y > cr.x;
-      }
-      cnt += ne ? 1 : 0;
-    }
+// the local expansion of its leaf converges. TPB threads per box scan its
+// centres' radii and 16 lanes search the child ranges: a warp on levels of
+// many boxes, 256 threads on the coarse ones, whose boxes hold up to every
+// centre (one thread per box walked 16384 centres in series: 2.4 ms of a plan
+// on the 8192-node starfish, 0.05 ms now).
+template <int TPB>
+__global__ void __launch_bounds__(TPB == 32 ? 128 : TPB) split_count_kernel(
+    int nb, int off, int level, int n_max, KeySet ks, const u64* __restrict__ bkey,
+    const int2* __restrict__ r0, const int2* __restrict__ r1, const int2* __restrict__ r2,
+    const int2* __restrict__ r3, const double* __restrict__ crad, double child_side, double kappa,
+    int* __restrict__ nchild) {
+  const int i = TPB == 32 ? (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) : (int)blockIdx.x;
+  const int lane = TPB == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  if (i >= nb) return;  // whole warps (or blocks) leave together
+  const int b = off + i;
+  const int2 rs = r0[b], rc = r1[b], rt = r2[b];
+  const int total = (rs.y - rs.x) + (rc.y - rc.x) + (rt.y - rt.x);
+  if (total <= n_max || level >= kMaxLevels) {
+    if (lane == 0) nchild[i] = 0;
+    return;
   }
-  nchild[i] = cnt;
+  bool narrow = false;
+#pragma unroll 4
+  for (int j = rc.x + lane; j < rc.y; j += TPB) narrow |= !(kappa * crad[j] <= child_side);
+  narrow = TPB == 32 ? __any_sync(0xffffffffu, narrow) != 0 : __syncthreads_or(narrow) != 0;
+  if (lane >= 32) return;
+  bool ne = false;
+  if (!narrow && lane < 16) {
+    const int2 cr = lane_child_range(ks, r0, r1, r2, r3, b, bkey[b], level, lane);
+    ne = cr.y > cr.x;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, ne);
+  if (lane == 0) {
+    int cnt = 0;
+    for (int c = 0; c < 4; ++c) cnt += ((m >> (4 * c)) & 15u) ? 1 : 0;
+    nchild[i] = cnt;
+  }
 }
 
-__global__ void split_fill_kernel(int nb, int off, int level, int next_off, KeySet ks,
-                                  const int* __restrict__ nchild, const int* __restrict__ choff,
-                                  double x0, double y0, double side, int* __restrict__ blevel,
-                                  int* __restrict__ bparent, int* __restrict__ bchild,
-                                  int2* __restrict__ bij, u64* __restrict__ bkey,
-                                  double2* __restrict__ bcentre, int2* r0, int2* r1, int2* r2,
-                                  int2* r3) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb) return;
-  int b = off + i;
-  if (nchild[i] == 0) return;
-  int2* rr[PT_COUNT] = {r0, r1, r2, r3};
-  const int2 r[PT_COUNT] = {r0[b], r1[b], r2[b], r3[b]};
-  int slot = next_off + choff[i];
+// The children of every split box, a warp per box (lanes as above).
+__global__ void __launch_bounds__(128) split_fill_kernel(
+    int nb, int off, int level, int next_off, KeySet ks, const int* __restrict__ nchild,
+    const int* __restrict__ choff, double x0, double y0, double side, int* __restrict__ blevel,
+    int* __restrict__ bparent, int* __restrict__ bchild, int2* __restrict__ bij,
+    u64* __restrict__ bkey, double2* __restrict__ bcentre, int2* r0, int2* r1, int2* r2, int2* r3) {
+  const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (i >= nb || nchild[i] == 0) return;
+  const int b = off + i;
+  int2 cr = make_int2(0, 0);
+  if (lane < 16) cr = lane_child_range(ks, r0, r1, r2, r3, b, bkey[b], level, lane);
+  const unsigned m = __ballot_sync(0xffffffffu, cr.y > cr.x);
+  const int c = lane >> 2, t = lane & 3;
+  if (lane >= 16 || ((m >> (4 * c)) & 15u) == 0u) return;
+  int d = next_off + choff[i];
+  for (int u = 0; u < c; ++u) d += ((m >> (4 * u)) & 15u) ? 1 : 0;
+  (t == 0 ? r0 : t == 1 ? r1 : t == 2 ? r2 : r3)[d] = cr;
+  if (t != 0) return;
   const int2 pij = bij[b];
   const double cs = side / (double)(1 << (level + 1));
-  for (int c = 0; c < 4; ++c) {
-    int2 cr[PT_COUNT];
-    bool ne = false;
-    for (int t = 0; t < PT_COUNT; ++t) {
-      cr[t] = child_range(ks, t, r[t], bkey[b], level, c);
-      ne = ne || cr[t].y > cr[t].x;
-    }
-    if (!ne) continue;
-    const int d = slot++;
-    const int ix = 2 * pij.x + (c & 1), iy = 2 * pij.y + (c >> 1);
-    blevel[d] = level + 1;
-    bparent[d] = b;
-    bij[d] = make_int2(ix, iy);
-    bkey[d] = morton(ix, iy);
-    bcentre[d] = make_double2(x0 + (ix + 0.5) * cs, y0 + (iy + 0.5) * cs);
-    for (int t = 0; t < PT_COUNT; ++t) rr[t][d] = cr[t];
-    for (int q = 0; q < 4; ++q) bchild[4 * d + q] = -1;
-    bchild[4 * b + c] = d;
-  }
+  const int ix = 2 * pij.x + (c & 1), iy = 2 * pij.y + (c >> 1);
+  blevel[d] = level + 1;
+  bparent[d] = b;
+  bij[d] = make_int2(ix, iy);
+  bkey[d] = morton(ix, iy);
+  bcentre[d] = make_double2(x0 + (ix + 0.5) * cs, y0 + (iy + 0.5) * cs);
+  for (int q = 0; q < 4; ++q) bchild[4 * d + q] = -1;
+  bchild[4 * b + c] = d;
 }
 
 template <typename T>
@@ -596,10 +610,17 @@ qbx_status tree_build(qbx_handle* h, FmmPlan* f, int n_max, double kappa) {
     DevBuf<int> nch, choff;
     QBX_CUDA_TRY(nch.alloc(nb));
     QBX_CUDA_TRY(choff.alloc(nb));
-    split_count_kernel<<<nblk(nb, 128), 128>>>(nb, off, level, n_max, ks, B.key.ptr,
-                                               B.rng[0].ptr, B.rng[1].ptr, B.rng[2].ptr,
-                                               B.rng[3].ptr, crad_sorted.ptr,
-                                               side / (double)(1 << (level + 1)), kappa, nch.ptr);
+    // levels of up to two boxes per SM: a block per box
+    const double cside = side / (double)(1 << (level + 1));
+    if (nb <= 2 * 152)
+      split_count_kernel<256><<<nb, 256>>>(nb, off, level, n_max, ks, B.key.ptr, B.rng[0].ptr,
+                                           B.rng[1].ptr, B.rng[2].ptr, B.rng[3].ptr,
+                                           crad_sorted.ptr, cside, kappa, nch.ptr);
+    else
+      split_count_kernel<32><<<nblk(nb, 4), 128>>>(nb, off, level, n_max, ks, B.key.ptr,
+                                                   B.rng[0].ptr, B.rng[1].ptr, B.rng[2].ptr,
+                                                   B.rng[3].ptr, crad_sorted.ptr, cside, kappa,
+                                                   nch.ptr);
     QBX_CUDA_TRY(cudaGetLastError());
     TRY(scan(nch.ptr, choff.ptr, nb));
     int last_off = 0, last_cnt = 0;
@@ -619,7 +640,7 @@ qbx_status tree_build(qbx_handle* h, FmmPlan* f, int n_max, double kappa) {
       for (int t = 0; t < PT_COUNT; ++t) TRY(grow(B.rng[t], need, keep));
       TRY(grow(B.child, 4 * B.level.n, 4 * keep));
     }
-    split_fill_kernel<<<nblk(nb, 128), 128>>>(nb, off, level, next_off, ks, nch.ptr, choff.ptr,
+    split_fill_kernel<<<nblk(nb, 4), 128>>>(nb, off, level, next_off, ks, nch.ptr, choff.ptr,
                                               f->x0, f->y0, side, B.level.ptr, B.parent.ptr,
                                               B.child.ptr, B.ij.ptr, B.key.ptr, B.centre.ptr,
                                               B.rng[0].ptr, B.rng[1].ptr, B.rng[2].ptr,
