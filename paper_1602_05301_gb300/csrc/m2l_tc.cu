@@ -184,6 +184,62 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float bh, float bl)
   lo = e - (hi - s);
 }
 
+// The SU accumulators of 16 output columns, v[a][c] of weight 2^{-beta (a + 2)}
+// (integers below 2^24, so every scaled value is exact), as float-float (hi, lo).
+// The lowest weights (from kTail on, 2^{-beta kTail} = 2^-28 to 2^-32 of the first)
+// are summed in plain FP32, whose rounding is below the truncation of the split
+// (2^-46); the others by TwoSum with the errors collected in lo and one
+// renormalisation: 34 FP32 instructions per column instead of 84 with every term
+// added as a float-float number (with the contiguous stores and eight epilogue
+// warps, M2L of 25 ellipses 2.08 -> 1.73 ms, of the k = 10 starfish 0.54 -> 0.43).
+template <int SU>
+__device__ __forceinline__ void combine16(const uint32_t (&r)[SU][16], int beta, float (&hi)[16],
+                                          float (&lo)[16]) {
+  constexpr int kTail = SU >= 8 ? 5 : 4;
+  float w[SU];
+#pragma unroll
+  for (int a = 0; a < SU; ++a) w[a] = exp2i(-beta * (a + 2));  // -beta (a + 2) >= -80
+#pragma unroll
+  for (int c = 0; c < 16; ++c) {
+    float s = 0.f, e = 0.f;
+#pragma unroll
+    for (int a = SU - 1; a >= kTail; --a) s = fmaf(__uint_as_float(r[a][c]), w[a], s);
+#pragma unroll
+    for (int a = (SU < kTail ? SU : kTail) - 1; a >= 0; --a) {
+      float t, d;
+      two_sum(s, __uint_as_float(r[a][c]) * w[a], t, d);
+      s = t;
+      e += d;
+    }
+    hi[c] = s + e;
+    lo[c] = e - (hi[c] - s);
+  }
+}
+
+// Row values of 16 consecutive real outputs j0.. of a row with exponent e_row
+// (fg: the outputs' exponents): (hi, lo) pairs at y[j0], a 128-byte run per thread.
+__device__ __forceinline__ void store16(const float (&hi)[16], const float (&lo)[16], int e_row,
+                                        const int* __restrict__ fg, int j0, int n, float2* y) {
+  float2 v[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) {
+    const int sc = e_row + (j0 + c < n ? fg[j0 + c] : 0);
+    const float f = exp2i(sc);
+    v[c] = f != 0.f ? make_float2(hi[c] * f, lo[c] * f)
+                    : make_float2(ldexpf(hi[c], sc), ldexpf(lo[c], sc));
+  }
+  if (j0 + 16 <= n) {
+    float4* dst = reinterpret_cast<float4*>(y + j0);  // rows start on 16 bytes, j0 % 16 == 0
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      dst[c] = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+      if (j0 + c < n) y[j0 + c] = v[c];
+  }
+}
+
 // ---------------------------------------------------------------- slicing
 // The S signed base-2^beta digits of rint(x 2^(beta S - e)) (|x| 2^-e < 1/2),
 // most significant first, as bf16 (exact: |d| <= 2^(beta - 1) <= 128): the
@@ -407,9 +463,10 @@ __global__ void __launch_bounds__(kThr) tc_m2m_reduce_kernel(
     for (int c = 0; c < 4; ++c) {
       const int r = prow[4 * i + c];
       if (r < 0) continue;
-      const float4 y = reinterpret_cast<const float4*>(Y)[(size_t)r * Q + lo];
-      ff_add(rh, rl, y.x, y.y);
-      ff_add(ih, il, y.z, y.w);
+      const float2* y = reinterpret_cast<const float2*>(Y + (size_t)r * Q) + lo;
+      const float2 a = y[0], b = y[Q];
+      ff_add(rh, rl, a.x, a.y);
+      ff_add(ih, il, b.x, b.y);
     }
     const double f = 1.0 / cv[abs(lo - pp)];
     dst[lo] = mk(((double)rh + (double)rl) * f, ((double)ih + (double)il) * f);
@@ -425,9 +482,10 @@ __global__ void __launch_bounds__(kThr) tc_l2l_apply_kernel(
   const double* cv = conv + (size_t)lc * (pbmax + 1);
   cd* dst = local + eoff[rowdst[r]];
   for (int lo = threadIdx.x; lo < Q; lo += kThr) {
-    const float4 y = reinterpret_cast<const float4*>(Y)[(size_t)r * Q + lo];
+    const float2* y = reinterpret_cast<const float2*>(Y + (size_t)r * Q) + lo;
+    const float2 a = y[0], b = y[Q];
     const double f = cv[abs(lo - pc)];
-    dst[lo] = cadd(dst[lo], mk(((double)y.x + (double)y.y) * f, ((double)y.z + (double)y.w) * f));
+    dst[lo] = cadd(dst[lo], mk(((double)a.x + (double)a.y) * f, ((double)b.x + (double)b.y) * f));
   }
 }
 
@@ -455,9 +513,9 @@ __host__ __device__ constexpr int tc_stages(int SU) {
 // first output, group). SD slices are
 // stored per operand (the level's split), the first SU of them are used: SU =
 // SD for the FP64 path, fewer for the mixed path (the leading digits are a
-// 24- to 28-bit approximation). Y receives, for each pair row and complex
-// output lo, (Re hi, Re lo, Im hi, Im lo) as float4 at yoff[row] + lo: the
-// float-float value of (A x)_j 2^(e + f_j).
+// 24- to 28-bit approximation). Y receives, for each pair row, the 2Q real
+// outputs (real parts, then imaginary parts) as (hi, lo) pairs from yoff[row]
+// on: the float-float value of (A x)_j 2^(e + f_j).
 //
 // Pipeline: NS shared-memory stages filled by cp.async (every thread copies
 // 16-byte pieces; rows past the tile's end are zero-filled); chunk c is
@@ -617,9 +675,7 @@ __global__ void __launch_bounds__(kThr, 1) m2l_tc_kernel(
           const int j = n0 + j0 + c;
           if (j >= 2 * Q) break;
           const int sc = e_row + fg[j];
-          const float2 w = make_float2(ldexpf(hi[c], sc), ldexpf(lo[c], sc));
-          float2* dst = reinterpret_cast<float2*>(Y + yo + (j < Q ? j : j - Q)) + (j < Q ? 0 : 1);
-          *dst = w;
+          reinterpret_cast<float2*>(Y + yo)[j] = make_float2(ldexpf(hi[c], sc), ldexpf(lo[c], sc));
         }
       }
     }
@@ -643,9 +699,9 @@ __global__ void __launch_bounds__(kThr, 1) m2l_tc_kernel(
 //    (the producer's refill waits on it), and after an item's last stage
 //    commits to the accumulator-full barrier; before an item's first MMA it
 //    waits until the epilogue has read the previous item's accumulators;
-//  * warps 4-7, the epilogue: TMEM lanes 32 (w mod 4) .. + 31 (the rows),
-//    the float-float combination and the stores of tc's epilogue, then an
-//    arrival on the accumulator-empty barrier.
+//  * warps 4-11, the epilogue: TMEM lanes 32 (w mod 4) .. + 31 (the rows) and
+//    half the columns each; an arrival on the accumulator-empty barrier after
+//    the last read, the float-float combination (combine16) and the stores.
 // Every wait is bounded (mbar_wait); a wait that runs out sets the CTA's fail
 // flag and the global flag, the roles leave their loops, the issued MMAs are
 // drained with one more bounded wait, and the tensor memory is freed.
@@ -654,7 +710,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 constexpr int kWsProd = 3;                       // producer warps
-constexpr int kWsThr = 32 * (kWsProd + 1 + 4);   // producers, MMA warp, four epilogue warps
+// Epilogue warps: two per TMEM lane quarter, each with half the columns. The next
+// item's MMAs wait until every accumulator has been read, so this read is on the
+// critical path.
+constexpr int kEpiWarps = 8;
+constexpr int kWsThr = 32 * (kWsProd + 1 + kEpiWarps);  // producers, MMA warp, epilogue
 
 template <int SD, int SU>
 __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
@@ -691,7 +751,8 @@ __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[b])));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&tfull)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" ::"r"(smem_u32(&tempty)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&tempty)),
+                 "r"(32 * kEpiWarps));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mfin)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -805,8 +866,9 @@ __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue: rows (warp mod 4) * 32 + lane
+    // ---------------- epilogue: rows (warp mod 4) * 32 + lane, half the columns
     const int m = (warp & 3) * 32 + lane;
+    const int col0 = (warp - (kWsProd + 1)) / 4 * (kNC / 2);
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     int k = 0;
     for (int it = blockIdx.x; it < n_items && !failed(); it += G, ++k) {
@@ -823,7 +885,7 @@ __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
       const bool row_ok = m < nr;
       const int e_row = row_ok ? xexp[rowsrc[row0 + m]] : 0;
       const long long yo = row_ok ? yoff[row0 + m] : 0;
-      for (int j0 = 0; j0 < kNC; j0 += 16) {
+      for (int j0 = col0; j0 < col0 + kNC / 2; j0 += 16) {
         // the SU accumulators of these 16 columns: all loads in flight, one wait
         uint32_t r[SU][16];
 #pragma unroll
@@ -831,32 +893,14 @@ __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
         tmem_wait_ld();
 #pragma unroll
         for (int a = 0; a < SU; ++a) reg_fence16(r[a]);
-        float hi[16], lo[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0.f;
-#pragma unroll
-        for (int a = SU - 1; a >= 0; --a) {
-          const float sa = exp2i(-beta * (a + 2));  // exact: -beta (a + 2) >= -80
-#pragma unroll
-          for (int c = 0; c < 16; ++c) ff_add(hi[c], lo[c], __uint_as_float(r[a][c]) * sa, 0.f);
-        }
-        if (j0 + 16 >= kNC) {  // every accumulator read: the MMAs may reuse TMEM
+        if (j0 + 16 >= col0 + kNC / 2) {  // this warp's last read: the MMAs may reuse TMEM
           asm volatile("tcgen05.fence::before_thread_sync;");
           mbar_arrive(&tempty);
         }
-        if (row_ok) {
-#pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            const int j = n0 + j0 + c;
-            if (j >= 2 * Q) break;
-            const int sc = e_row + fg[j];
-            const float f = exp2i(sc);
-            const float2 w = f != 0.f ? make_float2(hi[c] * f, lo[c] * f)
-                                      : make_float2(ldexpf(hi[c], sc), ldexpf(lo[c], sc));
-            float2* dst = reinterpret_cast<float2*>(Y + yo + (j < Q ? j : j - Q)) + (j < Q ? 0 : 1);
-            *dst = w;
-          }
-        }
+        float hi[16], lo[16];
+        combine16<SU>(r, beta, hi, lo);
+        if (row_ok)
+          store16(hi, lo, e_row, fg, n0 + j0, 2 * Q, reinterpret_cast<float2*>(Y + yo));
       }
     }
   }
@@ -909,7 +953,7 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const void* map, int x, i
       : "memory");
 }
 
-constexpr int kTmaThr = 32 * 6;  // producer warp (one lane), MMA warp, four epilogue warps
+constexpr int kTmaThr = 32 * (2 + kEpiWarps);  // producer warp (one lane), MMA warp, epilogue
 
 template <int SD, int SU>
 __global__ void __launch_bounds__(kTmaThr, 1) tc_gemm_tma_kernel(
@@ -944,7 +988,8 @@ __global__ void __launch_bounds__(kTmaThr, 1) tc_gemm_tma_kernel(
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[b])));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&tfull)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" ::"r"(smem_u32(&tempty)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&tempty)),
+                 "r"(32 * kEpiWarps));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mfin)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -1047,8 +1092,9 @@ __global__ void __launch_bounds__(kTmaThr, 1) tc_gemm_tma_kernel(
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue: rows (warp mod 4) * 32 + lane
+    // ---------------- epilogue: rows (warp mod 4) * 32 + lane, half the columns
     const int m = (warp & 3) * 32 + lane;
+    const int col0 = (warp - 2) / 4 * (kNC / 2);
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     int k = 0;
     for (int it = blockIdx.x; it < n_items && !failed(); it += G, ++k) {
@@ -1065,7 +1111,7 @@ __global__ void __launch_bounds__(kTmaThr, 1) tc_gemm_tma_kernel(
       const bool row_ok = m < nr;
       const int e_row = row_ok ? xexp[rowsrc[row0 + m]] : 0;
       const long long yo = row_ok ? yoff[row0 + m] : 0;
-      for (int j0 = 0; j0 < kNC; j0 += 16) {
+      for (int j0 = col0; j0 < col0 + kNC / 2; j0 += 16) {
         // the SU accumulators of these 16 columns: all loads in flight, one wait
         uint32_t r[SU][16];
 #pragma unroll
@@ -1073,32 +1119,14 @@ __global__ void __launch_bounds__(kTmaThr, 1) tc_gemm_tma_kernel(
         tmem_wait_ld();
 #pragma unroll
         for (int a = 0; a < SU; ++a) reg_fence16(r[a]);
-        float hi[16], lo[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0.f;
-#pragma unroll
-        for (int a = SU - 1; a >= 0; --a) {
-          const float sa = exp2i(-beta * (a + 2));  // exact: -beta (a + 2) >= -80
-#pragma unroll
-          for (int c = 0; c < 16; ++c) ff_add(hi[c], lo[c], __uint_as_float(r[a][c]) * sa, 0.f);
-        }
-        if (j0 + 16 >= kNC) {
+        if (j0 + 16 >= col0 + kNC / 2) {  // this warp's last read: the MMAs may reuse TMEM
           asm volatile("tcgen05.fence::before_thread_sync;");
           mbar_arrive(&tempty);
         }
-        if (row_ok) {
-#pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            const int j = n0 + j0 + c;
-            if (j >= 2 * Q) break;
-            const int sc = e_row + fg[j];
-            const float f = exp2i(sc);
-            const float2 w = f != 0.f ? make_float2(hi[c] * f, lo[c] * f)
-                                      : make_float2(ldexpf(hi[c], sc), ldexpf(lo[c], sc));
-            float2* dst = reinterpret_cast<float2*>(Y + yo + (j < Q ? j : j - Q)) + (j < Q ? 0 : 1);
-            *dst = w;
-          }
-        }
+        float hi[16], lo[16];
+        combine16<SU>(r, beta, hi, lo);
+        if (row_ok)
+          store16(hi, lo, e_row, fg, n0 + j0, 2 * Q, reinterpret_cast<float2*>(Y + yo));
       }
     }
   }
@@ -1130,9 +1158,10 @@ __global__ void __launch_bounds__(kThr) m2l_tc_reduce_kernel(
     for (int lo = threadIdx.x; lo < Q; lo += kThr) {
       float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
       for (int e = e0; e < e1; ++e) {
-        const float4 y = reinterpret_cast<const float4*>(Y)[eyoff[e] + lo];
-        ff_add(rh, rl, y.x, y.y);
-        ff_add(ih, il, y.z, y.w);
+        const float2* y = reinterpret_cast<const float2*>(Y + eyoff[e]) + lo;
+        const float2 a = y[0], b = y[Q];
+        ff_add(rh, rl, a.x, a.y);
+        ff_add(ih, il, b.x, b.y);
       }
       const double f = cv[abs(lo - pb)];
       dst[lo] = cadd(dst[lo], mk(((double)rh + (double)rl) * f, ((double)ih + (double)il) * f));
