@@ -692,46 +692,92 @@ __global__ void __launch_bounds__(kThreads) l2p_kernel(Fmm F, const int* __restr
 }
 
 
+// The multipoles that M2P reads in cosine/sine form: at entry eoff[b] + b of pq
+// (2 pb + 2 entries per box) the pairs (P_m, Q_m), m = 0..pb, of
+//   a_m H_m e^{i m th} + a_{-m} H_{-m} e^{-i m th} = H_m (P_m cos m th + Q_m sin m th),
+//   P_m = a_m + (-1)^m a_{-m},  Q_m = i (a_m - (-1)^m a_{-m}),  P_0 = a_0, Q_0 = 0,
+// from the true coefficients a_n = mh_n s^|n| on levels whose H_pb stays in
+// FP64's range (big[l] == 0), from mh_n on the others.
+__global__ void __launch_bounds__(kThreads) mpole_pq_kernel(Fmm F, const int* __restrict__ boxes,
+                                                            const int* __restrict__ big,
+                                                            cd* __restrict__ pq) {
+  const int b = boxes[blockIdx.x];
+  const int l = F.level[b];
+  const int pb = F.lpb[l];
+  const bool sc = big[l] != 0;
+  const double* pwl = pw_row(F, l);
+  const cd* a = F.mpole + F.eoff[b] + pb;
+  cd* dst = pq + F.eoff[b] + b;
+  for (int m = threadIdx.x; m <= pb; m += kThreads) {
+    const double f = sc ? 1.0 : pwl[m];
+    cd g = m > 0 ? a[-m] : mk(0.0, 0.0);
+    if (m & 1) g = mk(-g.x, -g.y);
+    const cd d = csub(a[m], g);
+    dst[2 * m] = cscale(cadd(a[m], g), f);
+    dst[2 * m + 1] = m > 0 ? mk(-d.y * f, d.x * f) : mk(0.0, 0.0);
+  }
+}
+
 // M2P: one thread per (direct target, W-list box of its leaf) pair, ordered by
 // (leaf, box, target) so that the lanes of a warp read one box's coefficients;
 // the value goes to the pair's slot in target order, and m2p_sum_kernel adds
-// each target's pairs in order.
+// each target's pairs in order. Bound by the FP64 pipe: 15 instructions per
+// order (the angular turn 4, P cos + Q sin 4, the product 4, the unscaled
+// recurrence 3) against 27 with W_m and W_{-m} formed apart (25 ellipses, FP64:
+// 0.67 -> 0.48 ms).
 __global__ void __launch_bounds__(kThreads) m2p_pair_kernel(Fmm F, const int* __restrict__ pt,
                                                             const int* __restrict__ pbx,
                                                             const int* __restrict__ slot, int n,
+                                                            const int* __restrict__ big,
+                                                            const cd* __restrict__ pq,
                                                             cd* __restrict__ partial) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const int i = pt[t], c = pbx[t];
   const int lc = F.level[c];
   const int pb = F.lpb[lc];
-  const cd* a = F.mpole + F.eoff[c];
-  const double s = F.scale[lc];
+  const cd* a = pq + F.eoff[c] + c;
   const double2 mc = F.centre[c];
   const double dx = F.txy[i].x - mc.x, dy = F.txy[i].y - mc.y;
   // one reciprocal square root gives r, 1/r and 1/x: no division
   const double d2 = dx * dx + dy * dy;
   const double ir = rsqrt(d2), x = F.k * (d2 * ir), ix = ir * F.ik;
-  const cd e1 = mk(dx * ir, dy * ir);
+  const double co1 = dx * ir, si1 = dy * ir;
   cd h0, h1;
   hankel01(x, ix, h0, h1);
-  // Wh_m = s^m H_m: Wh_{m+1} = m c1 Wh_m - s^2 Wh_{m-1}, c1 = 2 s / x
-  const double c1 = 2.0 * s * ix, s2 = s * s;
-  cd hm1 = h0, hm = cscale(h1, s), ee = mk(1.0, 0.0);
-  cd sum = cmul(a[pb], h0);
-  double dm = 0.0;
-  for (int m = 1; m <= pb; ++m) {
-    ee = cmul(ee, e1);
-    // Wh_m e^{i m th} and Wh_m e^{-i m th} from the same four products
-    const double rr_ = hm.x * ee.x, ii_ = hm.y * ee.y, ri_ = hm.x * ee.y, ir_ = hm.y * ee.x;
-    cfma(sum, a[pb + m], mk(rr_ - ii_, ri_ + ir_));
-    const cd v = mk(rr_ + ii_, ir_ - ri_);
-    cfma(sum, a[pb - m], (m & 1) ? mk(-v.x, -v.y) : v);
-    dm += 1.0;
-    const double cm = dm * c1;
-    const cd hn = mk(fma(cm, hm.x, -s2 * hm1.x), fma(cm, hm.y, -s2 * hm1.y));
-    hm1 = hm;
-    hm = hn;
+  cd sum = cmul(a[0], h0);
+  double co = co1, si = si1;
+  auto add = [&](int m, cd h) {
+    const cd P = a[2 * m], Q = a[2 * m + 1];
+    cfma(sum, mk(fma(P.x, co, Q.x * si), fma(P.y, co, Q.y * si)), h);
+    const double u = fma(co, co1, -si * si1);
+    si = fma(co, si1, si * co1);
+    co = u;
+  };
+  if (!big[lc]) {  // H_{m+1} = (2m/x) H_m - H_{m-1}
+    const double c2 = 2.0 * ix;
+    double dm = 0.0;
+    cd hp = h0, hc = h1;
+    for (int m = 1; m <= pb; ++m) {
+      add(m, hc);
+      dm += 1.0;
+      const double cm = dm * c2;
+      const cd hn = mk(fma(cm, hc.x, -hp.x), fma(cm, hc.y, -hp.y));
+      hp = hc;
+      hc = hn;
+    }
+  } else {  // Wh_m = s^m H_m: Wh_{m+1} = m c1 Wh_m - s^2 Wh_{m-1}, c1 = 2 s / x
+    const double s = F.scale[lc], c1 = 2.0 * s * ix, s2 = s * s;
+    double dm = 0.0;
+    cd hp = h0, hc = cscale(h1, s);
+    for (int m = 1; m <= pb; ++m) {
+      add(m, hc);
+      dm += 1.0;
+      const double cm = dm * c1;
+      const cd hn = mk(fma(cm, hc.x, -s2 * hp.x), fma(cm, hc.y, -s2 * hp.y));
+      hp = hc;
+      hc = hn;
+    }
   }
   partial[slot[t]] = sum;
 }
@@ -2203,6 +2249,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
       TRY(up(f->m2p_wbox, wb));
       f->n_m2p_wbox = (int)wb.size();
       QBX_CUDA_TRY(f->m2p_mu.alloc(wb.empty() ? 2 : f->n_coef + f->n_boxes));
+      QBX_CUDA_TRY(f->m2p_pq.alloc(wb.empty() ? 2 : f->n_coef + f->n_boxes));
     }
     f->n_dtgt = (int)dt.size();
     f->n_utgt = (int)ut.size();
@@ -2744,8 +2791,13 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
           f->m2p_rec.ptr, f->m2p_part.ptr);
       h->launches += 1;
     } else {
+      mpole_pq_kernel<<<f->n_m2p_wbox, kThreads, 0, s2>>>(F, f->m2p_wbox.ptr, f->m2p_big.ptr,
+                                                         f->m2p_pq.ptr);
+      QBX_KCHECK("m2p_pq", s2);
       m2p_pair_kernel<<<nblk(f->n_m2p_pairs, kThreads), kThreads, 0, s2>>>(
-          F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->m2p_slot.ptr, f->n_m2p_pairs, f->m2p_part.ptr);
+          F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->m2p_slot.ptr, f->n_m2p_pairs, f->m2p_big.ptr,
+          f->m2p_pq.ptr, f->m2p_part.ptr);
+      h->launches += 1;
     }
     QBX_KCHECK("m2p", s2);
     m2p_sum_kernel<<<nblk(f->n_wtgt, kThreads), kThreads, 0, s2>>>(

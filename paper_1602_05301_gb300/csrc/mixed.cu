@@ -860,6 +860,17 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
   QBX_CUDA_TRY(f->sigr.alloc((size_t)f->n_levels * (pbm + 2)));
   sig_ratio_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->lsig.ptr, f->sigr.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
+  {  // |H_m(x)| <~ (m-1)! (2/x)^m; a W-list box's targets lie 1.5 sides away (taken as 0.5)
+    std::vector<int> big(f->n_levels, 0);
+    for (int l = 2; l < f->n_levels; ++l) {
+      const double x_lo = 0.5 * h->k * f->side / std::ldexp(1.0, l);
+      const int pb = std::max(1, f->h_pb[l]);
+      big[l] = std::lgamma((double)pb + 1.0) + (pb + 1) * std::log(2.0 / x_lo) > 650.0 ? 1 : 0;
+    }
+    QBX_CUDA_TRY(f->m2p_big.alloc(f->n_levels));
+    QBX_CUDA_TRY(cudaMemcpy(f->m2p_big.ptr, big.data(), f->n_levels * sizeof(int),
+                            cudaMemcpyHostToDevice));
+  }
   {
     std::vector<int> ffs(f->n_levels, kNoFf);
     for (int l = 2; l < f->n_levels; ++l)

@@ -126,6 +126,8 @@ struct FmmPlan {
   DevBuf<int> m2p_wbox;                  // boxes M2P reads (mixed path converts them)
   int n_m2p_wbox = 0;
   DevBuf<float2> m2p_mu;                 // [n_coef + n_boxes] their FP32 multipoles
+  DevBuf<cd> m2p_pq;                     // the same in cosine/sine form, FP64
+  DevBuf<int> m2p_big;                   // [n_levels] 1: H_pb could leave FP64's range
   DevBuf<double2> m2p_rec;               // [n_levels][pbmax + 2] sigma-scaled Hankel recurrence
   DevBuf<double2> sigr;                  // [n_levels][pbmax + 2] (sig_{m-1}/sig_m, sig_{m+1}/sig_m)
   // [n_levels] s of the scaling 2^{s m} H_m, 2^{-s m} J_m that keeps orders up to
