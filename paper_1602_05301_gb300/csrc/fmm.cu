@@ -389,41 +389,45 @@ __global__ void __launch_bounds__(kThreads) p2m_sum_kernel(Fmm F, const int* __r
 }
 
 // ---------------------------------------------------------------- M2M (Stage 2)
-// CTA per parent (level l, order pp) over its children (level l+1, order pc):
-// a_s = sum_{|n| <= pc} a'_n conj(V_{s-n}), |s| <= pp.
-__host__ __device__ inline size_t m2m_smem(int pp, int pc) {
-  return ((size_t)(2 * pc + 1) + (size_t)(2 * (pp + pc) + 1) + (size_t)(2 * pp + 1)) * sizeof(cd);
-}
+// Parents of level l (order pp), children of level l + 1 (order pc), FP64:
+// a_s = sum_{|n| <= pc} a'_n conj(V_{s-n}), |s| <= pp. A CTA takes a parent and
+// 32 output orders (chunk blockIdx.y); warp c sums child c's terms (its scaled
+// multipole staged in shared memory, the table read through L1: consecutive
+// lanes read consecutive entries), and the four sums are added in child order.
+// Bound by the FP64 pipe at about 1/2 complex product per clock and SM, so a
+// level costs nb Qp Qc 4 / 608 cycles spread over the SMs: the levels of few
+// boxes (mml_on_cuda_cores) run here, the others on the tensor cores.
+constexpr int kMmlCols = 32;
 
 __global__ void __launch_bounds__(kThreads) m2m_kernel(Fmm F, const int* __restrict__ boxes) {
-  extern __shared__ cd smem[];
+  extern __shared__ cd smem[];  // [4][Qc], then [4][kMmlCols]
   const int b = boxes[blockIdx.x];
   const int l = F.level[b];
   const int pp = F.lpb[l], pc = F.lpb[l + 1];
-  const int Qp = 2 * pp + 1, Qc = 2 * pc + 1, M = pp + pc, T = 2 * M + 1;
-  cd* a = smem;        // [Qc]
-  cd* t = a + Qc;      // [T]  t[m + M] = conj(V_m)
-  cd* acc = t + T;     // [Qp]
+  const int Qc = 2 * pc + 1;
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int s = (int)blockIdx.y * kMmlCols + lane - pp;
   const double* pwc = pw_row(F, l + 1);
-  const double* ipp = ipw_row(F, l);
-  for (int i = threadIdx.x; i < Qp; i += kThreads) acc[i] = mk(0.0, 0.0);
-  for (int c = 0; c < 4; ++c) {
-    const int d = F.child[4 * b + c];
-    if (d < 0) continue;
+  const int d = F.child[4 * b + c];
+  cd* a = smem + c * Qc;
+  if (d >= 0) {
     const cd* mp = F.mpole + F.eoff[d];
-    for (int i = threadIdx.x; i < Qc; i += kThreads) a[i] = cscale(mp[i], pwc[abs(i - pc)]);
-    const cd* tab = table(F, F.t_m2m, 4, l, c);
-    for (int i = threadIdx.x; i < T; i += kThreads) t[i] = tab[i - M];
-    __syncthreads();
-    for (int s = (int)threadIdx.x - pp; s <= pp; s += kThreads) {
-      cd sum = mk(0.0, 0.0);
-      for (int n = -pc; n <= pc; ++n) cfma(sum, t[s - n + M], a[n + pc]);
-      acc[s + pp] = cadd(acc[s + pp], sum);
-    }
-    __syncthreads();
+    for (int i = lane; i < Qc; i += 32) a[i] = cscale(mp[i], pwc[abs(i - pc)]);
   }
-  cd* dst = F.mpole + F.eoff[b];
-  for (int i = threadIdx.x; i < Qp; i += kThreads) dst[i] = cscale(acc[i], ipp[abs(i - pp)]);
+  __syncwarp();
+  cd sum = mk(0.0, 0.0);
+  if (d >= 0 && s <= pp) {
+    const cd* t = table(F, F.t_m2m, 4, l, c) + s;
+#pragma unroll 4
+    for (int n = -pc; n <= pc; ++n) cfma(sum, t[-n], a[n + pc]);
+  }
+  cd* red = smem + 4 * Qc;
+  red[c * kMmlCols + lane] = sum;
+  __syncthreads();
+  if (c == 0 && s <= pp) {
+    for (int u = 1; u < 4; ++u) sum = cadd(sum, red[u * kMmlCols + lane]);
+    F.mpole[F.eoff[b] + s + pp] = cscale(sum, ipw_row(F, l)[abs(s)]);
+  }
 }
 
 // ---------------------------------------------------------------- M2L (Stage 4)
@@ -522,39 +526,45 @@ __global__ void __launch_bounds__(kThreads) p2l_sum_kernel(Fmm F, const int* __r
 }
 
 // ---------------------------------------------------------------- L2L (Stage 7)
-// CTA per parent (level l, order pp) into its children (order pc):
-// gamma'_s = sum_{|n| <= pp} gamma_n (-1)^{s-n} V_{s-n}, |s| <= pc.
-__host__ __device__ inline size_t l2l_smem(int pp, int pc) {
-  return ((size_t)(2 * pp + 1) + (size_t)(2 * (pp + pc) + 1)) * sizeof(cd);
-}
-
+// Parents of level l (order pp) into their children (order pc), FP64:
+// gamma'_s = sum_{|n| <= pp} gamma_n (-1)^{s-n} V_{s-n}, |s| <= pc. A CTA takes a
+// parent, a child quadrant (blockIdx.y) and 32 output orders (blockIdx.z); warp w
+// sums the w-th quarter of the parent's orders, the four sums are added in warp
+// order. Same bound and levels as m2m_kernel.
 __global__ void __launch_bounds__(kThreads) l2l_kernel(Fmm F, const int* __restrict__ boxes) {
-  extern __shared__ cd smem[];
-  const int b = boxes[blockIdx.x];
+  extern __shared__ cd smem[];  // [Qp], then [4][kMmlCols]
+  const int b = boxes[blockIdx.x], c = blockIdx.y;
+  const int d = F.child[4 * b + c];
+  if (d < 0) return;
   const int l = F.level[b];
   const int pp = F.lpb[l], pc = F.lpb[l + 1];
-  const int Qp = 2 * pp + 1, M = pp + pc, T = 2 * M + 1;
-  cd* g = smem;   // true local coefficients gamma_n
-  cd* t = g + Qp;
+  const int Qp = 2 * pp + 1;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int s = (int)blockIdx.z * kMmlCols + lane - pc;
   const double* ipp = ipw_row(F, l);
-  const double* pwc = pw_row(F, l + 1);
   const cd* lp = F.local + F.eoff[b];
+  cd* g = smem;  // true local coefficients gamma_n
   for (int i = threadIdx.x; i < Qp; i += kThreads) g[i] = cscale(lp[i], ipp[abs(i - pp)]);
-  for (int c = 0; c < 4; ++c) {
-    const int d = F.child[4 * b + c];
-    if (d < 0) continue;
-    const cd* tab = table(F, F.t_l2l, 4, l, c);
-    for (int i = threadIdx.x; i < T; i += kThreads) t[i] = tab[i - M];
-    __syncthreads();
-    cd* dl = F.local + F.eoff[d];
-    for (int s = (int)threadIdx.x - pc; s <= pc; s += kThreads) {
-      cd sum = mk(0.0, 0.0);
-      for (int n = -pp; n <= pp; ++n) cfma(sum, t[s - n + M], g[n + pp]);
-      dl[s + pc] = cadd(dl[s + pc], cscale(sum, pwc[abs(s)]));
-    }
-    __syncthreads();
+  __syncthreads();
+  const int per = (Qp + 3) / 4, i0 = min(Qp, w * per), i1 = min(Qp, i0 + per);
+  cd sum = mk(0.0, 0.0);
+  if (s <= pc) {
+    const cd* t = table(F, F.t_l2l, 4, l, c) + s + pp;
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) cfma(sum, t[-i], g[i]);
+  }
+  cd* red = smem + Qp;
+  red[w * kMmlCols + lane] = sum;
+  __syncthreads();
+  if (w == 0 && s <= pc) {
+    for (int u = 1; u < 4; ++u) sum = cadd(sum, red[u * kMmlCols + lane]);
+    cd* dl = F.local + F.eoff[d] + s + pc;
+    *dl = cadd(*dl, cscale(sum, pw_row(F, l + 1)[abs(s)]));
   }
 }
+
+size_t m2m_smem(int pc) { return (4 * (size_t)(2 * pc + 1) + 4 * kMmlCols) * sizeof(cd); }
+size_t l2l_smem(int pp) { return ((size_t)(2 * pp + 1) + 4 * kMmlCols) * sizeof(cd); }
 
 // ---------------------------------------------------------------- targets (Stages 3, 5, 8)
 // CTA per leaf; one thread per target of the leaf (strided). Only targets that
@@ -2758,13 +2768,14 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     for (int l = f->n_levels - 2; l >= 2; --l) {
       const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
       if (nb == 0) continue;
-      bool done = false;  // tensor cores where the level's split is exact
+      bool done = false;  // tensor cores on wide levels whose split is exact
       TRY(launch_mml_tc(h, f, 0, l, &done, s));
       if (done) {
         QBX_KCHECK("m2m_tc", s);
         continue;
       }
-      m2m_kernel<<<nb, kThreads, m2m_smem(pb[l], pb[l + 1]), s>>>(F, f->nonleaf.ptr + f->nonleaf_off[l]);
+      m2m_kernel<<<dim3(nb, nblk(2 * pb[l] + 1, kMmlCols)), kThreads, m2m_smem(pb[l + 1]), s>>>(
+          F, f->nonleaf.ptr + f->nonleaf_off[l]);
       QBX_KCHECK("m2m", s);
       h->launches += 1;
     }
@@ -2827,13 +2838,14 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     for (int l = 2; l + 1 < f->n_levels; ++l) {
       const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
       if (nb == 0) continue;
-      bool done = false;  // tensor cores where the level's split is exact
+      bool done = false;  // tensor cores on wide levels whose split is exact
       TRY(launch_mml_tc(h, f, 1, l, &done, s));
       if (done) {
         QBX_KCHECK("l2l_tc", s);
         continue;
       }
-      l2l_kernel<<<nb, kThreads, l2l_smem(pb[l], pb[l + 1]), s>>>(F, f->nonleaf.ptr + f->nonleaf_off[l]);
+      l2l_kernel<<<dim3(nb, 4, nblk(2 * pb[l + 1] + 1, kMmlCols)), kThreads, l2l_smem(pb[l]), s>>>(
+          F, f->nonleaf.ptr + f->nonleaf_off[l]);
       QBX_KCHECK("l2l", s);
       h->launches += 1;
     }

@@ -1458,8 +1458,8 @@ qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f) {
 // L2L, padded to 64) admits an exact split, the matrix slices of the four
 // quadrant operators, the rows (one per child: quadrant-major, parents in
 // level order), the source boxes and the work items. Levels without one keep
-// the CUDA-core kernels; so do all levels with m2l_engine == 2 or
-// QBX_M2L_TENSOR=0.
+// the CUDA-core kernels; so do levels of few boxes (mml_on_cuda_cores) and all
+// levels with m2l_engine == 2 or QBX_M2L_TENSOR=0.
 qbx_status tc_mml_plan_build(qbx_handle* h, FmmPlan* f) {
   const int nl = f->n_levels;
   f->tc_m2m.clear();
@@ -1486,6 +1486,7 @@ qbx_status tc_mml_plan_build(qbx_handle* h, FmmPlan* f) {
       if (par.empty()) continue;
       TcLevelOp& op = kind == 0 ? f->tc_m2m[l] : f->tc_l2l[l];
       const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
+      if (mml_on_cuda_cores((int)par.size(), pp, pc)) continue;
       const int qin = kind == 0 ? 2 * pc + 1 : 2 * pp + 1;
       const int qout = kind == 0 ? 2 * pp + 1 : 2 * pc + 1;
       const int K = (2 * qin + kPad - 1) / kPad * kPad;

@@ -221,6 +221,17 @@ struct FmmPlan {
   int n_tc_items[3] = {0, 0, 0};
 };
 
+// FP64 M2M and L2L levels of few boxes stay on the CUDA cores: 4 FMAs per complex
+// product at 304 FMAs per clock over the chip, up to kMmlCycles; the tensor-core
+// path takes three launches and one tile's latency (45 us) however few boxes
+// there are. M2M and L2L of the 8192-node starfish with 971 boxes, FP64: 0.20 and
+// 0.22 ms all on the tensor cores, 0.10 and 0.07 ms with this rule; levels above the
+// line (25 ellipses) measured the same either way.
+constexpr double kMmlCycles = 50e3;
+inline bool mml_on_cuda_cores(int n_parents, int pp, int pc) {
+  return 16.0 * n_parents * (2.0 * pp + 1) * (2.0 * pc + 1) / 304.0 <= kMmlCycles;
+}
+
 qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f);
 qbx_status configure_mixed_kernels(int smem_optin);
 qbx_status launch_m2l_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s);
