@@ -26,7 +26,8 @@
 namespace {
 
 constexpr int kT = 256;
-constexpr int kBlocks = 304;   // 2 x 152 SMs: partial sums per dot product
+constexpr int kBlocks = 304;   // 2 x 152 SMs: most partial sums per dot product
+constexpr int kPerThread = 4;  // terms of a dot product that a thread takes at least
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)std::max<int64_t>(1, (n + b - 1) / b); }
 
@@ -57,13 +58,19 @@ __global__ void __launch_bounds__(kT) dots_kernel(int64_t n, const cd* __restric
   s = block_sum(s, sh);
   if (threadIdx.x == 0) part[(int64_t)i * gridDim.x + blockIdx.x] = s;
 }
-// out[i] = sum_b part[i][b], in block order
-__global__ void sum_parts_kernel(int m, int nb, const cd* __restrict__ part, cd* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
+// out[i] = sum_b part[i][b]: a warp per dot product, lane L adding blocks L, L +
+// 32, ..., then a shuffle tree (a fixed order; one thread walking the blocks took
+// 38 us; with as many blocks as the vectors fill and one fetch per step, the solve
+// on 1536 nodes fell from 53.1 to 46.1 ms)
+__global__ void __launch_bounds__(32) sum_parts_kernel(int nb, const cd* __restrict__ part,
+                                                       cd* __restrict__ out) {
   cd s = mk(0.0, 0.0);
-  for (int b = 0; b < nb; ++b) s = cadd(s, part[(int64_t)i * nb + b]);
-  out[i] = s;
+  for (int b = threadIdx.x; b < nb; b += 32) s = cadd(s, part[(int64_t)blockIdx.x * nb + b]);
+  for (int o = 16; o > 0; o >>= 1) {
+    s.x += __shfl_down_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_down_sync(0xffffffffu, s.y, o);
+  }
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 // w -= sum_{i < m} c_i V_i
 __global__ void sub_combo_kernel(int64_t n, int m, const cd* __restrict__ V, int64_t ldv,
@@ -97,18 +104,34 @@ struct Krylov {
   cudaStream_t s;
   DevBuf<cd> part, dots;
   std::vector<cd> host;
-  // c_i = <V_i, w>, i < m (fixed-order reduction), copied to host
-  qbx_status dot(const cd* V, int64_t ldv, int m, const cd* w) {
-    if (part.n < (size_t)m * kBlocks) QBX_CUDA_TRY(part.alloc((size_t)m * kBlocks));
-    if (dots.n < (size_t)m) QBX_CUDA_TRY(dots.alloc(std::max(m, 64)));
-    dots_kernel<<<dim3(kBlocks, m), kT, 0, s>>>(n, V, ldv, w, part.ptr);
+  // room for dot products of up to m vectors, `slots` results of them at once
+  qbx_status init(int m, int slots) {
+    QBX_CUDA_TRY(part.alloc((size_t)m * kBlocks));
+    QBX_CUDA_TRY(dots.alloc((size_t)m * slots));
+    return QBX_OK;
+  }
+  // out[i] = <V_i, w>, i < m, on the device (fixed-order reduction)
+  qbx_status dot_dev(const cd* V, int64_t ldv, int m, const cd* w, cd* out) {
+    const int nb = (int)std::min<int64_t>(kBlocks, nblk(n, kT * kPerThread));
+    cd* p = nb == 1 ? out : part.ptr;
+    dots_kernel<<<dim3(nb, m), kT, 0, s>>>(n, V, ldv, w, p);
     QBX_CUDA_TRY(cudaGetLastError());
-    sum_parts_kernel<<<nblk(m, 64), 64, 0, s>>>(m, kBlocks, part.ptr, dots.ptr);
-    QBX_CUDA_TRY(cudaGetLastError());
+    if (nb > 1) {
+      sum_parts_kernel<<<m, 32, 0, s>>>(nb, p, out);
+      QBX_CUDA_TRY(cudaGetLastError());
+    }
+    return QBX_OK;
+  }
+  // the first m results to the host
+  qbx_status fetch(int m) {
     host.resize(m);
     QBX_CUDA_TRY(cudaMemcpyAsync(host.data(), dots.ptr, m * sizeof(cd), cudaMemcpyDeviceToHost, s));
     QBX_CUDA_TRY(cudaStreamSynchronize(s));
     return QBX_OK;
+  }
+  qbx_status dot(const cd* V, int64_t ldv, int m, const cd* w) {
+    const qbx_status st = dot_dev(V, ldv, m, w, dots.ptr);
+    return st != QBX_OK ? st : fetch(m);
   }
 };
 
@@ -164,8 +187,9 @@ extern "C" qbx_status qbx_solve_dirichlet(qbx_handle* h, const double* rhs, doub
                                     (double*)out, nullptr, precision, s);
   };
   Krylov K{n, s, {}, {}, {}};
-  qbx_status st = K.dot(b.ptr, n, 1, b.ptr);
+  qbx_status st = K.init(m + 1, 3);
   if (st != QBX_OK) return st;
+  if ((st = K.dot(b.ptr, n, 1, b.ptr)) != QBX_OK) return st;
   const double bnorm = std::sqrt(K.host[0].x);
   int it = 0;
   double rel = 0.0;
@@ -180,10 +204,14 @@ extern "C" qbx_status qbx_solve_dirichlet(qbx_handle* h, const double* rhs, doub
   typedef std::complex<double> C;
   bool done = false;
   while (!done) {
-    // r = b - A x into V_0
-    if ((st = apply(x.ptr, V.ptr)) != QBX_OK) return st;
-    residual_kernel<<<nblk(n, kT), kT, 0, s>>>(n, b.ptr, V.ptr);
-    QBX_CUDA_TRY(cudaGetLastError());
+    // r = b - A x into V_0 (x = 0 at first, and A 0 = 0)
+    if (it == 0) {
+      QBX_CUDA_TRY(cudaMemcpyAsync(V.ptr, b.ptr, n * sizeof(cd), cudaMemcpyDeviceToDevice, s));
+    } else {
+      if ((st = apply(x.ptr, V.ptr)) != QBX_OK) return st;
+      residual_kernel<<<nblk(n, kT), kT, 0, s>>>(n, b.ptr, V.ptr);
+      QBX_CUDA_TRY(cudaGetLastError());
+    }
     if ((st = K.dot(V.ptr, n, 1, V.ptr)) != QBX_OK) return st;
     const double beta = std::sqrt(K.host[0].x);
     rel = beta / bnorm;
@@ -196,19 +224,21 @@ extern "C" qbx_status qbx_solve_dirichlet(qbx_handle* h, const double* rhs, doub
     for (; j < m && it < max_iter; ++j, ++it) {
       cd* vj1 = V.ptr + (int64_t)(j + 1) * n;
       if ((st = apply(V.ptr + (int64_t)j * n, vj1)) != QBX_OK) return st;
-      // classical Gram-Schmidt, twice
-      std::vector<C> hc(j + 1, C(0.0));
+      // classical Gram-Schmidt, twice, then the norm; one copy to the host for
+      // the three sets of dot products
+      const int nv = j + 1;
       for (int pass = 0; pass < 2; ++pass) {
-        if ((st = K.dot(V.ptr, n, j + 1, vj1)) != QBX_OK) return st;
-        std::vector<cd> c(K.host);
-        for (int i = 0; i <= j; ++i) hc[i] += C(c[i].x, c[i].y);
-        QBX_CUDA_TRY(cudaMemcpyAsync(K.dots.ptr, c.data(), (j + 1) * sizeof(cd),
-                                     cudaMemcpyHostToDevice, s));
-        sub_combo_kernel<<<nblk(n, kT), kT, 0, s>>>(n, j + 1, V.ptr, n, K.dots.ptr, vj1);
+        cd* c = K.dots.ptr + pass * nv;
+        if ((st = K.dot_dev(V.ptr, n, nv, vj1, c)) != QBX_OK) return st;
+        sub_combo_kernel<<<nblk(n, kT), kT, 0, s>>>(n, nv, V.ptr, n, c, vj1);
         QBX_CUDA_TRY(cudaGetLastError());
       }
-      if ((st = K.dot(vj1, n, 1, vj1)) != QBX_OK) return st;
-      const double hn = std::sqrt(K.host[0].x);
+      if ((st = K.dot_dev(vj1, n, 1, vj1, K.dots.ptr + 2 * nv)) != QBX_OK) return st;
+      if ((st = K.fetch(2 * nv + 1)) != QBX_OK) return st;
+      std::vector<C> hc(nv);
+      for (int i = 0; i < nv; ++i)
+        hc[i] = C(K.host[i].x, K.host[i].y) + C(K.host[nv + i].x, K.host[nv + i].y);
+      const double hn = std::sqrt(K.host[2 * nv].x);
       for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hc[i];
       H[(size_t)(j + 1) * m + j] = hn;
       if (hn > 0.0) {
