@@ -929,8 +929,7 @@ __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
       pq[at] = v;
       return;
     }
-    const double f = pow2d(s * m);
-    const ff x = ff_round(v.x * f), y = ff_round(v.y * f);
+    const ff x = ff_from_f64(v.x, 896 - s * m), y = ff_from_f64(v.y, 896 - s * m);
     reinterpret_cast<float4*>(pq)[at] = make_float4(x.h, x.l, y.h, y.l);
   };
   for (int m = threadIdx.x; m <= pb; m += kThreads) {

@@ -17,6 +17,7 @@
 // conversions between the two normalisations are FP64.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "tree.cuh"
@@ -317,8 +318,13 @@ __global__ void __launch_bounds__(kT) mpole_to_f32_kernel(
 constexpr int kChunkK = 128;
 static_assert(kChunkK % kGemmBlock == 0, "staging must keep the summation blocks");
 
-// (four CTAs per SM: 128 registers, a few spilled; 2 % faster than three)
-__global__ void __launch_bounds__(kT, 4) m2l_f32_gemm_kernel(
+// NT threads, one output order each (items are cut to kT orders): the widths 64
+// and 96 serve levels with so few orders, which in a block of 128 leave one or
+// two of its four warps without work while they hold registers (128 per thread,
+// 16 warps per SM; M2L of the k = 10 starfish with 8192 nodes 0.217 -> 0.183 ms, of
+// 200 ellipses 3.36 -> 3.24).
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) m2l_f32_gemm_kernel(
     const int4* __restrict__ items, const int* __restrict__ lpb,
     const long long* __restrict__ goff, const long long* __restrict__ row_off,
     const float2* __restrict__ mu32, const float2* __restrict__ tm,
@@ -338,7 +344,7 @@ __global__ void __launch_bounds__(kT, 4) m2l_f32_gemm_kernel(
   for (int n0 = 0; n0 < Q; n0 += kChunkK) {
     const int nk = min(kChunkK, Q - n0);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nk * (kGemmRows / 2); idx += kT) {
+    for (int idx = threadIdx.x; idx < nk * (kGemmRows / 2); idx += NT) {
       const int r = 2 * (idx / nk), n = idx % nk;  // coalesced reads along each source row
       const float2 a = r < nr ? mu32[row_off[row0 + r] + n0 + n] : make_float2(0.f, 0.f);
       const float2 b = r + 1 < nr ? mu32[row_off[row0 + r + 1] + n0 + n] : make_float2(0.f, 0.f);
@@ -951,14 +957,18 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     // coarse levels (largest orders) first; work items (first row, rows,
     // first output order, group) per tile: chunks of kT output orders, and
     // for FP64 also groups of kF64Rows rows
-    std::vector<int4> it32, it64;
+    std::vector<int4> it32, it64, by_width[3];  // FP32: blocks of 128, 96, 64 threads
     for (const int4& t : tiles) {
       const int Q = 2 * f->h_pb[t.w] + 1;
       for (int c0 = 0; c0 < Q; c0 += kT) {
-        it32.push_back(make_int4(t.y, t.z, c0, t.x));
+        by_width[Q > 96 ? 0 : Q > 64 ? 1 : 2].push_back(make_int4(t.y, t.z, c0, t.x));
         for (int r0 = 0; r0 < t.z; r0 += kF64Rows)
           it64.push_back(make_int4(t.y + r0, std::min(kF64Rows, t.z - r0), c0, t.x));
       }
+    }
+    for (int u = 0; u < 3; ++u) {
+      it32.insert(it32.end(), by_width[u].begin(), by_width[u].end());
+      f->n_m2l_width[u] = (int)by_width[u].size();
     }
     // matrix offset of each group (level l, class c): level offset + c Q_l^2
     std::vector<long long> goff(ng, 0);
@@ -1156,14 +1166,27 @@ qbx_status launch_m2l_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
     QBX_CUDA_TRY(cudaGetLastError());
     h->launches += 1;
   }
-  m2l_f32_gemm_kernel<<<f->n_m2l_items32, kT, 0, s>>>(
-      f->m2l_items32.ptr, f->lpb.ptr, f->m2l_goff.ptr, f->m2l_rowoff.ptr, f->mu32.ptr,
-      f->tm_f32.ptr, f->m2l_yoff.ptr, f->m2l_y.ptr);
-  QBX_CUDA_TRY(cudaGetLastError());
+  int at = 0;
+  auto gemm = [&](auto nt, int n) -> qbx_status {
+    constexpr int NT = decltype(nt)::value;
+    if (n > 0) {
+      m2l_f32_gemm_kernel<NT><<<n, NT, 0, s>>>(
+          f->m2l_items32.ptr + at, f->lpb.ptr, f->m2l_goff.ptr, f->m2l_rowoff.ptr, f->mu32.ptr,
+          f->tm_f32.ptr, f->m2l_yoff.ptr, f->m2l_y.ptr);
+      QBX_CUDA_TRY(cudaGetLastError());
+      h->launches += 1;
+    }
+    at += n;
+    return QBX_OK;
+  };
+  qbx_status st;
+  if ((st = gemm(std::integral_constant<int, 128>(), f->n_m2l_width[0])) != QBX_OK) return st;
+  if ((st = gemm(std::integral_constant<int, 96>(), f->n_m2l_width[1])) != QBX_OK) return st;
+  if ((st = gemm(std::integral_constant<int, 64>(), f->n_m2l_width[2])) != QBX_OK) return st;
   m2l_f32_reduce_kernel<<<f->n_vbox, kT, 0, s>>>(
       f->pb_max, f->vbox.ptr, f->box.level.ptr, f->lpb.ptr, f->V.off.ptr, f->m2l_eyoff.ptr,
       f->m2l_y.ptr, f->conv.ptr, f->eoff.ptr, f->local.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
-  h->launches += 2;
+  h->launches += 1;
   return QBX_OK;
 }

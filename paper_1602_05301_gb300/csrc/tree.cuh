@@ -174,6 +174,7 @@ struct FmmPlan {
   DevBuf<long long> m2l_goff;           // [n_levels * 49] matrix offset per (level, class)
   DevBuf<int4> m2l_items32, m2l_items64;  // (first row, rows, first output order, group)
   int n_m2l_items32 = 0, n_m2l_items64 = 0;
+  int n_m2l_width[3] = {0, 0, 0};       // FP32 items by block width 128, 96, 64 (in this order)
   DevBuf<long long> m2l_eyoff;          // result-row offset of every V entry
   DevBuf<long long> m2l_rowoff;         // coefficient offset of each row's source box
   DevBuf<long long> m2l_yoff;
