@@ -483,7 +483,7 @@ qbx_status replace_geometry(qbx_handle* h, int64_t n_panels, DevBuf<double>& nod
 
 extern "C" void qbx_destroy(qbx_handle* h) {
   if (!h) return;
-  cudaDeviceSynchronize();
+  DeviceQuiet quiet;  // synchronises
   if (h->fmm) fmm_plan_free(h->fmm);
   h->fmm = nullptr;
   for (int i = 0; i < 2 * QBX_STAGE_COUNT; ++i)

@@ -2879,7 +2879,10 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   return QBX_OK;
 }
 
-void fmm_plan_free(FmmPlan* f) { delete f; }
+void fmm_plan_free(FmmPlan* f) {
+  DeviceQuiet quiet;
+  delete f;
+}
 
 extern "C" qbx_status qbx_export_tree(const qbx_handle* h, int64_t* info, double* root,
                                       int32_t* box_level, int32_t* box_ij, int32_t* box_child,

@@ -41,6 +41,19 @@ void set_error(const char* fmt, ...);
   } while (0)
 
 // ---------------------------------------------------------------- device buffers
+// pool.cu: device memory for DevBuf, kept in size classes between buffers
+cudaError_t dev_alloc(void** p, size_t bytes);
+void dev_free(void* p);
+// Buffers released while one is alive share its device synchronisation: for
+// scopes that release many and launch nothing meanwhile.
+struct DeviceQuiet {
+  DeviceQuiet();
+  ~DeviceQuiet();
+  DeviceQuiet(const DeviceQuiet&) = delete;
+  DeviceQuiet& operator=(const DeviceQuiet&) = delete;
+  const bool quiet;
+};
+
 template <typename T>
 struct DevBuf {
   T* ptr = nullptr;
@@ -48,12 +61,12 @@ struct DevBuf {
   cudaError_t alloc(size_t count) {
     release();
     if (count == 0) return cudaSuccess;
-    cudaError_t e = cudaMalloc((void**)&ptr, count * sizeof(T));
+    cudaError_t e = dev_alloc((void**)&ptr, count * sizeof(T));
     if (e == cudaSuccess) n = count; else ptr = nullptr;
     return e;
   }
   void release() {
-    if (ptr) cudaFree(ptr);
+    if (ptr) dev_free(ptr);
     ptr = nullptr;
     n = 0;
   }
