@@ -206,3 +206,44 @@ __device__ __forceinline__ ff split17(ff a) {
   const float h = __uint_as_float(__float_as_uint(n.h) & 0xFFFFFF80u);
   return mkff(h, __fadd_rn(__fsub_rn(n.h, h), n.l));
 }
+
+// (a + i b) *= c + i d
+__device__ __forceinline__ void ff_turn(ff& a, ff& b, ff c, ff d) {
+  const ff t = ff_sub_raw(ff_mul_raw(a, c), ff_mul_raw(b, d));
+  const ff u = ff_add(ff_mul_raw(a, d), ff_mul_raw(b, c));
+  a = fast_two_sum(t.h, t.l);
+  b = u;
+}
+
+// Miller's backward recurrence on f_j ~ 2^{-s j} J_j(k r), j = 0..M, kept in row
+// (h, l) while it runs; returns 1 / norm (2^{-s j} J_j = row[j] / norm):
+//   f_{n-1} = (2 n 2^s / x) f_n - 4^s f_{n+1},  norm = f_0 + 2 4^s (f_2 + 4^s (f_4 + ...)).
+__device__ __forceinline__ ff ff_miller_row(float2* row, int M, int s, const FfPolar& D,
+                                            const FfUnits& U) {
+  const float sg2 = pow2f(2 * s);
+  ff c2 = ff_mul_raw(ff_scale(U.ik2, pow2f(s)), D.ir);  // 2 2^s / x
+  c2 = fast_two_sum(c2.h, c2.l);
+  const int N = miller_start_f32(M, D.z.h);  // N > M + 1
+  ff f1 = mkff(0.f, 0.f), f0 = mkff(0x1p-40f, 0.f), sum = f1;
+  float fn = (float)N;
+  for (int nn = N; nn >= 1; --nn) {
+    if ((nn & 1) == 0) sum = ff_add(f0, ff_scale(sum, sg2));
+    const float ch = __fmul_rn(fn, c2.h);
+    const ff cn = mkff(ch, __fmaf_rn(fn, c2.l, __fmaf_rn(fn, c2.h, -ch)));
+    const ff f = ff_sub_raw(ff_mul_raw(cn, f0), ff_scale(f1, sg2));
+    f1 = f0;
+    f0 = fast_two_sum(f.h, f.l);
+    fn -= 1.f;
+    if (nn - 1 <= M) row[nn - 1] = make_float2(f0.h, f0.l);
+    if (fabsf(f0.h) >= 0x1p20f) {
+      constexpr float d = 0x1p-60f;
+      f0 = ff_scale(f0, d);
+      f1 = ff_scale(f1, d);
+      sum = ff_scale(sum, d);
+      for (int u = nn - 1; u <= M; ++u) row[u] = make_float2(row[u].x * d, row[u].y * d);
+    }
+  }
+  const ff norm = ff_add(f0, ff_scale(sum, 2.f * sg2));
+  const float r = 1.0f / norm.h;  // 1 / norm by one Newton step
+  return mkff(r, __fmul_rn(r, __fmaf_rn(-norm.l, r, __fmaf_rn(-norm.h, r, 1.0f))));
+}

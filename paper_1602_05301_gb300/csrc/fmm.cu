@@ -98,6 +98,7 @@ struct Fmm {
   cd* local;
   cd* lpq;               // [n_coef] leaf cos/sin coefficients of L2P (see unscale_leaf_locals_kernel)
   const int* ffs;        // [n_levels] power-of-two scale exponent of the float-float kernels
+  float2* loc32;         // [n_coef] leaf locals gamma_n 2^{ffs |n|} (mixed L2QBXL)
   const double* conv;    // [n_levels][pbmax + 1] s^j / sig_j (mixed path)
   const double* lsig;    // [n_levels][pbmax + 1] log sig_j
   const double* isig;    // [n_levels][pbmax + 2] 1 / sig_min(j, pb) (mixed P2M)
@@ -913,7 +914,8 @@ __global__ void __launch_bounds__(32) l2qbxl_kernel(Fmm F, const int* __restrict
 // stored as lpq[eoff + m] = P_m (m = 0..pb), lpq[eoff + pb + m] = Q_m (m = 1..pb).
 // With ff32 set (mixed path), leaves on float-float levels (ffs[l] = s) get
 // 2^{s m} P_m and 2^{s m} Q_m as float4 (re h, re l, im h, im l) in the same
-// places, for l2p_mixed_kernel.
+// places, for l2p_mixed_kernel, and 2^{s |n|} gamma_n in FP32 in loc32, for
+// l2qbxl_ff_kernel.
 __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
                                                                        const int* __restrict__ leaves,
                                                                        bool ff32) {
@@ -932,15 +934,22 @@ __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
     const ff x = ff_from_f64(v.x, 896 - s * m), y = ff_from_f64(v.y, 896 - s * m);
     reinterpret_cast<float4*>(pq)[at] = make_float4(x.h, x.l, y.h, y.l);
   };
+  float2* g32 = F.loc32 + F.eoff[b] + pb;
+  auto put32 = [&](int n, int m, cd v) {
+    if (s != kNoFf)
+      g32[n] = make_float2(f32_from_f64_sh(v.x, s * m), f32_from_f64_sh(v.y, s * m));
+  };
   for (int m = threadIdx.x; m <= pb; m += kThreads) {
     const cd gp = cscale(lp[pb + m], ipp[m]);
     lp[pb + m] = gp;
+    put32(m, m, gp);
     if (m == 0) {
       put(0, 0, gp);
       continue;
     }
     const cd gn = cscale(lp[pb - m], ipp[m]);
     lp[pb - m] = gn;
+    put32(-m, m, gn);
     const cd sg = (m & 1) ? mk(-gn.x, -gn.y) : gn;
     put(m, m, cadd(gp, sg));
     const cd d = csub(sg, gp);
@@ -1385,6 +1394,202 @@ __global__ void __launch_bounds__(32) l2qbxl_mixed_kernel(Fmm F, const int* __re
   }
 }
 
+// ---------------------------------------------------------------- L2QBXL, M2QBXL on float-float levels
+// The two translations above when every leaf (W-list box) of the launch is on a
+// level with a power-of-two scaling s = ffs (almost always): the scaled
+// coefficients and rows fit FP32, so a term is a plain FP32 product and no
+// exponents are carried. With g_n = 2^{s|n|} gamma_n and v_m = 2^{-s|m|} V_m,
+//   alpha_l = 2^{-s|l|} sum_n g_n t_{l-n} 2^{s(|l-n| - |n| + |l|)},
+// and for n' = n sgn(l) the exponent is 2 s |l| for n' <= 0 and 2 s max(|l| - n', 0)
+// for n' > 0: two Kahan sums, joined in FP64. M2QBXL has the same form with the
+// roles of the sides exchanged. Rows by the float-float recurrences; angular
+// factors FP32 between float-float anchors every eighth order. (200 ellipses: L2QBXL
+// 1.02 -> 0.47 ms, M2QBXL 0.67 -> 0.24, against the FP64 rows and split exponents.)
+__global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restrict__ cleaf,
+                                                       const int* __restrict__ clist, int n_ctr,
+                                                       int G, int TW, cd* __restrict__ alpha) {
+  extern __shared__ __align__(16) float2 frow[];  // [G][TW], TW > max M + 1
+  const int lane = threadIdx.x;
+  const int c0 = blockIdx.x * G;
+  const int p = F.p, P = 2 * p + 1;
+  if (lane < G && c0 + lane < n_ctr) {
+    const int i = clist[c0 + lane];
+    const int b = cleaf[i];
+    const int l = F.level[b], M = F.lpb[l] + p, s = F.ffs[l];
+    const double2 mb = F.centre[b], z = F.cxy[i];
+    const FfUnits U(F.k);
+    FfPolar D;
+    const bool off = D.set(z.x - mb.x, z.y - mb.y, U);
+    float2* row = frow + (size_t)lane * TW;
+    if (!off || D.z.h < 1e-8f) {  // J_m(x) = (x/2)^m / m!
+      float t = 1.f;
+      const float hx = off ? 0.5f * D.z.h * pow2f(-s) : 0.f;
+      float2 e = make_float2(1.f, 0.f);
+      for (int m = 0; m <= M; ++m) {
+        row[m] = make_float2(e.x * t, e.y * t);
+        t *= hx / (float)(m + 1);
+        if (off) e = fmul(e, make_float2(D.c, D.s));
+      }
+    } else {
+      const ff inv = ff_miller_row(row, M, s, D, U);
+      const ff c1 = ff_mul(D.x, D.ir), s1 = ff_mul(D.y, D.ir);
+      ff c8 = c1, s8 = s1;
+#pragma unroll
+      for (int u = 0; u < 3; ++u) ff_turn(c8, s8, c8, s8);
+      const float2 e1 = make_float2(ff_f32(c1), ff_f32(s1));
+      ff ex = mkff(1.f, 0.f), ey = mkff(0.f, 0.f);
+      float2 e = make_float2(1.f, 0.f);
+      for (int m = 0; m <= M; ++m) {
+        if ((m & 7) == 0) {
+          e = make_float2(ff_f32(ex), ff_f32(ey));
+          ff_turn(ex, ey, c8, s8);
+        } else {
+          e = fmul(e, e1);
+        }
+        const float2 f = row[m];
+        const float v = ff_f32(ff_mul_raw(mkff(f.x, f.y), inv));
+        row[m] = make_float2(e.x * v, e.y * v);
+      }
+    }
+  }
+  __syncwarp();
+  const int nG = min(G, n_ctr - c0);
+  for (int o = lane; o < nG * P; o += 32) {
+    const int u = o / P, so = o % P - p;
+    const int i = clist[c0 + u];
+    const int b = cleaf[i];
+    const int l = F.level[b], pb = F.lpb[l], s = F.ffs[l];
+    const float2* row = frow + (size_t)u * TW;
+    const float2* g = F.loc32 + F.eoff[b] + pb;
+    const int a = abs(so), dir = so < 0 ? -1 : 1;
+    // t_m = (-1)^m V_m for m >= 0, conj(V_{-m}) for m < 0 (signs on the bits)
+    auto term = [](float2 gn, float2 v, bool neg, int m) {
+      const unsigned fx = !neg && (m & 1) ? 0x80000000u : 0u;
+      const unsigned fy = neg ? 0x80000000u : fx;
+      return fmul(gn, make_float2(__uint_as_float(__float_as_uint(v.x) ^ fx),
+                                  __uint_as_float(__float_as_uint(v.y) ^ fy)));
+    };
+    float2 S1 = make_float2(0.f, 0.f), C1 = S1, S2 = S1, C2 = S1;
+    for (int j = 0; j <= pb; ++j)  // n' = -j: m = dir (a + j)
+      kahan2(S1, C1, term(g[-dir * j], row[a + j], so < 0, a + j));
+    for (int j = 1; j <= pb; ++j) {  // n' = j: m = dir (a - j)
+      const int m = abs(a - j);
+      const bool neg = (a > j) ? so < 0 : (a < j) ? so >= 0 : false;
+      float2 v = term(g[dir * j], row[m], neg, m);
+      if (j < a) {
+        const float f = pow2f(2 * s * (a - j));
+        v = make_float2(v.x * f, v.y * f);
+      }
+      kahan2(S2, C2, v);
+    }
+    const double f1 = pow2d(s * a), f2 = pow2d(-s * a);
+    cd* dst = alpha + (size_t)F.cid[i] * P + p + so;
+    *dst = cadd(*dst, mk(((double)S1.x - (double)C1.x) * f1 + ((double)S2.x - (double)C2.x) * f2,
+                         ((double)S1.y - (double)C1.y) * f1 + ((double)S2.y - (double)C2.y) * f2));
+  }
+}
+
+// a_n 2^{-s|n|} in FP32 of the boxes listed (a_n = mh_n s_l^|n|), for M2QBXL
+__global__ void __launch_bounds__(kThreads) mpole_scaled_kernel(Fmm F, const int* __restrict__ boxes,
+                                                                float2* __restrict__ out) {
+  const int b = boxes[blockIdx.x];
+  const int l = F.level[b], pb = F.lpb[l], s = F.ffs[l];
+  const double* pwl = pw_row(F, l);
+  const cd* a = F.mpole + F.eoff[b] + pb;
+  float2* dst = out + F.eoff[b] + pb;
+  for (int n = (int)threadIdx.x - pb; n <= pb; n += kThreads) {
+    const double f = pwl[abs(n)];
+    dst[n] = make_float2(f32_from_f64_sh(a[n].x * f, -s * abs(n)),
+                         f32_from_f64_sh(a[n].y * f, -s * abs(n)));
+  }
+}
+
+// M2QBXL: alpha_l += (-1)^l sum_n a_n W_{n+l} over (centre, W box) pairs, PW per
+// warp. With A_n = 2^{-s|n|} a_n, w_m = 2^{s|m|} W_m and n' = n sgn(l) the exponent
+// of a term is -s|l| plus 0 for n' >= 0 and 2 s min(-n', |l|) for n' < 0.
+__global__ void __launch_bounds__(32) m2qbxl_ff_kernel(
+    Fmm F, const int* __restrict__ pair_ctr, const int* __restrict__ pair_box, int n_pairs, int PW,
+    int TW, const float2* __restrict__ A, cd* __restrict__ partial) {
+  extern __shared__ __align__(16) float4 qrow[];  // [PW][TW]: w_m, w_{-m}
+  const int lane = threadIdx.x;
+  const int t0 = blockIdx.x * PW;
+  const int p = F.p, P = 2 * p + 1;
+  const int npw = min(PW, n_pairs - t0);
+  if (lane < npw) {
+    const int i = pair_ctr[t0 + lane], c = pair_box[t0 + lane];
+    const int l = F.level[c], M = F.lpb[l] + p, s = F.ffs[l];
+    const double2 z = F.cxy[i], mc = F.centre[c];
+    const FfUnits U(F.k);
+    FfPolar D;
+    D.set(z.x - mc.x, z.y - mc.y, U);
+    ffh hp, hc;
+    hankel01_ff_any<3>(D.z, hp, hc);
+    const float sg = pow2f(s), sg2 = pow2f(2 * s);
+    hc.x = ff_scale(hc.x, sg);
+    hc.y = ff_scale(hc.y, sg);
+    const ff c2 = split17(ff_mul_raw(ff_scale(U.ik2, sg), D.ir));  // 2 2^s / x
+    const ff c1 = ff_mul(D.x, D.ir), s1 = ff_mul(D.y, D.ir);
+    ff c8 = c1, s8 = s1;
+#pragma unroll
+    for (int u = 0; u < 3; ++u) ff_turn(c8, s8, c8, s8);
+    const float2 e1 = make_float2(ff_f32(c1), ff_f32(s1));
+    ff ex = c8, ey = s8;
+    float2 e = e1;
+    float4* row = qrow + (size_t)lane * TW;
+    const float2 h0 = make_float2(ff_f32(hp.x), ff_f32(hp.y));
+    row[0] = make_float4(h0.x, h0.y, h0.x, h0.y);
+    for (int m = 1; m <= M; ++m) {
+      if ((m & 7) == 0) {
+        e = make_float2(ff_f32(ex), ff_f32(ey));
+        ff_turn(ex, ey, c8, s8);
+      } else if (m > 1) {
+        e = fmul(e, e1);
+      }
+      const float2 hm = make_float2(ff_f32(hc.x), ff_f32(hc.y));
+      const float2 wp = fmul(hm, e), wq = fmul(hm, make_float2(e.x, -e.y));
+      row[m] = (m & 1) ? make_float4(wp.x, wp.y, -wq.x, -wq.y) : make_float4(wp.x, wp.y, wq.x, wq.y);
+      const ff cm = mkff((float)m * c2.h, (float)m * c2.l);
+      const ff nx = ff_sub_raw(ff_mul_raw(cm, hc.x), ff_scale(hp.x, sg2));
+      const ff ny = ff_sub_raw(ff_mul_raw(cm, hc.y), ff_scale(hp.y, sg2));
+      hp = hc;
+      hc.x = nx;
+      hc.y = ny;
+    }
+  }
+  __syncwarp();
+  for (int o = lane; o < npw * P; o += 32) {
+    const int u = o / P, lo = o % P - p;
+    const int c = pair_box[t0 + u];
+    const int l = F.level[c], pb = F.lpb[l], s = F.ffs[l];
+    const float4* row = qrow + (size_t)u * TW;
+    const float2* an = A + F.eoff[c] + pb;
+    const int a = abs(lo), dir = lo < 0 ? -1 : 1;
+    auto w = [&](int m, bool neg) {
+      const float4 v = row[m];
+      return neg ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+    };
+    float2 S1 = make_float2(0.f, 0.f), C1 = S1, S2 = S1, C2 = S1;
+    for (int j = 0; j <= pb; ++j)  // n' = j: m = dir (a + j)
+      kahan2(S1, C1, fmul(an[dir * j], w(a + j, lo < 0)));
+    for (int j = 1; j <= pb; ++j) {  // n' = -j: m = dir (a - j)
+      const bool neg = (a > j) ? lo < 0 : lo >= 0;
+      const float2 v = fmul(an[-dir * j], w(abs(a - j), neg));
+      if (j < a) {  // the exponent grows from n' = 0's by 2 s j (s < 0)
+        const float f = pow2f(2 * s * j);
+        kahan2(S1, C1, make_float2(v.x * f, v.y * f));
+      } else {
+        kahan2(S2, C2, v);
+      }
+    }
+    // exponents -s a for n' > -a (after the factors), s a for n' <= -a
+    double f1 = pow2d(-s * a), f2 = pow2d(s * a);
+    if (lo & 1) f1 = -f1, f2 = -f2;
+    partial[(size_t)(t0 + u) * P + lo + p] =
+        mk(((double)S1.x - (double)C1.x) * f1 + ((double)S2.x - (double)C2.x) * f2,
+           ((double)S1.y - (double)C1.y) * f1 + ((double)S2.y - (double)C2.y) * f2);
+  }
+}
+
 // ---------------------------------------------------------------- P2P in mixed precision
 // p2p_warp_kernel with everything but the two coordinate differences in
 // float-float (strengths, normals, tables to degree-6 second parts, the lanes'
@@ -1691,32 +1896,7 @@ __device__ __forceinline__ void p2m_fill_row_mixed(const Fmm& F, const FfUnits& 
   int en = 0;
   float imn = 0.f;
   if (in) {
-    const float sg2 = pow2f(2 * s);
-    ff c2 = ff_mul_raw(ff_scale(U.ik2, pow2f(s)), D.ir);  // 2 2^s / x
-    c2 = fast_two_sum(c2.h, c2.l);
-    const int M = pb + 1, N = miller_start_f32(M, D.z.h);  // N > M + 1
-    ff f1 = mkff(0.f, 0.f), f0 = mkff(0x1p-40f, 0.f), sum = f1;
-    float fn = (float)N;
-    for (int nn = N; nn >= 1; --nn) {
-      if ((nn & 1) == 0) sum = ff_add(f0, ff_scale(sum, sg2));
-      const float ch = __fmul_rn(fn, c2.h);
-      const ff cn = mkff(ch, __fmaf_rn(fn, c2.l, __fmaf_rn(fn, c2.h, -ch)));
-      const ff f = ff_sub_raw(ff_mul_raw(cn, f0), ff_scale(f1, sg2));
-      f1 = f0;
-      f0 = fast_two_sum(f.h, f.l);
-      fn -= 1.f;
-      if (nn - 1 <= M) row[nn - 1] = make_float2(f0.h, f0.l);
-      if (fabsf(f0.h) >= 0x1p20f) {
-        constexpr float d = 0x1p-60f;
-        f0 = ff_scale(f0, d);
-        f1 = ff_scale(f1, d);
-        sum = ff_scale(sum, d);
-        for (int u = nn - 1; u <= M; ++u) row[u] = make_float2(row[u].x * d, row[u].y * d);
-      }
-    }
-    const ff norm = ff_add(f0, ff_scale(sum, 2.f * sg2));
-    const float r = 1.0f / norm.h;  // 1 / norm by one Newton step
-    inv = mkff(r, __fmul_rn(r, __fmaf_rn(-norm.l, r, __fmaf_rn(-norm.h, r, 1.0f))));
+    inv = ff_miller_row(row, pb + 1, s, D, U);
   } else {
     const double dx = y.x - m.x, dy = y.y - m.y;
     const double d2 = dx * dx + dy * dy;
@@ -1728,22 +1908,16 @@ __device__ __forceinline__ void p2m_fill_row_mixed(const Fmm& F, const FfUnits& 
   const float2* isf = F.isf + (size_t)l * (F.pbmax + 2);
   const ff c1 = off ? ff_mul(D.x, D.ir) : mkff(1.f, 0.f);
   const ff s1 = off ? ff_mul(D.y, D.ir) : mkff(0.f, 0.f);
-  auto turn = [](ff& a, ff& b, ff c, ff d) {  // (a + i b) *= c + i d
-    const ff t = ff_sub_raw(ff_mul_raw(a, c), ff_mul_raw(b, d));
-    const ff u = ff_add(ff_mul_raw(a, d), ff_mul_raw(b, c));
-    a = fast_two_sum(t.h, t.l);
-    b = u;
-  };
   ff c8 = c1, s8 = mkff(-s1.h, -s1.l);  // e^{-8 i th} by three squarings
 #pragma unroll
-  for (int u = 0; u < 3; ++u) turn(c8, s8, c8, s8);
+  for (int u = 0; u < 3; ++u) ff_turn(c8, s8, c8, s8);
   const float2 emf = make_float2(ff_f32(c1), -ff_f32(s1));
   ff ex = mkff(1.f, 0.f), ey = mkff(0.f, 0.f);
   float2 ef = make_float2(1.f, 0.f);
   for (int j = 0; j <= pb + 1; ++j) {
     if ((j & 7) == 0) {
       ef = make_float2(ff_f32(ex), ff_f32(ey));
-      turn(ex, ey, c8, s8);
+      ff_turn(ex, ey, c8, s8);
     } else {
       ef = fmul(ef, emf);
     }
@@ -2334,6 +2508,29 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
       for (int64_t i = 0; i < h->n_ctr; ++i)
         if (mark[i]) used.push_back((int)i);
     }
+    // the W-list boxes of any centre, and whether every level the mixed L2QBXL
+    // (M2QBXL) meets has a float-float scaling (M2QBXL's rows go p orders further)
+    {
+      std::vector<char> seen(f->n_boxes, 0);
+      std::vector<int> cw;
+      f->ff_wboxes = true;
+      for (const std::vector<int>& w : wtrans)
+        for (int c : w)
+          if (!seen[c]) {
+            seen[c] = 1;
+            cw.push_back(c);
+            const int l = blev[c];
+            f->ff_wboxes = f->ff_wboxes && f->h_ffs[l] != kNoFf && f->h_pb[l] + h->p <= 100;
+          }
+      f->ff_leaves = true;
+      for (int b : leaves)
+        if (rc[b].y > rc[b].x && f->h_ffs[blev[b]] == kNoFf) f->ff_leaves = false;
+      f->n_cw_box = (int)cw.size();
+      QBX_CUDA_TRY(f->cw_box.alloc(std::max<size_t>(1, cw.size())));
+      if (!cw.empty())
+        QBX_CUDA_TRY(cudaMemcpy(f->cw_box.ptr, cw.data(), cw.size() * 4, cudaMemcpyHostToDevice));
+      QBX_CUDA_TRY(f->loc32.alloc(std::max<int64_t>(1, f->n_coef)));
+    }
     size_t max_pairs = 1;
     for (int k = 0; k < 2; ++k) {
       const std::vector<int>& list = k == 0 ? all : used;
@@ -2515,7 +2712,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.scale = f->scale.ptr; F.pw = f->pw.ptr; F.ipw = f->ipw.ptr;
   F.t_m2l = f->t_m2l.ptr; F.t_m2m = f->t_m2m.ptr; F.t_l2l = f->t_l2l.ptr;
   F.mpole = f->mpole.ptr; F.local = f->local.ptr; F.lpq = f->lpq.ptr;
-  F.ffs = f->ff_s.ptr;
+  F.ffs = f->ff_s.ptr; F.loc32 = f->loc32.ptr;
   F.conv = f->conv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.isf = f->isf.ptr; F.sigr = f->sigr.ptr;
   F.k = h->k; F.ik = 1.0 / h->k; F.side = f->side; F.pbmax = f->pb_max; F.p = h->p; F.n_levels = f->n_levels;
   F.has_S = S ? 1 : 0; F.has_D = D ? 1 : 0;
@@ -2539,10 +2736,14 @@ qbx_status launch_l2qbxl(const Fmm& F, FmmPlan* f, qbx_handle* h, const CentreSe
       while (!h->batched && G > 1 && (C.n + G - 1) / G < 152 * 2) G /= 2;
     // (batched handles share the SMs with other curves' stages and keep the
     // larger rows)
+    const bool ff32 = mixed && f->ff_leaves;
     const size_t lim = (mixed && !h->batched) ? kL2qbxlMixedSmem : kL2qbxlSmem;
-    while (G > 1 && (size_t)G * TW * sizeof(cd) > lim) G /= 2;
-    const size_t sm = (size_t)G * TW * sizeof(cd);
-    if (mixed) {
+    const size_t slot = ff32 ? sizeof(float2) : sizeof(cd);
+    while (G > 1 && (size_t)G * TW * slot > lim) G /= 2;
+    const size_t sm = (size_t)G * TW * slot;
+    if (ff32) {
+      l2qbxl_ff_kernel<<<nblk(C.n, G), 32, sm, s>>>(F, f->cleaf.ptr, C.clist.ptr, C.n, G, TW, alpha);
+    } else if (mixed) {
       split_coef_kernel<<<nblk(f->n_coef, 256), 256, 0, s>>>(f->local.ptr, f->n_coef, f->sp_m.ptr,
                                                              f->sp_e.ptr);
       l2qbxl_mixed_kernel<<<nblk(C.n, G), 32, sm, s>>>(F, f->cleaf.ptr, C.clist.ptr, C.n, G, TW,
@@ -2577,7 +2778,12 @@ qbx_status launch_m2qbxl(const Fmm& F, FmmPlan* f, qbx_handle* h, bool S, bool D
     int PW = h->batched ? 32 : kM2qbxlMixedPairs;
     while (PW > 1 && (size_t)PW * TW * 20 > kM2qbxlMixedSmem) PW /= 2;
     while (!h->batched && PW > 1 && (np + PW - 1) / PW < 152 * 2) PW /= 2;
-    if (mixed && (size_t)PW * TW * 20 <= kM2qbxlMixedSmem) {
+    if (mixed && f->ff_wboxes && (size_t)PW * TW * 16 <= kM2qbxlMixedSmem) {
+      mpole_scaled_kernel<<<f->n_cw_box, kThreads, 0, s>>>(F, f->cw_box.ptr, f->sp_m.ptr);
+      m2qbxl_ff_kernel<<<nblk(np, PW), 32, (size_t)PW * TW * 16, s>>>(
+          F, C.wp_ctr.ptr, C.wp_box.ptr, np, PW, TW, f->sp_m.ptr, part);
+      h->launches += 1;
+    } else if (mixed && (size_t)PW * TW * 20 <= kM2qbxlMixedSmem) {
       const long long ncoef = f->n_coef;
       split_coef_kernel<<<nblk(ncoef, 256), 256, 0, s>>>(f->mpole.ptr, ncoef, f->sp_m.ptr,
                                                         f->sp_e.ptr);

@@ -881,6 +881,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     std::vector<int> ffs(f->n_levels, kNoFf);
     for (int l = 2; l < f->n_levels; ++l)
       ffs[l] = float_float_scale(h->k * f->side / std::ldexp(1.0, l), f->h_pb[l]);
+    f->h_ffs = ffs;
     QBX_CUDA_TRY(f->ff_s.alloc(f->n_levels));
     QBX_CUDA_TRY(cudaMemcpy(f->ff_s.ptr, ffs.data(), f->n_levels * sizeof(int),
                             cudaMemcpyHostToDevice));

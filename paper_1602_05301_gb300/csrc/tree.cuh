@@ -133,6 +133,11 @@ struct FmmPlan {
   // [n_levels] s of the scaling 2^{s m} H_m, 2^{-s m} J_m that keeps orders up to
   // the level's in FP32's range (float-float kernels), or kNoFf
   DevBuf<int> ff_s;
+  std::vector<int> h_ffs;
+  bool ff_leaves = false, ff_wboxes = false;  // every centre leaf (W box) is on such a level
+  DevBuf<int> cw_box;                    // W-list boxes of the centres
+  int n_cw_box = 0;
+  DevBuf<float2> loc32;                  // [n_coef] scaled FP32 leaf locals (mixed L2QBXL)
   // Centre sets: [0] every centre, [1] the centres some target uses. Each
   // lists sorted centre indices (clist) and its M2QBXL work items, the
   // (sorted centre, W-list box) pairs grouped by list position (CSR wp_off).
