@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(32 * SW) p2qbxl_direct_kernel(
                             HD ? src_nrm[2 * j + 1] : 0.0, k, ik, p);
   }
   cd x32, x33;
-  warp_reduce_scatter<NC>(acc, lane, x32, x33);
+  group_reduce_scatter<32, NC>(acc, lane, x32, x33);
   cd v = acc[0];
   if (SW > 1) {
     __shared__ cd part[SW][34];
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(32 * SW) p2qbxl_direct_kernel(
     }
   }
   cd* dst = alpha + c * (2 * p + 1) + p;
-  pair_coefficients<PM>(v, x32, x33, lane, p, [&](int l, cd a) { dst[l] = a; });
+  pair_coefficients<32, PM>(v, v, x32, x33, lane, p, [&](int l, cd a) { dst[l] = a; });
 }
 
 // Smooth quadrature: u(t) = sum_j q_j H_0(k r) + d_j k H_1(k r) n_j.(t - s_j)/r.

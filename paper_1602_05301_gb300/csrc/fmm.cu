@@ -25,6 +25,7 @@
 #include <cstdio>
 #include <mutex>
 #include <set>
+#include <type_traits>
 #include <vector>
 
 #include "ff.cuh"
@@ -592,12 +593,12 @@ struct SourceCursor {
   }
 };
 
-template <typename Fn>
+template <int W = 32, typename Fn>
 __device__ __forceinline__ void deal_sources(const SourceCursor& sc, int lane, Fn&& fn) {
   const int tot = sc.total();
   int e = 0, base = 0;
   int2 r = sc.nu + sc.nx > 0 ? sc.rsrc[sc.box(0)] : make_int2(0, 0);
-  for (int t = lane; t < tot; t += 32) {
+  for (int t = lane; t < tot; t += W) {
     while (t >= base + (r.y - r.x)) {  // advance to the box holding source t
       base += r.y - r.x;
       r = sc.rsrc[sc.box(++e)];
@@ -1126,58 +1127,46 @@ __device__ __forceinline__ void p2qbxl_pair_mixed(float2 (&S)[2 * PM + 2], float
   hc.x = ff_scale(hc.x, sg);
   hc.y = ff_scale(hc.y, sg);
   const ff c2 = split17(ff_mul_raw(c2s, D.ir));  // 2 sigma / x
-  float cpsi = 0.f, spsi = 0.f;
-  const float2 dk = make_float2(dn.x, dn.y);
+  // D cos psi, D sin psi (psi = th - arg nu)
+  float2 dc = make_float2(0.f, 0.f), ds = dc;
   {
     float2 v = make_float2(0.f, 0.f);
     if (HS) v = fmul(q, make_float2(ff_f32(hp.x), ff_f32(hp.y)));
     if (HD) {
-      cpsi = fmaf(D.c, dn.z, D.s * dn.w);
-      spsi = fmaf(D.s, dn.z, -D.c * dn.w);
-      const float2 u = fmul(dk, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
-      const float t = -2.f * cpsi;  // E_0 = -2 H_1, K_0 = 0
-      v = make_float2(fmaf(u.x, t, v.x), fmaf(u.y, t, v.y));
+      const float cpsi = fmaf(D.c, dn.z, D.s * dn.w), spsi = fmaf(D.s, dn.z, -D.c * dn.w);
+      dc = make_float2(dn.x * cpsi, dn.y * cpsi);
+      ds = make_float2(dn.x * spsi, dn.y * spsi);
+      const float2 u = fmul(dc, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
+      v = make_float2(fmaf(-2.f, u.x, v.x), fmaf(-2.f, u.y, v.y));  // E_0 = -2 H_1
     }
     kahan2(S[0], C[0], v);
   }
-  float c = D.c, sn = D.s;
-  float ac = cpsi * c, as = cpsi * sn, bc = spsi * c, bs = spsi * sn;
-  auto turn = [&](float& u, float& v) {
-    const float t = fmaf(u, D.c, -v * D.s);
-    v = fmaf(u, D.s, v * D.c);
-    u = t;
-  };
+  float c = D.c, sn = D.s;  // cos m th, sin m th
 #pragma unroll
   for (int m = 1; m <= PM; ++m) {
     if (m > p) break;
     if (m > 1) {
-      if (HS) {
-        turn(c, sn);
-        if (HD) {
-          ac = cpsi * c;
-          as = cpsi * sn;
-          bc = spsi * c;
-          bs = spsi * sn;
-        }
-      } else {
-        turn(ac, as);
-        turn(bc, bs);
-      }
+      const float t = fmaf(c, D.c, -sn * D.s);
+      sn = fmaf(c, D.s, sn * D.c);
+      c = t;
     }
     const ff cm = mkff((float)m * c2.h, (float)m * c2.l);
     const ff Px = ff_mul_raw(cm, hc.x), Py = ff_mul_raw(cm, hc.y);
     const ff Zx = ff_scale(hp.x, sg2), Zy = ff_scale(hp.y, sg2);
-    float2 va = make_float2(0.f, 0.f), vb = va;
+    // G = q Ht + D cos psi E, L = D sin psi K: A = G cos + L sin, B = G sin - L cos
+    float2 G = make_float2(0.f, 0.f), va, vb;
+    if (HS) G = fmul(q, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
     if (HD) {
       const float px = ff_f32(Px), py = ff_f32(Py);
       const float ex = fmaf(2.f, ff_f32(Zx), -px), ey = fmaf(2.f, ff_f32(Zy), -py);
-      va = fmul(dk, make_float2(fmaf(ex, ac, px * bs), fmaf(ey, ac, py * bs)));
-      vb = fmul(dk, make_float2(fmaf(ex, as, -px * bc), fmaf(ey, as, -py * bc)));
-    }
-    if (HS) {
-      const float2 t = fmul(q, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
-      va = make_float2(fmaf(t.x, c, va.x), fmaf(t.y, c, va.y));
-      vb = make_float2(fmaf(t.x, sn, vb.x), fmaf(t.y, sn, vb.y));
+      G.x = fmaf(dc.x, ex, fmaf(-dc.y, ey, G.x));
+      G.y = fmaf(dc.x, ey, fmaf(dc.y, ex, G.y));
+      const float2 L = fmul(ds, make_float2(px, py));
+      va = make_float2(fmaf(G.x, c, L.x * sn), fmaf(G.y, c, L.y * sn));
+      vb = make_float2(fmaf(G.x, sn, -L.x * c), fmaf(G.y, sn, -L.y * c));
+    } else {
+      va = make_float2(G.x * c, G.y * c);
+      vb = make_float2(G.x * sn, G.y * sn);
     }
     kahan2(S[2 * m], C[2 * m], va);
     kahan2(S[2 * m + 1], C[2 * m + 1], vb);
@@ -2119,21 +2108,33 @@ qbx_status configure_kernels() {
   return QBX_OK;
 }
 
-// ---------------------------------------------------------------- P2QBXL, one warp per centre
-// Lanes stride over the concatenated sources of the centre's U-list boxes (so
-// the load is balanced to within one source), each lane keeps partial
-// coefficients (p2qbxl_pair), and a reduce-scatter of shuffles adds them.
-template <int PM, bool HS, bool HD>
+// ---------------------------------------------------------------- P2QBXL, W lanes per centre
+// The lanes of a centre stride over the concatenated sources of its U-list boxes
+// (so the load is balanced to within one source), each keeps partial coefficients
+// (p2qbxl_pair), and a reduce-scatter of shuffles adds them. A pass over a centre's
+// sources ends with a partly filled step (150 sources are 4.7 steps of 32 lanes), so
+// where centres are plenty half a warp takes one (W = 16, two centres per warp); with
+// few centres a warp each keeps more of the SMs' pipes fed. The rule takes all centres
+// of the handle, of which a launch may form only those that targets use, so that a
+// coefficient is the same sum whichever are formed. Measured with a warp and half a
+// warp each: 200 ellipses, mixed, 2.37 and 2.03 ms; 32 curves of 512 to 32768 centres in
+// a batch 5.99 and 5.34 ms in all; the GMRES solve with 3072 centres 38.3 and 42.6 ms.
+constexpr int kHalfWarpCentres = 6144;
+// Launches of fewer centres than this run one-warp blocks, which spread over the SMs
+// more evenly.
+constexpr int kSmallBlockCentres = 8192;
+template <int PM, bool HS, bool HD, int W>
 __global__ void __launch_bounds__(kThreads) p2qbxl_warp_kernel(Fmm F, const int* __restrict__ cleaf,
                                                                const int* __restrict__ wdoff,
                                                                const int* __restrict__ wdbox,
                                                                const int* __restrict__ clist,
                                                                int n_ctr, cd* __restrict__ alpha) {
   constexpr int NC = 2 * PM + 2;
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // position in clist
-  const int lane = threadIdx.x & 31;
-  if (w >= n_ctr) return;  // whole warps leave together
-  const int i = clist[w];  // sorted centre
+  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) / W);  // position in clist
+  const int lane = threadIdx.x & (W - 1);
+  if ((w & ~(32 / W - 1)) >= n_ctr) return;  // whole warps leave together
+  const bool live = w < n_ctr;  // the last warp's second half may be without a centre
+  const int i = clist[live ? w : n_ctr - 1];  // sorted centre
   const int b = cleaf[i];
   const double k = F.k, ik = F.ik, hk = 0.5 * k;
   const int p = F.p;
@@ -2151,25 +2152,28 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_kernel(Fmm F, const int*
   // U-list boxes of the leaf, then the W-list boxes summed directly for this centre
   const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], wdoff[i],
                         wdoff[i + 1] - wdoff[i], wdbox};
-  deal_sources(sc, lane, one);
+  if (live) deal_sources<W>(sc, lane, one);
+  __syncwarp();
   cd x32, x33;
-  warp_reduce_scatter<NC>(acc, lane, x32, x33);
+  group_reduce_scatter<W, NC>(acc, lane, x32, x33);
   cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
-  pair_coefficients<PM>(acc[0], x32, x33, lane, p,
-                        [&](int l, cd a) { dst[l] = cadd(dst[l], a); });
+  pair_coefficients<W, PM>(acc[0], acc[1], x32, x33, lane, p, [&](int l, cd a) {
+    if (live) dst[l] = cadd(dst[l], a);
+  });
 }
 
-template <int PM, bool HS, bool HD>
+template <int PM, bool HS, bool HD, int W>
 __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, const int* __restrict__ cleaf,
                                                                      const int* __restrict__ wdoff,
                                                                      const int* __restrict__ wdbox,
                                                                      const int* __restrict__ clist,
                                                                      int n_ctr, cd* __restrict__ alpha) {
   constexpr int NC = 2 * PM + 2;
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // position in clist
-  const int lane = threadIdx.x & 31;
-  if (w >= n_ctr) return;
-  const int i = clist[w];
+  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) / W);  // position in clist
+  const int lane = threadIdx.x & (W - 1);
+  if ((w & ~(32 / W - 1)) >= n_ctr) return;
+  const bool live = w < n_ctr;
+  const int i = clist[live ? w : n_ctr - 1];
   const int b = cleaf[i];
   const double k = F.k;
   const int p = F.p;
@@ -2195,17 +2199,19 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
   };
   const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], wdoff[i],
                         wdoff[i + 1] - wdoff[i], wdbox};
-  deal_sources(sc, lane, one);
-  // lane partial sums (compensation removed) in FP64, then the warp sum
+  if (live) deal_sources<W>(sc, lane, one);
+  __syncwarp();
+  // lane partial sums (compensation removed) in FP64, then the group's sum
   cd acc[NC];
 #pragma unroll
   for (int j = 0; j < NC; ++j)
     acc[j] = mk((double)S[j].x - (double)C[j].x, (double)S[j].y - (double)C[j].y);
   cd x32, x33;
-  warp_reduce_scatter<NC>(acc, lane, x32, x33);
+  group_reduce_scatter<W, NC>(acc, lane, x32, x33);
   cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
-  pair_coefficients<PM>(acc[0], x32, x33, lane, p, [&](int l, cd a) {
-    dst[l] = cadd(dst[l], cscale(a, pow2d(-s * (abs(l) + 1))));  // the sums carry sigma^{|l|+1}
+  pair_coefficients<W, PM>(acc[0], acc[1], x32, x33, lane, p, [&](int l, cd a) {
+    // the sums carry sigma^{|l|+1}
+    if (live) dst[l] = cadd(dst[l], cscale(a, pow2d(-s * (abs(l) + 1))));
   });
 }
 
@@ -2819,19 +2825,25 @@ qbx_status launch_centre_near(const Fmm& F, FmmPlan* f, qbx_handle* h, bool S, b
   if (!(S || D) || C.n == 0) return QBX_OK;
   stage_begin(h, QBX_STAGE_P2QBXL, s);
   const int nc = C.n;
-  const unsigned gw = nblk(nc, kThreads / 32);  // one warp per centre
-  const int* wo = f->wd_off.ptr;
-  const int* wb = f->wd_box.ptr;
   const int* cl = C.clist.ptr;
-  if (mixed) {
-    if (S && D) p2qbxl_warp_mixed_kernel<PM, true, true><<<gw, kThreads, 0, s>>>(F, f->cleaf.ptr, wo, wb, cl, nc, alpha);
-    else if (S) p2qbxl_warp_mixed_kernel<PM, true, false><<<gw, kThreads, 0, s>>>(F, f->cleaf.ptr, wo, wb, cl, nc, alpha);
-    else p2qbxl_warp_mixed_kernel<PM, false, true><<<gw, kThreads, 0, s>>>(F, f->cleaf.ptr, wo, wb, cl, nc, alpha);
-  } else {
-    if (S && D) p2qbxl_warp_kernel<PM, true, true><<<gw, kThreads, 0, s>>>(F, f->cleaf.ptr, wo, wb, cl, nc, alpha);
-    else if (S) p2qbxl_warp_kernel<PM, true, false><<<gw, kThreads, 0, s>>>(F, f->cleaf.ptr, wo, wb, cl, nc, alpha);
-    else p2qbxl_warp_kernel<PM, false, true><<<gw, kThreads, 0, s>>>(F, f->cleaf.ptr, wo, wb, cl, nc, alpha);
-  }
+  auto launch = [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    const int bt = nc < kSmallBlockCentres ? 32 : kThreads;
+    const unsigned g = nblk(nc, bt / W);
+#define P2QBXL_ARGS <<<g, bt, 0, s>>>(F, f->cleaf.ptr, f->wd_off.ptr, f->wd_box.ptr, cl, nc, alpha)
+    if (mixed) {
+      if (S && D) p2qbxl_warp_mixed_kernel<PM, true, true, W> P2QBXL_ARGS;
+      else if (S) p2qbxl_warp_mixed_kernel<PM, true, false, W> P2QBXL_ARGS;
+      else p2qbxl_warp_mixed_kernel<PM, false, true, W> P2QBXL_ARGS;
+    } else {
+      if (S && D) p2qbxl_warp_kernel<PM, true, true, W> P2QBXL_ARGS;
+      else if (S) p2qbxl_warp_kernel<PM, true, false, W> P2QBXL_ARGS;
+      else p2qbxl_warp_kernel<PM, false, true, W> P2QBXL_ARGS;
+    }
+#undef P2QBXL_ARGS
+  };
+  if (h->n_ctr >= kHalfWarpCentres) launch(std::integral_constant<int, 16>());
+  else launch(std::integral_constant<int, 32>());
   QBX_KCHECK("p2qbxl", s);
   stage_end(h, QBX_STAGE_P2QBXL, s);
   h->launches += 1;
