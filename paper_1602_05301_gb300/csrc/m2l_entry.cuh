@@ -1,8 +1,8 @@
 // Entries of the sigma-normalised M2L operator of one (level, offset class),
 //     T[n][lo] = sig_lo sig_n (-1)^lo W_{n+lo}(D) s^-|n+lo| (scale factors of
 //     the level's power-scaled Hankel table What_m = s^|m| W_m(D)),
-// computed in FP64 through logarithms (the table entries reach 1e155, the
-// sigma products are tiny): of order one or smaller for every n, lo. Used by
+// computed in FP64 through the logarithms of the scale factors (the table entries
+// reach 1e155, the sigma products are tiny): of order one or smaller for every n, lo. Used by
 // the FP32 M2L of the mixed path and by the tensor-core M2L of the FP64 path.
 #pragma once
 #include "qbx_internal.h"
@@ -20,14 +20,14 @@ struct M2lNorm {
     const int dx = cls / 7 - 3, dy = cls % 7 - 3;
     used = max(abs(dx), abs(dy)) >= 2;
   }
+  // the factor is at most 1 / |What|, so it may underflow where the product does
+  // not: its square root is applied twice
   __device__ cd entry(int n, int lo) const {
     if (!used) return mk(0.0, 0.0);
     const cd v = w[n + lo];
-    const double mag = hypot(v.x, v.y);  // no squares: entries reach 1e155
-    if (!(mag > 0.0)) return mk(0.0, 0.0);
-    const double lf = sg[abs(lo)] + sg[abs(n)] - abs(n + lo) * ls + log(mag);
-    const double f = lf < -700.0 ? 0.0 : exp(lf) / mag;
-    const double sgn = (lo & 1) ? -f : f;
-    return mk(v.x * sgn, v.y * sgn);
+    const double lf = sg[abs(lo)] + sg[abs(n)] - abs(n + lo) * ls;
+    double f = lf < -1400.0 ? 0.0 : exp(0.5 * lf);
+    const double g = (lo & 1) ? -f : f;
+    return mk(v.x * f * g, v.y * f * g);
   }
 };

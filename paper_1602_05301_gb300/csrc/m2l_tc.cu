@@ -281,7 +281,9 @@ __device__ double block_max(double v, double* red) {
 //   A[j][k] = Re T[n][lo] (j < Q, k < Q), -Im T[n][lo] (j < Q, k >= Q),
 //             Im T[n][lo] (j >= Q, k < Q), Re T[n][lo] (j >= Q, k >= Q),
 // lo = j mod Q, n = k mod Q, T the sigma-normalised M2L matrix; zero padding.
-// Grid (used groups, Np), threads over k. Slices [S][Np][Kp] at aoff.
+// Grid (used groups, Qmax + 1), threads over n: block lo forms T[.][lo] once for
+// the rows j = lo and lo + Q (which have the same largest entry, so one exponent);
+// block Q zeroes the padding rows. Slices [S][Np][Kp] at aoff.
 __global__ void __launch_bounds__(kThr) tc_matrix_kernel(
     const int* __restrict__ groups, const long long* __restrict__ aoff,
     const long long* __restrict__ foff, const int4* __restrict__ lvl, const int* __restrict__ lpb,
@@ -293,33 +295,46 @@ __global__ void __launch_bounds__(kThr) tc_matrix_kernel(
   const int4 P = lvl[l];  // (use, beta, S, Kp)
   const int Kp = P.w, beta = P.y, S = P.z;
   const int pb = lpb[l], Q = 2 * pb + 1;
-  const int j = blockIdx.y;
-  if (j >= Kp) return;
-  const int lo = (j < Q ? j : j - Q) - pb;
-  const bool im_out = j >= Q;
+  const int lo = blockIdx.y;
+  if (lo > Q) return;
+  __nv_bfloat16* base = A + aoff[blockIdx.x];
+  const size_t slice = (size_t)Kp * Kp;
+  if (lo == Q) {
+    for (int j = 2 * Q + (int)threadIdx.x; j < Kp; j += kThr) fexp[foff[blockIdx.x] + j] = 0;
+    for (int t = 0; t < S; ++t)
+      for (size_t i = (size_t)2 * Q * Kp + threadIdx.x; i < slice; i += kThr)
+        base[t * slice + i] = __float2bfloat16_rn(0.f);
+    return;
+  }
   const M2lNorm nm(t_m2l, scale, lsig, l, cls, pbmax);
-  double vals[16];  // k = threadIdx.x + 128 t, Kp <= 2048
+  cd vals[8];  // n = threadIdx.x + 128 t, Q <= Kp / 2 <= 1024
   double m = 0.0;
-  for (int t = 0; t < 16; ++t) {
-    const int k = threadIdx.x + kThr * t;
-    double v = 0.0;
-    if (j < 2 * Q && k < 2 * Q) {
-      const int n = (k < Q ? k : k - Q) - pb;
-      const cd T = nm.entry(n, lo);
-      const bool im_in = k >= Q;
-      v = im_out ? (im_in ? T.x : T.y) : (im_in ? -T.y : T.x);
-    }
-    vals[t] = v;
-    m = fmax(m, fabs(v));
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int n = threadIdx.x + kThr * t;
+    vals[t] = n < Q ? nm.entry(n - pb, lo - pb) : mk(0.0, 0.0);
+    m = fmax(m, fmax(fabs(vals[t].x), fabs(vals[t].y)));
   }
   m = block_max(m, red);
   const int e = scale_exponent(m);
-  if (threadIdx.x == 0) fexp[foff[blockIdx.x] + j] = e;
-  __nv_bfloat16* dst = A + aoff[blockIdx.x] + (size_t)j * Kp;
-  for (int t = 0; t < 16; ++t) {
-    const int k = threadIdx.x + kThr * t;
-    if (k < Kp) split_digits(vals[t], e, beta, S, dst + k, (size_t)Kp * Kp);
+  if (threadIdx.x == 0) {
+    fexp[foff[blockIdx.x] + lo] = e;
+    fexp[foff[blockIdx.x] + lo + Q] = e;
   }
+  __nv_bfloat16* r0 = base + (size_t)lo * Kp;
+  __nv_bfloat16* r1 = base + (size_t)(lo + Q) * Kp;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int n = threadIdx.x + kThr * t;
+    if (n >= Q) break;
+    split_digits(vals[t].x, e, beta, S, r0 + n, slice);
+    split_digits(-vals[t].y, e, beta, S, r0 + Q + n, slice);
+    split_digits(vals[t].y, e, beta, S, r1 + n, slice);
+    split_digits(vals[t].x, e, beta, S, r1 + Q + n, slice);
+  }
+  for (int k = 2 * Q + (int)threadIdx.x; k < Kp; k += kThr)
+    for (int t = 0; t < S; ++t)
+      r0[t * slice + k] = r1[t * slice + k] = __float2bfloat16_rn(0.f);
 }
 
 // Vector slices of the V-list sources: mu_n = mh_n conv_|n| (FP64), x = (Re mu,
@@ -1391,9 +1406,10 @@ qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f) {
     QBX_CUDA_TRY(cudaMemcpy(dg.ptr, groups.data(), groups.size() * 4, cudaMemcpyHostToDevice));
     QBX_CUDA_TRY(cudaMemcpy(da.ptr, g_aoff.data(), groups.size() * 8, cudaMemcpyHostToDevice));
     QBX_CUDA_TRY(cudaMemcpy(df.ptr, g_foff.data(), groups.size() * 8, cudaMemcpyHostToDevice));
-    int kpmax = 0;  // <= 2048 = 16 entries per thread (tc_params)
-    for (int l = 0; l < nl; ++l) kpmax = std::max(kpmax, lv[l].w);
-    dim3 grid((unsigned)groups.size(), (unsigned)kpmax);
+    int qmax = 0;  // 2 Q <= Kp <= 2048: 8 entries per thread (tc_params)
+    for (int l = 0; l < nl; ++l)
+      if (lv[l].x) qmax = std::max(qmax, 2 * f->h_pb[l] + 1);
+    dim3 grid((unsigned)groups.size(), (unsigned)qmax + 1);
     tc_matrix_kernel<<<grid, kThr>>>(dg.ptr, da.ptr, df.ptr, f->tc_lvl.ptr, f->lpb.ptr,
                                      f->pb_max, f->t_m2l.ptr, f->scale.ptr, f->lsig.ptr,
                                      reinterpret_cast<__nv_bfloat16*>(f->tc_A.ptr),

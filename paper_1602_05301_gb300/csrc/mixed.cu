@@ -35,18 +35,16 @@ __global__ void sigma_tables_kernel(int n_levels, int pbmax, const int* __restri
                                     double k, double side, const double* __restrict__ scale,
                                     double* __restrict__ lsig, double* __restrict__ conv,
                                     double* __restrict__ isig) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= n_levels) return;
+  const int l = blockIdx.x, pb = lpb[l];
   const double x = k * side / (double)(1 << l);
   const double ls = log(scale[l]);
-  double v = 0.0;
-  for (int j = 0; j <= lpb[l]; ++j) {
-    v = fmin(0.0, j * log(0.5 * x) - lgamma((double)j + 1.0));
+  for (int j = threadIdx.x; j <= pb; j += blockDim.x) {
+    const double v = fmin(0.0, j * log(0.5 * x) - lgamma((double)j + 1.0));
     lsig[(size_t)l * (pbmax + 1) + j] = v;
     conv[(size_t)l * (pbmax + 1) + j] = exp(j * ls - v);
     isig[(size_t)l * (pbmax + 2) + j] = exp(-v);
+    if (j == pb) isig[(size_t)l * (pbmax + 2) + pb + 1] = exp(-v);
   }
-  isig[(size_t)l * (pbmax + 2) + lpb[l] + 1] = exp(-v);
 }
 
 // Recurrence factors of G_m = sig_m H_m on level l (mixed M2P and P2L):
@@ -857,7 +855,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
   QBX_CUDA_TRY(f->lsig.alloc((size_t)f->n_levels * (pbm + 1)));
   QBX_CUDA_TRY(f->conv.alloc((size_t)f->n_levels * (pbm + 1)));
   QBX_CUDA_TRY(f->isig.alloc((size_t)f->n_levels * (pbm + 2)));
-  sigma_tables_kernel<<<1, 64>>>(f->n_levels, pbm, f->lpb.ptr, h->k, f->side, f->scale.ptr,
+  sigma_tables_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, h->k, f->side, f->scale.ptr,
                                  f->lsig.ptr, f->conv.ptr, f->isig.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
   QBX_CUDA_TRY(f->m2p_rec.alloc((size_t)f->n_levels * (pbm + 2)));
