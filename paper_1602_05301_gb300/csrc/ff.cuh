@@ -9,6 +9,8 @@
 //
 // Also H_0, H_1 from the tables of hankel_table_ff.h in float-float.
 #pragma once
+#include <cmath>
+
 #include "special.cuh"
 #include "hankel_table_ff.h"
 
@@ -73,6 +75,10 @@ __device__ __forceinline__ ff ff_from_f64(double v, int off) {
   r.l = (e <= 24 || e >= 255) ? 0.f : __fsub_rn(rest, one);
   return r;
 }
+// ff_from_f64 that keeps a NaN (which it makes infinite): coefficients, once each
+__device__ __forceinline__ ff ff_from_f64_nan(double v, int off) {
+  return v == v ? ff_from_f64(v, off) : mkff(__int_as_float(0x7FC00000), 0.f);
+}
 // FP64 constant (any magnitude FP32 holds) as float-float, for kernel arguments
 // and per-thread set-up
 __device__ __forceinline__ ff ff_round(double v) {
@@ -103,6 +109,22 @@ __device__ __forceinline__ ff ff_horner(ff p, ff t, float ch, float cl) {
 struct ffh {  // a complex float-float value
   ff x, y;
 };
+// keep += the value send of lane ^ off, not renormalised (group_reduce_scatter)
+__device__ __forceinline__ ffh lane_zero(const ffh*) {
+  ffh z;
+  z.x = z.y = mkff(0.f, 0.f);
+  return z;
+}
+__device__ __forceinline__ void lane_add(ff& keep, ff send, int off) {
+  const float h = __shfl_xor_sync(0xffffffffu, send.h, off);
+  const float l = __shfl_xor_sync(0xffffffffu, send.l, off);
+  const ff s = two_sum(keep.h, h);
+  keep = mkff(s.h, __fadd_rn(s.l, __fadd_rn(keep.l, l)));
+}
+__device__ __forceinline__ void lane_add(ffh& keep, const ffh& send, int off) {
+  lane_add(keep.x, send.x, off);
+  lane_add(keep.y, send.y, off);
+}
 
 // H_0, H_1 at 2^-16 <= x < 32 (x normalised) from the tables: the degrees
 // kHankDegFf .. ND in FP32, the lowest ND in float-float. The coefficients
@@ -167,18 +189,27 @@ __device__ __forceinline__ void hankel01_ff_any(ff x, ffh& h0, ffh& h1) {
 
 // Lengths in the float-float kernels are in units of 2^-sh (sh = floor(log2 k)), so
 // that the wavenumber is kk in [1, 2) and every quantity of order x = k r: off =
-// 896 - sh is ff_from_f64's offset.
+// 896 - sh is ff_from_f64's offset. Made on the host and passed to the kernels (a
+// thread forming it spends two dozen FP64 instructions).
 struct FfUnits {
   int off;
   ff kk, ik2;  // kk and 2 / kk
-  __device__ __forceinline__ explicit FfUnits(double k) {
-    const int sh = ilogb(k);
-    const double q = k * pow2d(-sh);
-    off = 896 - sh;
-    kk = ff_round(q);
-    ik2 = ff_round(2.0 / q);
-  }
 };
+inline FfUnits make_ff_units(double k) {
+  auto round2 = [](double v) {
+    ff r;
+    r.h = (float)v;
+    r.l = (float)(v - (double)r.h);
+    return r;
+  };
+  FfUnits U;
+  const int sh = std::ilogb(k);
+  const double q = std::ldexp(k, -sh);
+  U.off = 896 - sh;
+  U.kk = round2(q);
+  U.ik2 = round2(2.0 / q);
+  return U;
+}
 
 // (x, y) = a displacement in those units; x = k r, ir = 1 / r and the direction
 // e^{i th} in FP32. False at r = 0.

@@ -106,6 +106,7 @@ struct Fmm {
   const float2* isf;     // the same times 2^{ffs j}, float-float
   const double2* sigr;   // [n_levels][pbmax + 2] (sig_{j-1} / sig_j, sig_{j+1} / sig_j)
   double k, ik, side;    // wavenumber, 1 / k, root box side
+  FfUnits U;             // units of the float-float kernels
   int pbmax, p, n_levels, has_S, has_D;
 };
 
@@ -932,7 +933,7 @@ __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
       pq[at] = v;
       return;
     }
-    const ff x = ff_from_f64(v.x, 896 - s * m), y = ff_from_f64(v.y, 896 - s * m);
+    const ff x = ff_from_f64_nan(v.x, 896 - s * m), y = ff_from_f64_nan(v.y, 896 - s * m);
     reinterpret_cast<float4*>(pq)[at] = make_float4(x.h, x.l, y.h, y.l);
   };
   float2* g32 = F.loc32 + F.eoff[b] + pb;
@@ -1406,7 +1407,7 @@ __global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restr
     const int b = cleaf[i];
     const int l = F.level[b], M = F.lpb[l] + p, s = F.ffs[l];
     const double2 mb = F.centre[b], z = F.cxy[i];
-    const FfUnits U(F.k);
+    const FfUnits& U = F.U;
     FfPolar D;
     const bool off = D.set(z.x - mb.x, z.y - mb.y, U);
     float2* row = frow + (size_t)lane * TW;
@@ -1508,7 +1509,7 @@ __global__ void __launch_bounds__(32) m2qbxl_ff_kernel(
     const int i = pair_ctr[t0 + lane], c = pair_box[t0 + lane];
     const int l = F.level[c], M = F.lpb[l] + p, s = F.ffs[l];
     const double2 z = F.cxy[i], mc = F.centre[c];
-    const FfUnits U(F.k);
+    const FfUnits& U = F.U;
     FfPolar D;
     D.set(z.x - mc.x, z.y - mc.y, U);
     ffh hp, hc;
@@ -1606,7 +1607,7 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_mixed_kernel(Fmm F, const i
   const int i = utgt[t];
   const int b = tleaf[i];
   const double2 tp = F.txy[i];
-  const FfUnits U(F.k);
+  const FfUnits& U = F.U;
   FfSum acc;
   const SourceCursor sc{F.uidx, F.rsrc, F.uoff[b], F.uoff[b + 1] - F.uoff[b], 0, 0, nullptr};
   deal_sources(sc, lane, [&](int j) {
@@ -1660,7 +1661,7 @@ __global__ void __launch_bounds__(kThreads) l2p_mixed_kernel(Fmm F, const int* _
   const int pb = F.lpb[l], s = F.ffs[l];
   cd* dst = out + F.tid[i];
   const double2 mc = F.centre[b], tp = F.txy[i];
-  const FfUnits U(F.k);
+  const FfUnits& U = F.U;
   FfPolar D;
   const bool in = s != kNoFf && D.set(tp.x - mc.x, tp.y - mc.y, U) && D.z.h >= 1e-8f;
   if (!in) {
@@ -1801,7 +1802,7 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
   float2 S, C = make_float2(0.f, 0.f);
   if (s != kNoFf) {
     const float4* a = reinterpret_cast<const float4*>(mu + F.eoff[c] + c);
-    const FfUnits U(F.k);
+    const FfUnits& U = F.U;
     FfPolar D;
     D.set(dx, dy, U);
     ffh hp, hc;
@@ -1939,7 +1940,7 @@ __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
   float2* sb = sa + chunk;                // [chunk]
   if ((int)threadIdx.x < it.w) {
     const int j = threadIdx.x, i = src[it.z + j];
-    const FfUnits U(F.k);
+    const FfUnits& U = F.U;
     p2m_fill_row_mixed(F, U, i, F.centre[src_leaf[it.z + j]], l, pb, rows + j * RW + (pb + 1));
     const float4 ab = F.ab32[i];
     sq[j] = F.q32[i];
@@ -1960,14 +1961,17 @@ __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
         kahan2(Sb, Cb, fmul(sb[j], r[1]));
       }
     }
-    // sig_|n-1| / sig_|n| and sig_|n+1| / sig_|n| (1 beyond order pb)
-    const int an = abs(n);
-    const double2 rt = sr[an];  // (sig_{an-1} / sig_an, sig_{an+1} / sig_an)
-    const double fm = n > 0 ? rt.x : rt.y, fp = n < 0 ? rt.x : rt.y;
-    const double re = ((double)Sq.x - (double)Cq.x) + fm * ((double)Sa.x - (double)Ca.x) -
-                      fp * ((double)Sb.x - (double)Cb.x);
-    const double im = ((double)Sq.y - (double)Cq.y) + fm * ((double)Sa.y - (double)Ca.y) -
-                      fp * ((double)Sb.y - (double)Cb.y);
+    // sig_|n-1| / sig_|n| and sig_|n+1| / sig_|n| (1 beyond order pb); the three sums
+    // are joined in float-float
+    const double2 rt = sr[abs(n)];
+    const ff fm = ff_from_f64_nan(n > 0 ? rt.x : rt.y, 896),
+             fp = ff_from_f64_nan(n < 0 ? rt.x : rt.y, 896);
+    auto join = [&](float q, float cq, float a, float ca, float b, float cb) {
+      const ff t = ff_sub_raw(ff_mul_raw(mkff(a, -ca), fm), ff_mul_raw(mkff(b, -cb), fp));
+      return ff_f64(ff_add(mkff(q, -cq), t));
+    };
+    const double re = join(Sq.x, Cq.x, Sa.x, Ca.x, Sb.x, Cb.x);
+    const double im = join(Sq.y, Cq.y, Sa.y, Ca.y, Sb.y, Cb.y);
     partial[seg_poff[it.x + u] + n + pb] = mk(re, im);
   }
 }
@@ -2181,7 +2185,7 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
   // sigma = 2^s within a factor sqrt 2 of k r_c
   const int s = ilogb(k * F.crad[i] * 1.4142135623730951);
   const float sg = pow2f(s), sg2 = pow2f(2 * s);
-  const FfUnits U(k);
+  const FfUnits& U = F.U;
   const ff c2s = ff_scale(U.ik2, sg);
   float2 S[NC], C[NC];
 #pragma unroll
@@ -2201,15 +2205,22 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
                         wdoff[i + 1] - wdoff[i], wdbox};
   if (live) deal_sources<W>(sc, lane, one);
   __syncwarp();
-  // lane partial sums (compensation removed) in FP64, then the group's sum
-  cd acc[NC];
+  // the lanes' sums (S - C) added over the group in float-float: in FP64 the
+  // conversions and additions of one centre were 290 FP64 instructions, as many as
+  // 145 of its pairs
+  ffh acc[NC];
 #pragma unroll
-  for (int j = 0; j < NC; ++j)
-    acc[j] = mk((double)S[j].x - (double)C[j].x, (double)S[j].y - (double)C[j].y);
-  cd x32, x33;
-  group_reduce_scatter<W, NC>(acc, lane, x32, x33);
+  for (int j = 0; j < NC; ++j) {
+    acc[j].x = mkff(S[j].x, -C[j].x);
+    acc[j].y = mkff(S[j].y, -C[j].y);
+  }
+  ffh y32, y33;
+  group_reduce_scatter<W, NC>(acc, lane, y32, y33);
+  auto f64 = [](ffh v) { return mk(ff_f64(v.x), ff_f64(v.y)); };
+  const cd a0 = f64(acc[0]), a1 = W == 16 ? f64(acc[1]) : a0;
+  const cd x32 = PM == 16 ? f64(y32) : a0, x33 = PM == 16 ? f64(y33) : a0;
   cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
-  pair_coefficients<W, PM>(acc[0], acc[1], x32, x33, lane, p, [&](int l, cd a) {
+  pair_coefficients<W, PM>(a0, a1, x32, x33, lane, p, [&](int l, cd a) {
     // the sums carry sigma^{|l|+1}
     if (live) dst[l] = cadd(dst[l], cscale(a, pow2d(-s * (abs(l) + 1))));
   });
@@ -2720,6 +2731,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.mpole = f->mpole.ptr; F.local = f->local.ptr; F.lpq = f->lpq.ptr;
   F.ffs = f->ff_s.ptr; F.loc32 = f->loc32.ptr;
   F.conv = f->conv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.isf = f->isf.ptr; F.sigr = f->sigr.ptr;
+  F.U = make_ff_units(h->k);
   F.k = h->k; F.ik = 1.0 / h->k; F.side = f->side; F.pbmax = f->pb_max; F.p = h->p; F.n_levels = f->n_levels;
   F.has_S = S ? 1 : 0; F.has_D = D ? 1 : 0;
   return F;

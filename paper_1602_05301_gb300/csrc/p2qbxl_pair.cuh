@@ -95,25 +95,32 @@ __device__ __forceinline__ void p2qbxl_pair(cd (&acc)[2 * PM + 2], double dx, do
   }
 }
 
+// keep += the value send of lane ^ off (complex FP64, and float-float in ff.cuh)
+__device__ __forceinline__ cd lane_zero(const cd*) { return mk(0.0, 0.0); }
+__device__ __forceinline__ void lane_add(cd& keep, const cd& send, int off) {
+  const double x = __shfl_xor_sync(0xffffffffu, send.x, off);
+  const double y = __shfl_xor_sync(0xffffffffu, send.y, off);
+  keep.x += x;
+  keep.y += y;
+}
+
 // Sums the partial coefficients of a group of W lanes (32, or 16: two centres per
 // warp) by a reduce-scatter of shuffles (31 or 30 complex shuffles for 32 entries
 // instead of 160 for a butterfly): afterwards lane g of the group holds the sums of
 // entries (32 / W) g .. in acc[0..32 / W). Entries 32 and 33 (order 16) are summed by
 // a butterfly into x32, x33 on every lane; padding both of them to a second 32
 // would double the shuffles.
-template <int W, int NC>
-__device__ __forceinline__ void group_reduce_scatter(cd (&acc)[NC], int lane, cd& x32, cd& x33) {
+template <int W, int NC, typename V>
+__device__ __forceinline__ void group_reduce_scatter(V (&acc)[NC], int lane, V& x32, V& x33) {
   static_assert(NC <= 34, "at most order 16");
-  constexpr unsigned kAll = 0xffffffffu;
-  x32 = NC > 32 ? acc[NC - 2] : mk(0.0, 0.0);
-  x33 = NC > 32 ? acc[NC - 1] : mk(0.0, 0.0);
+  const V zero = lane_zero((const V*)nullptr);
+  x32 = NC > 32 ? acc[NC - 2] : zero;
+  x33 = NC > 32 ? acc[NC - 1] : zero;
   if (NC > 32) {
 #pragma unroll
     for (int off = W / 2; off >= 1; off >>= 1) {
-      x32.x += __shfl_xor_sync(kAll, x32.x, off);
-      x32.y += __shfl_xor_sync(kAll, x32.y, off);
-      x33.x += __shfl_xor_sync(kAll, x33.x, off);
-      x33.y += __shfl_xor_sync(kAll, x33.y, off);
+      lane_add(x32, x32, off);
+      lane_add(x33, x33, off);
     }
   }
   constexpr int N = NC < 32 ? NC : 32;
@@ -123,12 +130,11 @@ __device__ __forceinline__ void group_reduce_scatter(cd (&acc)[NC], int lane, cd
     const bool upper = (lane & off) != 0;
 #pragma unroll
     for (int i = 0; i < h; ++i) {
-      const cd lo = i < N ? acc[i] : mk(0.0, 0.0);
-      const cd hi = i + h < N ? acc[i + h] : mk(0.0, 0.0);
-      const cd send = upper ? lo : hi;
-      cd keep = upper ? hi : lo;
-      keep.x += __shfl_xor_sync(kAll, send.x, off);
-      keep.y += __shfl_xor_sync(kAll, send.y, off);
+      const V lo = i < N ? acc[i] : zero;
+      const V hi = i + h < N ? acc[i + h] : zero;
+      const V send = upper ? lo : hi;
+      V keep = upper ? hi : lo;
+      lane_add(keep, send, off);
       if (i < N) acc[i] = keep;
     }
   }
