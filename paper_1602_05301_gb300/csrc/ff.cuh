@@ -247,8 +247,18 @@ __device__ __forceinline__ void ff_turn(ff& a, ff& b, ff c, ff d) {
 }
 
 // Miller's backward recurrence on f_j ~ 2^{-s j} J_j(k r), j = 0..M, kept in row
-// (h, l) while it runs; returns 1 / norm (2^{-s j} J_j = row[j] / norm):
+// (h, l); returns 1 / norm:
 //   f_{n-1} = (2 n 2^s / x) f_n - 4^s f_{n+1},  norm = f_0 + 2 4^s (f_2 + 4^s (f_4 + ...)).
+// Where f outgrows its range it is scaled by kMillerDown, and the order at which that
+// happened is marked in the row (the lowest bit of l): ff_miller_value, called for j =
+// 0, 1, ... M in this order, gives 2^{-s j} J_j / inv. (Scaling the stored orders at
+// once, a loop over them, was over half of the fill's instructions: the lanes of a
+// warp outgrow the range at different orders.)
+constexpr float kMillerDown = 0x1p-60f;
+__device__ __forceinline__ ff ff_miller_value(float2 v, float& scale) {
+  if (__float_as_uint(v.y) & 1u) scale *= kMillerDown;
+  return mkff(v.x * scale, v.y * scale);
+}
 __device__ __forceinline__ ff ff_miller_row(float2* row, int M, int s, const FfPolar& D,
                                             const FfUnits& U) {
   const float sg2 = pow2f(2 * s);
@@ -265,13 +275,14 @@ __device__ __forceinline__ ff ff_miller_row(float2* row, int M, int s, const FfP
     f1 = f0;
     f0 = fast_two_sum(f.h, f.l);
     fn -= 1.f;
-    if (nn - 1 <= M) row[nn - 1] = make_float2(f0.h, f0.l);
-    if (fabsf(f0.h) >= 0x1p20f) {
-      constexpr float d = 0x1p-60f;
-      f0 = ff_scale(f0, d);
-      f1 = ff_scale(f1, d);
-      sum = ff_scale(sum, d);
-      for (int u = nn - 1; u <= M; ++u) row[u] = make_float2(row[u].x * d, row[u].y * d);
+    const bool over = fabsf(f0.h) >= 0x1p20f;
+    if (nn - 1 <= M)
+      row[nn - 1] = make_float2(
+          f0.h, __uint_as_float((__float_as_uint(f0.l) & ~1u) | (over ? 1u : 0u)));
+    if (over) {
+      f0 = ff_scale(f0, kMillerDown);
+      f1 = ff_scale(f1, kMillerDown);
+      sum = ff_scale(sum, kMillerDown);
     }
   }
   const ff norm = ff_add(f0, ff_scale(sum, 2.f * sg2));

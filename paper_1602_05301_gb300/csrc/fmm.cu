@@ -1429,6 +1429,7 @@ __global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restr
       const float2 e1 = make_float2(ff_f32(c1), ff_f32(s1));
       ff ex = mkff(1.f, 0.f), ey = mkff(0.f, 0.f);
       float2 e = make_float2(1.f, 0.f);
+      float sc = 1.f;
       for (int m = 0; m <= M; ++m) {
         if ((m & 7) == 0) {
           e = make_float2(ff_f32(ex), ff_f32(ey));
@@ -1436,8 +1437,7 @@ __global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restr
         } else {
           e = fmul(e, e1);
         }
-        const float2 f = row[m];
-        const float v = ff_f32(ff_mul_raw(mkff(f.x, f.y), inv));
+        const float v = ff_f32(ff_mul_raw(ff_miller_value(row[m], sc), inv));
         row[m] = make_float2(e.x * v, e.y * v);
       }
     }
@@ -1866,8 +1866,8 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
 // A = d (k/2) conj(nu), B = d (k/2) nu; mu_n = a_n / sig_|n|, of order one.
 // p2m_sum_mixed_kernel adds a leaf's segments in FP64 and forms mh_n = mu_n /
 // conv_|n| (conv = s^j / sig_j).
-// Row of source i for a box of level l with centre m: row[t] = R_t, |t| <= pb + 1
-// (row points at t = 0). On float-float levels the Miller recurrence of
+// Row of source i for a box of level l with centre m: row[t] = R_t, 0 <= t <= pb + 1
+// (R_{-t} = (-1)^t conj(R_t)). On float-float levels the Miller recurrence of
 // l2p_mixed_kernel on 2^{-s j} J_j (its values kept in the row while it runs),
 // normalised and brought to J_j / sig_j by isf[j] = 2^{s j} / sig_j; elsewhere in
 // FP64, one product per order, the normalisation as an exponent offset and an
@@ -1904,6 +1904,7 @@ __device__ __forceinline__ void p2m_fill_row_mixed(const Fmm& F, const FfUnits& 
   const float2 emf = make_float2(ff_f32(c1), -ff_f32(s1));
   ff ex = mkff(1.f, 0.f), ey = mkff(0.f, 0.f);
   float2 ef = make_float2(1.f, 0.f);
+  float sc = 1.f;
   for (int j = 0; j <= pb + 1; ++j) {
     if ((j & 7) == 0) {
       ef = make_float2(ff_f32(ex), ff_f32(ey));
@@ -1913,19 +1914,32 @@ __device__ __forceinline__ void p2m_fill_row_mixed(const Fmm& F, const FfUnits& 
     }
     float v;
     if (in) {
-      const float2 f = row[j], g = isf[j];
-      v = ff_f32(ff_mul_raw(ff_mul_raw(mkff(f.x, f.y), mkff(g.x, g.y)), inv));
+      const float2 g = isf[j];
+      v = ff_f32(ff_mul_raw(ff_mul_raw(ff_miller_value(row[j], sc), mkff(g.x, g.y)), inv));
     } else {
       v = f32_from_f64_sh(reinterpret_cast<const double*>(row)[j] * isg[j], -en) * imn;
     }
-    const float2 c = make_float2(ef.x * v, ef.y * v);  // R_j
-    row[j] = c;
-    if (j > 0) row[-j] = (j & 1) ? make_float2(-c.x, c.y) : make_float2(c.x, -c.y);
+    row[j] = make_float2(ef.x * v, ef.y * v);  // R_j
   }
 }
 
-// Rows and strengths of an item in shared memory: FP32, half the FP64 form's.
-__global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
+// v, or its conjugate where neg is the sign bit
+__device__ __forceinline__ float2 fconj_if(float2 v, unsigned neg) {
+  return make_float2(v.x, __uint_as_float(__float_as_uint(v.y) ^ neg));
+}
+
+// Rows and strengths of an item in shared memory: FP32 and t >= 0 only, a quarter of
+// the FP64 form's. One warp fills an item's rows while the others wait, so blocks of
+// 64 threads, of which twice as many share an SM. (With this, and with the orders that
+// Miller's recurrence outgrows marked instead of rescaled at once, 200 ellipses 0.84 ->
+// 0.51 ms, the starfish at k = 50 0.135 -> 0.088.)
+constexpr int kP2mMixedThreads = 64;
+static_assert(kP2mMixedThreads >= kChunk, "a thread per source of an item");
+__host__ __device__ inline int p2m_mixed_row(int pb) { return (pb + 2) | 1; }
+inline size_t p2m_mixed_smem(int pb, int chunk) {
+  return (size_t)chunk * (p2m_mixed_row(pb) + 3) * sizeof(float2);
+}
+__global__ void __launch_bounds__(kP2mMixedThreads) p2m_item_mixed_kernel(
     Fmm F, const int4* __restrict__ items, const int* __restrict__ seg_leaf,
     const int2* __restrict__ seg_row, const long long* __restrict__ seg_poff,
     const int* __restrict__ src, const int* __restrict__ src_leaf, cd* __restrict__ partial,
@@ -1933,7 +1947,7 @@ __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
   extern __shared__ __align__(16) float2 fsmem[];
   const int4 it = items[blockIdx.x];
   const int l = F.level[seg_leaf[it.x]];
-  const int pb = F.lpb[l], Q = 2 * pb + 1, RW = 2 * pb + 3;
+  const int pb = F.lpb[l], Q = 2 * pb + 1, RW = p2m_mixed_row(pb);
   float2* rows = fsmem;                   // [chunk][RW], it.w <= chunk
   float2* sq = rows + chunk * RW;         // [chunk]
   float2* sa = sq + chunk;                // [chunk]
@@ -1941,7 +1955,7 @@ __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
   if ((int)threadIdx.x < it.w) {
     const int j = threadIdx.x, i = src[it.z + j];
     const FfUnits& U = F.U;
-    p2m_fill_row_mixed(F, U, i, F.centre[src_leaf[it.z + j]], l, pb, rows + j * RW + (pb + 1));
+    p2m_fill_row_mixed(F, U, i, F.centre[src_leaf[it.z + j]], l, pb, rows + j * RW);
     const float4 ab = F.ab32[i];
     sq[j] = F.q32[i];
     sa[j] = make_float2(ab.z, ab.w);  // d (k/2) conj(nu)
@@ -1949,26 +1963,33 @@ __global__ void __launch_bounds__(kThreads) p2m_item_mixed_kernel(
   }
   __syncthreads();
   const double2* sr = F.sigr + (size_t)l * (F.pbmax + 2);
-  for (int idx = threadIdx.x; idx < it.y * Q; idx += kThreads) {
+  for (int idx = threadIdx.x; idx < it.y * Q; idx += kP2mMixedThreads) {
     const int u = idx / Q, n = idx % Q - pb;
     const int2 rg = seg_row[it.x + u];
     float2 Sq = make_float2(0.f, 0.f), Cq = Sq, Sa = Sq, Ca = Sq, Sb = Sq, Cb = Sq;
+    const int an = abs(n), aa = abs(n - 1), ab = abs(n + 1);
+    const unsigned gq = n < 0 ? 0x80000000u : 0u, ga = n < 1 ? 0x80000000u : 0u,
+                   gb = n < -1 ? 0x80000000u : 0u;
     for (int j = rg.x; j < rg.x + rg.y; ++j) {
-      const float2* r = rows + j * RW + (pb + 1) + n;
-      if (F.has_S) kahan2(Sq, Cq, fmul(sq[j], r[0]));
+      const float2* r = rows + j * RW;
+      if (F.has_S) kahan2(Sq, Cq, fmul(sq[j], fconj_if(r[an], gq)));
       if (F.has_D) {
-        kahan2(Sa, Ca, fmul(sa[j], r[-1]));
-        kahan2(Sb, Cb, fmul(sb[j], r[1]));
+        kahan2(Sa, Ca, fmul(sa[j], fconj_if(r[aa], ga)));
+        kahan2(Sb, Cb, fmul(sb[j], fconj_if(r[ab], gb)));
       }
     }
+    // the sign (-1)^t of the negative orders t
+    const float zq = gq && (an & 1) ? -1.f : 1.f, za = ga && (aa & 1) ? -1.f : 1.f,
+                zb = gb && (ab & 1) ? -1.f : 1.f;
     // sig_|n-1| / sig_|n| and sig_|n+1| / sig_|n| (1 beyond order pb); the three sums
     // are joined in float-float
-    const double2 rt = sr[abs(n)];
+    const double2 rt = sr[an];
     const ff fm = ff_from_f64_nan(n > 0 ? rt.x : rt.y, 896),
              fp = ff_from_f64_nan(n < 0 ? rt.x : rt.y, 896);
     auto join = [&](float q, float cq, float a, float ca, float b, float cb) {
-      const ff t = ff_sub_raw(ff_mul_raw(mkff(a, -ca), fm), ff_mul_raw(mkff(b, -cb), fp));
-      return ff_f64(ff_add(mkff(q, -cq), t));
+      const ff t = ff_sub_raw(ff_mul_raw(mkff(za * a, -za * ca), fm),
+                              ff_mul_raw(mkff(zb * b, -zb * cb), fp));
+      return ff_f64(ff_add(mkff(zq * q, -zq * cq), t));
     };
     const double re = join(Sq.x, Cq.x, Sa.x, Ca.x, Sb.x, Cb.x);
     const double im = join(Sq.y, Cq.y, Sa.y, Ca.y, Sb.y, Cb.y);
@@ -2588,6 +2609,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
     f->p2m_sm = rows_launch_smem(pbs);
     const int chunk = rows_chunk(pbs, f->p2m_sm);  // the least capacity over the leaf levels
     f->p2m_chunk = chunk;
+    f->p2m_pb = pbs;
     std::vector<int> sleaf, psrc, psleaf, lseg(src_leaves.size() + 1, 0);
     std::vector<int2> srow;
     std::vector<long long> spoff;
@@ -2972,7 +2994,8 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   stage_begin(h, QBX_STAGE_P2M, s);
   if ((S || D) && f->n_p2m_items > 0) {
     if (mixed) {
-      p2m_item_mixed_kernel<<<f->n_p2m_items, kThreads, f->p2m_sm / 2, s>>>(
+      p2m_item_mixed_kernel<<<f->n_p2m_items, kP2mMixedThreads,
+                              p2m_mixed_smem(f->p2m_pb, f->p2m_chunk), s>>>(
           F, f->p2m_items.ptr, f->p2m_segleaf.ptr, f->p2m_segrow.ptr, f->p2m_segpoff.ptr,
           f->p2m_src.ptr, f->p2m_srcleaf.ptr, f->p2m_part.ptr, f->p2m_chunk);
       QBX_KCHECK("p2m", s);

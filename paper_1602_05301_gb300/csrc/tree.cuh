@@ -109,7 +109,7 @@ struct FmmPlan {
   DevBuf<cd> p2m_part;
   int n_p2m_items = 0;
   size_t p2m_sm = 0;
-  int p2m_chunk = 0;                    // most sources of an item
+  int p2m_chunk = 0, p2m_pb = 0;        // most sources of an item, largest leaf order
   // xbox and vbox are ordered by level; [n_levels + 1] offsets
   std::vector<int> xbox_off, vbox_off;
   int q_leaf = 1, q_w = 1;              // largest Q_l among leaves / W-list boxes
