@@ -2014,83 +2014,140 @@ __global__ void __launch_bounds__(kThreads) p2m_sum_mixed_kernel(
 
 // P2L in mixed precision: the item structure of p2l_item_kernel with FP32
 // rows and sums. Row j of a source holds G_j e^{i j th} (j >= 0) and
-// (-1)^j G_j e^{-i j th} (j < 0), G_j = sig_j H_j(k r) by the FP64 recurrence
-// G_{j+1} = rec[j].x (1/x) G_j - rec[j].y G_{j-1} (sig of the box's level,
+// (-1)^j G_j e^{-i j th} (j < 0), G_j = sig_j H_j(k r) (sig of the box's level,
 // sig_{pb+1} taken as sig_pb); X-list sources lie at least 1.5 box sides from
-// the centre, so G_j is of order one or smaller. The angular factors are FP32
-// between FP64 anchors every eighth order. Per output order n the charge and
-// the two dipole sums are FP32 with Kahan compensation over the item's
+// the centre, so G_j is of order one or smaller. On float-float levels
+// G_j = w_j / isf[j], w_j = 2^{s j} H_j by the float-float recurrence
+//   w_{j+1} = (2 j 2^s / x) w_j - 4^s w_{j-1};
+// elsewhere in FP64, G_{j+1} = rec[j].x (1/x) G_j - rec[j].y G_{j-1}. The angular
+// factors are FP32 between anchors every eighth order. Per output order n the charge
+// and the two dipole sums are FP32 with Kahan compensation over the item's
 // sources; lambda_n = sig_n gamma_n = Sq + (sig_n / sig_|n-1|) Sa -
 // (sig_n / sig_|n+1|) Sb and lh_n = lambda_n conv_|n| are formed in FP64.
-__global__ void __launch_bounds__(kThreads) p2l_item_mixed_kernel(
+// (One warp of a block fills its rows: bound by that recurrence's latency and by how
+// many blocks share an SM. Against FP64 recurrences, rows in 16-byte slots and blocks
+// of 128 threads, 200 ellipses 0.64 -> 0.31 ms, the starfish at k = 50 0.073 -> 0.043.)
+constexpr int kP2lMixedThreads = 64;
+static_assert(kP2lMixedThreads >= kChunk, "a thread per source of an item");
+inline size_t p2l_mixed_smem(int pb, int chunk) {
+  return (size_t)chunk * (2 * pb + 6) * sizeof(float2);
+}
+// The row (at j = 0) of one source; R = rec, g = isf of the box's level.
+__device__ __forceinline__ void p2l_fill_row_mixed(const Fmm& F, double dx, double dy, int l, int pb,
+                                                   const double2* __restrict__ R, float2* row) {
+  const int s = F.ffs[l];
+  auto put = [&](int j, float2 g, float2 e) {
+    const float2 wp = fmul(g, e);
+    const float2 wq = fmul(g, make_float2(e.x, -e.y));
+    row[j] = wp;
+    row[-j] = (j & 1) ? make_float2(-wq.x, -wq.y) : wq;
+  };
+  if (s != kNoFf) {
+    const float2* isf = F.isf + (size_t)l * (F.pbmax + 2);
+    const FfUnits& U = F.U;
+    FfPolar D;
+    D.set(dx, dy, U);
+    ffh hp, hc;
+    hankel01_ff_any<3>(D.z, hp, hc);
+    const float sg = pow2f(s), sg2 = pow2f(2 * s);
+    hc.x = ff_scale(hc.x, sg);
+    hc.y = ff_scale(hc.y, sg);
+    const ff c2 = split17(ff_mul_raw(ff_scale(U.ik2, sg), D.ir));  // 2 2^s / x
+    const ff c1 = ff_mul(D.x, D.ir), s1 = ff_mul(D.y, D.ir);
+    ff c8 = c1, s8 = s1;
+#pragma unroll
+    for (int u = 0; u < 3; ++u) ff_turn(c8, s8, c8, s8);
+    const float2 e1 = make_float2(ff_f32(c1), ff_f32(s1));
+    ff ex = c8, ey = s8;
+    float2 e = e1;
+    auto scaled = [&](int j, ffh w) {  // w / isf[j]
+      const float2 g = isf[j];
+      const float r = 1.0f / g.x;
+      const ff ig = mkff(r, __fmul_rn(r, __fmaf_rn(-g.y, r, __fmaf_rn(-g.x, r, 1.0f))));
+      return make_float2(ff_f32(ff_mul_raw(w.x, ig)), ff_f32(ff_mul_raw(w.y, ig)));
+    };
+    row[0] = scaled(0, hp);
+    for (int j = 1; j <= pb + 1; ++j) {
+      if ((j & 7) == 0) {
+        e = make_float2(ff_f32(ex), ff_f32(ey));
+        ff_turn(ex, ey, c8, s8);
+      } else if (j > 1) {
+        e = fmul(e, e1);
+      }
+      put(j, scaled(j, hc), e);
+      const ff cj = mkff((float)j * c2.h, (float)j * c2.l);
+      const ff nx = ff_sub_raw(ff_mul_raw(cj, hc.x), ff_scale(hp.x, sg2));
+      const ff ny = ff_sub_raw(ff_mul_raw(cj, hc.y), ff_scale(hp.y, sg2));
+      hp = hc;
+      hc.x = nx;
+      hc.y = ny;
+    }
+    return;
+  }
+  const double d2 = dx * dx + dy * dy;
+  const double ir = rsqrt(d2), x = F.k * (d2 * ir), ix = ir * F.ik;
+  cd h0, h1;
+  hankel01_wide(x, ix, h0, h1);
+  const cd e1 = mk(dx * ir, dy * ir);
+  cd e8 = cmul(e1, e1);
+  e8 = cmul(e8, e8);
+  e8 = cmul(e8, e8);
+  const float2 e1f = f2(e1);
+  cd gprev = h0, gcur = cscale(h1, R[0].x);  // G_0, G_1
+  cd E = mk(1.0, 0.0);
+  float2 ef = make_float2(1.f, 0.f);
+  row[0] = f2(h0);
+  for (int j = 1; j <= pb + 1; ++j) {
+    if ((j & 7) == 0) {  // e^{i j th}: an FP64 anchor every eighth order
+      E = cmul(E, e8);
+      ef = f2(E);
+    } else {
+      ef = fmul(ef, e1f);
+    }
+    put(j, f2(gcur), ef);
+    if (j <= pb) {
+      const double c1 = R[j].x * ix, c2 = R[j].y;
+      const cd gn = mk(fma(c1, gcur.x, -c2 * gprev.x), fma(c1, gcur.y, -c2 * gprev.y));
+      gprev = gcur;
+      gcur = gn;
+    }
+  }
+}
+__global__ void __launch_bounds__(kP2lMixedThreads) p2l_item_mixed_kernel(
     Fmm F, const int4* __restrict__ items, const int* __restrict__ src,
-    const long long* __restrict__ poff, cd* __restrict__ partial, unsigned sm_bytes,
+    const long long* __restrict__ poff, cd* __restrict__ partial, int chunk,
     const double2* __restrict__ rec) {
-  extern __shared__ cd smem[];
-  const int4 it = items[blockIdx.x];  // (box, first position in src, sources, -)
+  extern __shared__ __align__(16) float2 fsmem[];
+  const int4 it = items[blockIdx.x];  // (box, first position in src, sources <= chunk, -)
   const int b = it.x, cnt = it.z;
   const int l = F.level[b];
   const int pb = F.lpb[l], RW = 2 * pb + 3;  // row: |t| <= pb+1
-  const int chunk = rows_chunk(pb, sm_bytes);
-  cd* rows = smem;                        // [chunk][RW], FP32 entries in the first half of each slot
-  cd* sq = rows + chunk * RW;             // [chunk]
-  cd* sa = sq + chunk;                    // [chunk]  A = d (k/2) nu
-  cd* sb = sa + chunk;                    // [chunk]  B = d (k/2) conj(nu)
+  float2* rows = fsmem;                   // [chunk][RW]
+  float2* sq = rows + chunk * RW;         // [chunk]
+  float2* sa = sq + chunk;                // [chunk]  A = d (k/2) nu
+  float2* sb = sa + chunk;                // [chunk]  B = d (k/2) conj(nu)
   const double2 m = F.centre[b];
   if ((int)threadIdx.x < cnt) {
     const int i = src[it.y + threadIdx.x];
-    const double dx = F.sxy[i].x - m.x, dy = F.sxy[i].y - m.y;
-    const double d2 = dx * dx + dy * dy;
-    const double ir = rsqrt(d2), x = F.k * (d2 * ir), ix = ir * F.ik;
-    cd h0, h1;
-    hankel01_wide(x, ix, h0, h1);
-    const double2* R = rec + (size_t)l * (F.pbmax + 2);
-    const cd e1 = mk(dx * ir, dy * ir);
-    cd e8 = cmul(e1, e1);
-    e8 = cmul(e8, e8);
-    e8 = cmul(e8, e8);
-    const float2 e1f = f2(e1);
-    float2* row = reinterpret_cast<float2*>(rows + threadIdx.x * RW + (pb + 1));
-    cd gprev = h0, gcur = cscale(h1, R[0].x);  // G_0, G_1
-    cd E = mk(1.0, 0.0);
-    float2 ef = make_float2(1.f, 0.f);
-    row[0] = f2(h0);
-    for (int j = 1; j <= pb + 1; ++j) {
-      if ((j & 7) == 0) {  // e^{i j th}: an FP64 anchor every eighth order
-        E = cmul(E, e8);
-        ef = f2(E);
-      } else {
-        ef = fmul(ef, e1f);
-      }
-      const float2 g = f2(gcur);
-      const float2 wp = fmul(g, ef);
-      const float2 wq = fmul(g, make_float2(ef.x, -ef.y));
-      row[2 * j] = wp;
-      row[-2 * j] = (j & 1) ? make_float2(-wq.x, -wq.y) : wq;
-      if (j <= pb) {
-        const double c1 = R[j].x * ix, c2 = R[j].y;
-        const cd gn = mk(fma(c1, gcur.x, -c2 * gprev.x), fma(c1, gcur.y, -c2 * gprev.y));
-        gprev = gcur;
-        gcur = gn;
-      }
-    }
+    p2l_fill_row_mixed(F, F.sxy[i].x - m.x, F.sxy[i].y - m.y, l, pb,
+                       rec + (size_t)l * (F.pbmax + 2), rows + threadIdx.x * RW + (pb + 1));
     const float4 ab = F.ab32[i];
-    reinterpret_cast<float2*>(sq + threadIdx.x)[0] = F.q32[i];
-    reinterpret_cast<float2*>(sa + threadIdx.x)[0] = make_float2(ab.x, ab.y);  // d (k/2) nu
-    reinterpret_cast<float2*>(sb + threadIdx.x)[0] = make_float2(ab.z, ab.w);  // d (k/2) conj(nu)
+    sq[threadIdx.x] = F.q32[i];
+    sa[threadIdx.x] = make_float2(ab.x, ab.y);  // d (k/2) nu
+    sb[threadIdx.x] = make_float2(ab.z, ab.w);  // d (k/2) conj(nu)
   }
   __syncthreads();
   const double2* sr = F.sigr + (size_t)l * (F.pbmax + 2);
   const double* cv = F.conv + (size_t)l * (F.pbmax + 1);
   cd* dst = partial + poff[blockIdx.x] + pb;
-  for (int n = (int)threadIdx.x - pb; n <= pb; n += kThreads) {
+  for (int n = (int)threadIdx.x - pb; n <= pb; n += kP2lMixedThreads) {
     float2 Sq = make_float2(0.f, 0.f), Cq = Sq, Sa = Sq, Ca = Sq, Sb = Sq, Cb = Sq;
     for (int j = 0; j < cnt; ++j) {
-      const float2* r = reinterpret_cast<const float2*>(rows + j * RW + (pb + 1));
-      if (F.has_S) kahan2(Sq, Cq, fmul(reinterpret_cast<const float2*>(sq + j)[0], r[2 * n]));
+      const float2* r = rows + j * RW + (pb + 1) + n;
+      if (F.has_S) kahan2(Sq, Cq, fmul(sq[j], r[0]));
       if (F.has_D) {
-        kahan2(Sa, Ca, fmul(reinterpret_cast<const float2*>(sa + j)[0], r[2 * (n - 1)]));
-        kahan2(Sb, Cb, fmul(reinterpret_cast<const float2*>(sb + j)[0], r[2 * (n + 1)]));
+        kahan2(Sa, Ca, fmul(sa[j], r[-1]));
+        kahan2(Sb, Cb, fmul(sb[j], r[1]));
       }
     }
     // sig_|n| / sig_|n-1| and sig_|n| / sig_|n+1| from the ratio table (which
@@ -2669,6 +2726,8 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
     const int pbx = max_order(f->h_pb, f->xbox_off);
     f->p2l_sm = rows_launch_smem(pbx);
     const int chunk = rows_chunk(pbx, f->p2l_sm);  // the least capacity over the X levels
+    f->p2l_chunk = chunk;
+    f->p2l_pb = pbx;
     std::vector<int> src, boff(f->n_xbox + 1, 0);
     std::vector<int4> items;
     std::vector<long long> poff;
@@ -2950,9 +3009,10 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
   stage_begin(h, QBX_STAGE_P2L, s2);
   if ((S || D) && f->n_p2l_items > 0) {  // X lists without sources add nothing
     if (mixed)
-      p2l_item_mixed_kernel<<<f->n_p2l_items, kThreads, f->p2l_sm, s2>>>(
-          F, f->p2l_items.ptr, f->p2l_src.ptr, f->p2l_poff.ptr, f->p2l_part.ptr,
-          (unsigned)f->p2l_sm, f->m2p_rec.ptr);
+      p2l_item_mixed_kernel<<<f->n_p2l_items, kP2lMixedThreads,
+                              p2l_mixed_smem(f->p2l_pb, f->p2l_chunk), s2>>>(
+          F, f->p2l_items.ptr, f->p2l_src.ptr, f->p2l_poff.ptr, f->p2l_part.ptr, f->p2l_chunk,
+          f->m2p_rec.ptr);
     else
       p2l_item_kernel<<<f->n_p2l_items, kThreads, f->p2l_sm, s2>>>(
           F, f->p2l_items.ptr, f->p2l_src.ptr, f->p2l_poff.ptr, f->p2l_part.ptr, (unsigned)f->p2l_sm);

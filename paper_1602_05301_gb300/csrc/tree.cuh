@@ -110,6 +110,7 @@ struct FmmPlan {
   int n_p2m_items = 0;
   size_t p2m_sm = 0;
   int p2m_chunk = 0, p2m_pb = 0;        // most sources of an item, largest leaf order
+  int p2l_chunk = 0, p2l_pb = 0;        // the same of the X boxes
   // xbox and vbox are ordered by level; [n_levels + 1] offsets
   std::vector<int> xbox_off, vbox_off;
   int q_leaf = 1, q_w = 1;              // largest Q_l among leaves / W-list boxes
