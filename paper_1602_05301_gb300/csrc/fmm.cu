@@ -100,7 +100,7 @@ struct Fmm {
   cd* lpq;               // [n_coef] leaf cos/sin coefficients of L2P (see unscale_leaf_locals_kernel)
   const int* ffs;        // [n_levels] power-of-two scale exponent of the float-float kernels
   float2* loc32;         // [n_coef] leaf locals gamma_n 2^{ffs |n|} (mixed L2QBXL)
-  const double* conv;    // [n_levels][pbmax + 1] s^j / sig_j (mixed path)
+  const double *conv, *iconv;  // [n_levels][pbmax + 1] s^j / sig_j and its inverse (mixed path)
   const double* lsig;    // [n_levels][pbmax + 1] log sig_j
   const double* isig;    // [n_levels][pbmax + 2] 1 / sig_min(j, pb) (mixed P2M)
   const float2* isf;     // the same times 2^{ffs j}, float-float
@@ -2003,12 +2003,12 @@ __global__ void __launch_bounds__(kThreads) p2m_sum_mixed_kernel(
   const int t = blockIdx.x, b = leaves[t];
   const int l = F.level[b];
   const int pb = F.lpb[l], Q = 2 * pb + 1;
-  const double* cv = F.conv + (size_t)l * (F.pbmax + 1);
+  const double* icv = F.iconv + (size_t)l * (F.pbmax + 1);
   cd* dst = F.mpole + F.eoff[b];
   for (int n = threadIdx.x; n < Q; n += kThreads) {
     cd sum = mk(0.0, 0.0);
     for (int g = lseg[t]; g < lseg[t + 1]; ++g) sum = cadd(sum, partial[seg_poff[g] + n]);
-    dst[n] = cscale(sum, 1.0 / cv[abs(n - pb)]);
+    dst[n] = cscale(sum, icv[abs(n - pb)]);
   }
 }
 
@@ -2023,7 +2023,7 @@ __global__ void __launch_bounds__(kThreads) p2m_sum_mixed_kernel(
 // factors are FP32 between anchors every eighth order. Per output order n the charge
 // and the two dipole sums are FP32 with Kahan compensation over the item's
 // sources; lambda_n = sig_n gamma_n = Sq + (sig_n / sig_|n-1|) Sa -
-// (sig_n / sig_|n+1|) Sb and lh_n = lambda_n conv_|n| are formed in FP64.
+// (sig_n / sig_|n+1|) Sb and lh_n = lambda_n conv_|n|.
 // (One warp of a block fills its rows: bound by that recurrence's latency and by how
 // many blocks share an SM. Against FP64 recurrences, rows in 16-byte slots and blocks
 // of 128 threads, 200 ellipses 0.64 -> 0.31 ms, the starfish at k = 50 0.073 -> 0.043.)
@@ -2150,16 +2150,19 @@ __global__ void __launch_bounds__(kP2lMixedThreads) p2l_item_mixed_kernel(
         kahan2(Sb, Cb, fmul(sb[j], r[1]));
       }
     }
-    // sig_|n| / sig_|n-1| and sig_|n| / sig_|n+1| from the ratio table (which
-    // holds sig_|n-1| / sig_|n| and sig_|n+1| / sig_|n|, 1 beyond order pb)
+    // sig_|n| / sig_|n-1| and sig_|n| / sig_|n+1|: the ratio table holds sig_{m-1} /
+    // sig_m and sig_{m+1} / sig_m at m (1 beyond order pb); the three sums are joined
+    // in float-float
     const int an = abs(n);
-    const double2 rt = sr[an];
-    const double fm = 1.0 / (n > 0 ? rt.x : rt.y), fp = 1.0 / (n < 0 ? rt.x : rt.y);
+    const double up = sr[an + 1].x, dn = an > 0 ? sr[an - 1].y : up;
+    const ff fm = ff_from_f64_nan(n > 0 ? dn : up, 896), fp = ff_from_f64_nan(n < 0 ? dn : up, 896);
     const double c = cv[an];
-    const double re = ((double)Sq.x - (double)Cq.x) + fm * ((double)Sa.x - (double)Ca.x) -
-                      fp * ((double)Sb.x - (double)Cb.x);
-    const double im = ((double)Sq.y - (double)Cq.y) + fm * ((double)Sa.y - (double)Ca.y) -
-                      fp * ((double)Sb.y - (double)Cb.y);
+    auto join = [&](float q, float cq, float a, float ca, float b, float cb) {
+      const ff t = ff_sub_raw(ff_mul_raw(mkff(a, -ca), fm), ff_mul_raw(mkff(b, -cb), fp));
+      return ff_f64(ff_add(mkff(q, -cq), t));
+    };
+    const double re = join(Sq.x, Cq.x, Sa.x, Ca.x, Sb.x, Cb.x);
+    const double im = join(Sq.y, Cq.y, Sa.y, Ca.y, Sb.y, Cb.y);
     dst[n] = mk(re * c, im * c);
   }
 }
@@ -2811,7 +2814,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.t_m2l = f->t_m2l.ptr; F.t_m2m = f->t_m2m.ptr; F.t_l2l = f->t_l2l.ptr;
   F.mpole = f->mpole.ptr; F.local = f->local.ptr; F.lpq = f->lpq.ptr;
   F.ffs = f->ff_s.ptr; F.loc32 = f->loc32.ptr;
-  F.conv = f->conv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.isf = f->isf.ptr; F.sigr = f->sigr.ptr;
+  F.conv = f->conv.ptr; F.iconv = f->iconv.ptr; F.lsig = f->lsig.ptr; F.isig = f->isig.ptr; F.isf = f->isf.ptr; F.sigr = f->sigr.ptr;
   F.U = make_ff_units(h->k);
   F.k = h->k; F.ik = 1.0 / h->k; F.side = f->side; F.pbmax = f->pb_max; F.p = h->p; F.n_levels = f->n_levels;
   F.has_S = S ? 1 : 0; F.has_D = D ? 1 : 0;

@@ -30,18 +30,20 @@ constexpr int kT = 128;
 inline unsigned nblk(int64_t n, int b) { return (unsigned)std::max<int64_t>(1, (n + b - 1) / b); }
 
 // per level: lsig[j] = log sig_j, conv[j] = s^j / sig_j  (j = 0..pb_l; stride
-// pbmax + 1), isig[j] = 1 / sig_min(j, pb_l) (j = 0..pb_l + 1; stride pbmax + 2)
+// pbmax + 1), iconv = 1 / conv, isig[j] = 1 / sig_min(j, pb_l) (j = 0..pb_l + 1; stride pbmax + 2)
 __global__ void sigma_tables_kernel(int n_levels, int pbmax, const int* __restrict__ lpb,
                                     double k, double side, const double* __restrict__ scale,
                                     double* __restrict__ lsig, double* __restrict__ conv,
-                                    double* __restrict__ isig) {
+                                    double* __restrict__ iconv, double* __restrict__ isig) {
   const int l = blockIdx.x, pb = lpb[l];
   const double x = k * side / (double)(1 << l);
   const double ls = log(scale[l]);
   for (int j = threadIdx.x; j <= pb; j += blockDim.x) {
     const double v = fmin(0.0, j * log(0.5 * x) - lgamma((double)j + 1.0));
     lsig[(size_t)l * (pbmax + 1) + j] = v;
-    conv[(size_t)l * (pbmax + 1) + j] = exp(j * ls - v);
+    const double c = exp(j * ls - v);
+    conv[(size_t)l * (pbmax + 1) + j] = c;
+    iconv[(size_t)l * (pbmax + 1) + j] = 1.0 / c;
     isig[(size_t)l * (pbmax + 2) + j] = exp(-v);
     if (j == pb) isig[(size_t)l * (pbmax + 2) + pb + 1] = exp(-v);
   }
@@ -87,19 +89,51 @@ __global__ void sig_ratio_kernel(int n_levels, int pbmax, const int* __restrict_
   }
 }
 
-// Level l's matrices Tm[cls][n][lo] = sig_lo sig_n (-1)^lo W_{n+lo}(D) (orders
-// up to pb = pb_l; M2lNorm), stored in FP32. Grid: (cls, n), threads over lo.
-__global__ void m2l_f32_matrix_kernel(int l, int pb, int pbmax, const cd* __restrict__ t_m2l,
-                                      const double* __restrict__ scale,
-                                      const double* __restrict__ lsig, float2* __restrict__ Tm) {
+// The FP32 M2L matrices. An offset D = |D| e^{i phi} acts on sigma-normalised
+// coefficients as T[n][l] = (-1)^l sig_l sig_n W_{n+l}(D), W_m = H_m(k |D|) e^{i m phi}.
+// With x_n = e^{i n phi} mu_n the angle is gone, and because H_{-m} = (-1)^m H_m the
+// matrix splits into one for the even parts e_n = x_n + (-1)^n x_{-n} and one for the
+// odd parts o_n = x_n - (-1)^n x_{-n} (0 <= n, l <= pb; e_0 = x_0):
+//   y_l    = (-1)^l e^{ i l phi} (E_l + O_l),   E_l = sum_n Te[n][l] e_n,
+//   y_{-l} =        e^{-i l phi} (E_l - O_l),   O_l = sum_n To[n][l] o_n,
+//   Te, To = sig_l sig_n (H_{n+l} +- (-1)^l H_{n-l}) / 2:
+// half the products, and the 40 offsets of a V list share the matrices of their
+// kM2lDist distances. Tm[d][2][n][l] of level l here; grid (d, n), threads over l.
+constexpr int kM2lDist = 7;  // |D| of (2,0) (2,1) (2,2) (3,0) (3,1) (3,2) (3,3) box sides
+__host__ __device__ constexpr int m2l_dist(int cls) {  // of offset class (dx + 3) * 7 + dy + 3
+  const int dx = cls / 7 - 3, dy = cls % 7 - 3;
+  const int ax = dx < 0 ? -dx : dx, ay = dy < 0 ? -dy : dy;
+  const int hi = ax > ay ? ax : ay, lo = ax > ay ? ay : ax;
+  return hi == 2 ? lo : hi == 3 ? 3 + lo : -1;
+}
+__global__ void m2l_fold_matrix_kernel(int l, int pb, int pbmax, const cd* __restrict__ t_m2l,
+                                       const double* __restrict__ scale,
+                                       const double* __restrict__ lsig, float2* __restrict__ Tm) {
+  const int d = blockIdx.x, n = blockIdx.y, P = pb + 1;
+  const int dx = d < 3 ? 2 : 3, dy = d < 3 ? d : d - 3;
+  const M2lNorm nm(t_m2l, scale, lsig, l, (dx + 3) * 7 + dy + 3, pbmax);
+  const double turn = -atan2((double)dy, (double)dx) * 0.31830988618379067154;  // -phi / pi
+  float2* te = Tm + ((size_t)2 * d * P + n) * P;
+  float2* to = te + (size_t)P * P;
+  for (int lo = threadIdx.x; lo <= pb; lo += blockDim.x) {
+    cd ra, rb;
+    sincospi((n + lo) * turn, &ra.y, &ra.x);
+    sincospi((n - lo) * turn, &rb.y, &rb.x);
+    cd a = cmul(nm.entry(n, lo), ra);         // (-1)^lo sig sig H_{n+lo}
+    const cd b = cmul(nm.entry(n, -lo), rb);  // (-1)^lo sig sig H_{n-lo}
+    if (lo & 1) a = mk(-a.x, -a.y);
+    te[lo] = make_float2((float)(0.5 * (a.x + b.x)), (float)(0.5 * (a.y + b.y)));
+    to[lo] = make_float2((float)(0.5 * (a.x - b.x)), (float)(0.5 * (a.y - b.y)));
+  }
+}
+// rot[cls][m] = e^{i m phi}, m <= pbmax
+__global__ void m2l_rot_kernel(int pbmax, float2* __restrict__ rot) {
   const int cls = blockIdx.x;
-  const int n = (int)blockIdx.y - pb;
-  const int Q = 2 * pb + 1;
-  const M2lNorm nm(t_m2l, scale, lsig, l, cls, pbmax);
-  float2* dst = Tm + ((size_t)cls * Q + (n + pb)) * Q;
-  for (int lo = (int)threadIdx.x - pb; lo <= pb; lo += blockDim.x) {
-    const cd v = nm.entry(n, lo);
-    dst[lo + pb] = make_float2((float)v.x, (float)v.y);
+  const double turn = atan2((double)(cls % 7 - 3), (double)(cls / 7 - 3)) * 0.31830988618379067154;
+  for (int m = threadIdx.x; m <= pbmax; m += blockDim.x) {
+    double c, sn;
+    sincospi(m * turn, &sn, &c);
+    rot[(size_t)cls * (pbmax + 1) + m] = make_float2((float)c, (float)sn);
   }
 }
 
@@ -141,21 +175,17 @@ __device__ __forceinline__ f32p fma2(f32p a, f32p b, f32p c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
-__device__ __forceinline__ f32p mul2(f32p a, f32p b) {
-  f32p r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
 __device__ __forceinline__ f32p add2(f32p a, f32p b) {
   f32p r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 __device__ __forceinline__ f32p sub2(f32p a, f32p b) { return fma2(b, pk(-1.f, -1.f), a); }
-__device__ __forceinline__ void kahan_add2(f32p& s, f32p& c, f32p v) {
-  const f32p y = sub2(v, c);
+// s += y, where y holds the lost part n of the sum so far (s + n is the sum); the new
+// lost part
+__device__ __forceinline__ void kahan_add2(f32p& s, f32p& n, f32p y) {
   const f32p t = add2(s, y);
-  c = sub2(sub2(t, s), y);
+  n = sub2(y, sub2(t, s));
   s = t;
 }
 
@@ -166,23 +196,13 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
   s = t;
 }
 
-// M2L as batched complex GEMMs. The V-list pairs (target box b, source box c)
-// are grouped by (level, offset class) at plan time; all pairs of a group use
-// the same matrix Tm[cls]. A CTA takes kGemmRows pairs of one group: their
-// sigma-normalised source coefficients mu (FP32) go to shared memory ([n][row],
-// n-major), and each thread computes one output order lo for all the rows,
-// streaming matrix row n once for all of them (so the matrix is read once per
-// kGemmRows pairs instead of once per pair). Sums: plain FP32 FMAs over blocks
-// of kGemmBlock terms, blocks added with Kahan compensation. Each pair's result
-// goes to its row of Y (FP32); m2l_f32_reduce_kernel adds each target box's
-// rows in its V-list order with Kahan compensation (deterministic).
+// The tile GEMMs. A CTA takes some rows (M2L: V-list pairs; M2M, L2L: parents) that
+// share a matrix: their FP32 coefficients go to shared memory ([n][row], n-major), and
+// each thread computes one output order for R rows, streaming the matrix once for all
+// of them. Sums: plain FP32 FMAs over blocks of kGemmBlock terms, blocks added with
+// Kahan compensation.
 constexpr int kGemmRows = 16;
 constexpr int kGemmBlock = 8;
-// M2M / L2L levels with fewer parents than kWideLevel use tiles of kNarrowRows
-// parents, so that the launch still spreads over the SMs.
-constexpr int kNarrowRows = 4;
-constexpr int kWideLevel = kGemmRows * 2 * 152;
-
 // Staged rows: order n of the row pair (r, r + 1), r even, is the float4 (re r,
 // re r+1, im r, im r+1) at x + n * stage_stride(R) + r, so that each half is an
 // operand of the packed FMAs. Two float2 of padding per n keep the row pairs
@@ -194,18 +214,18 @@ __device__ __forceinline__ void stage_put(float2* x, size_t n, int r, int RS, fl
   f[2] = v.y;
 }
 
-// Sums of R rows, row pairs packed: value s, Kahan compensation c (the sum is s - c).
+// Sums of R rows, row pairs packed: value s, lost part n (the sum is s + n).
 template <int R>
 struct RowSums {
-  f32p sr[R / 2], si[R / 2], cr[R / 2], ci[R / 2];
+  f32p sr[R / 2], si[R / 2], nr[R / 2], ni[R / 2];
   __device__ __forceinline__ RowSums() {
 #pragma unroll
-    for (int r = 0; r < R / 2; ++r) sr[r] = si[r] = cr[r] = ci[r] = 0ull;
+    for (int r = 0; r < R / 2; ++r) sr[r] = si[r] = nr[r] = ni[r] = 0ull;
   }
   __device__ __forceinline__ float sum_r(int r) const { return part(sr[r / 2], r); }
   __device__ __forceinline__ float sum_i(int r) const { return part(si[r / 2], r); }
-  __device__ __forceinline__ float comp_r(int r) const { return part(cr[r / 2], r); }
-  __device__ __forceinline__ float comp_i(int r) const { return part(ci[r / 2], r); }
+  __device__ __forceinline__ float lost_r(int r) const { return part(nr[r / 2], r); }
+  __device__ __forceinline__ float lost_i(int r) const { return part(ni[r / 2], r); }
   __device__ static __forceinline__ float part(f32p v, int r) {
     const float2 u = unpk(v);
     return (r & 1) ? u.y : u.x;
@@ -213,8 +233,8 @@ struct RowSums {
 };
 
 // One block of nj (1 <= nj <= kGemmBlock) terms of a tile product column,
-// sum_{j < nj} tb[j] * x[j], started from the first term and added to S with
-// Kahan compensation.
+// sum_{j < nj} tb[j] * x[j], started from the lost part of S and added to S (Kahan
+// compensation in three operations per block).
 template <int R>
 __device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], int nj,
                                                const float2* __restrict__ x, RowSums<R>& S) {
@@ -231,8 +251,8 @@ __device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], i
       for (int r = 0; r < R / 2; ++r) {
         const ulonglong2 v = m[r];  // (re, re), (im, im) of rows 2r, 2r + 1
         if (j == 0) {
-          tr[r] = fma2(tx, v.x, mul2(my, v.y));
-          ti[r] = fma2(tx, v.y, mul2(ty, v.x));
+          tr[r] = fma2(tx, v.x, fma2(my, v.y, S.nr[r]));
+          ti[r] = fma2(tx, v.y, fma2(ty, v.x, S.ni[r]));
         } else {
           tr[r] = fma2(tx, v.x, fma2(my, v.y, tr[r]));
           ti[r] = fma2(tx, v.y, fma2(ty, v.x, ti[r]));
@@ -242,8 +262,8 @@ __device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], i
   }
 #pragma unroll
   for (int r = 0; r < R / 2; ++r) {
-    kahan_add2(S.sr[r], S.cr[r], tr[r]);
-    kahan_add2(S.si[r], S.ci[r], ti[r]);
+    kahan_add2(S.sr[r], S.nr[r], tr[r]);
+    kahan_add2(S.si[r], S.ni[r], ti[r]);
   }
 }
 
@@ -288,75 +308,122 @@ __device__ __forceinline__ void tile_gemm_column(const float2* __restrict__ M, s
   }
 }
 
-// mu32 = mh * conv (sigma-normalised multipoles in FP32), once per box that
-// is a V-list source; the GEMM tiles gather these rows.
+// Programmatic dependent launch: a kernel launched with the attribute starts while
+// its predecessor in the stream still runs, prepares what does not depend on it
+// and waits here for its completion; the predecessor allows that at its start.
+// Both are no-ops in an ordinary launch.
+__device__ __forceinline__ void pdl_allow_next() {
+  asm volatile("griddepcontrol.launch_dependents;");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The sigma-normalised multipoles mu_n = mh_n conv_|n| of the boxes that are V-list
+// sources, as the FP32 sums that m2l_fold_kernel turns by a pair's angle: float4
+// (mu_n + (-1)^n mu_{-n}, mu_n - (-1)^n mu_{-n}), n = 0..pb (mu_0, 0 at n = 0), at
+// entry eoff[b] + b of mu32.
 __global__ void __launch_bounds__(kT) mpole_to_f32_kernel(
     int pbmax, const int* __restrict__ boxes, const int* __restrict__ level,
     const int* __restrict__ lpb, const long long* __restrict__ eoff,
     const double* __restrict__ conv, const cd* __restrict__ mpole, float2* __restrict__ mu32) {
   const int b = boxes[blockIdx.x];
   const int l = level[b];
-  const int pb = lpb[l], Q = 2 * pb + 1;
+  const int pb = lpb[l];
   const double* cv = conv + (size_t)l * (pbmax + 1);
-  const cd* a = mpole + eoff[b];
-  float2* dst = mu32 + eoff[b];
-  for (int n = threadIdx.x; n < Q; n += kT) {
-    const double f = cv[abs(n - pb)];
-    dst[n] = make_float2((float)(a[n].x * f), (float)(a[n].y * f));
+  const cd* a = mpole + eoff[b] + pb;
+  float4* dst = reinterpret_cast<float4*>(mu32 + eoff[b] + b);
+  for (int n = threadIdx.x; n <= pb; n += kT) {
+    const double f = cv[n];
+    cd m = n > 0 ? a[-n] : mk(0.0, 0.0);
+    if (n & 1) m = mk(-m.x, -m.y);
+    const cd s = cadd(a[n], m), d = n > 0 ? csub(a[n], m) : mk(0.0, 0.0);
+    dst[n] = make_float4((float)(s.x * f), (float)(s.y * f), (float)(d.x * f), (float)(d.y * f));
   }
 }
 
-// M2L work items: (first row, rows, first output order, group) over the tiles
-// of kGemmRows rows of one group. Each CTA computes kT consecutive output
-// orders (one per thread) of its rows and
-// stages the source rows through shared memory kChunkK orders at a time, so
-// its footprint does not grow with the box order. kChunkK is a multiple of
-// kGemmBlock: the compensated blocks, and so the result bits, do not depend on
-// the staging.
-constexpr int kChunkK = 128;
-static_assert(kChunkK % kGemmBlock == 0, "staging must keep the summation blocks");
-
-// NT threads, one output order each (items are cut to kT orders): the widths 64
-// and 96 serve levels with so few orders, which in a block of 128 leave one or
-// two of its four warps without work while they hold registers (128 per thread,
-// 16 warps per SM; M2L of the k = 10 starfish with 8192 nodes 0.217 -> 0.183 ms, of
-// 200 ellipses 3.36 -> 3.24).
+// M2L of V-list pairs grouped by (level, distance), in the even / odd form above.
+// Items: (first row, rows, first output order, level * kM2lDist + distance). A thread
+// computes E_l and O_l of one order l for kFoldRows rows. With P = pb + 1 <= NT orders
+// the CTA's threads are G = NT / P row groups of P orders (NT is chosen by level so
+// that few threads are left over); with more, one row group, NT orders per item and
+// the source orders staged NT at a time. row.x: entry of the source in mu; row.y: 64
+// times the entry of the pair's results in Y, plus its offset class (for the angle).
+// m2l_f32_reduce_kernel adds each target box's rows in its V-list order with Kahan
+// compensation (deterministic).
+// Bound by FP32 issue. M2L of 200 ellipses 3.23 -> 2.45 ms against one matrix per
+// offset class, 16 rows per thread; starfish at k = 10 0.18 -> 0.15, at k = 50 0.45 ->
+// 0.37 ms. (Three blocks of 128 threads per SM: at four, 128 registers, the two sets of
+// sums spill, and 200 ellipses take 2.88 ms.)
+constexpr int kFoldRows = 8;
+constexpr int kFoldWidth[3] = {128, 96, 64};  // NT
+constexpr int fold_groups(int NT, int P) { return P <= NT ? NT / P : 1; }
 template <int NT>
-__global__ void __launch_bounds__(NT, 512 / NT) m2l_f32_gemm_kernel(
+__global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
     const int4* __restrict__ items, const int* __restrict__ lpb,
-    const long long* __restrict__ goff, const long long* __restrict__ row_off,
-    const float2* __restrict__ mu32, const float2* __restrict__ tm,
-    const long long* __restrict__ yoff, float2* __restrict__ Y) {
-  constexpr int RS = stage_stride(kGemmRows);
-  __shared__ __align__(16) float2 mu[kChunkK * RS];  // [n][row]
-  const int4 I = items[blockIdx.x];  // (first row, rows, first output order, group)
+    const long long* __restrict__ toff, const longlong2* __restrict__ rows, int pbmax,
+    const float2* __restrict__ rot, const float2* __restrict__ mu, const float2* __restrict__ tm,
+    float2* __restrict__ Y) {
+  constexpr int R = kFoldRows, RS = stage_stride(R);
+  static_assert(NT % kGemmBlock == 0, "staging must keep the summation blocks");
+  __shared__ __align__(16) float2 xs[2 * NT * RS];  // e, then o: [row group][n][row]
+  const int4 I = items[blockIdx.x];
   const int row0 = I.x, nr = I.y;
-  const int Q = 2 * lpb[I.w / 49] + 1;
-  const int lo = I.z + (int)threadIdx.x;
-  const bool act = lo < Q;
-  // warps past the last output order only help stage the sources: an FMA
-  // costs its warp the same however few lanes are active
-  const bool warp_act = I.z + (int)(threadIdx.x & ~31u) < Q;
-  const float2* M = tm + goff[I.w];
-  RowSums<kGemmRows> S;
-  for (int n0 = 0; n0 < Q; n0 += kChunkK) {
-    const int nk = min(kChunkK, Q - n0);
+  const int pb = lpb[I.w / kM2lDist], P = pb + 1;
+  const int G = P <= NT ? NT / P : 1;
+  int rg = P <= NT ? (int)threadIdx.x / P : 0;
+  const int lo = P <= NT ? (int)threadIdx.x % P : I.z + (int)threadIdx.x;
+  const bool act = rg < G && rg * R < nr && lo < P;
+  if (!act) rg = 0;
+  const bool warp_act = __any_sync(0xffffffffu, act);
+  const float2* te = tm + toff[I.w];
+  const float2* to = te + (size_t)P * P;
+  const int used = (nr + R - 1) / R * R;  // rows staged
+  RowSums<R> E, O;
+  for (int n0 = 0; n0 < P; n0 += NT) {
+    const int nk = min(NT, P - n0);
+    float2* xe = xs;
+    float2* xo = xs + (size_t)G * nk * RS;
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nk * (kGemmRows / 2); idx += NT) {
+    for (int idx = threadIdx.x; idx < nk * (used / 2); idx += NT) {
       const int r = 2 * (idx / nk), n = idx % nk;  // coalesced reads along each source row
-      const float2 a = r < nr ? mu32[row_off[row0 + r] + n0 + n] : make_float2(0.f, 0.f);
-      const float2 b = r + 1 < nr ? mu32[row_off[row0 + r + 1] + n0 + n] : make_float2(0.f, 0.f);
-      *reinterpret_cast<float4*>(mu + n * RS + r) = make_float4(a.x, b.x, a.y, b.y);
+      float4 e, o;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float2 ev = make_float2(0.f, 0.f), ov = ev;
+        if (r + u < nr) {
+          const longlong2 q = rows[row0 + r + u];
+          const float4 v = reinterpret_cast<const float4*>(mu + q.x)[n0 + n];
+          const float2 w = rot[(size_t)(q.y & 63) * (pbmax + 1) + n0 + n];
+          ev = make_float2(fmaf(w.x, v.x, -w.y * v.w), fmaf(w.x, v.y, w.y * v.z));
+          ov = make_float2(fmaf(w.x, v.z, -w.y * v.y), fmaf(w.x, v.w, w.y * v.x));
+        }
+        if (u == 0) e.x = ev.x, e.z = ev.y, o.x = ov.x, o.z = ov.y;
+        else e.y = ev.x, e.w = ev.y, o.y = ov.x, o.w = ov.y;
+      }
+      const int at = ((r / R) * nk + n) * RS + r % R;
+      *reinterpret_cast<float4*>(xe + at) = e;
+      *reinterpret_cast<float4*>(xo + at) = o;
     }
     __syncthreads();
-    if (warp_act) tile_gemm_column(M + (size_t)n0 * Q, Q, nk, mu, lo, act, S);
+    if (warp_act) {
+      const size_t m0 = (size_t)n0 * P;
+      tile_gemm_column<R>(te + m0, P, nk, xe + (size_t)rg * nk * RS, lo, act, E);
+      tile_gemm_column<R>(to + m0, P, nk, xo + (size_t)rg * nk * RS, lo, act, O);
+    }
   }
-  if (act) {
+  if (!act) return;
 #pragma unroll
-    for (int r = 0; r < kGemmRows; ++r)
-      if (r < nr)
-        Y[yoff[row0 + r] + lo] =
-            make_float2(S.sum_r(r) - S.comp_r(r), S.sum_i(r) - S.comp_i(r));
+  for (int r = 0; r < R; ++r) {
+    if (rg * R + r >= nr) break;
+    const long long q = rows[row0 + rg * R + r].y;
+    const float2 w = rot[(size_t)(q & 63) * (pbmax + 1) + lo];
+    float2* y = Y + (q >> 6) + pb;
+    const float2 p = make_float2((E.sum_r(r) + O.sum_r(r)) + (E.lost_r(r) + O.lost_r(r)),
+                                 (E.sum_i(r) + O.sum_i(r)) + (E.lost_i(r) + O.lost_i(r)));
+    const float2 m = make_float2((E.sum_r(r) - O.sum_r(r)) + (E.lost_r(r) - O.lost_r(r)),
+                                 (E.sum_i(r) - O.sum_i(r)) + (E.lost_i(r) - O.lost_i(r)));
+    const float2 yp = make_float2(fmaf(w.x, p.x, -w.y * p.y), fmaf(w.x, p.y, w.y * p.x));
+    y[lo] = (lo & 1) ? make_float2(-yp.x, -yp.y) : yp;
+    if (lo > 0) y[-lo] = make_float2(fmaf(w.x, m.x, w.y * m.y), fmaf(w.x, m.y, -w.y * m.x));
   }
 }
 
@@ -428,6 +495,7 @@ __global__ void m2l_f64_matrix_kernel(int l, int pb, int pbmax, const cd* __rest
 // rows would not fit in registers), kT output orders and the same staging as
 // the FP32 items. Results go to the FP64 rows of Y64, added per target box by
 // m2l_f64_reduce_kernel in V-list order.
+constexpr int kChunkK = 128;  // source orders staged at a time
 constexpr int kF64Rows = 8;
 __global__ void __launch_bounds__(kT) m2l_f64_gemm_kernel(
     const int4* __restrict__ items, const int* __restrict__ lpb,
@@ -499,306 +567,302 @@ __global__ void __launch_bounds__(kT) m2l_f64_reduce_kernel(
   }
 }
 
-// L2L matrices of parent level l (order pp) and quadrant c, child order pc:
-// Tl[c][n][s] = (sig'_s / sig_n) (-1)^{s-n} V_{s-n}(d), sig' on level l+1,
-// sig on level l, from the FP64 table of (-1)^m V_m(d) (row stride
-// 4 pbmax + 1, order m at m + 2 pbmax). Grid: (quadrant, n), threads over s.
-__global__ void l2l_f32_matrix_kernel(int l, int pp, int pc, int pbmax, const cd* __restrict__ t_l2l,
-                                      const double* __restrict__ lsig, float2* __restrict__ Tl) {
-  const int c = blockIdx.x;
-  const int n = (int)blockIdx.y - pp;
-  const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
-  const cd* v = t_l2l + ((size_t)l * 4 + c) * (4 * pbmax + 1) + 2 * pbmax;
+// ---------------------------------------------------------------- FP32 M2M and L2L
+// The four children of a box lie at the same distance d and at the angles
+// pi/4 + rho pi/2, so that the translation by a child's offset is a real matrix
+// J_{s-n}(k d) between rotations by eighth turns, and the rotations of the four differ
+// by quarter turns i^{rho (s-n)}, which depend on (s - n) mod 4 only:
+//   M2M  mu'_s = e^{-i s pi/4} sum_n J_{s-n} b_{(n-s) mod 4, n},
+//        b_{j,n} = sum_rho i^{rho j} e^{i n pi/4} mu_{rho,n};
+//   L2L  lambda'_{rho,s} = e^{i s pi/4} sum_k i^{rho k} t_k,
+//        t_k = sum over n = s - k mod 4 of J_{n-s} e^{-i n pi/4} lambda_n:
+// one real matrix product and a four-point transform in place of four complex matrix
+// products, an eighth of the multiplications (200 ellipses: M2M 0.69 -> 0.38 ms, L2L with
+// the leaves' unscaling 0.97 -> 0.50; starfish at k = 50 0.18 -> 0.11 and 0.20 -> 0.11).
+// What is left is the FP64 conversion of the coefficients. Coefficients sigma-normalised (mu_n =
+// mh_n conv_n, lambda_n = lh_n / conv_n); the matrices T[n][s] hold the ratio of sigmas
+// and 1/sqrt 2 for each odd order of the eighth turns (turn8 leaves it out).
+constexpr int child_at(int rho) { return (0x4B >> (2 * rho)) & 3; }  // quadrant at pi/4 + rho pi/2
+// Their sums carry the rounding errors along (fe: value and error, fec: complex), so
+// that a coefficient is rounded to FP32 once before and once after the product.
+struct fe {
+  float h, l;
+};
+struct fec {
+  fe x, y;
+};
+__device__ __forceinline__ fe add(fe a, fe b) {
+  const float s = a.h + b.h, t = s - a.h;
+  return {s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
+}
+__device__ __forceinline__ fe neg(fe a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ fec add(fec a, fec b) { return {add(a.x, b.x), add(a.y, b.y)}; }
+__device__ __forceinline__ fec sub(fec a, fec b) { return {add(a.x, neg(b.x)), add(a.y, neg(b.y))}; }
+__device__ __forceinline__ fec turn4(fec v, int q) {  // i^q v
+  if (q & 1) v = {neg(v.y), v.x};
+  if (q & 2) v = {neg(v.x), neg(v.y)};
+  return v;
+}
+__device__ __forceinline__ fec turn8(fec v, int m) {  // e^{i m pi/4} v, sqrt 2 times for odd m
+  if (m & 1) v = {add(v.x, neg(v.y)), add(v.x, v.y)};
+  return turn4(v, m >> 1);
+}
+__device__ __forceinline__ void dft4(fec (&v)[4]) {  // v_j <- sum_rho i^{rho j} v_rho
+  const fec a = add(v[0], v[2]), b = sub(v[0], v[2]);
+  const fec c = add(v[1], v[3]), d = turn4(sub(v[1], v[3]), 1);
+  v[0] = add(a, c);
+  v[2] = sub(a, c);
+  v[1] = add(b, d);
+  v[3] = sub(b, d);
+}
+__device__ __forceinline__ float2 f32(fec v) { return make_float2(v.x.h + v.x.l, v.y.h + v.y.l); }
+
+// The matrix of parent level l (M2M: from child order n to parent order s; L2L: from
+// parent to child), from the tables of the quadrant at pi/4 (row stride 4 pbmax + 1,
+// order m at m + 2 pbmax): J_m e^{-i m pi/4} for M2M, J_{-m} e^{i m pi/4} for L2L at
+// m = s - n. Grid: n, threads over s.
+template <bool M2M>
+__global__ void fold_matrix_kernel(int l, int pp, int pc, int pbmax, const cd* __restrict__ table,
+                                   const double* __restrict__ lsig, float* __restrict__ T) {
+  const int pn = M2M ? pc : pp, ps = M2M ? pp : pc;
+  const int n = (int)blockIdx.x - pn;
+  const cd* v = table + ((size_t)l * 4 + child_at(0)) * (4 * pbmax + 1) + 2 * pbmax;
   const double* sp = lsig + (size_t)l * (pbmax + 1);
   const double* sc = lsig + (size_t)(l + 1) * (pbmax + 1);
-  float2* dst = Tl + ((size_t)c * Qp + (n + pp)) * Qc;
-  for (int so = (int)threadIdx.x - pc; so <= pc; so += blockDim.x) {
-    const cd e = v[so - n];
-    const double mag = hypot(e.x, e.y);
-    float2 out = make_float2(0.f, 0.f);
-    if (mag > 0.0) {
-      const double lf = sc[abs(so)] - sp[abs(n)] + log(mag);
-      const double f = lf < -700.0 ? 0.0 : exp(lf) / mag;
-      out = make_float2((float)(e.x * f), (float)(e.y * f));
+  float* dst = T + (size_t)(n + pn) * (2 * ps + 1) + ps;
+  for (int s = (int)threadIdx.x - ps; s <= ps; s += blockDim.x) {
+    const cd e = v[s - n];
+    double c, sn;
+    sincospi(0.25 * (M2M ? s - n : n - s), &sn, &c);
+    const double J = e.x * c - e.y * sn;
+    double out = 0.0;
+    if (J != 0.0) {
+      const double lf = (M2M ? sc[abs(n)] - sp[abs(s)] : sc[abs(s)] - sp[abs(n)]) + log(fabs(J));
+      out = lf < -700.0 ? 0.0 : copysign(exp(lf), J);
     }
-    dst[so + pc] = out;
+    if (n & 1) out *= 0.70710678118654752440;
+    if (s & 1) out *= 0.70710678118654752440;
+    dst[s] = (float)out;
   }
 }
 
-// L2L on level l as tile GEMMs: a CTA takes R parents, one child quadrant
-// c = blockIdx.y and kT child orders (chunk blockIdx.z), stages the parents' sigma-normalised locals
-// lambda_n = lh_n / conv_n (FP32) in shared memory, and computes
-// lambda'_s = sum_n Tl[c][n][s] lambda_n for all of them at once (threads over
-// s); the quadrant-c children get lh'_s += lambda'_s conv'_s in FP64.
-template <int R>
-__global__ void __launch_bounds__(kT) l2l_f32_kernel(
-    int l, int pp, int pc, int pbmax, const int* __restrict__ parents, int nb,
-    const int* __restrict__ child, const long long* __restrict__ eoff,
-    const float2* __restrict__ Tl, const double* __restrict__ conv, cd* __restrict__ local) {
-  extern __shared__ __align__(16) float2 lam[];  // [Qp][stage_stride(R)]
-  const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
-  const int p0 = blockIdx.x * R, nr = min(R, nb - p0);
-  const double* cvp = conv + (size_t)l * (pbmax + 1);
-  const double* cvc = conv + (size_t)(l + 1) * (pbmax + 1);
-  for (int idx = threadIdx.x; idx < Qp * R; idx += kT) {
-    const int r = idx / Qp, n = idx % Qp;
-    float2 v = make_float2(0.f, 0.f);
-    if (r < nr) {
-      const cd g = local[eoff[parents[p0 + r]] + n];
-      const double f = 1.0 / cvp[abs(n - pp)];
-      v = make_float2((float)(g.x * f), (float)(g.y * f));
-    }
-    stage_put(lam, n, r, stage_stride(R), v);
-  }
-  __syncthreads();
-  {
-    const int c = blockIdx.y;
-    const float2* M = Tl + (size_t)c * Qp * Qc;
-    {
-      const int so = (int)blockIdx.z * kT + threadIdx.x;  // output chunk blockIdx.z
-      const bool act = so < Qc;
-      RowSums<R> S;
-      tile_gemm_column<R>(M, Qc, Qp, lam, so, act, S);
-      if (act) {
-        const double f = cvc[abs(so - pc)];
+// S[r] += sum_{j < N} M[j * ld + lo] * x[j * XS][r] with a real matrix, otherwise as
+// tile_gemm_column.
+template <int R, int XS>
+__device__ __forceinline__ void real_block_add(const float (&tb)[kGemmBlock], int nj,
+                                               const float2* __restrict__ x, RowSums<R>& S) {
+  f32p tr[R / 2], ti[R / 2];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (r >= nr) break;
-          const int d = child[4 * parents[p0 + r] + c];
-          if (d < 0) continue;
-          cd* dl = local + eoff[d] + so;
-          dl->x += ((double)S.sum_r(r) - (double)S.comp_r(r)) * f;
-          dl->y += ((double)S.sum_i(r) - (double)S.comp_i(r)) * f;
-        }
-      }
-    }
-  }
-}
-
-// M2M matrices of parent level l (order pp) and quadrant c, child order pc:
-// Tm2m[c][n][s] = (sig_n / sig'_s) conj(V_{s-n}(d)), sig on the child level
-// l+1, sig' on level l, from the FP64 table of conj(V_m(d)). Grid: (quadrant,
-// n), threads over s.
-__global__ void m2m_f32_matrix_kernel(int l, int pp, int pc, int pbmax, const cd* __restrict__ t_m2m,
-                                      const double* __restrict__ lsig, float2* __restrict__ Tmm) {
-  const int c = blockIdx.x;
-  const int n = (int)blockIdx.y - pc;
-  const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
-  const cd* v = t_m2m + ((size_t)l * 4 + c) * (4 * pbmax + 1) + 2 * pbmax;
-  const double* sp = lsig + (size_t)l * (pbmax + 1);
-  const double* sc = lsig + (size_t)(l + 1) * (pbmax + 1);
-  float2* dst = Tmm + ((size_t)c * Qc + (n + pc)) * Qp;
-  for (int so = (int)threadIdx.x - pp; so <= pp; so += blockDim.x) {
-    const cd e = v[so - n];
-    const double mag = hypot(e.x, e.y);
-    float2 out = make_float2(0.f, 0.f);
-    if (mag > 0.0) {
-      const double lf = sc[abs(n)] - sp[abs(so)] + log(mag);
-      const double f = lf < -700.0 ? 0.0 : exp(lf) / mag;
-      out = make_float2((float)(e.x * f), (float)(e.y * f));
-    }
-    dst[so + pp] = out;
-  }
-}
-
-// M2M on level l as tile GEMMs: a CTA takes R parents and kT output orders
-// (chunk blockIdx.y, so that the few wide boxes of coarse levels spread over
-// many CTAs); for each quadrant it stages the children's sigma-normalised
-// multipoles mu_n = mh_n conv_n (FP32) and adds sum_n Tm2m[c][n][s] mu_n to the
-// parents' compensated sums (threads over s); mh'_s = mu'_s / conv'_s in FP64.
-template <int R>
-__global__ void __launch_bounds__(kT) m2m_f32_kernel(
-    int l, int pp, int pc, int pbmax, const int* __restrict__ parents, int nb,
-    const int* __restrict__ child, const long long* __restrict__ eoff,
-    const float2* __restrict__ Tmm, const double* __restrict__ conv, cd* __restrict__ mpole) {
-  extern __shared__ __align__(16) float2 mus[];  // [Qc][stage_stride(R)]
-  __shared__ long long coff[4][R], poff[R];       // children's (-1: none) and parents' offsets
-  const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
-  const int p0 = blockIdx.x * R, nr = min(R, nb - p0);
-  const double* cvp = conv + (size_t)l * (pbmax + 1);
-  const double* cvc = conv + (size_t)(l + 1) * (pbmax + 1);
-  for (int idx = threadIdx.x; idx < 5 * R; idx += kT) {
-    const int r = idx % R, c = idx / R;
-    long long o = -1;
-    if (r < nr) {
-      if (c == 4) {
-        o = eoff[parents[p0 + r]];
-      } else {
-        const int d = child[4 * parents[p0 + r] + c];
-        if (d >= 0) o = eoff[d];
-      }
-    }
-    if (c == 4) poff[r] = o; else coff[c][r] = o;
-  }
-  {
-    const int so = (int)blockIdx.y * kT + threadIdx.x;  // output chunk blockIdx.y
-    const bool act = so < Qp;
-    RowSums<R> S;
-    for (int c = 0; c < 4; ++c) {
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < Qc * R; idx += kT) {
-        const int r = idx / Qc, n = idx % Qc;
-        float2 v = make_float2(0.f, 0.f);
-        const long long o = coff[c][r];
-        if (o >= 0) {
-          const cd a = mpole[o + n];
-          const double f = cvc[abs(n - pc)];
-          v = make_float2((float)(a.x * f), (float)(a.y * f));
-        }
-        stage_put(mus, n, r, stage_stride(R), v);
-      }
-      __syncthreads();
-      tile_gemm_column<R>(Tmm + (size_t)c * Qc * Qp, Qp, Qc, mus, so, act, S);
-    }
-    if (act) {
-      const double f = 1.0 / cvp[abs(so - pp)];
+  for (int j = 0; j < kGemmBlock; ++j) {
+    if (j < nj) {
+      const f32p t = pk(tb[j], tb[j]);
+      const ulonglong2* m = reinterpret_cast<const ulonglong2*>(x + j * XS);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (r >= nr) break;
-        cd* dst = mpole + poff[r] + so;
-        dst->x = ((double)S.sum_r(r) - (double)S.comp_r(r)) * f;
-        dst->y = ((double)S.sum_i(r) - (double)S.comp_i(r)) * f;
+      for (int r = 0; r < R / 2; ++r) {
+        const ulonglong2 v = m[r];
+        tr[r] = fma2(t, v.x, j == 0 ? S.nr[r] : tr[r]);
+        ti[r] = fma2(t, v.y, j == 0 ? S.ni[r] : ti[r]);
       }
     }
   }
+#pragma unroll
+  for (int r = 0; r < R / 2; ++r) {
+    kahan_add2(S.sr[r], S.nr[r], tr[r]);
+    kahan_add2(S.si[r], S.ni[r], ti[r]);
+  }
+}
+template <int R, int XS>
+__device__ __forceinline__ void real_column(const float* __restrict__ M, size_t ld, int N,
+                                            const float2* __restrict__ x, int lo, bool act,
+                                            RowSums<R>& S) {
+  const float* Mc = M + (act ? lo : 0);
+  float ta[kGemmBlock], tb[kGemmBlock];
+  auto load = [&](float (&t)[kGemmBlock], int n0) {
+#pragma unroll
+    for (int j = 0; j < kGemmBlock; ++j) t[j] = n0 + j < N ? Mc[(size_t)(n0 + j) * ld] : 0.f;
+  };
+  load(ta, 0);
+  for (int n0 = 0; n0 < N; n0 += 2 * kGemmBlock) {
+    const int n1 = n0 + kGemmBlock;
+    if (n1 < N) load(tb, n1);
+    real_block_add<R, XS>(ta, min(kGemmBlock, N - n0), x + (size_t)n0 * XS, S);
+    if (n1 >= N) break;
+    if (n1 + kGemmBlock < N) load(ta, n1 + kGemmBlock);
+    real_block_add<R, XS>(tb, min(kGemmBlock, N - n1), x + (size_t)n1 * XS, S);
+  }
 }
 
-// Coarse levels (few parents, high orders) as split-K tile GEMMs: the two
-// kernels above give each thread one output column and the whole K range, so
-// a level of a few dozen boxes runs a few CTAs with K-long dependent chains.
-// Here a CTA of kT threads takes R parents and 32 output orders (chunk
-// blockIdx.y or blockIdx.z); warp w sums its quarter of K (M2M: child quadrant
-// w; L2L: the w-th quarter of the parent's orders) for the 32 orders, and the
-// four partial sums are added in FP64 in warp order (deterministic).
-constexpr int kSplitCols = 32, kSplitWarps = kT / 32;
-
+// A CTA takes R parents. Warp w sums the terms n = w mod 4 (counted from the lowest
+// order) of 32 orders s, one per lane, for all R; the CTA's warps then join the four
+// sums. The orders s are taken 32 at a time, gridDim.y apart. Source orders are staged
+// kFoldK at a time (all at once but for orders beyond any ordinary box).
+constexpr int kFoldK = 256;
+static_assert(kT == 128 && kFoldK % (4 * kGemmBlock) == 0, "four warps, whole summation blocks");
+__host__ __device__ constexpr size_t fold_staged(int Q, int per, int R) {  // float2 words
+  return (size_t)(Q < kFoldK ? Q : kFoldK) * per * stage_stride(R);
+}
+constexpr size_t fold_smem(int Q, int per, int R) {  // the rows and the joint's fec[4][R][32]
+  return fold_staged(Q, per, R) * sizeof(float2) + 128 * (size_t)R * sizeof(fec);
+}
 template <int R>
-__device__ __forceinline__ void split_reduce(const RowSums<R>& S, float2* red, int warp, int lane,
-                                             double (&outr)[R], double (&outi)[R]) {
-  // red: [kSplitWarps][R][32]
+__device__ __forceinline__ void put_sums(const RowSums<R>& S, fec* red, int warp, int lane) {
 #pragma unroll
   for (int r = 0; r < R; ++r)
-    red[(warp * R + r) * 32 + lane] =
-        make_float2(S.sum_r(r) - S.comp_r(r), S.sum_i(r) - S.comp_i(r));
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < kSplitWarps; ++w) {
-      const float2 v = red[(w * R + r) * 32 + lane];
-      a += (double)v.x;
-      b += (double)v.y;
-    }
-    outr[r] = a;
-    outi[r] = b;
-  }
+    red[(warp * R + r) * 32 + lane] = {{S.sum_r(r), S.lost_r(r)}, {S.sum_i(r), S.lost_i(r)}};
 }
 
 template <int R>
-__global__ void __launch_bounds__(kT) m2m_f32_split_kernel(
+__global__ void __launch_bounds__(kT, 4) m2m_fold_kernel(
     int l, int pp, int pc, int pbmax, const int* __restrict__ parents, int nb,
-    const int* __restrict__ child, const long long* __restrict__ eoff,
-    const float2* __restrict__ Tmm, const double* __restrict__ conv, cd* __restrict__ mpole) {
-  extern __shared__ __align__(16) float2 mus4[];  // [4][Qc][stage_stride(R)], then red
-  __shared__ long long coff[4][R], poff[R];
+    const int* __restrict__ child, const long long* __restrict__ eoff, const float* __restrict__ T,
+    const double* __restrict__ conv, const double* __restrict__ iconv, cd* __restrict__ mpole) {
+  constexpr int RS = stage_stride(R);
+  extern __shared__ __align__(16) float2 fx[];  // [n][j][RS], then the joint's fec[4][R][32]
+  __shared__ long long coff[4][R], poff[R];     // children by rho
   const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
-  const int RS = stage_stride(R);
+  fec* red = reinterpret_cast<fec*>(fx + fold_staged(Qc, 4, R));
   const int p0 = blockIdx.x * R, nr = min(R, nb - p0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double* cvp = conv + (size_t)l * (pbmax + 1);
-  const double* cvc = conv + (size_t)(l + 1) * (pbmax + 1);
+  pdl_allow_next();
   for (int idx = threadIdx.x; idx < 5 * R; idx += kT) {
     const int r = idx % R, c = idx / R;
     long long o = -1;
     if (r < nr) {
-      if (c == 4) {
-        o = eoff[parents[p0 + r]];
-      } else {
-        const int d = child[4 * parents[p0 + r] + c];
-        if (d >= 0) o = eoff[d];
-      }
+      const int b = parents[p0 + r];
+      const int d = c == 4 ? b : child[4 * b + child_at(c)];
+      if (d >= 0) o = eoff[d];
     }
     if (c == 4) poff[r] = o; else coff[c][r] = o;
   }
+  const double* cvc = conv + (size_t)(l + 1) * (pbmax + 1);
+  const double* icp = iconv + (size_t)l * (pbmax + 1);
   __syncthreads();
-  for (int idx = threadIdx.x; idx < 4 * Qc * R; idx += kT) {
-    const int c = idx / (Qc * R), rem = idx % (Qc * R), r = rem / Qc, n = rem % Qc;
-    float2 v = make_float2(0.f, 0.f);
-    const long long o = coff[c][r];
-    if (o >= 0) {
-      const cd a = mpole[o + n];
-      const double f = cvc[abs(n - pc)];
-      v = make_float2((float)(a.x * f), (float)(a.y * f));
-    }
-    stage_put(mus4, (size_t)c * Qc + n, r, RS, v);
-  }
-  __syncthreads();
-  const int so = (int)blockIdx.y * kSplitCols + lane;
-  const bool act = so < Qp;
-  RowSums<R> S;
-  tile_gemm_column<R>(Tmm + (size_t)warp * Qc * Qp, Qp, Qc, mus4 + (size_t)warp * Qc * RS, so,
-                      act, S);
-  __syncthreads();  // the staged rows are dead: the reduction reuses the space
-  double outr[R], outi[R];
-  split_reduce<R>(S, mus4, warp, lane, outr, outi);
-  if (warp == 0 && act) {
-    const double f = 1.0 / cvp[abs(so - pp)];
+  pdl_wait();
+  bool staged = false;
+  for (int s0 = blockIdx.y * 32; s0 < Qp; s0 += 32 * gridDim.y) {
+    const int at = s0 + lane, s = at - pp;
+    const bool act = at < Qp;
+    const int j = (warp - pc - s) & 3;
+    RowSums<R> S;
+    for (int n0 = 0; n0 < Qc; n0 += kFoldK) {
+      const int nk = min(kFoldK, Qc - n0);
+      if (!staged || Qc > kFoldK) {
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < nk * R; idx += kT) {
+          const int r = idx / nk, n = idx % nk, m = n0 + n - pc;
+          const double f = cvc[abs(m)];
+          fec v[4];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (r >= nr) break;
-      cd* dst = mpole + poff[r] + so;
-      dst->x = outr[r] * f;
-      dst->y = outi[r] * f;
+          for (int c = 0; c < 4; ++c) {
+            v[c] = {{0.f, 0.f}, {0.f, 0.f}};
+            if (coff[c][r] >= 0) {
+              const cd a = mpole[coff[c][r] + n0 + n];
+              v[c] = turn8({{(float)(a.x * f), 0.f}, {(float)(a.y * f), 0.f}}, m);
+            }
+          }
+          dft4(v);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) stage_put(fx, (size_t)n * 4 + q, r, RS, f32(v[q]));
+        }
+        __syncthreads();
+        staged = true;
+      }
+      const int N = (nk - warp + 3) / 4;
+      if (N > 0)
+        real_column<R, 16 * RS>(T + (size_t)(n0 + warp) * Qp, 4 * (size_t)Qp, N,
+                                fx + (warp * 4 + j) * RS, at, act, S);
+    }
+    __syncthreads();
+    put_sums<R>(S, red, warp, lane);
+    __syncthreads();
+    if (act) {
+      const double f = icp[abs(s)];
+      for (int r = warp; r < nr; r += 4) {
+        fec v[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) v[w] = red[(w * R + r) * 32 + lane];
+        const fec u = turn8(add(add(v[0], v[1]), add(v[2], v[3])), -s);
+        mpole[poff[r] + at] =
+            mk(((double)u.x.h + (double)u.x.l) * f, ((double)u.y.h + (double)u.y.l) * f);
+      }
     }
   }
 }
 
 template <int R>
-__global__ void __launch_bounds__(kT) l2l_f32_split_kernel(
+__global__ void __launch_bounds__(kT, 4) l2l_fold_kernel(
     int l, int pp, int pc, int pbmax, const int* __restrict__ parents, int nb,
-    const int* __restrict__ child, const long long* __restrict__ eoff,
-    const float2* __restrict__ Tl, const double* __restrict__ conv, cd* __restrict__ local) {
-  extern __shared__ __align__(16) float2 lam2[];  // [Qp][stage_stride(R)], then red
+    const int* __restrict__ child, const long long* __restrict__ eoff, const float* __restrict__ T,
+    const double* __restrict__ conv, const double* __restrict__ iconv, cd* __restrict__ local) {
+  constexpr int RS = stage_stride(R);
+  extern __shared__ __align__(16) float2 fx[];  // [n][RS], then the joint's fec[4][R][32]
+  __shared__ long long coff[4][R], poff[R];     // children by rho
   const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
-  const int RS = stage_stride(R);
+  fec* red = reinterpret_cast<fec*>(fx + fold_staged(Qp, 1, R));
   const int p0 = blockIdx.x * R, nr = min(R, nb - p0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double* cvp = conv + (size_t)l * (pbmax + 1);
-  const double* cvc = conv + (size_t)(l + 1) * (pbmax + 1);
-  for (int idx = threadIdx.x; idx < Qp * R; idx += kT) {
-    const int r = idx / Qp, n = idx % Qp;
-    float2 v = make_float2(0.f, 0.f);
+  pdl_allow_next();
+  for (int idx = threadIdx.x; idx < 5 * R; idx += kT) {
+    const int r = idx % R, c = idx / R;
+    long long o = -1;
     if (r < nr) {
-      const cd g = local[eoff[parents[p0 + r]] + n];
-      const double f = 1.0 / cvp[abs(n - pp)];
-      v = make_float2((float)(g.x * f), (float)(g.y * f));
+      const int b = parents[p0 + r];
+      const int d = c == 4 ? b : child[4 * b + child_at(c)];
+      if (d >= 0) o = eoff[d];
     }
-    stage_put(lam2, n, r, RS, v);
+    if (c == 4) poff[r] = o; else coff[c][r] = o;
   }
+  const double* cvc = conv + (size_t)(l + 1) * (pbmax + 1);
+  const double* icp = iconv + (size_t)l * (pbmax + 1);
   __syncthreads();
-  const int c = blockIdx.y;
-  const int so = (int)blockIdx.z * kSplitCols + lane;
-  const bool act = so < Qc;
-  // warp w: parent orders [n0, n1)
-  const int per = (Qp + kSplitWarps - 1) / kSplitWarps;
-  const int n0 = min(Qp, warp * per), n1 = min(Qp, n0 + per);
-  RowSums<R> S;
-  if (n1 > n0)
-    tile_gemm_column<R>(Tl + (size_t)c * Qp * Qc + (size_t)n0 * Qc, Qc, n1 - n0, lam2 + n0 * RS,
-                        so, act, S);
-  __syncthreads();
-  double outr[R], outi[R];
-  split_reduce<R>(S, lam2, warp, lane, outr, outi);
-  if (warp == 0 && act) {
-    const double f = cvc[abs(so - pc)];
+  pdl_wait();
+  bool staged = false;
+  for (int s0 = blockIdx.y * 32; s0 < Qc; s0 += 32 * gridDim.y) {
+    const int at = s0 + lane, s = at - pc;
+    const bool act = at < Qc;
+    RowSums<R> S;
+    for (int n0 = 0; n0 < Qp; n0 += kFoldK) {
+      const int nk = min(kFoldK, Qp - n0);
+      if (!staged || Qp > kFoldK) {
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < nk * R; idx += kT) {
+          const int r = idx / nk, n = idx % nk, m = n0 + n - pp;
+          float2 v = make_float2(0.f, 0.f);
+          if (r < nr) {
+            const cd g = local[poff[r] + n0 + n];
+            const double f = icp[abs(m)];
+            const fec u = turn8({{(float)(g.x * f), 0.f}, {(float)(g.y * f), 0.f}}, -m);
+            v = f32(u);
+          }
+          stage_put(fx, n, r, RS, v);
+        }
+        __syncthreads();
+        staged = true;
+      }
+      const int N = (nk - warp + 3) / 4;
+      if (N > 0)
+        real_column<R, 4 * RS>(T + (size_t)(n0 + warp) * Qc, 4 * (size_t)Qc, N, fx + warp * RS, at,
+                               act, S);
+    }
+    __syncthreads();
+    put_sums<R>(S, red, warp, lane);
+    __syncthreads();
+    if (act) {
+      const double f = cvc[abs(s)];
+      for (int r = warp; r < nr; r += 4) {
+        fec v[4];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (r >= nr) break;
-      const int d = child[4 * parents[p0 + r] + c];
-      if (d < 0) continue;
-      cd* dl = local + eoff[d] + so;
-      dl->x += outr[r] * f;
-      dl->y += outi[r] * f;
+        for (int k = 0; k < 4; ++k) v[k] = red[(((s + pp - k) & 3) * R + r) * 32 + lane];
+        dft4(v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (coff[c][r] < 0) continue;
+          const float2 u = f32(turn8(v[c], s));
+          cd* dst = local + coff[c][r] + at;
+          dst->x += (double)u.x * f;
+          dst->y += (double)u.y * f;
+        }
+      }
     }
   }
 }
@@ -812,14 +876,10 @@ __global__ void gather_offsets_kernel(const int* __restrict__ idx, const long lo
 
 }  // namespace
 
-static int g_mixed_smem_optin = 48 * 1024;  // the device's opt-in limit once configured
-
 qbx_status configure_mixed_kernels(int smem_optin) {
-  g_mixed_smem_optin = smem_optin;
-  const void* k[] = {(const void*)l2l_f32_kernel<kGemmRows>, (const void*)l2l_f32_kernel<kNarrowRows>,
-                     (const void*)m2m_f32_kernel<kGemmRows>, (const void*)m2m_f32_kernel<kNarrowRows>,
-                     (const void*)m2m_f32_split_kernel<kNarrowRows>,
-                     (const void*)l2l_f32_split_kernel<kNarrowRows>};
+  const void* k[] = {(const void*)m2m_fold_kernel<2>, (const void*)m2m_fold_kernel<4>,
+                     (const void*)m2m_fold_kernel<8>, (const void*)l2l_fold_kernel<2>,
+                     (const void*)l2l_fold_kernel<4>, (const void*)l2l_fold_kernel<8>};
   for (const void* fn : k) {
     cudaFuncAttributes a;
     QBX_CUDA_TRY(cudaFuncGetAttributes(&a, fn));  // dynamic + static must fit the opt-in size
@@ -854,9 +914,10 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
   const int pbm = f->pb_max;
   QBX_CUDA_TRY(f->lsig.alloc((size_t)f->n_levels * (pbm + 1)));
   QBX_CUDA_TRY(f->conv.alloc((size_t)f->n_levels * (pbm + 1)));
+  QBX_CUDA_TRY(f->iconv.alloc((size_t)f->n_levels * (pbm + 1)));
   QBX_CUDA_TRY(f->isig.alloc((size_t)f->n_levels * (pbm + 2)));
   sigma_tables_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, h->k, f->side, f->scale.ptr,
-                                 f->lsig.ptr, f->conv.ptr, f->isig.ptr);
+                                 f->lsig.ptr, f->conv.ptr, f->iconv.ptr, f->isig.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
   QBX_CUDA_TRY(f->m2p_rec.alloc((size_t)f->n_levels * (pbm + 2)));
   m2p_rec_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->lsig.ptr, f->m2p_rec.ptr);
@@ -898,18 +959,33 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
       tot += 49 * Q * Q;
     }
   }
-  QBX_CUDA_TRY(f->tm_f32.alloc(std::max<long long>(1, tot)));
-  f->h_tm_off = off;
+  std::vector<long long> foff((size_t)f->n_levels * kM2lDist, 0);  // FP32, per (level, distance)
+  long long ftot = 0;
+  for (int l = 0; l < f->n_levels; ++l) {
+    if (f->vbox_off[l + 1] == f->vbox_off[l]) continue;
+    const long long P = f->h_pb[l] + 1;
+    for (int d = 0; d < kM2lDist; ++d) {
+      foff[(size_t)l * kM2lDist + d] = ftot;
+      ftot += 2 * P * P;
+    }
+  }
+  QBX_CUDA_TRY(f->tm_f32.alloc(std::max<long long>(1, ftot)));
   for (int l = 2; l < f->n_levels; ++l) {
     if (f->vbox_off[l + 1] == f->vbox_off[l]) continue;
     const int pb = f->h_pb[l];
-    dim3 grid(49, 2 * pb + 1);
-    m2l_f32_matrix_kernel<<<grid, kT>>>(l, pb, pbm, f->t_m2l.ptr, f->scale.ptr, f->lsig.ptr,
-                                        f->tm_f32.ptr + off[l]);
+    m2l_fold_matrix_kernel<<<dim3(kM2lDist, pb + 1), kT>>>(
+        l, pb, pbm, f->t_m2l.ptr, f->scale.ptr, f->lsig.ptr,
+        f->tm_f32.ptr + foff[(size_t)l * kM2lDist]);
     QBX_CUDA_TRY(cudaGetLastError());
   }
-  // M2L work: V-list pairs grouped by (level, offset class), cut into tiles
-  // of kGemmRows rows; the row of V entry e is vrow[e], its output at yoff[row]
+  QBX_CUDA_TRY(f->m2l_toff.alloc(foff.size()));
+  QBX_CUDA_TRY(cudaMemcpy(f->m2l_toff.ptr, foff.data(), foff.size() * sizeof(long long),
+                          cudaMemcpyHostToDevice));
+  QBX_CUDA_TRY(f->m2l_rot.alloc((size_t)49 * (pbm + 1)));
+  m2l_rot_kernel<<<49, 128>>>(pbm, f->m2l_rot.ptr);
+  QBX_CUDA_TRY(cudaGetLastError());
+  // M2L work: V-list pairs grouped by (level, offset class); the row of V entry e is
+  // vrow[e], its output at yoff[row]
   {
     const int nb = f->n_boxes;
     const int64_t nv = f->V.nnz;
@@ -930,6 +1006,8 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
         gcount[egroup[e] + 1] += 1;
       }
     for (int g = 0; g < ng; ++g) gcount[g + 1] += gcount[g];
+    std::vector<long long> eo(nb);
+    QBX_CUDA_TRY(cudaMemcpy(eo.data(), f->eoff.ptr, nb * sizeof(long long), cudaMemcpyDeviceToHost));
     std::vector<int> vrow(std::max<int64_t>(1, nv)), row_src(std::max<int64_t>(1, nv));
     std::vector<long long> yoff(std::max<int64_t>(1, nv));
     std::vector<int64_t> fill(gcount.begin(), gcount.end() - 1);
@@ -953,22 +1031,52 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
       for (int64_t r = gcount[g]; r < gcount[g + 1]; r += kGemmRows)
         tiles.push_back(make_int4(g, (int)r, (int)std::min<int64_t>(kGemmRows, gcount[g + 1] - r), l));
     }
-    // coarse levels (largest orders) first; work items (first row, rows,
-    // first output order, group) per tile: chunks of kT output orders, and
-    // for FP64 also groups of kF64Rows rows
-    std::vector<int4> it32, it64, by_width[3];  // FP32: blocks of 128, 96, 64 threads
+    // FP64 work items, coarse levels (largest orders) first: (first row, rows, first
+    // output order, group), tiles in groups of kF64Rows rows and kT output orders
+    std::vector<int4> it64;
     for (const int4& t : tiles) {
       const int Q = 2 * f->h_pb[t.w] + 1;
-      for (int c0 = 0; c0 < Q; c0 += kT) {
-        by_width[Q > 96 ? 0 : Q > 64 ? 1 : 2].push_back(make_int4(t.y, t.z, c0, t.x));
+      for (int c0 = 0; c0 < Q; c0 += kT)
         for (int r0 = 0; r0 < t.z; r0 += kF64Rows)
           it64.push_back(make_int4(t.y + r0, std::min(kF64Rows, t.z - r0), c0, t.x));
+    }
+    // FP32: the rows in order of (level, distance), classes side by side; items by
+    // block width
+    std::vector<longlong2> frow;
+    std::vector<int4> it32, by_width[3];  // blocks of 128, 96, 64 threads
+    frow.reserve(gcount[ng]);
+    for (int l = 0; l < f->n_levels; ++l) {
+      const int P = f->h_pb[l] + 1;
+      int u = 0, best = -1;  // the width that leaves the fewest threads without an order
+      for (int v = 2; v >= 0; --v) {
+        const int nt = kFoldWidth[v];
+        const int full = P <= nt ? 1000 * (nt / P * P) / nt : 1000 * P / (nblk(P, nt) * nt);
+        if (full > best) best = full, u = v;
+      }
+      const int nt = kFoldWidth[u], most = kFoldRows * fold_groups(nt, P);
+      for (int d = 0; d < kM2lDist; ++d) {
+        const int64_t r0 = (int64_t)frow.size();
+        for (int c = 0; c < 49; ++c) {
+          if (m2l_dist(c) != d) continue;
+          const int g = l * 49 + c;
+          for (int64_t r = gcount[g]; r < gcount[g + 1]; ++r)
+            frow.push_back(make_longlong2(eo[row_src[r]] + row_src[r], yoff[r] * 64 + c));
+        }
+        const int64_t r1 = (int64_t)frow.size();
+        for (int64_t r = r0; r < r1; r += most)
+          for (int c0 = 0; c0 < P; c0 += P <= nt ? P : nt)
+            by_width[u].push_back(
+                make_int4((int)r, (int)std::min<int64_t>(most, r1 - r), c0, l * kM2lDist + d));
       }
     }
     for (int u = 0; u < 3; ++u) {
       it32.insert(it32.end(), by_width[u].begin(), by_width[u].end());
       f->n_m2l_width[u] = (int)by_width[u].size();
     }
+    QBX_CUDA_TRY(f->m2l_frow.alloc(std::max<size_t>(1, frow.size())));
+    if (!frow.empty())
+      QBX_CUDA_TRY(cudaMemcpy(f->m2l_frow.ptr, frow.data(), frow.size() * sizeof(longlong2),
+                              cudaMemcpyHostToDevice));
     // matrix offset of each group (level l, class c): level offset + c Q_l^2
     std::vector<long long> goff(ng, 0);
     for (int g = 0; g < ng; ++g) {
@@ -999,7 +1107,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     QBX_CUDA_TRY(f->m2l_vsrc.alloc(std::max<size_t>(1, vsrc.size())));
     if (!vsrc.empty())
       QBX_CUDA_TRY(cudaMemcpy(f->m2l_vsrc.ptr, vsrc.data(), vsrc.size() * sizeof(int), cudaMemcpyHostToDevice));
-    QBX_CUDA_TRY(f->mu32.alloc(std::max<int64_t>(1, f->n_coef)));
+    QBX_CUDA_TRY(f->mu32.alloc(std::max<int64_t>(1, f->n_coef + nb)));
     {  // result-row offset of every V entry
       std::vector<long long> eyoff(vrow.size(), 0);
       for (int64_t e = 0; e < nv; ++e) eyoff[e] = yoff[vrow[e]];
@@ -1018,7 +1126,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     }
     QBX_CUDA_TRY(cudaMemcpy(f->m2l_yoff.ptr, yoff.data(), yoff.size() * sizeof(long long), cudaMemcpyHostToDevice));
   }
-  // FP64 M2L matrices (same offsets as the FP32 ones) and result rows
+  // FP64 M2L matrices and result rows
   QBX_CUDA_TRY(f->tm_f64.alloc(std::max<long long>(1, tot)));
   for (int l = 2; l < f->n_levels; ++l) {
     if (f->vbox_off[l + 1] == f->vbox_off[l]) continue;
@@ -1028,38 +1136,23 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     QBX_CUDA_TRY(cudaGetLastError());
   }
   QBX_CUDA_TRY(f->m2l_y64.alloc(std::max<size_t>(1, f->m2l_y.n)));
-  // M2M matrices for parents on levels 2 .. n_levels - 2
-  {
-    std::vector<long long> moff(f->n_levels, 0);
-    long long mtot = 0;
-    for (int l = 2; l + 1 < f->n_levels; ++l) {
-      moff[l] = mtot;
-      mtot += 4LL * (2 * f->h_pb[l] + 1) * (2 * f->h_pb[l + 1] + 1);
-    }
-    QBX_CUDA_TRY(f->tmm_f32.alloc(std::max<long long>(1, mtot)));
-    f->h_tmm_off = moff;
-    for (int l = 2; l + 1 < f->n_levels; ++l) {
-      const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
-      dim3 grid(4, 2 * pc + 1);
-      m2m_f32_matrix_kernel<<<grid, kT>>>(l, pp, pc, pbm, f->t_m2m.ptr, f->lsig.ptr,
-                                          f->tmm_f32.ptr + moff[l]);
-      QBX_CUDA_TRY(cudaGetLastError());
-    }
-  }
-  // L2L matrices for parents on levels 2 .. n_levels - 2
-  std::vector<long long> loff(f->n_levels, 0);
-  long long ltot = 0;
+  // M2M and L2L matrices for parents on levels 2 .. n_levels - 2
+  std::vector<long long> moff(f->n_levels, 0);
+  long long mtot = 0;
   for (int l = 2; l + 1 < f->n_levels; ++l) {
-    loff[l] = ltot;
-    ltot += 4LL * (2 * f->h_pb[l] + 1) * (2 * f->h_pb[l + 1] + 1);
+    moff[l] = mtot;
+    mtot += (2LL * f->h_pb[l] + 1) * (2 * f->h_pb[l + 1] + 1);
   }
-  QBX_CUDA_TRY(f->tl_f32.alloc(std::max<long long>(1, ltot)));
-  f->h_tl_off = loff;
+  QBX_CUDA_TRY(f->tmm_f32.alloc(std::max<long long>(1, mtot)));
+  QBX_CUDA_TRY(f->tl_f32.alloc(std::max<long long>(1, mtot)));
+  f->h_fold_off = moff;
   for (int l = 2; l + 1 < f->n_levels; ++l) {
     const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
-    dim3 grid(4, 2 * pp + 1);
-    l2l_f32_matrix_kernel<<<grid, kT>>>(l, pp, pc, pbm, f->t_l2l.ptr, f->lsig.ptr,
-                                        f->tl_f32.ptr + loff[l]);
+    fold_matrix_kernel<true><<<2 * pc + 1, kT>>>(l, pp, pc, pbm, f->t_m2m.ptr, f->lsig.ptr,
+                                                 f->tmm_f32.ptr + moff[l]);
+    QBX_CUDA_TRY(cudaGetLastError());
+    fold_matrix_kernel<false><<<2 * pp + 1, kT>>>(l, pp, pc, pbm, f->t_l2l.ptr, f->lsig.ptr,
+                                                  f->tl_f32.ptr + moff[l]);
     QBX_CUDA_TRY(cudaGetLastError());
   }
   return QBX_OK;
@@ -1097,63 +1190,66 @@ qbx_status launch_m2l_f64_gemm_rest(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
   return QBX_OK;
 }
 
-// Dynamic shared memory of a split-K M2M / L2L CTA staging `rows` coefficient
-// rows of kNarrowRows boxes (the reduction reuses the space); split_fits: within
-// the opt-in limit with room for the kernels' static shared memory.
-static size_t split_smem(int rows) {
-  const size_t stage = (size_t)rows * stage_stride(kNarrowRows) * sizeof(float2);
-  const size_t red = (size_t)kSplitWarps * kNarrowRows * 32 * sizeof(float2);
-  return std::max(stage, red);
+// A launch that may start before its predecessor in the stream has finished
+// (pdl_wait in the kernel); ordinary for batched handles, whose streams share the
+// SMs with other problems.
+template <typename... P, typename... A>
+static cudaError_t launch_chained(void (*k)(P...), dim3 g, size_t smem, cudaStream_t s, bool chain,
+                                  A... a) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = g;
+  c.blockDim = dim3(kT);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(a)...);
 }
-static bool split_fits(int rows) { return split_smem(rows) + 1024 <= (size_t)g_mixed_smem_optin; }
-// The split kernels serve levels whose one-column-per-thread grid would have
-// fewer than four CTAs per SM (GB300: 152 SMs); wider levels keep the others.
-constexpr long long kSplitBelow = 4 * 152;
-
+// FP32 M2M (from the child level up) or L2L of all levels. Parents per CTA: 8 where
+// that gives the SMs two CTAs each, fewer on narrower levels, whose CTAs also share a
+// parent's orders out (so that it is staged several times). A level's launch may
+// overlap the one before it (only such kernels allow it).
+template <bool M2M>
+static qbx_status launch_fold(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
+  bool prev = false;
+  const int n = f->n_levels - 3;  // levels 2 .. n_levels - 2
+  for (int i = 0; i < n; ++i) {
+    const int l = M2M ? f->n_levels - 2 - i : 2 + i;
+    const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
+    if (nb == 0) continue;
+    const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
+    const int Qi = 2 * (M2M ? pc : pp) + 1, Qo = 2 * (M2M ? pp : pc) + 1;
+    auto launch = [&](auto rows) -> cudaError_t {
+      constexpr int R = decltype(rows)::value;
+      const unsigned gx = nblk(nb, R), chunks = nblk(Qo, 32);
+      const unsigned gy = h->batched ? 1u : std::min(chunks, std::max(1u, 4 * 152 / gx));
+      return launch_chained(M2M ? m2m_fold_kernel<R> : l2l_fold_kernel<R>, dim3(gx, gy),
+                            fold_smem(Qi, M2M ? 4 : 1, R), s, prev && !h->batched, l, pp, pc,
+                            f->pb_max, (const int*)f->nonleaf.ptr + f->nonleaf_off[l], nb,
+                            (const int*)f->box.child.ptr, (const long long*)f->eoff.ptr,
+                            (const float*)(M2M ? f->tmm_f32.ptr : f->tl_f32.ptr) + f->h_fold_off[l],
+                            (const double*)f->conv.ptr, (const double*)f->iconv.ptr,
+                            M2M ? f->mpole.ptr : f->local.ptr);
+    };
+    if (nb >= 8 * 2 * 152 || (h->batched && nb >= 64))
+      QBX_CUDA_TRY(launch(std::integral_constant<int, 8>()));
+    else if (nb >= 4 * 152)
+      QBX_CUDA_TRY(launch(std::integral_constant<int, 4>()));
+    else
+      QBX_CUDA_TRY(launch(std::integral_constant<int, 2>()));
+    prev = !debug_sync();
+    h->launches += 1;
+  }
+  return QBX_OK;
+}
 qbx_status launch_m2m_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
-  for (int l = f->n_levels - 2; l >= 2; --l) {
-    const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
-    if (nb == 0) continue;
-    const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
-    const int* par = f->nonleaf.ptr + f->nonleaf_off[l];
-    const float2* T = f->tmm_f32.ptr + f->h_tmm_off[l];
-    if (nb >= kWideLevel || h->batched)
-      m2m_f32_kernel<kGemmRows><<<dim3(nblk(nb, kGemmRows), nblk(2 * pp + 1, kT)), kT, (size_t)(2 * pc + 1) * stage_stride(kGemmRows) * sizeof(float2), s>>>(
-          l, pp, pc, f->pb_max, par, nb, f->box.child.ptr, f->eoff.ptr, T, f->conv.ptr, f->mpole.ptr);
-    else if ((long long)nblk(nb, kNarrowRows) * nblk(2 * pp + 1, kT) < kSplitBelow &&
-             split_fits(4 * (2 * pc + 1)))
-      m2m_f32_split_kernel<kNarrowRows><<<dim3(nblk(nb, kNarrowRows), nblk(2 * pp + 1, kSplitCols)), kT, split_smem(4 * (2 * pc + 1)), s>>>(
-          l, pp, pc, f->pb_max, par, nb, f->box.child.ptr, f->eoff.ptr, T, f->conv.ptr, f->mpole.ptr);
-    else
-      m2m_f32_kernel<kNarrowRows><<<dim3(nblk(nb, kNarrowRows), nblk(2 * pp + 1, kT)), kT, (size_t)(2 * pc + 1) * stage_stride(kNarrowRows) * sizeof(float2), s>>>(
-          l, pp, pc, f->pb_max, par, nb, f->box.child.ptr, f->eoff.ptr, T, f->conv.ptr, f->mpole.ptr);
-    QBX_CUDA_TRY(cudaGetLastError());
-    h->launches += 1;
-  }
-  return QBX_OK;
+  return launch_fold<true>(h, f, s);
 }
-
 qbx_status launch_l2l_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
-  for (int l = 2; l + 1 < f->n_levels; ++l) {
-    const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
-    if (nb == 0) continue;
-    const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
-    const int* par = f->nonleaf.ptr + f->nonleaf_off[l];
-    const float2* T = f->tl_f32.ptr + f->h_tl_off[l];
-    if (nb >= kWideLevel || h->batched)
-      l2l_f32_kernel<kGemmRows><<<dim3(nblk(nb, kGemmRows), 4, nblk(2 * pc + 1, kT)), kT, (size_t)(2 * pp + 1) * stage_stride(kGemmRows) * sizeof(float2), s>>>(
-          l, pp, pc, f->pb_max, par, nb, f->box.child.ptr, f->eoff.ptr, T, f->conv.ptr, f->local.ptr);
-    else if ((long long)nblk(nb, kNarrowRows) * 4 * nblk(2 * pc + 1, kT) < kSplitBelow &&
-             split_fits(2 * pp + 1))
-      l2l_f32_split_kernel<kNarrowRows><<<dim3(nblk(nb, kNarrowRows), 4, nblk(2 * pc + 1, kSplitCols)), kT, split_smem(2 * pp + 1), s>>>(
-          l, pp, pc, f->pb_max, par, nb, f->box.child.ptr, f->eoff.ptr, T, f->conv.ptr, f->local.ptr);
-    else
-      l2l_f32_kernel<kNarrowRows><<<dim3(nblk(nb, kNarrowRows), 4, nblk(2 * pc + 1, kT)), kT, (size_t)(2 * pp + 1) * stage_stride(kNarrowRows) * sizeof(float2), s>>>(
-          l, pp, pc, f->pb_max, par, nb, f->box.child.ptr, f->eoff.ptr, T, f->conv.ptr, f->local.ptr);
-    QBX_CUDA_TRY(cudaGetLastError());
-    h->launches += 1;
-  }
-  return QBX_OK;
+  return launch_fold<false>(h, f, s);
 }
 
 qbx_status launch_m2l_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
@@ -1169,9 +1265,9 @@ qbx_status launch_m2l_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s) {
   auto gemm = [&](auto nt, int n) -> qbx_status {
     constexpr int NT = decltype(nt)::value;
     if (n > 0) {
-      m2l_f32_gemm_kernel<NT><<<n, NT, 0, s>>>(
-          f->m2l_items32.ptr + at, f->lpb.ptr, f->m2l_goff.ptr, f->m2l_rowoff.ptr, f->mu32.ptr,
-          f->tm_f32.ptr, f->m2l_yoff.ptr, f->m2l_y.ptr);
+      m2l_fold_kernel<NT><<<n, NT, 0, s>>>(
+          f->m2l_items32.ptr + at, f->lpb.ptr, f->m2l_toff.ptr, f->m2l_frow.ptr, f->pb_max,
+          f->m2l_rot.ptr, f->mu32.ptr, f->tm_f32.ptr, f->m2l_y.ptr);
       QBX_CUDA_TRY(cudaGetLastError());
       h->launches += 1;
     }

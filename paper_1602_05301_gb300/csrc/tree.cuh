@@ -169,11 +169,13 @@ struct FmmPlan {
   DevBuf<float4> dn32, qf, df, nf;      // FP32 (d k/2, nu); float-float charges, d k, normals
   DevBuf<int> err;                      // device error flags
   // mixed precision (sigma-normalised FP32 M2L)
-  DevBuf<double> lsig, conv;            // [n_levels][pb_max+1] log sig_j, s^j / sig_j
+  DevBuf<double> lsig, conv, iconv;     // [n_levels][pb_max+1] log sig_j, s^j / sig_j, its inverse
   DevBuf<double> isig;                  // [n_levels][pb_max+2] 1 / sig_min(j, pb) (mixed P2M)
   DevBuf<float2> isf;                   // the same times 2^{s j} (s = ff_s), float-float
-  DevBuf<float2> tm_f32;                // per level l >= 2: [49][Q_l][Q_l] M2L matrices
-  std::vector<long long> h_tm_off;      // [n_levels] offset of level l's matrices
+  DevBuf<float2> tm_f32;                // per (level l >= 2, distance): Te, To [P_l][P_l]
+  DevBuf<long long> m2l_toff;           // their offsets
+  DevBuf<longlong2> m2l_frow;           // FP32 M2L rows (m2l_fold_kernel)
+  DevBuf<float2> m2l_rot;               // [49][pb_max + 1] e^{i m phi} of the offset classes
   // M2L as batched GEMMs: V entries grouped by (level, offset class) into
   // rows; work items over tiles of rows, row offsets into the result
   // buffers, and the result row of every V entry
@@ -189,11 +191,9 @@ struct FmmPlan {
   DevBuf<cd> m2l_y64;                   // FP64 result rows of the FP64 M2L GEMM
   DevBuf<int> m2l_vsrc;                 // boxes that are V-list sources
   int n_vsrc = 0;
-  DevBuf<float2> mu32;                  // [n_coef] their sigma-normalised FP32 multipoles
-  DevBuf<float2> tl_f32;                // per parent level l: [4][Q_l][Q_{l+1}] L2L matrices
-  std::vector<long long> h_tl_off;
-  DevBuf<float2> tmm_f32;               // per parent level l: [4][Q_{l+1}][Q_l] M2M matrices
-  std::vector<long long> h_tmm_off;
+  DevBuf<float2> mu32;                  // [n_coef + n_boxes] their FP32 multipoles (mpole_to_f32_kernel)
+  DevBuf<float> tmm_f32, tl_f32;        // per parent level: M2M [Q_{l+1}][Q_l], L2L [Q_l][Q_{l+1}]
+  std::vector<long long> h_fold_off;    // offsets of both
   // tensor-core M2L of the FP64 path (m2l_tc.cu)
   std::vector<int> h_row_src;           // source box of every M2L row
   std::vector<int64_t> h_gcount;        // [n_levels * 49 + 1] first row of every group
