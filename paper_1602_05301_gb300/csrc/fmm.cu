@@ -35,11 +35,6 @@
 namespace {
 
 constexpr int kThreads = 128;
-// CTA size of the per-leaf kernels (threads over the centres or targets of one
-// leaf). Leaves that hold centres are kept at least kLeafOverRadius disk radii
-// wide, so they carry many centres (about 65 on the starfish workloads) and few
-// leaves hold any: one warp per leaf left most SMs idle (measured 2x slower).
-constexpr int kLeafThreads = 128;
 // Sources per shared-memory chunk in P2M / P2L. Their rows (one FP64 recurrence
 // per source) are built by threads 0..kChunk-1, a full warp: the SM's FP64
 // rate is shared by its warps and a warp instruction costs the same with few
@@ -112,10 +107,6 @@ struct Fmm {
 
 __device__ __forceinline__ const double* pw_row(const Fmm& F, int l) { return F.pw + (size_t)l * (2 * F.pbmax + 3); }
 __device__ __forceinline__ const double* ipw_row(const Fmm& F, int l) { return F.ipw + (size_t)l * (F.pbmax + 2); }
-// Centred translation table of (level l, item): entry m at [m].
-__device__ __forceinline__ const cd* table(const Fmm& F, const cd* t, int items, int l, int item) {
-  return t + ((size_t)l * items + item) * (4 * F.pbmax + 1) + 2 * F.pbmax;
-}
 
 // Unnormalised Miller recurrence for J_0..J_M of x into row[0..M]; returns the
 // normalisation (divide by it). Rescales the stored part when values grow.
@@ -391,46 +382,158 @@ __global__ void __launch_bounds__(kThreads) p2m_sum_kernel(Fmm F, const int* __r
   }
 }
 
-// ---------------------------------------------------------------- M2M (Stage 2)
-// Parents of level l (order pp), children of level l + 1 (order pc), FP64:
-// a_s = sum_{|n| <= pc} a'_n conj(V_{s-n}), |s| <= pp. A CTA takes a parent and
-// 32 output orders (chunk blockIdx.y); warp c sums child c's terms (its scaled
-// multipole staged in shared memory, the table read through L1: consecutive
-// lanes read consecutive entries), and the four sums are added in child order.
-// Bound by the FP64 pipe at about 1/2 complex product per clock and SM, so a
-// level costs nb Qp Qc 4 / 608 cycles spread over the SMs: the levels of few
-// boxes (mml_on_cuda_cores) run here, the others on the tensor cores.
-constexpr int kMmlCols = 32;
-
-__global__ void __launch_bounds__(kThreads) m2m_kernel(Fmm F, const int* __restrict__ boxes) {
-  extern __shared__ cd smem[];  // [4][Qc], then [4][kMmlCols]
+// ---------------------------------------------------------------- M2M (Stage 2), L2L (Stage 7)
+// FP64. a_s = sum over the children and |n| <= pc of a'_n conj(V_{s-n}), and
+// gamma'_s = sum_{|n| <= pp} gamma_n (-1)^{s-n} V_{s-n}. The four children of a box lie
+// at the same distance and at the angles pi/4 + rho pi/2, so that with rotations by
+// eighth turns both are a real matrix product J_{s-n}, and the rotations of the four
+// children differ by quarter turns, which depend on s - n mod 4 only:
+//   M2M  a_s = e^{-i s pi/4} sum_n J_{s-n} b_{(n-s) mod 4, n},
+//        b_{j,n} = sum_rho i^{rho j} e^{i n pi/4} a'_{rho,n};
+//   L2L  gamma'_{rho,s} = e^{i s pi/4} sum_k i^{rho k} t_k,
+//        t_k = sum over n = s - k mod 4 of J_{n-s} e^{-i n pi/4} gamma_n.
+// 2 FMAs per (n, s) and parent where the four complex products take 16. The matrices
+// T[n][s] hold the powers of the scaled coefficients and 1/sqrt 2 for each odd order of
+// the eighth turns (turn8 leaves it out).
+// A CTA takes a parent; warp w sums the terms n = w mod 4 (counted from the lowest
+// order) of 32 orders s, one per lane, and the warps join the four sums. The orders s
+// are taken 32 at a time, gridDim.y apart. Bound by the FP64 pipe (304 FMAs per clock
+// over the chip). M2M and L2L of 25 ellipses 0.73 and 0.72 ms -> 0.28 and 0.32 against
+// the exact split of the four complex products on the tensor cores, which this replaces
+// (its conversions to and from digits cost more than the products), of 200 ellipses
+// 2.57 -> 1.48 and 1.98 -> 1.81, of the 8192-node starfish 0.19 and 0.15 -> 0.07 and
+// 0.08; also the faster one at box orders of 573.
+constexpr int child_at(int rho) { return (0x4B >> (2 * rho)) & 3; }  // quadrant at pi/4 + rho pi/2
+__device__ __forceinline__ cd turn4(cd v, int q) {  // i^q v
+  if (q & 1) v = mk(-v.y, v.x);
+  if (q & 2) v = mk(-v.x, -v.y);
+  return v;
+}
+__device__ __forceinline__ cd turn8(cd v, int m) {  // e^{i m pi/4} v, sqrt 2 times for odd m
+  if (m & 1) v = mk(v.x - v.y, v.x + v.y);
+  return turn4(v, m >> 1);
+}
+__device__ __forceinline__ void dft4(cd (&v)[4]) {  // v_j <- sum_rho i^{rho j} v_rho
+  const cd a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+  const cd c = cadd(v[1], v[3]), d = mk(v[3].y - v[1].y, v[1].x - v[3].x);
+  v[0] = cadd(a, c);
+  v[2] = csub(a, c);
+  v[1] = cadd(b, d);
+  v[3] = csub(b, d);
+}
+// The matrix of parent level l: M2M from child order n to parent order s, L2L from
+// parent to child; from the tables of the quadrant at pi/4. Grid: n, threads over s.
+template <bool M2M>
+__global__ void fold64_matrix_kernel(int l, int pp, int pc, int pbmax, const cd* __restrict__ table,
+                                     const double* __restrict__ pw, const double* __restrict__ ipw,
+                                     double* __restrict__ T) {
+  const int pn = M2M ? pc : pp, ps = M2M ? pp : pc;
+  const int n = (int)blockIdx.x - pn;
+  const cd* v = table + ((size_t)l * 4 + child_at(0)) * (4 * pbmax + 1) + 2 * pbmax;
+  const double* pwc = pw + (size_t)(l + 1) * (2 * pbmax + 3);
+  const double* ipp = ipw + (size_t)l * (pbmax + 2);
+  double* dst = T + (size_t)(n + pn) * (2 * ps + 1) + ps;
+  for (int s = (int)threadIdx.x - ps; s <= ps; s += blockDim.x) {
+    const cd e = v[s - n];  // J_{s-n} e^{-i (s-n) pi/4} (M2M), J_{n-s} e^{i (s-n) pi/4} (L2L)
+    double c, sn;
+    sincospi(0.25 * (M2M ? s - n : n - s), &sn, &c);
+    double f = M2M ? pwc[abs(n)] * ipp[abs(s)] : pwc[abs(s)] * ipp[abs(n)];
+    if ((n & 1) && (s & 1)) f *= 0.5;
+    else if ((n | s) & 1) f *= 0.70710678118654752440;
+    dst[s] = (e.x * c - e.y * sn) * f;
+  }
+}
+constexpr int kFoldCols = 32;
+// sum_{j < N} M[j * ld] x[j * xs]
+__device__ __forceinline__ cd real_sum(const double* __restrict__ M, size_t ld, int N,
+                                       const cd* __restrict__ x, int xs) {
+  cd sum = mk(0.0, 0.0);
+#pragma unroll 4
+  for (int j = 0; j < N; ++j) {
+    const double t = M[(size_t)j * ld];
+    const cd v = x[(size_t)j * xs];
+    sum.x = fma(t, v.x, sum.x);
+    sum.y = fma(t, v.y, sum.y);
+  }
+  return sum;
+}
+__global__ void __launch_bounds__(kThreads) m2m_kernel(Fmm F, const int* __restrict__ boxes,
+                                                       const double* __restrict__ T) {
+  extern __shared__ cd smem[];  // [Qc][4], then [4][kFoldCols]
   const int b = boxes[blockIdx.x];
   const int l = F.level[b];
   const int pp = F.lpb[l], pc = F.lpb[l + 1];
-  const int Qc = 2 * pc + 1;
-  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = (int)blockIdx.y * kMmlCols + lane - pp;
-  const double* pwc = pw_row(F, l + 1);
-  const int d = F.child[4 * b + c];
-  cd* a = smem + c * Qc;
-  if (d >= 0) {
-    const cd* mp = F.mpole + F.eoff[d];
-    for (int i = lane; i < Qc; i += 32) a[i] = cscale(mp[i], pwc[abs(i - pc)]);
-  }
-  __syncwarp();
-  cd sum = mk(0.0, 0.0);
-  if (d >= 0 && s <= pp) {
-    const cd* t = table(F, F.t_m2m, 4, l, c) + s;
-#pragma unroll 4
-    for (int n = -pc; n <= pc; ++n) cfma(sum, t[-n], a[n + pc]);
-  }
+  const int Qc = 2 * pc + 1, Qp = 2 * pp + 1;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   cd* red = smem + 4 * Qc;
-  red[c * kMmlCols + lane] = sum;
-  __syncthreads();
-  if (c == 0 && s <= pp) {
-    for (int u = 1; u < 4; ++u) sum = cadd(sum, red[u * kMmlCols + lane]);
-    F.mpole[F.eoff[b] + s + pp] = cscale(sum, ipw_row(F, l)[abs(s)]);
+  const cd* src[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int d = F.child[4 * b + child_at(c)];
+    src[c] = d >= 0 ? F.mpole + F.eoff[d] : nullptr;
   }
+  for (int i = threadIdx.x; i < Qc; i += kThreads) {
+    cd v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = src[c] ? turn8(src[c][i], i - pc) : mk(0.0, 0.0);
+    dft4(v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) smem[4 * i + j] = v[j];
+  }
+  __syncthreads();
+  for (int s0 = blockIdx.y * kFoldCols; s0 < Qp; s0 += kFoldCols * gridDim.y) {
+    const int at = s0 + lane, s = at - pp;
+    const int j = (w - pc - s) & 3;
+    cd sum = mk(0.0, 0.0);
+    if (at < Qp && w < Qc)
+      sum = real_sum(T + (size_t)w * Qp + at, 4 * (size_t)Qp, (Qc - w + 3) / 4, smem + 4 * w + j, 16);
+    __syncthreads();
+    red[w * kFoldCols + lane] = sum;
+    __syncthreads();
+    if (w == (s0 / kFoldCols & 3) && at < Qp) {
+      cd v = cadd(cadd(red[lane], red[kFoldCols + lane]),
+                  cadd(red[2 * kFoldCols + lane], red[3 * kFoldCols + lane]));
+      F.mpole[F.eoff[b] + at] = turn8(v, -s);
+    }
+  }
+}
+__global__ void __launch_bounds__(kThreads) l2l_kernel(Fmm F, const int* __restrict__ boxes,
+                                                       const double* __restrict__ T) {
+  extern __shared__ cd smem[];  // [Qp], then [4][kFoldCols]
+  const int b = boxes[blockIdx.x];
+  const int l = F.level[b];
+  const int pp = F.lpb[l], pc = F.lpb[l + 1];
+  const int Qp = 2 * pp + 1, Qc = 2 * pc + 1;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  cd* red = smem + Qp;
+  const cd* lp = F.local + F.eoff[b];
+  for (int i = threadIdx.x; i < Qp; i += kThreads) smem[i] = turn8(lp[i], pp - i);
+  const int d = F.child[4 * b + child_at(w)];  // warp w stores the child at rho = w
+  cd* dl = d >= 0 ? F.local + F.eoff[d] : nullptr;
+  __syncthreads();
+  for (int s0 = blockIdx.y * kFoldCols; s0 < Qc; s0 += kFoldCols * gridDim.y) {
+    const int at = s0 + lane, s = at - pc;
+    cd sum = mk(0.0, 0.0);
+    if (at < Qc && w < Qp)
+      sum = real_sum(T + (size_t)w * Qc + at, 4 * (size_t)Qc, (Qp - w + 3) / 4, smem + w, 4);
+    __syncthreads();
+    red[w * kFoldCols + lane] = sum;
+    __syncthreads();
+    if (dl && at < Qc) {  // sum_k i^{w k} t_k, t_k in the sums of warp (s + pp - k) mod 4
+      cd v = red[((s + pp) & 3) * kFoldCols + lane];
+#pragma unroll
+      for (int k = 1; k < 4; ++k)
+        v = cadd(v, turn4(red[((s + pp - k) & 3) * kFoldCols + lane], w * k));
+      dl[at] = cadd(dl[at], turn8(v, s));
+    }
+  }
+}
+size_t m2m_smem(int pc) { return (4 * (size_t)(2 * pc + 1) + 4 * kFoldCols) * sizeof(cd); }
+size_t l2l_smem(int pp) { return ((size_t)(2 * pp + 1) + 4 * kFoldCols) * sizeof(cd); }
+// blocks along the orders: all of a parent's orders in one where there are parents
+// enough, so that they are staged once
+unsigned fold_split(int nb, int Q) {
+  return std::min(nblk(Q, kFoldCols), std::max(1u, 8u * 152u / (unsigned)nb));
 }
 
 // ---------------------------------------------------------------- M2L (Stage 4)
@@ -527,47 +630,6 @@ __global__ void __launch_bounds__(kThreads) p2l_sum_kernel(Fmm F, const int* __r
     dst[n] = cadd(dst[n], sum);
   }
 }
-
-// ---------------------------------------------------------------- L2L (Stage 7)
-// Parents of level l (order pp) into their children (order pc), FP64:
-// gamma'_s = sum_{|n| <= pp} gamma_n (-1)^{s-n} V_{s-n}, |s| <= pc. A CTA takes a
-// parent, a child quadrant (blockIdx.y) and 32 output orders (blockIdx.z); warp w
-// sums the w-th quarter of the parent's orders, the four sums are added in warp
-// order. Same bound and levels as m2m_kernel.
-__global__ void __launch_bounds__(kThreads) l2l_kernel(Fmm F, const int* __restrict__ boxes) {
-  extern __shared__ cd smem[];  // [Qp], then [4][kMmlCols]
-  const int b = boxes[blockIdx.x], c = blockIdx.y;
-  const int d = F.child[4 * b + c];
-  if (d < 0) return;
-  const int l = F.level[b];
-  const int pp = F.lpb[l], pc = F.lpb[l + 1];
-  const int Qp = 2 * pp + 1;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = (int)blockIdx.z * kMmlCols + lane - pc;
-  const double* ipp = ipw_row(F, l);
-  const cd* lp = F.local + F.eoff[b];
-  cd* g = smem;  // true local coefficients gamma_n
-  for (int i = threadIdx.x; i < Qp; i += kThreads) g[i] = cscale(lp[i], ipp[abs(i - pp)]);
-  __syncthreads();
-  const int per = (Qp + 3) / 4, i0 = min(Qp, w * per), i1 = min(Qp, i0 + per);
-  cd sum = mk(0.0, 0.0);
-  if (s <= pc) {
-    const cd* t = table(F, F.t_l2l, 4, l, c) + s + pp;
-#pragma unroll 4
-    for (int i = i0; i < i1; ++i) cfma(sum, t[-i], g[i]);
-  }
-  cd* red = smem + Qp;
-  red[w * kMmlCols + lane] = sum;
-  __syncthreads();
-  if (w == 0 && s <= pc) {
-    for (int u = 1; u < 4; ++u) sum = cadd(sum, red[u * kMmlCols + lane]);
-    cd* dl = F.local + F.eoff[d] + s + pc;
-    *dl = cadd(*dl, cscale(sum, pw_row(F, l + 1)[abs(s)]));
-  }
-}
-
-size_t m2m_smem(int pc) { return (4 * (size_t)(2 * pc + 1) + 4 * kMmlCols) * sizeof(cd); }
-size_t l2l_smem(int pp) { return ((size_t)(2 * pp + 1) + 4 * kMmlCols) * sizeof(cd); }
 
 // ---------------------------------------------------------------- targets (Stages 3, 5, 8)
 // CTA per leaf; one thread per target of the leaf (strided). Only targets that
@@ -1105,7 +1167,6 @@ __device__ __forceinline__ void kahan2(float2& s, float2& c, float2 v) {
 __device__ __forceinline__ float2 fmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ float2 fsub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 f2(cd a) { return make_float2(f32_from_f64(a.x), f32_from_f64(a.y)); }
 
 // One source's contribution to the scaled sums of a centre, in the split of
@@ -2423,8 +2484,18 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
     return QBX_ERR_ARG;
   }
   TRY(mixed_plan_build(h, f));
+  QBX_CUDA_TRY(f->tmm_f64.alloc(f->tmm_f32.n));
+  QBX_CUDA_TRY(f->tl_f64.alloc(f->tl_f32.n));
+  for (int l = 2; l + 1 < f->n_levels; ++l) {
+    const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
+    fold64_matrix_kernel<true><<<2 * pc + 1, kThreads>>>(l, pp, pc, pbm, f->t_m2m.ptr, f->pw.ptr,
+                                                         f->ipw.ptr, f->tmm_f64.ptr + f->h_fold_off[l]);
+    QBX_CUDA_TRY(cudaGetLastError());
+    fold64_matrix_kernel<false><<<2 * pp + 1, kThreads>>>(l, pp, pc, pbm, f->t_l2l.ptr, f->pw.ptr,
+                                                          f->ipw.ptr, f->tl_f64.ptr + f->h_fold_off[l]);
+    QBX_CUDA_TRY(cudaGetLastError());
+  }
   TRY(tc_plan_build(h, f));
-  TRY(tc_mml_plan_build(h, f));
   QBX_CUDA_TRY(f->qs.alloc(std::max<int64_t>(1, h->n_src)));
   QBX_CUDA_TRY(f->ds.alloc(std::max<int64_t>(1, h->n_src)));
   QBX_CUDA_TRY(f->q32.alloc(std::max<int64_t>(1, h->n_src)));
@@ -3083,14 +3154,8 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     for (int l = f->n_levels - 2; l >= 2; --l) {
       const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
       if (nb == 0) continue;
-      bool done = false;  // tensor cores on wide levels whose split is exact
-      TRY(launch_mml_tc(h, f, 0, l, &done, s));
-      if (done) {
-        QBX_KCHECK("m2m_tc", s);
-        continue;
-      }
-      m2m_kernel<<<dim3(nb, nblk(2 * pb[l] + 1, kMmlCols)), kThreads, m2m_smem(pb[l + 1]), s>>>(
-          F, f->nonleaf.ptr + f->nonleaf_off[l]);
+      m2m_kernel<<<dim3(nb, fold_split(nb, 2 * pb[l] + 1)), kThreads, m2m_smem(pb[l + 1]), s>>>(
+          F, f->nonleaf.ptr + f->nonleaf_off[l], f->tmm_f64.ptr + f->h_fold_off[l]);
       QBX_KCHECK("m2m", s);
       h->launches += 1;
     }
@@ -3153,14 +3218,8 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     for (int l = 2; l + 1 < f->n_levels; ++l) {
       const int nb = f->nonleaf_off[l + 1] - f->nonleaf_off[l];
       if (nb == 0) continue;
-      bool done = false;  // tensor cores on wide levels whose split is exact
-      TRY(launch_mml_tc(h, f, 1, l, &done, s));
-      if (done) {
-        QBX_KCHECK("l2l_tc", s);
-        continue;
-      }
-      l2l_kernel<<<dim3(nb, 4, nblk(2 * pb[l + 1] + 1, kMmlCols)), kThreads, l2l_smem(pb[l]), s>>>(
-          F, f->nonleaf.ptr + f->nonleaf_off[l]);
+      l2l_kernel<<<dim3(nb, fold_split(nb, 2 * pb[l + 1] + 1)), kThreads, l2l_smem(pb[l]), s>>>(
+          F, f->nonleaf.ptr + f->nonleaf_off[l], f->tl_f64.ptr + f->h_fold_off[l]);
       QBX_KCHECK("l2l", s);
       h->launches += 1;
     }

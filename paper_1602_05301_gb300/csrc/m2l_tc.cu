@@ -74,7 +74,6 @@ constexpr int kThr = 128;
 constexpr long long kSpin = 1LL << 26;
 constexpr unsigned long long kWaitNs = 1000000000ull;  // 1 s
 
-inline unsigned nblk(int64_t n, int b) { return (unsigned)std::max<int64_t>(1, (n + b - 1) / b); }
 
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -372,135 +371,6 @@ __global__ void __launch_bounds__(kThr) tc_mu_kernel(
   for (int t = 0; t < 16; ++t) {
     const int k = threadIdx.x + kThr * t;
     if (k < Kp) split_digits(vals[t], e, beta, S, dst + k, (size_t)Kp);
-  }
-}
-
-// Matrix slices of the four quadrant groups of one parent level l of M2M
-// (kind 0: child orders in, parent orders out) or L2L (kind 1: parent orders
-// in, child orders out), from the FP64 tables of conj(V_m) (M2M) and
-// (-1)^m V_m (L2L) of the quadrant's shift, sigma-normalised:
-//   M2M  T[so][n] = (sig_{l+1,|n|} / sig_{l,|so|}) conj(V_{so-n}),
-//   L2L  T[so][n] = (sig_{l+1,|so|} / sig_{l,|n|}) (-1)^{so-n} V_{so-n},
-// in the real form of tc_matrix_kernel. Grid (4, Np), threads over k < K.
-// Slices [quadrant][S][Np][K], row exponents [quadrant][Np].
-__global__ void __launch_bounds__(kThr) tc_mml_matrix_kernel(
-    int kind, int l, int pp, int pc, int pbmax, const cd* __restrict__ tab,
-    const double* __restrict__ lsig, int K, int Np, int beta, int S, __nv_bfloat16* __restrict__ A,
-    int* __restrict__ fexp) {
-  __shared__ double red[kThr / 32];
-  const int c = blockIdx.x, j = blockIdx.y;
-  const int pin = kind == 0 ? pc : pp, pout = kind == 0 ? pp : pc;
-  const int Qin = 2 * pin + 1, Qout = 2 * pout + 1;
-  const cd* v = tab + ((size_t)l * 4 + c) * (4 * pbmax + 1) + 2 * pbmax;
-  const double* sp = lsig + (size_t)l * (pbmax + 1);        // parent level
-  const double* sc = lsig + (size_t)(l + 1) * (pbmax + 1);  // child level
-  const int so = (j < Qout ? j : j - Qout) - pout;
-  const bool im_out = j >= Qout;
-  double vals[16];  // k = threadIdx.x + 128 t, K <= 2048
-  double m = 0.0;
-  for (int t = 0; t < 16; ++t) {
-    const int k = threadIdx.x + kThr * t;
-    double val = 0.0;
-    if (j < 2 * Qout && k < 2 * Qin) {
-      const int n = (k < Qin ? k : k - Qin) - pin;
-      const cd e = v[so - n];
-      const double mag = hypot(e.x, e.y);
-      cd T = mk(0.0, 0.0);
-      if (mag > 0.0) {
-        const double lf = (kind == 0 ? sc[abs(n)] - sp[abs(so)] : sc[abs(so)] - sp[abs(n)]) + log(mag);
-        const double f = lf < -700.0 ? 0.0 : exp(lf) / mag;
-        T = mk(e.x * f, e.y * f);
-      }
-      const bool im_in = k >= Qin;
-      val = im_out ? (im_in ? T.x : T.y) : (im_in ? -T.y : T.x);
-    }
-    vals[t] = val;
-    m = fmax(m, fabs(val));
-  }
-  m = block_max(m, red);
-  const int e = scale_exponent(m);
-  if (threadIdx.x == 0) fexp[(size_t)c * Np + j] = e;
-  __nv_bfloat16* dst = A + (size_t)c * S * Np * K + (size_t)j * K;
-  for (int t = 0; t < 16; ++t) {
-    const int k = threadIdx.x + kThr * t;
-    if (k < K) split_digits(vals[t], e, beta, S, dst + k, (size_t)Np * K);
-  }
-}
-
-// Vector slices of the source boxes of one M2M / L2L level: M2M the children's
-// multipoles mu_n = mh_n conv_|n| (level l+1), L2L the parents' locals
-// lambda_n = lh_n / conv_|n| (level l); x = (Re, Im) padded to K, one exponent
-// per box, slices [S][K] at xoff[i]. One block per source box.
-__global__ void __launch_bounds__(kThr) tc_mml_vec_kernel(
-    int kind, const int* __restrict__ boxes, const cd* __restrict__ coef, int lsrc, int pb, int K,
-    int beta, int S, const double* __restrict__ conv, int pbmax, const long long* __restrict__ eoff,
-    const long long* __restrict__ xoff, __nv_bfloat16* __restrict__ X, int* __restrict__ xexp) {
-  __shared__ double red[kThr / 32];
-  const int b = boxes[blockIdx.x];
-  const int Q = 2 * pb + 1;
-  const double* cv = conv + (size_t)lsrc * (pbmax + 1);
-  const cd* a = coef + eoff[b];
-  double vals[16];  // K <= 2048
-  double m = 0.0;
-  for (int t = 0; t < 16; ++t) {
-    const int k = threadIdx.x + kThr * t;
-    double v = 0.0;
-    if (k < 2 * Q) {
-      const int n = k < Q ? k : k - Q;
-      const double f = kind == 0 ? cv[abs(n - pb)] : 1.0 / cv[abs(n - pb)];
-      v = (k < Q ? a[n].x : a[n].y) * f;
-    }
-    vals[t] = v;
-    m = fmax(m, fabs(v));
-  }
-  m = block_max(m, red);
-  const int e = scale_exponent(m);
-  if (threadIdx.x == 0) xexp[blockIdx.x] = e;
-  __nv_bfloat16* dst = X + xoff[blockIdx.x];
-  for (int t = 0; t < 16; ++t) {
-    const int k = threadIdx.x + kThr * t;
-    if (k < K) split_digits(vals[t], e, beta, S, dst + k, (size_t)K);
-  }
-}
-
-// M2M: mh_p[so] = (sum over the parent's child rows, quadrant order, float-float)
-// / conv_l[|so|]. prow[i][c]: the row of parent i's quadrant-c child (-1: none).
-__global__ void __launch_bounds__(kThr) tc_m2m_reduce_kernel(
-    const int* __restrict__ parents, const int* __restrict__ prow, int pp, int l, int pbmax,
-    const double* __restrict__ conv, const cd* __restrict__ Y, const long long* __restrict__ eoff,
-    cd* __restrict__ mpole) {
-  const int i = blockIdx.x;
-  const int Q = 2 * pp + 1;
-  const double* cv = conv + (size_t)l * (pbmax + 1);
-  cd* dst = mpole + eoff[parents[i]];
-  for (int lo = threadIdx.x; lo < Q; lo += kThr) {
-    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-    for (int c = 0; c < 4; ++c) {
-      const int r = prow[4 * i + c];
-      if (r < 0) continue;
-      const float2* y = reinterpret_cast<const float2*>(Y + (size_t)r * Q) + lo;
-      const float2 a = y[0], b = y[Q];
-      ff_add(rh, rl, a.x, a.y);
-      ff_add(ih, il, b.x, b.y);
-    }
-    const double f = 1.0 / cv[abs(lo - pp)];
-    dst[lo] = mk(((double)rh + (double)rl) * f, ((double)ih + (double)il) * f);
-  }
-}
-
-// L2L: lh_child[so] += row value * conv_{l+1}[|so|]. One block per row (child).
-__global__ void __launch_bounds__(kThr) tc_l2l_apply_kernel(
-    const int* __restrict__ rowdst, int pc, int lc, int pbmax, const double* __restrict__ conv,
-    const cd* __restrict__ Y, const long long* __restrict__ eoff, cd* __restrict__ local) {
-  const int r = blockIdx.x;
-  const int Q = 2 * pc + 1;
-  const double* cv = conv + (size_t)lc * (pbmax + 1);
-  cd* dst = local + eoff[rowdst[r]];
-  for (int lo = threadIdx.x; lo < Q; lo += kThr) {
-    const float2* y = reinterpret_cast<const float2*>(Y + (size_t)r * Q) + lo;
-    const float2 a = y[0], b = y[Q];
-    const double f = cv[abs(lo - pc)];
-    dst[lo] = cadd(dst[lo], mk(((double)a.x + (double)a.y) * f, ((double)b.x + (double)b.y) * f));
   }
 }
 
@@ -1465,157 +1335,6 @@ qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f) {
                               cudaMemcpyHostToDevice));
   }
   return tc_tma_plan_build(h, f, groups, lv, aoff, rowsrc, xoff);
-}
-
-
-
-// Plan of the FP64 M2M and L2L on the tensor cores: for every parent level l
-// whose contraction width K (2 Q of the child level for M2M, of level l for
-// L2L, padded to 64) admits an exact split, the matrix slices of the four
-// quadrant operators, the rows (one per child: quadrant-major, parents in
-// level order), the source boxes and the work items. Levels without one keep
-// the CUDA-core kernels; so do levels of few boxes (mml_on_cuda_cores) and all
-// levels with m2l_engine == 2 or QBX_M2L_TENSOR=0.
-qbx_status tc_mml_plan_build(qbx_handle* h, FmmPlan* f) {
-  const int nl = f->n_levels;
-  f->tc_m2m.clear();
-  f->tc_l2l.clear();
-  f->tc_m2m.resize(nl);
-  f->tc_l2l.resize(nl);
-  {
-    const char* env = getenv("QBX_M2L_TENSOR");
-    if ((env && env[0] == '0') || h->m2l_engine == 2) return QBX_OK;
-  }
-  std::vector<int> child((size_t)4 * f->n_boxes), nonleaf(std::max(1, f->nonleaf_off[nl]));
-  QBX_CUDA_TRY(cudaMemcpy(child.data(), f->box.child.ptr, child.size() * sizeof(int),
-                          cudaMemcpyDeviceToHost));
-  if (f->nonleaf_off[nl] > 0)
-    QBX_CUDA_TRY(cudaMemcpy(nonleaf.data(), f->nonleaf.ptr, f->nonleaf_off[nl] * sizeof(int),
-                            cudaMemcpyDeviceToHost));
-  size_t ymax = 1;
-  for (int kind = 0; kind < 2; ++kind) {
-    for (int l = 2; l + 1 < nl; ++l) {
-      // the level's parents, in the order of the device list (the reduce
-      // kernel walks that list)
-      const std::vector<int> par(nonleaf.begin() + f->nonleaf_off[l],
-                                 nonleaf.begin() + f->nonleaf_off[l + 1]);
-      if (par.empty()) continue;
-      TcLevelOp& op = kind == 0 ? f->tc_m2m[l] : f->tc_l2l[l];
-      const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
-      if (mml_on_cuda_cores((int)par.size(), pp, pc)) continue;
-      const int qin = kind == 0 ? 2 * pc + 1 : 2 * pp + 1;
-      const int qout = kind == 0 ? 2 * pp + 1 : 2 * pc + 1;
-      const int K = (2 * qin + kPad - 1) / kPad * kPad;
-      const int Np = (2 * qout + kPad - 1) / kPad * kPad;
-      const int2 bs = tc_params(K);
-      if (bs.x == 0) continue;
-      op.use = true;
-      op.beta = bs.x;
-      op.S = bs.y;
-      op.K = K;
-      op.Np = Np;
-      op.Q = qout;
-      op.n_par = (int)par.size();
-      // rows: quadrant-major, parents in level order; sources
-      std::vector<int> rowsrc, rowdst, prow((size_t)4 * par.size(), -1), src;
-      std::vector<int64_t> gcount(5, 0);
-      for (int c = 0; c < 4; ++c) {
-        gcount[c] = (int64_t)rowdst.size();
-        for (size_t i = 0; i < par.size(); ++i) {
-          const int d = child[4 * (size_t)par[i] + c];
-          if (d < 0) continue;
-          prow[4 * i + c] = (int)rowdst.size();
-          if (kind == 0) {  // M2M: the row's source is the child
-            rowsrc.push_back((int)src.size());
-            src.push_back(d);
-            rowdst.push_back(par[i]);
-          } else {          // L2L: the parent (one source per parent)
-            rowsrc.push_back((int)i);
-            rowdst.push_back(d);
-          }
-        }
-      }
-      gcount[4] = (int64_t)rowdst.size();
-      if (kind == 1) src = par;
-      op.n_rows = (int)rowdst.size();
-      op.n_src = (int)src.size();
-      ymax = std::max(ymax, (size_t)op.n_rows * qout);
-      std::vector<int4> gp(4, make_int4(K, qout, bs.x, Np));
-      std::vector<long long> gaoff(4), gfoff(4), xoff(src.size()), yoff(rowdst.size());
-      for (int c = 0; c < 4; ++c) {
-        gaoff[c] = (long long)c * bs.y * Np * K;
-        gfoff[c] = (long long)c * Np;
-      }
-      for (size_t i = 0; i < src.size(); ++i) xoff[i] = (long long)i * bs.y * K;
-      for (size_t r = 0; r < rowdst.size(); ++r) yoff[r] = (long long)r * qout;
-      std::vector<int4> items;
-      for (int c = 0; c < 4; ++c)
-        for (int64_t r = gcount[c]; r < gcount[c + 1]; r += kRows)
-          for (int n0 = 0; n0 < 2 * qout; n0 += kNC)
-            items.push_back(make_int4((int)r, (int)std::min<int64_t>(kRows, gcount[c + 1] - r), n0, c));
-      op.n_items = (int)items.size();
-      TRY_TC(upload(op.gp, gp));
-      TRY_TC(upload(op.items, items));
-      TRY_TC(upload(op.gaoff, gaoff));
-      TRY_TC(upload(op.gfoff, gfoff));
-      TRY_TC(upload(op.xoff, xoff));
-      TRY_TC(upload(op.yoff, yoff));
-      TRY_TC(upload(op.src, src));
-      TRY_TC(upload(op.rowsrc, rowsrc));
-      TRY_TC(upload(op.rowdst, rowdst));
-      TRY_TC(upload(op.prow, prow));
-      QBX_CUDA_TRY(op.A.alloc((size_t)4 * bs.y * Np * K));
-      QBX_CUDA_TRY(op.fexp.alloc((size_t)4 * Np));
-      QBX_CUDA_TRY(op.X.alloc(std::max<size_t>(1, src.size() * (size_t)bs.y * K)));
-      QBX_CUDA_TRY(op.xexp.alloc(std::max<size_t>(1, src.size())));
-      tc_mml_matrix_kernel<<<dim3(4, Np), kThr>>>(
-          kind, l, pp, pc, f->pb_max, kind == 0 ? f->t_m2m.ptr : f->t_l2l.ptr, f->lsig.ptr, K, Np,
-          bs.x, bs.y, reinterpret_cast<__nv_bfloat16*>(op.A.ptr), op.fexp.ptr);
-      QBX_CUDA_TRY(cudaGetLastError());
-    }
-  }
-  QBX_CUDA_TRY(f->tc_mml_y.alloc(ymax));
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
-  return QBX_OK;
-}
-
-qbx_status launch_mml_tc(qbx_handle* h, FmmPlan* f, int kind, int l, bool* done, cudaStream_t s) {
-  *done = false;
-  if (l >= (int)f->tc_m2m.size()) return QBX_OK;
-  TcLevelOp& op = kind == 0 ? f->tc_m2m[l] : f->tc_l2l[l];
-  if (!op.use) return QBX_OK;
-  const int pp = f->h_pb[l], pc = f->h_pb[l + 1];
-  if (op.n_src > 0) {
-    tc_mml_vec_kernel<<<op.n_src, kThr, 0, s>>>(
-        kind, op.src.ptr, kind == 0 ? f->mpole.ptr : f->local.ptr, kind == 0 ? l + 1 : l,
-        kind == 0 ? pc : pp, op.K, op.beta, op.S, f->conv.ptr, f->pb_max, f->eoff.ptr,
-        op.xoff.ptr, reinterpret_cast<__nv_bfloat16*>(op.X.ptr), op.xexp.ptr);
-    QBX_CUDA_TRY(cudaGetLastError());
-  }
-#define TC_MML(S_)                                                                              \
-  tc_gemm_ws_kernel<S_, S_><<<std::min(op.n_items, g_tc_sms), kWsThr, tc_smem_bytes<S_>(), s>>>(  \
-      op.items.ptr, op.n_items, op.gp.ptr, op.gaoff.ptr, op.gfoff.ptr,                          \
-      reinterpret_cast<const __nv_bfloat16*>(op.A.ptr), op.fexp.ptr, op.rowsrc.ptr, op.xoff.ptr, \
-      op.xexp.ptr, reinterpret_cast<const __nv_bfloat16*>(op.X.ptr), op.yoff.ptr,               \
-      f->tc_mml_y.ptr, f->err.ptr + 1)
-  if (op.n_items > 0) {
-    if (op.S == 6) TC_MML(6);
-    else if (op.S == 7) TC_MML(7);
-    else TC_MML(8);
-    QBX_CUDA_TRY(cudaGetLastError());
-  }
-#undef TC_MML
-  if (kind == 0)
-    tc_m2m_reduce_kernel<<<op.n_par, kThr, 0, s>>>(f->nonleaf.ptr + f->nonleaf_off[l], op.prow.ptr,
-                                                   pp, l, f->pb_max, f->conv.ptr, f->tc_mml_y.ptr,
-                                                   f->eoff.ptr, f->mpole.ptr);
-  else if (op.n_rows > 0)
-    tc_l2l_apply_kernel<<<op.n_rows, kThr, 0, s>>>(op.rowdst.ptr, pc, l + 1, f->pb_max, f->conv.ptr,
-                                                   f->tc_mml_y.ptr, f->eoff.ptr, f->local.ptr);
-  QBX_CUDA_TRY(cudaGetLastError());
-  h->launches += 3;
-  *done = true;
-  return QBX_OK;
 }
 
 qbx_status launch_m2l_tc(qbx_handle* h, FmmPlan* f, bool mixed, cudaStream_t s) {

@@ -32,19 +32,6 @@ struct alignas(64) TmapBlob {
   unsigned char b[128];
 };
 
-// One parent level of the FP64 M2M or L2L on the tensor cores: four groups
-// (the child quadrants), the bf16 matrix slices of their sigma-normalised
-// operators, the source vectors' slices, and the rows (one per child).
-struct TcLevelOp {
-  bool use = false;
-  int S = 0, beta = 0, K = 0, Np = 0, Q = 0;  // slices, digit bits, input width, output rows, outputs
-  int n_rows = 0, n_src = 0, n_items = 0, n_par = 0;
-  DevBuf<int4> gp, items;
-  DevBuf<long long> gaoff, gfoff, xoff, yoff;
-  DevBuf<uint16_t> A, X;
-  DevBuf<int> fexp, xexp, src, rowsrc, rowdst, prow;
-};
-
 // No power-of-two scaling of a level fits FP32 (see float_float_scale).
 constexpr int kNoFf = -100000;
 
@@ -193,7 +180,8 @@ struct FmmPlan {
   int n_vsrc = 0;
   DevBuf<float2> mu32;                  // [n_coef + n_boxes] their FP32 multipoles (mpole_to_f32_kernel)
   DevBuf<float> tmm_f32, tl_f32;        // per parent level: M2M [Q_{l+1}][Q_l], L2L [Q_l][Q_{l+1}]
-  std::vector<long long> h_fold_off;    // offsets of both
+  DevBuf<double> tmm_f64, tl_f64;       // the same for the FP64 kernels
+  std::vector<long long> h_fold_off;    // offsets of all four
   // tensor-core M2L of the FP64 path (m2l_tc.cu)
   std::vector<int> h_row_src;           // source box of every M2L row
   std::vector<int64_t> h_gcount;        // [n_levels * 49 + 1] first row of every group
@@ -203,7 +191,6 @@ struct FmmPlan {
   std::vector<int4> h_tc_lvl;           // per level (use, beta, S, padded 2Q)
   DevBuf<int4> tc_lvl;
   DevBuf<int4> tc_gp;                   // per group (K, Q, beta, Np) of the tile product
-  std::vector<TcLevelOp> tc_m2m, tc_l2l;  // per parent level (FP64 path)
   // FP64 M2L through TMA: the rows' source slices copied into row order per
   // group ([S][rows][K] at x2off), and the tensor maps of those copies and of
   // the matrix slices, per group
@@ -213,7 +200,6 @@ struct FmmPlan {
   DevBuf<long long> tc_x2src, tc_x2dst, tc_x2ts, tc_gstart;
   DevBuf<int2> tc_x2sk;
   DevBuf<TmapBlob> tc_mapA, tc_mapX;
-  DevBuf<cd> tc_mml_y;                  // their result rows (one level at a time)
   bool tc_any = false;
   DevBuf<uint16_t> tc_A;                // bf16 matrix slices [S][Kp][Kp] per group
   DevBuf<int> tc_fexp;                  // row exponents [Kp] per group
@@ -228,17 +214,6 @@ struct FmmPlan {
   int n_tc_items[3] = {0, 0, 0};
 };
 
-// FP64 M2M and L2L levels of few boxes stay on the CUDA cores: 4 FMAs per complex
-// product at 304 FMAs per clock over the chip, up to kMmlCycles; the tensor-core
-// path takes three launches and one tile's latency (45 us) however few boxes
-// there are. M2M and L2L of the 8192-node starfish with 971 boxes, FP64: 0.20 and
-// 0.22 ms all on the tensor cores, 0.10 and 0.07 ms with this rule; levels above the
-// line (25 ellipses) measured the same either way.
-constexpr double kMmlCycles = 50e3;
-inline bool mml_on_cuda_cores(int n_parents, int pp, int pc) {
-  return 16.0 * n_parents * (2.0 * pp + 1) * (2.0 * pc + 1) / 304.0 <= kMmlCycles;
-}
-
 qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f);
 qbx_status configure_mixed_kernels(int smem_optin);
 qbx_status launch_m2l_f32(qbx_handle* h, FmmPlan* f, cudaStream_t s);
@@ -249,10 +224,6 @@ qbx_status launch_m2l_f64_gemm_rest(qbx_handle* h, FmmPlan* f, cudaStream_t s);
 // m2l_tc.cu
 qbx_status configure_tc_kernels(int smem_optin);
 qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f);
-qbx_status tc_mml_plan_build(qbx_handle* h, FmmPlan* f);
-// FP64 M2M (kind 0) or L2L (kind 1) of parent level l on the tensor cores;
-// *done = false when the level stays on the CUDA-core kernel
-qbx_status launch_mml_tc(qbx_handle* h, FmmPlan* f, int kind, int l, bool* done, cudaStream_t s);
 qbx_status launch_m2l_tc(qbx_handle* h, FmmPlan* f, bool mixed, cudaStream_t s);
 // shared memory of one M2M / L2L tile-GEMM block at box order pb
 size_t gemm_smem_bytes(int pb);
