@@ -337,13 +337,19 @@ __global__ void __launch_bounds__(kThr) tc_matrix_kernel(
 }
 
 // Vector slices of the V-list sources: mu_n = mh_n conv_|n| (FP64), x = (Re mu,
-// Im mu) padded to Kp, one exponent per box. One block per box.
+// Im mu) padded to Kp, one exponent per box. One block per box. Into X ([S][Kp] at
+// xoff), or with rowoff into row order for the TMA product: box i's slices go to its
+// rows j = rowoff[i] .. rowoff[i + 1], slice t at X2 + rows[j].x + t rows[j].y. (As a
+// kernel of its own, the copy from X to the rows was bound by the latency of its index
+// loads, 82 us of the 430 us M2L of the 8192-node starfish.)
 __global__ void __launch_bounds__(kThr) tc_mu_kernel(
     const int* __restrict__ boxes, const int* __restrict__ level, const int* __restrict__ lpb,
     const long long* __restrict__ eoff, const double* __restrict__ conv, int pbmax,
     const int4* __restrict__ lvl, const cd* __restrict__ mpole, const long long* __restrict__ xoff,
-    __nv_bfloat16* __restrict__ X, int* __restrict__ xexp) {
+    __nv_bfloat16* __restrict__ X, int* __restrict__ xexp, const int* __restrict__ rowoff,
+    const longlong2* __restrict__ rows, uint16_t* __restrict__ X2) {
   __shared__ double red[kThr / 32];
+  extern __shared__ __align__(16) __nv_bfloat16 slices[];  // [S][Kp] with rowoff
   const int b = boxes[blockIdx.x];
   const int l = level[b];
   const int4 P = lvl[l];
@@ -367,10 +373,20 @@ __global__ void __launch_bounds__(kThr) tc_mu_kernel(
   m = block_max(m, red);
   const int e = scale_exponent(m);
   if (threadIdx.x == 0) xexp[blockIdx.x] = e;
-  __nv_bfloat16* dst = X + xoff[blockIdx.x];
+  __nv_bfloat16* dst = rowoff ? slices : X + xoff[blockIdx.x];
   for (int t = 0; t < 16; ++t) {
     const int k = threadIdx.x + kThr * t;
     if (k < Kp) split_digits(vals[t], e, beta, S, dst + k, (size_t)Kp);
+  }
+  if (!rowoff) return;
+  __syncthreads();
+  const int V = Kp / 8, SV = S * V;  // 16-byte vectors of a slice, of a row
+  const uint4* in = reinterpret_cast<const uint4*>(slices);
+  const int j0 = rowoff[blockIdx.x], n = (rowoff[blockIdx.x + 1] - j0) * SV;
+  for (int i = threadIdx.x; i < n; i += kThr) {
+    const int j = i / SV, u = i % SV;
+    const longlong2 r = rows[j0 + j];
+    reinterpret_cast<uint4*>(X2 + r.x + (u / V) * r.y)[u % V] = in[u];
   }
 }
 
@@ -801,7 +817,7 @@ __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
 }
 
 // The FP64 M2L's tile product fed by TMA. The source slices of the rows are
-// first copied into row order per group (tc_x2_fill_kernel: [S][rows][K], a
+// first written in row order per group (tc_mu_kernel: [S][rows][K], a
 // TMA-tileable 2D array); then a single producer lane loads a stage as 4 S
 // boxes of 128 rows x 16 bytes (rows) and 4 S boxes of 64 rows x 16 bytes
 // (matrix), one per slice and 8-wide k-group, with one expect-tx arrival on
@@ -809,21 +825,6 @@ __global__ void __launch_bounds__(kWsThr, 1) tc_gemm_ws_kernel(
 // 128 x 16 B at kg * 2 KB (rows; 1 KB for the matrix's 64), i.e. core matrices
 // adjacent in M 128 B apart and in K 2 KB (1 KB) apart. The MMA warp and the
 // epilogue warps are those of tc_gemm_ws_kernel.
-__global__ void tc_x2_fill_kernel(int n_rows, const long long* __restrict__ src,
-                                  const long long* __restrict__ dst,
-                                  const long long* __restrict__ tstride,
-                                  const int2* __restrict__ sk, const uint16_t* __restrict__ X,
-                                  uint16_t* __restrict__ X2) {
-  const int r = blockIdx.x;
-  if (r >= n_rows) return;
-  const int S = sk[r].x, K = sk[r].y, V = K / 8;  // 16-byte vectors per slice row
-  const uint4* in = reinterpret_cast<const uint4*>(X + src[r]);
-  for (int i = threadIdx.x; i < S * V; i += blockDim.x) {
-    const int t = i / V, v = i % V;
-    *reinterpret_cast<uint4*>(X2 + dst[r] + (size_t)t * tstride[r] + (size_t)v * 8) = in[(size_t)t * V + v];
-  }
-}
-
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                "r"(bytes)
@@ -1155,7 +1156,7 @@ bool encode_map(PFN_cuTensorMapEncodeTiled_v12000 enc, const void* base, uint64_
 // environment keeps the cp.async kernel (for comparisons).
 qbx_status tc_tma_plan_build(qbx_handle* h, FmmPlan* f, const std::vector<int>& groups,
                              const std::vector<int4>& lv, const std::vector<long long>& aoff,
-                             const std::vector<int>& rowsrc, const std::vector<long long>& xoff) {
+                             const std::vector<int>& rowsrc) {
   (void)h;
   f->tc_tma = false;
   const char* env = getenv("QBX_TC_TMA");
@@ -1165,20 +1166,24 @@ qbx_status tc_tma_plan_build(qbx_handle* h, FmmPlan* f, const std::vector<int>& 
   const int ng = f->n_levels * 49;
   std::vector<long long> gstart(ng + 1, 0), x2off(ng, 0);
   for (int g = 0; g <= ng; ++g) gstart[g] = f->h_gcount[g];
-  std::vector<long long> src, dst, ts;
-  std::vector<int2> sk;
+  // (group row, slice stride) of every row, by source
+  std::vector<int> rowoff(f->n_tc_src + 1, 0);
+  std::vector<longlong2> rows_of;
+  for (int g : groups)
+    for (long long r = gstart[g]; r < gstart[g + 1]; ++r) rowoff[rowsrc[r] + 1] += 1;
+  for (int i = 0; i < f->n_tc_src; ++i) rowoff[i + 1] += rowoff[i];
+  rows_of.resize(rowoff.back());
+  std::vector<int> at(rowoff.begin(), rowoff.end() - 1);
   long long tot = 0;
+  size_t smem = 0;
   for (int g : groups) {
     const int l = g / 49, S = lv[l].z, K = lv[l].w;
     const long long rows = gstart[g + 1] - gstart[g];
     x2off[g] = tot;
-    for (long long r = gstart[g]; r < gstart[g + 1]; ++r) {
-      src.push_back(xoff[rowsrc[r]]);
-      dst.push_back(tot + (r - gstart[g]) * K);
-      ts.push_back(rows * K);
-      sk.push_back(make_int2(S, K));
-    }
+    for (long long r = gstart[g]; r < gstart[g + 1]; ++r)
+      rows_of[at[rowsrc[r]]++] = make_longlong2(tot + (r - gstart[g]) * K, rows * K);
     tot += (long long)S * rows * K;
+    smem = std::max(smem, (size_t)S * K * sizeof(uint16_t));
   }
   QBX_CUDA_TRY(f->tc_X2.alloc(std::max<long long>(1, tot)));
   std::vector<TmapBlob> ma(ng), mx(ng);
@@ -1192,11 +1197,9 @@ qbx_status tc_tma_plan_build(qbx_handle* h, FmmPlan* f, const std::vector<int>& 
         !encode_map(enc, f->tc_X2.ptr + x2off[g], K, (uint64_t)S * rows, kRows, &mx[g]))
       return QBX_OK;  // no TMA maps: the cp.async kernel serves
   }
-  f->n_tc_rows = (int)src.size();
-  TRY_TC(upload(f->tc_x2src, src));
-  TRY_TC(upload(f->tc_x2dst, dst));
-  TRY_TC(upload(f->tc_x2ts, ts));
-  TRY_TC(upload(f->tc_x2sk, sk));
+  f->tc_mu_smem = smem;
+  TRY_TC(upload(f->tc_rowoff, rowoff));
+  TRY_TC(upload(f->tc_rows, rows_of));
   TRY_TC(upload(f->tc_gstart, gstart));
   TRY_TC(upload(f->tc_mapA, ma));
   TRY_TC(upload(f->tc_mapX, mx));
@@ -1334,17 +1337,18 @@ qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f) {
       QBX_CUDA_TRY(cudaMemcpy(f->tc_items[s].ptr, items[s].data(), items[s].size() * sizeof(int4),
                               cudaMemcpyHostToDevice));
   }
-  return tc_tma_plan_build(h, f, groups, lv, aoff, rowsrc, xoff);
+  return tc_tma_plan_build(h, f, groups, lv, aoff, rowsrc);
 }
 
 qbx_status launch_m2l_tc(qbx_handle* h, FmmPlan* f, bool mixed, cudaStream_t s) {
   if (f->n_vbox == 0) return QBX_OK;
   if (f->n_tc_src > 0) {
-    tc_mu_kernel<<<f->n_tc_src, kThr, 0, s>>>(f->tc_src.ptr, f->box.level.ptr, f->lpb.ptr,
-                                              f->eoff.ptr, f->conv.ptr, f->pb_max, f->tc_lvl.ptr,
-                                              f->mpole.ptr, f->tc_xoff.ptr,
-                                              reinterpret_cast<__nv_bfloat16*>(f->tc_X.ptr),
-                                              f->tc_xexp.ptr);
+    const bool to_rows = f->tc_tma && !mixed;
+    tc_mu_kernel<<<f->n_tc_src, kThr, to_rows ? f->tc_mu_smem : 0, s>>>(
+        f->tc_src.ptr, f->box.level.ptr, f->lpb.ptr, f->eoff.ptr, f->conv.ptr, f->pb_max,
+        f->tc_lvl.ptr, f->mpole.ptr, f->tc_xoff.ptr,
+        reinterpret_cast<__nv_bfloat16*>(f->tc_X.ptr), f->tc_xexp.ptr,
+        to_rows ? f->tc_rowoff.ptr : nullptr, f->tc_rows.ptr, f->tc_X2.ptr);
     QBX_CUDA_TRY(cudaGetLastError());
     h->launches += 1;
   }
@@ -1374,12 +1378,7 @@ qbx_status launch_m2l_tc(qbx_handle* h, FmmPlan* f, bool mixed, cudaStream_t s) 
     TC_LAUNCH(6, 3)
     TC_LAUNCH(7, 4)
     TC_LAUNCH(8, 4)
-  } else if (f->tc_tma) {  // TMA-fed: the rows' slices in row order first
-    tc_x2_fill_kernel<<<f->n_tc_rows, 128, 0, s>>>(f->n_tc_rows, f->tc_x2src.ptr, f->tc_x2dst.ptr,
-                                                  f->tc_x2ts.ptr, f->tc_x2sk.ptr, f->tc_X.ptr,
-                                                  f->tc_X2.ptr);
-    QBX_CUDA_TRY(cudaGetLastError());
-    h->launches += 1;
+  } else if (f->tc_tma) {  // TMA-fed from the rows' slices
 #define TC_LAUNCH_TMA(S_)                                                                       \
     if (f->n_tc_items[S_ - 6] > 0) {                                                            \
       tc_gemm_tma_kernel<S_, S_><<<std::min(f->n_tc_items[S_ - 6], g_tc_sms), kTmaThr,          \

@@ -191,14 +191,15 @@ struct FmmPlan {
   std::vector<int4> h_tc_lvl;           // per level (use, beta, S, padded 2Q)
   DevBuf<int4> tc_lvl;
   DevBuf<int4> tc_gp;                   // per group (K, Q, beta, Np) of the tile product
-  // FP64 M2L through TMA: the rows' source slices copied into row order per
-  // group ([S][rows][K] at x2off), and the tensor maps of those copies and of
-  // the matrix slices, per group
+  // FP64 M2L through TMA: the rows' source slices in row order per group
+  // ([S][rows][K] at x2off), and the tensor maps of those and of the matrix slices,
+  // per group
   bool tc_tma = false;
-  int n_tc_rows = 0;
+  size_t tc_mu_smem = 0;                // a source's slices in shared memory
   DevBuf<uint16_t> tc_X2;
-  DevBuf<long long> tc_x2src, tc_x2dst, tc_x2ts, tc_gstart;
-  DevBuf<int2> tc_x2sk;
+  DevBuf<int> tc_rowoff;                // per source: its rows in tc_rows
+  DevBuf<longlong2> tc_rows;            // (offset in tc_X2, slice stride)
+  DevBuf<long long> tc_gstart;
   DevBuf<TmapBlob> tc_mapA, tc_mapX;
   bool tc_any = false;
   DevBuf<uint16_t> tc_A;                // bf16 matrix slices [S][Kp][Kp] per group
