@@ -28,6 +28,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "f32x2.cuh"
 #include "ff.cuh"
 #include "p2qbxl_pair.cuh"
 #include "tree.cuh"
@@ -1175,35 +1176,54 @@ __device__ __forceinline__ float2 f2(cd a) { return make_float2(f32_from_f64(a.x
 // float-float on Ht_m = sigma^m H_m,
 //   P_m = (2 m sigma / x) Ht_m = sigma^{m+1} K_m,  Z_m = sigma^2 Ht_{m-1},
 //   Ht_{m+1} = P_m - Z_m,  sigma^{m+1} E_m = 2 Z_m - P_m,
-// everything after it (rounded to FP32) in FP32 with Kahan sums, as before.
-// q: sigma times the charge; dn: (d k/2, nu).
+// everything after it (rounded to FP32) in FP32 with Kahan sums. Real and imaginary
+// parts are packed pairs, two operations per issue slot (about 45 slots per order of a
+// dipole instead of 72, at two warps per scheduler: 200 ellipses 2.04 -> 1.26 ms, 32
+// curves in a batch 5.10 -> 4.22 in all). S: sums, N: their lost parts (the sum is
+// S + N). q: sigma times the charge; dn: (d k/2, nu).
 template <int PM, bool HS, bool HD>
-__device__ __forceinline__ void p2qbxl_pair_mixed(float2 (&S)[2 * PM + 2], float2 (&C)[2 * PM + 2],
+__device__ __forceinline__ void p2qbxl_pair_mixed(f32p (&S)[2 * PM + 2], f32p (&N)[2 * PM + 2],
                                                   double dx, double dy, float2 q, float4 dn,
                                                   const FfUnits& U, ff c2s, float sg, float sg2,
                                                   int p) {
   FfPolar D;
   if (!D.set(dx, dy, U)) return;
-  ffh hp, hc;
-  hankel01_ff_any<3>(D.z, hp, hc);
-  hc.x = ff_scale(hc.x, sg);
-  hc.y = ff_scale(hc.y, sg);
-  const ff c2 = split17(ff_mul_raw(c2s, D.ir));  // 2 sigma / x
-  // D cos psi, D sin psi (psi = th - arg nu)
-  float2 dc = make_float2(0.f, 0.f), ds = dc;
+  ffh h0, h1;
+  hankel01_ff_any<3>(D.z, h0, h1);
+  f32p ph = pk(h0.x.h, h0.y.h), pl = pk(h0.x.l, h0.y.l);  // Ht_{m-1}
+  f32p ch = mul2(pk(h1.x.h, h1.y.h), pk(sg, sg));         // Ht_m
+  f32p cl = mul2(pk(h1.x.l, h1.y.l), pk(sg, sg));
+  const ff c2 = split17(ff_mul_raw(c2s, D.ir));  // 2 sigma / x; m c2.h is exact
+  const f32p ah = pk(c2.h, c2.h), al = pk(c2.l, c2.l), nah = pk(-c2.h, -c2.h);
+  const f32p z2 = pk(sg2, sg2), nz2 = pk(-sg2, -sg2), nz4 = pk(-2.f * sg2, -2.f * sg2);
+  // - D cos psi, D sin psi (psi = th - arg nu)
+  f32p dcx = 0, dcy = 0, dsx = 0, dsy = 0, qx = 0, qy = 0;
+  auto swap = [](f32p v) {
+    const float2 u = unpk(v);
+    return pk(u.y, u.x);
+  };
   {
-    float2 v = make_float2(0.f, 0.f);
-    if (HS) v = fmul(q, make_float2(ff_f32(hp.x), ff_f32(hp.y)));
+    f32p v = N[0];
+    if (HS) {
+      const f32p h = add2(ph, pl);
+      qx = pk(q.x, q.x);
+      qy = pk(-q.y, q.y);
+      v = fma2(qx, h, fma2(qy, swap(h), v));
+    }
     if (HD) {
       const float cpsi = fmaf(D.c, dn.z, D.s * dn.w), spsi = fmaf(D.s, dn.z, -D.c * dn.w);
-      dc = make_float2(dn.x * cpsi, dn.y * cpsi);
-      ds = make_float2(dn.x * spsi, dn.y * spsi);
-      const float2 u = fmul(dc, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
-      v = make_float2(fmaf(-2.f, u.x, v.x), fmaf(-2.f, u.y, v.y));  // E_0 = -2 H_1
+      const float cx = dn.x * cpsi, cy = dn.y * cpsi, sx = dn.x * spsi, sy = dn.y * spsi;
+      dcx = pk(-cx, -cx);
+      dcy = pk(cy, -cy);
+      dsx = pk(sx, sx);
+      dsy = pk(-sy, sy);
+      const f32p h = add2(ch, cl), two = pk(2.f, 2.f);
+      v = fma2(two, fma2(dcx, h, mul2(dcy, swap(h))), v);  // E_0 = -2 H_1
     }
-    kahan2(S[0], C[0], v);
+    kahan_add2(S[0], N[0], v);
   }
   float c = D.c, sn = D.s;  // cos m th, sin m th
+  f32p mh = ah, ml = al, nmh = nah;
 #pragma unroll
   for (int m = 1; m <= PM; ++m) {
     if (m > p) break;
@@ -1211,31 +1231,43 @@ __device__ __forceinline__ void p2qbxl_pair_mixed(float2 (&S)[2 * PM + 2], float
       const float t = fmaf(c, D.c, -sn * D.s);
       sn = fmaf(c, D.s, sn * D.c);
       c = t;
+      mh = add2(mh, ah);
+      nmh = add2(nmh, nah);
+      ml = add2(ml, al);
     }
-    const ff cm = mkff((float)m * c2.h, (float)m * c2.l);
-    const ff Px = ff_mul_raw(cm, hc.x), Py = ff_mul_raw(cm, hc.y);
-    const ff Zx = ff_scale(hp.x, sg2), Zy = ff_scale(hp.y, sg2);
+    const f32p cc = pk(c, c), ss = pk(sn, sn);
+    // P = (mh + ml) (ch + cl)
+    const f32p Ph = mul2(mh, ch);
+    const f32p Pl = fma2(ml, ch, fma2(mh, cl, fma2(mh, ch, mul2(nmh, ch))));
     // G = q Ht + D cos psi E, L = D sin psi K: A = G cos + L sin, B = G sin - L cos
-    float2 G = make_float2(0.f, 0.f), va, vb;
-    if (HS) G = fmul(q, make_float2(ff_f32(hc.x), ff_f32(hc.y)));
+    f32p va, vb;
     if (HD) {
-      const float px = ff_f32(Px), py = ff_f32(Py);
-      const float ex = fmaf(2.f, ff_f32(Zx), -px), ey = fmaf(2.f, ff_f32(Zy), -py);
-      G.x = fmaf(dc.x, ex, fmaf(-dc.y, ey, G.x));
-      G.y = fmaf(dc.x, ey, fmaf(dc.y, ex, G.y));
-      const float2 L = fmul(ds, make_float2(px, py));
-      va = make_float2(fmaf(G.x, c, L.x * sn), fmaf(G.y, c, L.y * sn));
-      vb = make_float2(fmaf(G.x, sn, -L.x * c), fmaf(G.y, sn, -L.y * c));
+      const f32p P = add2(Ph, Pl);
+      const f32p E = fma2(add2(ph, pl), nz4, P);  // -E
+      f32p G = fma2(dcx, E, mul2(dcy, swap(E)));
+      if (HS) {
+        const f32p h = add2(ch, cl);
+        G = fma2(qx, h, fma2(qy, swap(h), G));
+      }
+      const f32p L = fma2(dsx, P, mul2(dsy, swap(P)));
+      va = fma2(G, cc, fma2(L, ss, N[2 * m]));
+      vb = fma2(G, ss, fma2(L, pk(-c, -c), N[2 * m + 1]));
     } else {
-      va = make_float2(G.x * c, G.y * c);
-      vb = make_float2(G.x * sn, G.y * sn);
+      const f32p h = add2(ch, cl);
+      const f32p G = fma2(qx, h, mul2(qy, swap(h)));
+      va = fma2(G, cc, N[2 * m]);
+      vb = fma2(G, ss, N[2 * m + 1]);
     }
-    kahan2(S[2 * m], C[2 * m], va);
-    kahan2(S[2 * m + 1], C[2 * m + 1], vb);
-    const ff nx = ff_sub_raw(Px, Zx), ny = ff_sub_raw(Py, Zy);
-    hp = hc;
-    hc.x = nx;
-    hc.y = ny;
+    kahan_add2(S[2 * m], N[2 * m], va);
+    kahan_add2(S[2 * m + 1], N[2 * m + 1], vb);
+    // Ht_{m+1} = P - sigma^2 Ht_{m-1}: the two_sum of the first parts, not renormalised
+    const f32p s = fma2(ph, nz2, Ph), t = sub2(s, Ph);
+    const f32p e = sub2(sub2(Ph, sub2(s, t)), fma2(ph, z2, t));
+    const f32p l = add2(e, fma2(pl, nz2, Pl));
+    ph = ch;
+    pl = cl;
+    ch = s;
+    cl = l;
   }
 }
 
@@ -2329,9 +2361,9 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
   const float sg = pow2f(s), sg2 = pow2f(2 * s);
   const FfUnits& U = F.U;
   const ff c2s = ff_scale(U.ik2, sg);
-  float2 S[NC], C[NC];
+  f32p S[NC], N[NC];
 #pragma unroll
-  for (int j = 0; j < NC; ++j) S[j] = C[j] = make_float2(0.f, 0.f);
+  for (int j = 0; j < NC; ++j) S[j] = N[j] = 0ull;
   auto one = [&](int j) {
     const double2 y = F.sxy[j];
     float2 q = make_float2(0.f, 0.f);
@@ -2339,7 +2371,7 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
       q = F.q32[j];
       q = make_float2(q.x * sg, q.y * sg);
     }
-    p2qbxl_pair_mixed<PM, HS, HD>(S, C, y.x - c.x, y.y - c.y, q,
+    p2qbxl_pair_mixed<PM, HS, HD>(S, N, y.x - c.x, y.y - c.y, q,
                                   HD ? F.dn32[j] : make_float4(0.f, 0.f, 0.f, 0.f), U, c2s, sg,
                                   sg2, p);
   };
@@ -2347,14 +2379,15 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
                         wdoff[i + 1] - wdoff[i], wdbox};
   if (live) deal_sources<W>(sc, lane, one);
   __syncwarp();
-  // the lanes' sums (S - C) added over the group in float-float: in FP64 the
+  // the lanes' sums (S + N) added over the group in float-float: in FP64 the
   // conversions and additions of one centre were 290 FP64 instructions, as many as
   // 145 of its pairs
   ffh acc[NC];
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
-    acc[j].x = mkff(S[j].x, -C[j].x);
-    acc[j].y = mkff(S[j].y, -C[j].y);
+    const float2 s = unpk(S[j]), n = unpk(N[j]);
+    acc[j].x = mkff(s.x, n.x);
+    acc[j].y = mkff(s.y, n.y);
   }
   ffh y32, y33;
   group_reduce_scatter<W, NC>(acc, lane, y32, y33);
