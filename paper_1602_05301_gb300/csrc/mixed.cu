@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kT) mpole_to_f32_kernel(
 // M2L of V-list pairs grouped by (level, distance), in the even / odd form above.
 // Items: (first row, rows, first output order, level * kM2lDist + distance). A thread
 // computes E_l and O_l of one order l for kFoldRows rows. With P = pb + 1 <= NT orders
-// the CTA's threads are G = NT / P row groups of P orders (NT is chosen by level so
+// the CTA's threads are G = NT / P <= 16 row groups of P orders (NT is chosen by level so
 // that few threads are left over); with more, one row group, NT orders per item and
 // the source orders staged NT at a time. row.x: entry of the source in mu; row.y: 64
 // times the entry of the pair's results in Y, plus its offset class (for the angle).
@@ -322,7 +322,10 @@ __global__ void __launch_bounds__(kT) mpole_to_f32_kernel(
 // sums spill, and 200 ellipses take 2.88 ms.)
 constexpr int kFoldRows = 8;
 constexpr int kFoldWidth[3] = {128, 96, 64};  // NT
-constexpr int fold_groups(int NT, int P) { return P <= NT ? NT / P : 1; }
+constexpr int kFoldGroups = 16;
+__host__ __device__ constexpr int fold_groups(int NT, int P) {
+  return P > NT ? 1 : NT / P < kFoldGroups ? NT / P : kFoldGroups;
+}
 template <int NT>
 __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
     const int4* __restrict__ items, const int* __restrict__ lpb,
@@ -332,10 +335,11 @@ __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
   constexpr int R = kFoldRows, RS = stage_stride(R);
   static_assert(NT % kGemmBlock == 0, "staging must keep the summation blocks");
   __shared__ __align__(16) float2 xs[2 * NT * RS];  // e, then o: [row group][n][row]
+  __shared__ longlong2 meta[kFoldGroups * R];
   const int4 I = items[blockIdx.x];
   const int row0 = I.x, nr = I.y;
   const int pb = lpb[I.w / kM2lDist], P = pb + 1;
-  const int G = P <= NT ? NT / P : 1;
+  const int G = fold_groups(NT, P);
   int rg = P <= NT ? (int)threadIdx.x / P : 0;
   const int lo = P <= NT ? (int)threadIdx.x % P : I.z + (int)threadIdx.x;
   const bool act = rg < G && rg * R < nr && lo < P;
@@ -344,31 +348,52 @@ __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
   const float2* te = tm + toff[I.w];
   const float2* to = te + (size_t)P * P;
   const int used = (nr + R - 1) / R * R;  // rows staged
+  for (int i = threadIdx.x; i < nr; i += NT) meta[i] = rows[row0 + i];
   RowSums<R> E, O;
   for (int n0 = 0; n0 < P; n0 += NT) {
     const int nk = min(NT, P - n0);
     float2* xe = xs;
     float2* xo = xs + (size_t)G * nk * RS;
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nk * (used / 2); idx += NT) {
-      const int r = 2 * (idx / nk), n = idx % nk;  // coalesced reads along each source row
-      float4 e, o;
+    // two row pairs at a time: their loads are in flight together
+    const int total = nk * (used / 2);
+    for (int i0 = threadIdx.x; i0 < total; i0 += 2 * NT) {
+      float4 v[2][2];
+      float2 w[2][2];
+      int r[2], n[2];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        float2 ev = make_float2(0.f, 0.f), ov = ev;
-        if (r + u < nr) {
-          const longlong2 q = rows[row0 + r + u];
-          const float4 v = reinterpret_cast<const float4*>(mu + q.x)[n0 + n];
-          const float2 w = rot[(size_t)(q.y & 63) * (pbmax + 1) + n0 + n];
-          ev = make_float2(fmaf(w.x, v.x, -w.y * v.w), fmaf(w.x, v.y, w.y * v.z));
-          ov = make_float2(fmaf(w.x, v.z, -w.y * v.y), fmaf(w.x, v.w, w.y * v.x));
+      for (int t = 0; t < 2; ++t) {
+        const int idx = i0 + t * NT;
+        r[t] = 2 * (idx / nk);  // coalesced reads along each source row
+        n[t] = idx % nk;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          v[t][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          w[t][u] = make_float2(0.f, 0.f);
+          if (idx < total && r[t] + u < nr) {
+            const longlong2 q = meta[r[t] + u];
+            v[t][u] = reinterpret_cast<const float4*>(mu + q.x)[n0 + n[t]];
+            w[t][u] = rot[(size_t)(q.y & 63) * (pbmax + 1) + n0 + n[t]];
+          }
         }
-        if (u == 0) e.x = ev.x, e.z = ev.y, o.x = ov.x, o.z = ov.y;
-        else e.y = ev.x, e.w = ev.y, o.y = ov.x, o.w = ov.y;
       }
-      const int at = ((r / R) * nk + n) * RS + r % R;
-      *reinterpret_cast<float4*>(xe + at) = e;
-      *reinterpret_cast<float4*>(xo + at) = o;
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (i0 + t * NT >= total) break;
+        float4 e, o;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float4 x = v[t][u];
+          const float2 z = w[t][u];
+          const float2 ev = make_float2(fmaf(z.x, x.x, -z.y * x.w), fmaf(z.x, x.y, z.y * x.z));
+          const float2 ov = make_float2(fmaf(z.x, x.z, -z.y * x.y), fmaf(z.x, x.w, z.y * x.x));
+          if (u == 0) e.x = ev.x, e.z = ev.y, o.x = ov.x, o.z = ov.y;
+          else e.y = ev.x, e.w = ev.y, o.y = ov.x, o.w = ov.y;
+        }
+        const int at = ((r[t] / R) * nk + n[t]) * RS + r[t] % R;
+        *reinterpret_cast<float4*>(xe + at) = e;
+        *reinterpret_cast<float4*>(xo + at) = o;
+      }
     }
     __syncthreads();
     if (warp_act) {
@@ -381,7 +406,7 @@ __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     if (rg * R + r >= nr) break;
-    const long long q = rows[row0 + rg * R + r].y;
+    const long long q = meta[rg * R + r].y;
     const float2 w = rot[(size_t)(q & 63) * (pbmax + 1) + lo];
     float2* y = Y + (q >> 6) + pb;
     const float2 p = make_float2((E.sum_r(r) + O.sum_r(r)) + (E.lost_r(r) + O.lost_r(r)),
