@@ -981,44 +981,48 @@ __global__ void __launch_bounds__(32) l2qbxl_kernel(Fmm F, const int* __restrict
 // 2^{s m} P_m and 2^{s m} Q_m as float4 (re h, re l, im h, im l) in the same
 // places, for l2p_mixed_kernel, and 2^{s |n|} gamma_n in FP32 in loc32, for
 // l2qbxl_ff_kernel.
+// A CTA takes kBoxGroup leaves (see BoxGroup): bound by the FP64 pipe, whose warps
+// one leaf's pb + 1 orders would not fill (L2L with this of 200 ellipses 0.51 -> 0.46 ms).
 __global__ void __launch_bounds__(kThreads) unscale_leaf_locals_kernel(Fmm F,
                                                                        const int* __restrict__ leaves,
-                                                                       bool ff32) {
-  const int b = leaves[blockIdx.x];
-  const int l = F.level[b];
-  const int pb = F.lpb[l];
-  const double* ipp = ipw_row(F, l);
-  cd* lp = F.local + F.eoff[b];
-  cd* pq = F.lpq + F.eoff[b];
-  const int s = ff32 ? F.ffs[l] : kNoFf;
-  auto put = [&](int at, int m, cd v) {
-    if (s == kNoFf) {
-      pq[at] = v;
-      return;
-    }
-    const ff x = ff_from_f64_nan(v.x, 896 - s * m), y = ff_from_f64_nan(v.y, 896 - s * m);
-    reinterpret_cast<float4*>(pq)[at] = make_float4(x.h, x.l, y.h, y.l);
-  };
-  float2* g32 = F.loc32 + F.eoff[b] + pb;
-  auto put32 = [&](int n, int m, cd v) {
-    if (s != kNoFf)
-      g32[n] = make_float2(f32_from_f64_sh(v.x, s * m), f32_from_f64_sh(v.y, s * m));
-  };
-  for (int m = threadIdx.x; m <= pb; m += kThreads) {
-    const cd gp = cscale(lp[pb + m], ipp[m]);
-    lp[pb + m] = gp;
-    put32(m, m, gp);
+                                                                       int n_leaves, bool ff32) {
+  __shared__ BoxGroup g;
+  g.fill(leaves, n_leaves, F.level, F.lpb);
+  for (int idx = threadIdx.x, u = 0; idx < g.start[kBoxGroup]; idx += kThreads) {
+    while (idx >= g.start[u + 1]) ++u;
+    const int b = g.box[u], m = idx - g.start[u], pb = g.start[u + 1] - g.start[u] - 1;
+    const int l = F.level[b];
+    const double ip = ipw_row(F, l)[m];
+    cd* lp = F.local + F.eoff[b] + pb;
+    cd* pq = F.lpq + F.eoff[b];
+    float2* g32 = F.loc32 + F.eoff[b] + pb;
+    const int s = ff32 ? F.ffs[l] : kNoFf;
+    auto put = [&](int at, cd v) {
+      if (s == kNoFf) {
+        pq[at] = v;
+        return;
+      }
+      const ff x = ff_from_f64_nan(v.x, 896 - s * m), y = ff_from_f64_nan(v.y, 896 - s * m);
+      reinterpret_cast<float4*>(pq)[at] = make_float4(x.h, x.l, y.h, y.l);
+    };
+    auto put32 = [&](int n, cd v) {
+      if (s != kNoFf)
+        g32[n] = make_float2(f32_from_f64_sh(v.x, s * m), f32_from_f64_sh(v.y, s * m));
+    };
+    const cd gp = cscale(lp[m], ip);
+    lp[m] = gp;
+    put32(m, gp);
     if (m == 0) {
-      put(0, 0, gp);
+      put(0, gp);
       continue;
     }
-    const cd gn = cscale(lp[pb - m], ipp[m]);
-    lp[pb - m] = gn;
-    put32(-m, m, gn);
+    const cd gn = cscale(lp[-m], ip);
+    lp[-m] = gn;
+    put32(-m, gn);
     const cd sg = (m & 1) ? mk(-gn.x, -gn.y) : gn;
-    put(m, m, cadd(gp, sg));
+    put(m, cadd(gp, sg));
     const cd d = csub(sg, gp);
-    put(pb + m, m, mk(-d.y, d.x));
+    put(pb + m, mk(-d.y, d.x));
   }
 }
 
@@ -1879,7 +1883,8 @@ __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
 //    sig_1) against mu_m = a_m / sig_m.
 // Angular factors, products and the compensated (Kahan) sum are FP32. With the
 // recurrence in FP64 on every level the kernel ran at 87 % of the FP64 pipe (4.8 M
-// pairs of 200 ellipses: 2.11 -> 0.76 ms).
+// pairs of 200 ellipses: 2.11 -> 0.76 ms; with packed pairs and the pairs' sums joined
+// in float-float 0.62).
 __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
     Fmm F, const int* __restrict__ pt, const int* __restrict__ pbx, const int* __restrict__ slot,
     int n, const float2* __restrict__ mu, const double2* __restrict__ rec,
@@ -3258,7 +3263,8 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     }
   }
   if (f->n_leaves > 0) {
-    unscale_leaf_locals_kernel<<<f->n_leaves, kThreads, 0, s>>>(F, f->leaves.ptr, mixed);
+    unscale_leaf_locals_kernel<<<nblk(f->n_leaves, kBoxGroup), kThreads, 0, s>>>(
+        F, f->leaves.ptr, f->n_leaves, mixed);
     QBX_KCHECK("unscale_leaf_locals", s);
     h->launches += 1;
   }

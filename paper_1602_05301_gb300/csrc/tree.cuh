@@ -32,6 +32,30 @@ struct alignas(64) TmapBlob {
   unsigned char b[128];
 };
 
+// The orders 0..pb of kBoxGroup boxes side by side, for kernels whose threads run over
+// (box, order): box u's are start[u] .. start[u + 1] - 1. One per CTA, in shared memory.
+constexpr int kBoxGroup = 8;
+struct BoxGroup {
+  int box[kBoxGroup], start[kBoxGroup + 1];
+  __device__ void fill(const int* boxes, int n, const int* level, const int* lpb) {
+    if (threadIdx.x < 32) {
+      const int u = threadIdx.x, i = (int)blockIdx.x * kBoxGroup + u;
+      int w = 0;
+      if (u < kBoxGroup && i < n) {
+        box[u] = boxes[i];
+        w = lpb[level[box[u]]] + 1;
+      }
+      for (int d = 1; d < kBoxGroup; d *= 2) {
+        const int v = __shfl_up_sync(0xffffffffu, w, d);
+        if (u >= d) w += v;
+      }
+      if (u < kBoxGroup) start[u + 1] = w;
+      if (u == 0) start[0] = 0;
+    }
+    __syncthreads();
+  }
+};
+
 // No power-of-two scaling of a level fits FP32 (see float_float_scale).
 constexpr int kNoFf = -100000;
 
