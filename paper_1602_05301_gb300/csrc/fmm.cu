@@ -1873,7 +1873,7 @@ __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
 
 // M2P: a thread per (direct target, W-list box) pair, pairs ordered by (leaf,
 // box, target) so that the lanes of a warp read the same box's coefficients;
-// slot[t] is the pair's place in target order, where m2p_sum_kernel adds.
+// slot[t] is the pair's place in target order, where m2p_sum_mixed_kernel adds.
 //  * float-float levels: Ht_m = 2^{s m} H_m(k r) by the float-float recurrence
 //      Ht_{m+1} = (2 m 2^s / x) Ht_m - 4^s Ht_{m-1};
 //  * levels whose orders do not fit FP32's range that way (hundreds of orders
@@ -1888,7 +1888,7 @@ __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
 __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
     Fmm F, const int* __restrict__ pt, const int* __restrict__ pbx, const int* __restrict__ slot,
     int n, const float2* __restrict__ mu, const double2* __restrict__ rec,
-    cd* __restrict__ partial) {
+    float4* __restrict__ partial) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const int i = pt[t], c = pbx[t];
@@ -1897,35 +1897,50 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
   const int s = F.ffs[lc];
   const double2 mc = F.centre[c];
   const double dx = F.txy[i].x - mc.x, dy = F.txy[i].y - mc.y;
-  float2 S, C = make_float2(0.f, 0.f);
-  if (s != kNoFf) {
-    const float4* a = reinterpret_cast<const float4*>(mu + F.eoff[c] + c);
+  float2 S, C = make_float2(0.f, 0.f);  // the sum is S - C
+  if (s != kNoFf) {  // packed (re, im) pairs, as in p2qbxl_pair_mixed
+    const ulonglong2* a = reinterpret_cast<const ulonglong2*>(mu + F.eoff[c] + c);  // (P_m, Q_m)
     const FfUnits& U = F.U;
     FfPolar D;
     D.set(dx, dy, U);
-    ffh hp, hc;
-    hankel01_ff_any<3>(D.z, hp, hc);
+    ffh h0, h1;
+    hankel01_ff_any<3>(D.z, h0, h1);
     const float sg = pow2f(s), sg2 = pow2f(2 * s);
-    hc.x = ff_scale(hc.x, sg);
-    hc.y = ff_scale(hc.y, sg);
     const ff c2 = split17(ff_mul_raw(ff_scale(U.ik2, sg), D.ir));  // 2 2^s / x
-    S = fmul(make_float2(a[0].x, a[0].y), make_float2(ff_f32(hp.x), ff_f32(hp.y)));
-    float co = D.c, si = D.s, fm = 1.f;
+    f32p ph = pk(h0.x.h, h0.y.h), pl = pk(h0.x.l, h0.y.l);
+    f32p ch = mul2(pk(h1.x.h, h1.y.h), pk(sg, sg)), cl = mul2(pk(h1.x.l, h1.y.l), pk(sg, sg));
+    const f32p ah = pk(c2.h, c2.h), al = pk(c2.l, c2.l), nah = pk(-c2.h, -c2.h);
+    const f32p z2 = pk(sg2, sg2), nz2 = pk(-sg2, -sg2);
+    const float2 p0 = unpk(a[0].x), w0 = unpk(add2(ph, pl));
+    const float2 v0 = fmul(p0, w0);
+    f32p sum = pk(v0.x, v0.y), lost = 0ull;
+    float co = D.c, si = D.s;
+    f32p mh = ah, ml = al, nmh = nah;
     for (int m = 1; m <= pb; ++m) {
-      const float4 pq = a[m];
-      const float2 v = make_float2(fmaf(pq.x, co, pq.z * si), fmaf(pq.y, co, pq.w * si));
-      kahan2(S, C, fmul(v, make_float2(ff_f32(hc.x), ff_f32(hc.y))));
-      const ff cm = mkff(fm * c2.h, fm * c2.l);
-      fm += 1.f;
-      const ff nx = ff_sub_raw(ff_mul_raw(cm, hc.x), ff_scale(hp.x, sg2));
-      const ff ny = ff_sub_raw(ff_mul_raw(cm, hc.y), ff_scale(hp.y, sg2));
-      hp = hc;
-      hc.x = nx;
-      hc.y = ny;
-      const float u = fmaf(co, D.c, -si * D.s);
+      const ulonglong2 pq = a[m];
+      const float2 v = unpk(fma2(pq.x, pk(co, co), mul2(pq.y, pk(si, si))));
+      const f32p h = add2(ch, cl);
+      const float2 u = unpk(h);
+      kahan_add2(sum, lost, fma2(pk(v.x, v.x), h, fma2(pk(-v.y, v.y), pk(u.y, u.x), lost)));
+      const f32p Ph = mul2(mh, ch);
+      const f32p Pl = fma2(ml, ch, fma2(mh, cl, fma2(mh, ch, mul2(nmh, ch))));
+      const f32p t1 = fma2(ph, nz2, Ph), t2 = sub2(t1, Ph);
+      const f32p e = sub2(sub2(Ph, sub2(t1, t2)), fma2(ph, z2, t2));
+      const f32p l = add2(e, fma2(pl, nz2, Pl));
+      ph = ch;
+      pl = cl;
+      ch = t1;
+      cl = l;
+      mh = add2(mh, ah);
+      nmh = add2(nmh, nah);
+      ml = add2(ml, al);
+      const float t = fmaf(co, D.c, -si * D.s);
       si = fmaf(co, D.s, si * D.c);
-      co = u;
+      co = t;
     }
+    S = unpk(sum);
+    C = unpk(lost);
+    C = make_float2(-C.x, -C.y);
   } else {
     const float2* a = mu + F.eoff[c] + c + pb;  // a[m], |m| <= pb
     const double d2 = dx * dx + dy * dy;
@@ -1954,7 +1969,23 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
       }
     }
   }
-  partial[slot[t]] = mk((double)S.x - (double)C.x, (double)S.y - (double)C.y);
+  partial[slot[t]] = make_float4(S.x, -C.x, S.y, -C.y);
+}
+
+// out[target] += sum of its pairs' float-float terms, in pair order.
+__global__ void m2p_sum_mixed_kernel(int n, const int* __restrict__ wtgt, const int* __restrict__ off,
+                                     const float4* __restrict__ partial, const int* __restrict__ tid,
+                                     cd* __restrict__ out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  ff x = mkff(0.f, 0.f), y = x;
+  for (int e = off[t]; e < off[t + 1]; ++e) {
+    const float4 v = partial[e];
+    x = ff_add(x, mkff(v.x, v.y));
+    y = ff_add(y, mkff(v.z, v.w));
+  }
+  cd* dst = out + tid[wtgt[t]];
+  *dst = cadd(*dst, mk(ff_f64(x), ff_f64(y)));
 }
 
 // ---------------------------------------------------------------- P2M in mixed precision
@@ -3217,8 +3248,11 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
       QBX_KCHECK("m2p_mu", s2);
       m2p_pair_mixed_kernel<<<nblk(f->n_m2p_pairs, kThreads), kThreads, 0, s2>>>(
           F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->m2p_slot.ptr, f->n_m2p_pairs, f->m2p_mu.ptr,
-          f->m2p_rec.ptr, f->m2p_part.ptr);
-      h->launches += 1;
+          f->m2p_rec.ptr, reinterpret_cast<float4*>(f->m2p_part.ptr));
+      QBX_KCHECK("m2p", s2);
+      m2p_sum_mixed_kernel<<<nblk(f->n_wtgt, kThreads), kThreads, 0, s2>>>(
+          f->n_wtgt, f->wtgt.ptr, f->m2p_off.ptr, reinterpret_cast<float4*>(f->m2p_part.ptr),
+          f->perm[PT_TGT].ptr, out);
     } else {
       mpole_pq_kernel<<<f->n_m2p_wbox, kThreads, 0, s2>>>(F, f->m2p_wbox.ptr, f->m2p_big.ptr,
                                                          f->m2p_pq.ptr);
@@ -3226,13 +3260,12 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
       m2p_pair_kernel<<<nblk(f->n_m2p_pairs, kThreads), kThreads, 0, s2>>>(
           F, f->m2p_tgt.ptr, f->m2p_box.ptr, f->m2p_slot.ptr, f->n_m2p_pairs, f->m2p_big.ptr,
           f->m2p_pq.ptr, f->m2p_part.ptr);
-      h->launches += 1;
+      QBX_KCHECK("m2p", s2);
+      m2p_sum_kernel<<<nblk(f->n_wtgt, kThreads), kThreads, 0, s2>>>(
+          f->n_wtgt, f->wtgt.ptr, f->m2p_off.ptr, f->m2p_part.ptr, f->perm[PT_TGT].ptr, out);
     }
-    QBX_KCHECK("m2p", s2);
-    m2p_sum_kernel<<<nblk(f->n_wtgt, kThreads), kThreads, 0, s2>>>(
-        f->n_wtgt, f->wtgt.ptr, f->m2p_off.ptr, f->m2p_part.ptr, f->perm[PT_TGT].ptr, out);
     QBX_KCHECK("m2p_sum", s2);
-    h->launches += 2;
+    h->launches += 3;
   }
   stage_end(h, QBX_STAGE_M2P, s2);
   TRY(signal(f->ev_out, s2));
