@@ -312,22 +312,24 @@ __global__ void __launch_bounds__(kT) mpole_to_f32_kernel(
 
 // M2L of V-list pairs grouped by (level, distance), in the even / odd form above.
 // Items: (first row, rows, first output order, level * kM2lDist + distance). A thread
-// computes E_l and O_l of one order l for kFoldRows rows. With P = pb + 1 <= NT orders
-// the CTA's threads are G = NT / P <= 16 row groups of P orders (NT is chosen by level so
-// that few threads are left over); with more, one row group, NT orders per item and
-// the source orders staged NT at a time. row.x: entry of the source in mu; row.y: 64
+// computes E_l or O_l of one order l for kFoldRows rows. With P = pb + 1 <= NT / 2
+// orders the CTA's threads are P for each half of G <= 16 row groups (NT is chosen by
+// level so that few threads are left over); with more, one row group, NT / 2 orders per
+// item and the source orders staged NT / 2 at a time. The two threads of an order then
+// exchange sums and finish half of the rows each. row.x: entry of the source in mu; row.y: 64
 // times the entry of the pair's results in Y, plus its offset class (for the angle).
 // m2l_f32_reduce_kernel adds each target box's rows in its V-list order with Kahan
 // compensation (deterministic).
-// Bound by FP32 issue. M2L of 200 ellipses 3.23 -> 2.45 ms against one matrix per
-// offset class, 16 rows per thread; starfish at k = 10 0.18 -> 0.15, at k = 50 0.45 ->
-// 0.37 ms. (Three blocks of 128 threads per SM: at four, 128 registers, the two sets of
-// sums spill, and 200 ellipses take 2.88 ms.)
-constexpr int kFoldRows = 8;
+// Bound by the matrix loads and the latencies of 12 warps per SM (FMA pipe about half
+// busy): every entry is loaded once per kFoldRows rows. M2L of 200 ellipses 3.23 -> 2.21
+// ms against one matrix per offset class; starfish at k = 10 0.18 -> 0.13, at k = 50 0.45
+// -> 0.32 ms. With E_l and O_l in one thread and 8 rows 2.36 ms, with two orders and 8
+// rows per thread (half the shared-memory reads) 2.37, with 4 rows and 20 warps 2.74.
+constexpr int kFoldRows = 16;
 constexpr int kFoldWidth[3] = {128, 96, 64};  // NT
 constexpr int kFoldGroups = 16;
 __host__ __device__ constexpr int fold_groups(int NT, int P) {
-  return P > NT ? 1 : NT / P < kFoldGroups ? NT / P : kFoldGroups;
+  return 2 * P > NT ? 1 : NT / (2 * P) < kFoldGroups ? NT / (2 * P) : kFoldGroups;
 }
 template <int NT>
 __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
@@ -336,25 +338,28 @@ __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
     const float2* __restrict__ rot, const float2* __restrict__ mu, const float2* __restrict__ tm,
     float2* __restrict__ Y) {
   constexpr int R = kFoldRows, RS = stage_stride(R);
-  static_assert(NT % kGemmBlock == 0, "staging must keep the summation blocks");
-  __shared__ __align__(16) float2 xs[2 * NT * RS];  // e, then o: [row group][n][row]
+  constexpr int NH = NT / 2;
+  static_assert(NH % kGemmBlock == 0, "staging must keep the summation blocks");
+  __shared__ __align__(16) float2 xs[NT * RS];  // e, then o: [row group][n][row]
   __shared__ longlong2 meta[kFoldGroups * R];
   const int4 I = items[blockIdx.x];
   const int row0 = I.x, nr = I.y;
   const int pb = lpb[I.w / kM2lDist], P = pb + 1;
-  const int G = fold_groups(NT, P);
-  int rg = P <= NT ? (int)threadIdx.x / P : 0;
-  const int lo = P <= NT ? (int)threadIdx.x % P : I.z + (int)threadIdx.x;
-  const bool act = rg < G && rg * R < nr && lo < P;
-  if (!act) rg = 0;
+  const int G = fold_groups(NT, P), W = P <= NH ? P : NH;
+  const int id = min((int)threadIdx.x, 2 * G * W - 1);  // threads left over repeat the last
+  const int unit = id % (G * W);
+  const bool odd = id >= G * W;  // the thread sums O
+  const int l = I.z + unit % W, lo = l < P ? l : 0;
+  int rg = unit / W;
+  const bool act = (int)threadIdx.x < 2 * G * W && rg * R < nr && l < P;
+  if (rg * R >= nr) rg = 0;
   const bool warp_act = __any_sync(0xffffffffu, act);
-  const float2* te = tm + toff[I.w];
-  const float2* to = te + (size_t)P * P;
+  const float2* te = tm + toff[I.w] + (odd ? (size_t)P * P : 0);
   const int used = (nr + R - 1) / R * R;  // rows staged
   for (int i = threadIdx.x; i < nr; i += NT) meta[i] = rows[row0 + i];
-  RowSums<R> E, O;
-  for (int n0 = 0; n0 < P; n0 += NT) {
-    const int nk = min(NT, P - n0);
+  RowSums<R> S;
+  for (int n0 = 0; n0 < P; n0 += NH) {
+    const int nk = min(NH, P - n0);
     float2* xe = xs;
     float2* xo = xs + (size_t)G * nk * RS;
     __syncthreads();
@@ -399,26 +404,41 @@ __global__ void __launch_bounds__(NT, 384 / NT) m2l_fold_kernel(
       }
     }
     __syncthreads();
-    if (warp_act) {
-      const size_t m0 = (size_t)n0 * P;
-      tile_gemm_column<R>(te + m0, P, nk, xe + (size_t)rg * nk * RS, lo, act, E);
-      tile_gemm_column<R>(to + m0, P, nk, xo + (size_t)rg * nk * RS, lo, act, O);
-    }
+    if (warp_act)
+      tile_gemm_column<R>(te + (size_t)n0 * P, P, nk, (odd ? xo : xe) + (size_t)rg * nk * RS, lo,
+                          true, S);
   }
+  // E gives its sums of the upper half of the rows for O's of the lower half
+  constexpr int RH = R / 2;
+  __syncthreads();
+  float4* ex = reinterpret_cast<float4*>(xs);  // [row][thread]
+  static_assert(sizeof(xs) >= sizeof(float4) * NT * RH, "room for the exchange");
+  auto sums = [&](int r) {
+    return make_float4(S.sum_r(r), S.sum_i(r), S.lost_r(r), S.lost_i(r));
+  };
+#pragma unroll
+  for (int r = 0; r < RH; ++r) {
+    const float4 a = sums(r), b = sums(r + RH);
+    ex[r * NT + threadIdx.x] = odd ? a : b;
+  }
+  __syncthreads();
+  const int mate = odd ? (int)threadIdx.x - G * W : (int)threadIdx.x + G * W;
   if (!act) return;
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    if (rg * R + r >= nr) break;
-    const long long q = meta[rg * R + r].y;
-    const float2 w = rot[(size_t)(q & 63) * (pbmax + 1) + lo];
+  for (int r = 0; r < RH; ++r) {
+    const int row = rg * R + r + (odd ? RH : 0);
+    if (row >= nr) break;
+    const long long q = meta[row].y;
+    const float2 w = rot[(size_t)(q & 63) * (pbmax + 1) + l];
     float2* y = Y + (q >> 6) + pb;
-    const float2 p = make_float2((E.sum_r(r) + O.sum_r(r)) + (E.lost_r(r) + O.lost_r(r)),
-                                 (E.sum_i(r) + O.sum_i(r)) + (E.lost_i(r) + O.lost_i(r)));
-    const float2 m = make_float2((E.sum_r(r) - O.sum_r(r)) + (E.lost_r(r) - O.lost_r(r)),
-                                 (E.sum_i(r) - O.sum_i(r)) + (E.lost_i(r) - O.lost_i(r)));
+    const float4 a0 = sums(r), a1 = sums(r + RH);
+    const float4 a = odd ? a1 : a0, o = ex[r * NT + mate];
+    const float2 p = make_float2((a.x + o.x) + (a.z + o.z), (a.y + o.y) + (a.w + o.w));
+    float2 m = make_float2((a.x - o.x) + (a.z - o.z), (a.y - o.y) + (a.w - o.w));  // E - O
+    if (odd) m = make_float2(-m.x, -m.y);
     const float2 yp = make_float2(fmaf(w.x, p.x, -w.y * p.y), fmaf(w.x, p.y, w.y * p.x));
-    y[lo] = (lo & 1) ? make_float2(-yp.x, -yp.y) : yp;
-    if (lo > 0) y[-lo] = make_float2(fmaf(w.x, m.x, w.y * m.y), fmaf(w.x, m.y, -w.y * m.x));
+    y[l] = (l & 1) ? make_float2(-yp.x, -yp.y) : yp;
+    if (l > 0) y[-l] = make_float2(fmaf(w.x, m.x, w.y * m.y), fmaf(w.x, m.y, -w.y * m.x));
   }
 }
 
@@ -1045,7 +1065,8 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
       int u = 0, best = -1;  // the width that leaves the fewest threads without an order
       for (int v = 2; v >= 0; --v) {
         const int nt = kFoldWidth[v];
-        const int full = P <= nt ? 1000 * (nt / P * P) / nt : 1000 * P / (nblk(P, nt) * nt);
+        const int full = 2 * P <= nt ? 2000 * fold_groups(nt, P) * P / nt
+                                     : 1000 * P / (nblk(P, nt / 2) * (nt / 2));
         if (full > best) best = full, u = v;
       }
       const int nt = kFoldWidth[u], most = kFoldRows * fold_groups(nt, P);
@@ -1059,7 +1080,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
         }
         const int64_t r1 = (int64_t)frow.size();
         for (int64_t r = r0; r < r1; r += most)
-          for (int c0 = 0; c0 < P; c0 += P <= nt ? P : nt)
+          for (int c0 = 0; c0 < P; c0 += 2 * P <= nt ? P : nt / 2)
             by_width[u].push_back(
                 make_int4((int)r, (int)std::min<int64_t>(most, r1 - r), c0, l * kM2lDist + d));
       }
