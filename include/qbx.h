@@ -22,7 +22,9 @@
  *    the CUDA runtime which it is. Device pointers must live on the current
  *    device. Host outputs are written before the call returns.
  *  - The caller owns every buffer it passes; the library copies what it keeps
- *    and never frees caller memory. The handle owns all memory it allocates.
+ *    and never frees caller memory. The handle owns all memory it allocates;
+ *    when it is destroyed the library may keep up to 256 MiB of it per device
+ *    for later handles.
  *  - No C++ exception crosses this boundary. Every call returns a status; on a
  *    non-OK status qbx_last_error() holds a message (thread-local).
  *  - One handle must not be used from two threads at once; distinct handles
@@ -135,8 +137,9 @@ qbx_status qbx_geometry_create(const qbx_geometry_desc *desc, qbx_handle **out);
  * (-1: direct quadrature).
  * m2l_engine: the M2L translations of FMM mode (Sec. 7.2, Stage 4): 0 the
  * default (FP64 on tensor cores for levels whose bf16 split is exact, mixed
- * precision on the FP32 CUDA-core GEMM), 1 tensor cores in both precisions,
- * 2 CUDA cores in both; every engine meets the precision's tolerance.
+ * precision in FP32 on the CUDA cores), 1 tensor cores in both precisions,
+ * 2 CUDA cores in both; every engine meets the precision's tolerance. M2M and
+ * L2L run on the CUDA cores with every engine.
  * Errors: QBX_ERR_ASSOCIATION (count and first target in qbx_last_error()),
  * QBX_ERR_ARG, QBX_ERR_OOM, QBX_ERR_CUDA. Synchronous.
  */
@@ -162,9 +165,10 @@ qbx_status qbx_tree_build(qbx_handle *h, const qbx_tree_desc *desc);
  * step 3). sigma_S / sigma_D: complex [n_src] on the source grid; either may be
  * NULL (that layer is absent). out: complex [n_targets]. alpha_out (optional):
  * complex [n_centres][2p+1], l = -p..p, the QBX coefficients of every centre.
- * Without alpha_out, FMM mode forms the coefficients only at the centres that
+ * Without alpha_out, the coefficients are formed only at the centres that
  * some target is associated with (the only ones the evaluation reads); with
- * it, at every centre. The potential at the targets is the same either way.
+ * it, at every centre. The potential at the targets is the same either way (in
+ * direct mode up to rounding).
  * precision: QBX_FP64 or QBX_MIXED. cuda_stream: a cudaStream_t (NULL: the
  * legacy default stream). With device buffers the call is asynchronous on the
  * stream; with any host buffer it copies through the stream and returns after

@@ -2544,8 +2544,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
   QBX_CUDA_TRY(cudaStreamCreateWithFlags(&f->near_stream, cudaStreamNonBlocking));
   for (cudaEvent_t* ev : {&f->ev_fork, &f->ev_join, &f->ev_p2l, &f->ev_m2m, &f->ev_out})
     QBX_CUDA_TRY(cudaEventCreateWithFlags(ev, cudaEventDisableTiming));
-  // the largest per-block footprint (the M2M / L2L GEMMs at the largest
-  // order) bounds all others
+  // the limit on box orders: no kernel stages more than this for its largest one
   const size_t smem_need = gemm_smem_bytes(f->pb_max);
   if (smem_need > (size_t)g_smem_optin) {
     set_error("box order %d needs %zu bytes of shared memory per block (device: %d)", f->pb_max,

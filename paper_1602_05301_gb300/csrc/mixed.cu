@@ -12,9 +12,9 @@
 // (sig' of the child level) and M2M entry (sig_n / sig'_s) conj(V_{s-n}(d))
 // (sig' of the parent level): the scale ratios are binomial-sized while
 // J_{s-n}(k d) decays factorially. The entries are computed in FP64 (through logarithms
-// of the scale factors) and stored as FP32 matrices, one per (level, offset
-// class) for M2L and per (level, quadrant) for L2L; the coefficient
-// conversions between the two normalisations are FP64.
+// of the scale factors), with the angles of the offsets taken out, and stored as FP32
+// matrices, two per (level, distance) for M2L and one per level for M2M and for L2L; the
+// coefficient conversions between the two normalisations are FP64.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -170,6 +170,10 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
 // Kahan compensation.
 constexpr int kGemmRows = 16;
 constexpr int kGemmBlock = 8;
+// Complex products of M2L between Kahan steps: with eight the rotated form's error
+// against FP64 (18 cases, geometric mean) is 1.71e-7, with four 1.62e-7 (1.75e-7 with
+// one matrix per offset class), at 2.32 ms instead of 2.21 on 200 ellipses.
+constexpr int kKahanBlock = 4;
 // Staged rows: order n of the row pair (r, r + 1), r even, is the float4 (re r,
 // re r+1, im r, im r+1) at x + n * stage_stride(R) + r, so that each half is an
 // operand of the packed FMAs. Two float2 of padding per n keep the row pairs
@@ -199,9 +203,9 @@ struct RowSums {
   }
 };
 
-// One block of nj (1 <= nj <= kGemmBlock) terms of a tile product column,
-// sum_{j < nj} tb[j] * x[j], started from the lost part of S and added to S (Kahan
-// compensation in three operations per block).
+// nj (1 <= nj <= kGemmBlock) terms of a tile product column, S += sum_{j < nj}
+// tb[j] * x[j]: every kKahanBlock of them summed from the lost part of S and added to S
+// (Kahan compensation in three operations).
 template <int R>
 __device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], int nj,
                                                const float2* __restrict__ x, RowSums<R>& S) {
@@ -217,7 +221,11 @@ __device__ __forceinline__ void gemm_block_add(const float2 (&tb)[kGemmBlock], i
 #pragma unroll
       for (int r = 0; r < R / 2; ++r) {
         const ulonglong2 v = m[r];  // (re, re), (im, im) of rows 2r, 2r + 1
-        if (j == 0) {
+        if (j > 0 && j % kKahanBlock == 0) {
+          kahan_add2(S.sr[r], S.nr[r], tr[r]);
+          kahan_add2(S.si[r], S.ni[r], ti[r]);
+        }
+        if (j % kKahanBlock == 0) {
           tr[r] = fma2(tx, v.x, fma2(my, v.y, S.nr[r]));
           ti[r] = fma2(tx, v.y, fma2(ty, v.x, S.ni[r]));
         } else {
@@ -323,7 +331,7 @@ __global__ void __launch_bounds__(kT) mpole_to_f32_kernel(
 // Bound by the matrix loads and the latencies of 12 warps per SM (FMA pipe about half
 // busy): every entry is loaded once per kFoldRows rows. M2L of 200 ellipses 3.23 -> 2.21
 // ms against one matrix per offset class; starfish at k = 10 0.18 -> 0.13, at k = 50 0.45
-// -> 0.32 ms. With E_l and O_l in one thread and 8 rows 2.36 ms, with two orders and 8
+// -> 0.32 ms (kKahanBlock = 8). With E_l and O_l in one thread and 8 rows 2.36 ms, with two orders and 8
 // rows per thread (half the shared-memory reads) 2.37, with 4 rows and 20 warps 2.74.
 constexpr int kFoldRows = 16;
 constexpr int kFoldWidth[3] = {128, 96, 64};  // NT
@@ -507,8 +515,8 @@ __global__ void m2l_f64_matrix_kernel(int l, int pb, int pbmax, const cd* __rest
 }
 
 // FP64 work items take kF64Rows rows of a tile (the accumulators of 16 FP64
-// rows would not fit in registers), kT output orders and the same staging as
-// the FP32 items. Results go to the FP64 rows of Y64, added per target box by
+// rows would not fit in registers) and kT output orders, the sources staged kChunkK
+// orders at a time. Results go to the FP64 rows of Y64, added per target box by
 // m2l_f64_reduce_kernel in V-list order.
 constexpr int kChunkK = 128;  // source orders staged at a time
 constexpr int kF64Rows = 8;

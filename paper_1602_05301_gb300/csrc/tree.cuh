@@ -250,7 +250,7 @@ qbx_status launch_m2l_f64_gemm_rest(qbx_handle* h, FmmPlan* f, cudaStream_t s);
 qbx_status configure_tc_kernels(int smem_optin);
 qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f);
 qbx_status launch_m2l_tc(qbx_handle* h, FmmPlan* f, bool mixed, cudaStream_t s);
-// shared memory of one M2M / L2L tile-GEMM block at box order pb
+// an upper bound of the shared memory that a translation block needs at box order pb
 size_t gemm_smem_bytes(int pb);
 
 qbx_status tree_build(qbx_handle* h, FmmPlan* f, int n_max, double kappa);
