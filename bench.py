@@ -268,20 +268,28 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# FP64 flops of the base Hankel values H0, H1 of one pair: four polynomials
-# of the library's tables by Horner's rule, degree 10 on the FP64 path and 8 on
+# Flops of the base Hankel values H0, H1 of one pair: four polynomials
+# of the library's tables by Horner's rule, degree 10 on the FP64 path and 9 on
 # the mixed one (the logarithm below x = 2 is not charged), and of one step of
 # the upward Hankel recurrence (a real-scaled complex step, 6 flops).
-HANKEL01_FLOPS = {False: 4 * 10 * 2, True: 4 * 8 * 2}
+HANKEL01_FLOPS = {False: 4 * 10 * 2, True: 4 * 9 * 2}
 REC_STEP_FLOPS = 6
+
+
+def as_run(f, mixed):
+    """The classes' (FP64, FP32) flops with float-float work counted as FP32."""
+    return {k: (0.0, v[0] + v[1]) if mixed and k != "qbxl2p" else v for k, v in f.items()}
 
 
 def flop_model(lp, stats, p, has_S, has_D, assoc, fmm, mixed=False, active_frac=1.0):
     """Algorithmic flops per kernel class as (FP64, FP32) pairs: complex
     multiply-add = 8 flops; special-function values as stated above. P = 2p+1
     QBX terms; a box on tree level l carries Q_l = 2 pb_l + 1 terms (per-level
-    orders), and every translation is charged with the orders of its boxes. In
-    mixed precision M2M, M2L, L2L and the P2QBXL accumulation are FP32.
+    orders), and every translation is charged with the orders of its boxes and
+    the products that are left once its symmetries are used (M2M and L2L: a real
+    matrix for the four children; FP32 M2L: even and odd halves). In mixed
+    precision all but QBXL2P is FP32: values and recurrences are float-float,
+    whose splitting is charged nothing.
     active_frac scales the centre stages to the centres whose coefficients are
     formed (those some target uses)."""
     P = 2 * p + 1
@@ -292,10 +300,10 @@ def flop_model(lp, stats, p, has_S, has_D, assoc, fmm, mixed=False, active_frac=
     f = {}
     f["p2qbxl"] = (base, pairs * acc) if mixed else (base + pairs * acc, 0.0)
     # P2P evaluates only the Hankel functions its layers read (H0 for S, H1 for D)
-    f["p2p"] = (stats["p2p_pairs"] * (HANKEL01_FLOPS[False] * lay / 2 + 8 * lay), 0.0)
+    f["p2p"] = (stats["p2p_pairs"] * (HANKEL01_FLOPS[mixed] * lay / 2 + 8 * lay), 0.0)
     f["qbxl2p"] = (stats["n_qbx_targets"] * 16 * P, 0.0)
     if not fmm:
-        return f
+        return as_run(f, mixed)
     t = lp.export_tree()
     pbl = lp.box_orders().astype(np.int64)
     lev = t["level"].astype(np.int64)
@@ -318,14 +326,14 @@ def flop_model(lp, stats, p, has_S, has_D, assoc, fmm, mixed=False, active_frac=
         return own, t["idx"][base[i]:base[i] + cnt.sum()].astype(np.int64)
     vb, _ = entries(1)
     tr = lambda v: (0.0, float(v)) if mixed else (float(v), 0.0)  # FP32 translations in mixed
-    f["m2l"] = tr(8 * np.sum(Qb[vb] ** 2))
+    f["m2l"] = tr((4 if mixed else 8) * np.sum(Qb[vb] ** 2))
     parent = np.full(nb, -1, np.int64)
     for q in range(4):
         has = child[:, q] >= 0
         parent[child[has, q]] = np.nonzero(has)[0]
     mm = (lev >= 3) & (parent >= 0)
-    f["m2m"] = f["l2l"] = tr(8 * np.sum(Qb[mm] * Qb[parent[mm]]))
-    # P2M: one FP64 Miller row per source (about pb + 8 orders, 6 flops each);
+    f["m2m"] = f["l2l"] = tr(np.sum(Qb[mm] * Qb[parent[mm]]))
+    # P2M: one Miller row per source (about pb + 8 orders, 6 flops each);
     # the sums over the sources, 8 flops per layer and coefficient, are FP64 on
     # the FP64 path and FP32 (with 8 more for the compensation) in mixed precision
     srcQ = np.sum((nsrc * Qb)[leaf & (lev >= 2)])
@@ -341,15 +349,15 @@ def flop_model(lp, stats, p, has_S, has_D, assoc, fmm, mixed=False, active_frac=
     w_q = float(np.sum((nctr * wq)[leaf]))
     mq = stats["m2qbxl_pairs"] * active_frac * (w_q / w_all if w_all else 0.0)
     lq = np.sum((nctr * Qb)[leaf]) * active_frac
-    # M2P: per (direct target, W box) pair the Hankel recurrence (6 FP64 flops
+    # M2P: per (direct target, W box) pair the Hankel recurrence (6 flops
     # per order, about Q/2 orders) and a complex product-sum per coefficient,
     # FP64 on the FP64 path, FP32 with compensation (16 flops) in mixed
     nw = np.bincount(wb, minlength=nb).astype(np.int64)
     w_pairs = float(np.sum((ndir * nw)[leaf]))
     w_coef = float(np.sum((ndir * wq)[leaf]))
     if mixed:
-        # M2QBXL / L2QBXL: products on split FP32 factors (about 16 flops per
-        # term with the scaling and compensation), recurrences in FP64
+        # M2QBXL / L2QBXL: FP32 products with compensation (about 16 flops per
+        # term)
         f["m2qbxl"] = (3.0 * mq, 16.0 * P * mq)
         f["m2p"] = (HANKEL01_FLOPS[True] * w_pairs + 3.0 * w_coef, 16.0 * w_coef)
         f["l2qbxl"] = (0.0, 16.0 * P * lq)
@@ -360,7 +368,7 @@ def flop_model(lp, stats, p, has_S, has_D, assoc, fmm, mixed=False, active_frac=
     # L2P: per order Miller's step (6 flops) and Clenshaw's two complex steps
     # (16 flops), for the two coefficients of orders +-m: 11 per coefficient
     f["l2p"] = (11.0 * np.sum((ndir * Qb)[leaf]), 0.0)
-    return f
+    return as_run(f, mixed)
 
 
 # ---------------------------------------------------------------- our arm
