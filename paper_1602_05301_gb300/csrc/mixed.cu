@@ -918,19 +918,24 @@ qbx_status configure_mixed_kernels(int smem_optin) {
 // (x >= 1.4 x0), its own points within 0.71 sides (y <= 0.71 x0). H_m grows like
 // (2 m / (e x))^m, so s puts the turn of (2 m 2^s / (e x))^m at 0.6 pb: it falls
 // to 2^{-0.32 pb} before and rises to 2^{0.44 pb} at pb. Refused (FP64 kernels)
-// when the largest |2^{s m} H_m| exceeds 2^60, or an order reaches 128 (the
-// recurrence's exact products m c hold 7 bits of m).
+// when the largest |2^{s m} H_m| exceeds 2^60, when 2^{s m} / sig_m (isf, larger than
+// that by pi m 1.4^m) comes within a factor four of FP32's largest value, which it does
+// from order 119 on, or an order reaches 128 (the recurrence's exact products m c hold 7
+// bits of m).
 static int float_float_scale(double x0, int pb) {
   if (pb < 1 || pb > 126) return kNoFf;
   const double xl = 1.4 * x0;
   const int s = (int)std::lrint(std::min(0.0, std::log2(xl * 1.3591409142295226 / (0.6 * pb))));
   if (s < -50) return kNoFf;
-  double top = 0.0;
-  for (int m = 1; m <= pb; ++m)  // |H_m(x)| <~ (m-1)!/pi (2/x)^m for m > x, of order one below
-    if (m > xl)
+  constexpr double kLn2 = 0.69314718055994531;
+  double top = 0.0, isf = 0.0;
+  for (int m = 1; m <= pb; ++m) {
+    if (m > xl)  // |H_m(x)| <~ (m-1)!/pi (2/x)^m for m > x, of order one below
       top = std::max(top, s * m + (std::lgamma((double)m) - 1.1447298858494002 +
-                                   m * std::log(2.0 / xl)) / 0.69314718055994531);
-  return top > 60.0 ? kNoFf : s;
+                                   m * std::log(2.0 / xl)) / kLn2);
+    isf = std::max(isf, s * m + std::max(0.0, std::lgamma(m + 1.0) - m * std::log(0.5 * x0)) / kLn2);
+  }
+  return top > 60.0 || isf > 126.0 ? kNoFf : s;
 }
 
 qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
