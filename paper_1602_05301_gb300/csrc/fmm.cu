@@ -1861,13 +1861,14 @@ __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
   }
   const double* pwl = pw_row(F, l);
   for (int m = threadIdx.x; m <= pb; m += kThreads) {
-    const double f = pwl[m] * pow2d(-s * m);
+    // s_l^m 2^{-s m}, the power of two (up to 2^1500) in two halves
+    const int sh = -s * m;
+    const double f = pwl[m] * pow2d(sh / 2), f2 = pow2d(sh - sh / 2);
     cd g = m > 0 ? a[-m] : mk(0.0, 0.0);
     if (m & 1) g = mk(-g.x, -g.y);
-    const cd P = cadd(a[m], g), d = csub(a[m], g);
+    const cd P = cscale(cscale(cadd(a[m], g), f), f2), d = cscale(cscale(csub(a[m], g), f), f2);
     reinterpret_cast<float4*>(dst)[m] =
-        make_float4((float)(P.x * f), (float)(P.y * f), m ? (float)(-d.y * f) : 0.f,
-                    m ? (float)(d.x * f) : 0.f);
+        make_float4((float)P.x, (float)P.y, m ? (float)-d.y : 0.f, m ? (float)d.x : 0.f);
   }
 }
 

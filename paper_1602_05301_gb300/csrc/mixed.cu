@@ -31,7 +31,11 @@ constexpr int kT = 128;
 inline unsigned nblk(int64_t n, int b) { return (unsigned)std::max<int64_t>(1, (n + b - 1) / b); }
 
 // per level: lsig[j] = log sig_j, conv[j] = s^j / sig_j  (j = 0..pb_l; stride
-// pbmax + 1), iconv = 1 / conv, isig[j] = 1 / sig_min(j, pb_l) (j = 0..pb_l + 1; stride pbmax + 2)
+// pbmax + 1), iconv = 1 / conv, isig[j] = 1 / sig_min(j, pb_l) (j = 0..pb_l + 1; stride
+// pbmax + 2). isig is held at e^kMaxLogIsig = 1e299: orders it would exceed that at lie
+// above 45 (the plan bounds s^pb), where a box's own points (0.71 sides away) and its
+// nearest partners (1.5 sides) leave less than (0.71 / 1.5)^45 = 2e-15 of a potential.
+constexpr double kMaxLogIsig = 690.0;
 __global__ void sigma_tables_kernel(int n_levels, int pbmax, const int* __restrict__ lpb,
                                     double k, double side, const double* __restrict__ scale,
                                     double* __restrict__ lsig, double* __restrict__ conv,
@@ -45,8 +49,9 @@ __global__ void sigma_tables_kernel(int n_levels, int pbmax, const int* __restri
     const double c = exp(j * ls - v);
     conv[(size_t)l * (pbmax + 1) + j] = c;
     iconv[(size_t)l * (pbmax + 1) + j] = 1.0 / c;
-    isig[(size_t)l * (pbmax + 2) + j] = exp(-v);
-    if (j == pb) isig[(size_t)l * (pbmax + 2) + pb + 1] = exp(-v);
+    const double i = exp(fmin(-v, kMaxLogIsig));
+    isig[(size_t)l * (pbmax + 2) + j] = i;
+    if (j == pb) isig[(size_t)l * (pbmax + 2) + pb + 1] = i;
   }
 }
 
@@ -138,9 +143,11 @@ __global__ void m2l_rot_kernel(int pbmax, float2* __restrict__ rot) {
   }
 }
 
-// isf[l][j] = 2^{s j} isig[l][j] as a pair of FP32, s = ffs[l] (0 on levels without)
+// isf[l][j] = 2^{s j} / sig_min(j, pb) as a pair of FP32, s = ffs[l] (0 on levels
+// without), from the logarithm: it fits FP32 (float_float_scale) where 1 / sig_j is
+// beyond FP64
 __global__ void isig_ff_kernel(int n_levels, int pbmax, const int* __restrict__ lpb,
-                               const int* __restrict__ ffs, const double* __restrict__ isig,
+                               const int* __restrict__ ffs, const double* __restrict__ lsig,
                                float2* __restrict__ isf) {
   const int l = blockIdx.x;
   if (l >= n_levels) return;
@@ -148,7 +155,8 @@ __global__ void isig_ff_kernel(int n_levels, int pbmax, const int* __restrict__ 
   for (int j = threadIdx.x; j < pbmax + 2; j += blockDim.x) {
     float2 v = make_float2(0.f, 0.f);
     if (s != kNoFf && j <= lpb[l] + 1) {
-      const double x = ldexp(isig[(size_t)l * (pbmax + 2) + j], s * j);
+      const double x = exp(fma((double)(s * j), 0.69314718055994530942,
+                               -lsig[(size_t)l * (pbmax + 1) + min(j, lpb[l])]));
       v.x = (float)x;
       v.y = (float)(x - (double)v.x);
     }
@@ -973,7 +981,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
     QBX_CUDA_TRY(cudaMemcpy(f->ff_s.ptr, ffs.data(), f->n_levels * sizeof(int),
                             cudaMemcpyHostToDevice));
     QBX_CUDA_TRY(f->isf.alloc((size_t)f->n_levels * (pbm + 2)));
-    isig_ff_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->ff_s.ptr, f->isig.ptr,
+    isig_ff_kernel<<<f->n_levels, 128>>>(f->n_levels, pbm, f->lpb.ptr, f->ff_s.ptr, f->lsig.ptr,
                                          f->isf.ptr);
     QBX_CUDA_TRY(cudaGetLastError());
   }

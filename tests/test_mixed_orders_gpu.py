@@ -63,3 +63,10 @@ def _check(qbxmod, order, x):
     (126, 5.856), (125, 5.7848), (124, 5.7144), (123, 5.6456), (122, 5.6)])
 def test_scaled_powers_beyond_fp32(qbxmod, order, x):
     _check(qbxmod, order, x)
+
+
+# 1 / sig_j beyond FP64
+@pytest.mark.parametrize("order,x", [
+    (54, 2.0 ** -13.7), (54, 2.0 ** -14), (64, 2.0 ** -10.5)])
+def test_inverse_sigma_beyond_fp64(qbxmod, order, x):
+    _check(qbxmod, order, x)
