@@ -21,10 +21,14 @@ struct M2lNorm {
     used = max(abs(dx), abs(dy)) >= 2;
   }
   // the factor is at most 1 / |What|, so it may underflow where the product does
-  // not: its square root is applied twice
+  // not: its square root is applied twice. Orders |n + lo| > 170 of boxes below a
+  // wavelength leave FP64's range in What; such an entry multiplies and makes
+  // coefficients below 0.71^|n| and 0.71^|lo| (a box's own points are that near), less
+  // than 1e-25 of a potential: zero
   __device__ cd entry(int n, int lo) const {
     if (!used) return mk(0.0, 0.0);
     const cd v = w[n + lo];
+    if (!isfinite(v.x) || !isfinite(v.y)) return mk(0.0, 0.0);
     const double lf = sg[abs(lo)] + sg[abs(n)] - abs(n + lo) * ls;
     double f = lf < -1400.0 ? 0.0 : exp(0.5 * lf);
     const double g = (lo & 1) ? -f : f;

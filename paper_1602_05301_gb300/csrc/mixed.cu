@@ -515,6 +515,7 @@ __global__ void m2l_f64_matrix_kernel(int l, int pb, int pbmax, const cd* __rest
     cd v = mk(0.0, 0.0);
     if (used) {
       v = w[n + lo];
+      if (!isfinite(v.x) || !isfinite(v.y)) v = mk(0.0, 0.0);  // as in M2lNorm::entry
       if ((n < 0 && lo > 0) || (n > 0 && lo < 0)) v = cscale(v, p2[2 * min(abs(n), abs(lo))]);
       if (lo & 1) v = mk(-v.x, -v.y);
     }

@@ -70,3 +70,25 @@ def test_scaled_powers_beyond_fp32(qbxmod, order, x):
     (54, 2.0 ** -13.7), (54, 2.0 ** -14), (64, 2.0 ** -10.5)])
 def test_inverse_sigma_beyond_fp64(qbxmod, order, x):
     _check(qbxmod, order, x)
+
+
+# H_m of the M2L, m <= 2 order, beyond FP64, with and without the above
+@pytest.mark.parametrize("order,x", [
+    (126, 0.732), (123, 0.7057), (120, 0.24), (130, 0.5)])
+def test_m2l_hankel_beyond_fp64(qbxmod, order, x):
+    _check(qbxmod, order, x)
+
+
+# the same in FP64 on the CUDA cores (m2l_engine 2)
+def test_m2l_hankel_beyond_fp64_cuda_cores(qbxmod):
+    g = discretise_curve(*fourier_radial(np.array([0.2]), np.array([0.3]), 1.0), 160, 8, k=4.0)
+    sig = np.exp(1j * np.arange(g.n))
+    u = []
+    for engine in (0, 2):
+        lp = qbxmod.LayerPotential(g.as_dict(), 6, sides=2)
+        lp.build(grid_targets(40, -3.0, 3.0), mode=qbxmod.QBX_FMM, p_fmm=126, p_add=0, n_max=12,
+                 m2l_engine=engine)
+        u.append(lp.eval(sigma_S=sig, cS=1.0))
+        lp.close()
+    assert np.isfinite(u[1]).all()
+    assert np.linalg.norm(u[1] - u[0]) < 1e-10 * np.linalg.norm(u[0])
