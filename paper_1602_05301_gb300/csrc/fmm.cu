@@ -1861,14 +1861,15 @@ __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
   }
   const double* pwl = pw_row(F, l);
   for (int m = threadIdx.x; m <= pb; m += kThreads) {
-    // s_l^m 2^{-s m}, the power of two (up to 2^1500) in two halves
+    // the power of two, up to 2^1500, as an exponent offset
     const int sh = -s * m;
-    const double f = pwl[m] * pow2d(sh / 2), f2 = pow2d(sh - sh / 2);
+    const double f = pwl[m];
     cd g = m > 0 ? a[-m] : mk(0.0, 0.0);
     if (m & 1) g = mk(-g.x, -g.y);
-    const cd P = cscale(cscale(cadd(a[m], g), f), f2), d = cscale(cscale(csub(a[m], g), f), f2);
+    const cd P = cscale(cadd(a[m], g), f), d = cscale(csub(a[m], g), f);
     reinterpret_cast<float4*>(dst)[m] =
-        make_float4((float)P.x, (float)P.y, m ? (float)-d.y : 0.f, m ? (float)d.x : 0.f);
+        make_float4(f32_from_f64_sh(P.x, sh), f32_from_f64_sh(P.y, sh),
+                    m ? f32_from_f64_sh(-d.y, sh) : 0.f, m ? f32_from_f64_sh(d.x, sh) : 0.f);
   }
 }
 
