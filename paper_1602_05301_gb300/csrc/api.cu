@@ -205,6 +205,7 @@ extern "C" qbx_status qbx_geometry_create(const qbx_geometry_desc* d, qbx_handle
       (e = h->ctr_r.alloc(h->n_ctr)) != cudaSuccess ||
       (e = h->q_str.alloc(h->n_src)) != cudaSuccess ||
       (e = h->d_str.alloc(h->n_src)) != cudaSuccess ||
+      (e = h->str_exp.alloc(kStrengthBlocks)) != cudaSuccess ||
       (e = h->alpha.alloc(h->n_ctr * (2 * h->p + 1))) != cudaSuccess ||
       (e = h->counters.alloc(16)) != cudaSuccess) {
     set_error("device allocation failed: %s", cudaGetErrorString(e));
@@ -470,6 +471,7 @@ qbx_status replace_geometry(qbx_handle* h, int64_t n_panels, DevBuf<double>& nod
       (e = h->ctr_r.alloc(h->n_ctr)) != cudaSuccess ||
       (e = h->q_str.alloc(h->n_src)) != cudaSuccess ||
       (e = h->d_str.alloc(h->n_src)) != cudaSuccess ||
+      (e = h->str_exp.alloc(kStrengthBlocks)) != cudaSuccess ||
       (e = h->alpha.alloc(h->n_ctr * (2 * h->p + 1))) != cudaSuccess) {
     set_error("device allocation failed: %s", cudaGetErrorString(e));
     return QBX_ERR_OOM;

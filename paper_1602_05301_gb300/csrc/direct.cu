@@ -8,6 +8,7 @@
 //   qbxl2p         truncated J-expansion at associated targets (Sec. 2.1, Eq. (phiapprox))
 //   associate      target association (Sec. 6.1) by exhaustive search
 //   place_centres  c = s + side (h/2) n (Sec. 2.2)
+#include <cmath>
 #include <cstdio>
 
 #include "qbx_internal.h"
@@ -15,15 +16,25 @@
 
 namespace {
 
-// q_j = (i/4) w_j cS sigmaS_j,  d_j = (i/4) w_j cD sigmaD_j
-__global__ void strengths_kernel(int64_t n, const double* __restrict__ w, cd cS,
-                                 const cd* __restrict__ sS, cd cD, const cd* __restrict__ sD,
-                                 cd* __restrict__ q, cd* __restrict__ d) {
-  int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const cd i4 = mk(0.0, 0.25 * w[j]);
-  q[j] = sS ? cmul(i4, cmul(cS, sS[j])) : mk(0.0, 0.0);
-  d[j] = sD ? cmul(i4, cmul(cD, sD[j])) : mk(0.0, 0.0);
+// q_j = (i/4) w_j cS sigmaS_j,  d_j = (i/4) w_j cD sigmaD_j; with str_exp each
+// block's largest exponent
+__global__ void __launch_bounds__(256) strengths_kernel(
+    int64_t n, const double* __restrict__ w, cd cS, const cd* __restrict__ sS, cd cD,
+    const cd* __restrict__ sD, cd* __restrict__ q, cd* __restrict__ d, int lk,
+    int* __restrict__ str_exp) {
+  int e = 0;
+#pragma unroll 4
+  for (int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x; j < n; j += (int64_t)256 * gridDim.x) {
+    const cd i4 = mk(0.0, 0.25 * w[j]);
+    const cd qj = sS ? cmul(i4, cmul(cS, sS[j])) : mk(0.0, 0.0);
+    const cd dj = sD ? cmul(i4, cmul(cD, sD[j])) : mk(0.0, 0.0);
+    q[j] = qj;
+    d[j] = dj;
+    e = max(e, strength_exponent(qj, dj, lk));
+  }
+  if (!str_exp) return;
+  e = block_exponent(e);
+  if (threadIdx.x == 0) str_exp[blockIdx.x] = e;
 }
 
 // alpha at the centres list[0..n) (every centre when list is NULL), SW warps per
@@ -274,8 +285,9 @@ void p2qbxl_direct(int64_t n, const int32_t* list, const double* cxy, int64_t n_
 qbx_status launch_strengths(qbx_handle* h, cd cS, const cd* sigS, cd cD, const cd* sigD,
                             cudaStream_t s) {
   if (h->n_src == 0) return QBX_OK;
-  strengths_kernel<<<nblk(h->n_src, 256), 256, 0, s>>>(h->n_src, h->src_w.ptr, cS, sigS, cD, sigD,
-                                                     h->q_str.ptr, h->d_str.ptr);
+  strengths_kernel<<<strength_blocks(h->n_src), 256, 0, s>>>(
+      h->n_src, h->src_w.ptr, cS, sigS, cD, sigD, h->q_str.ptr, h->d_str.ptr, std::ilogb(h->k),
+      h->str_exp.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
   h->launches += 1;
   return QBX_OK;
@@ -488,7 +500,7 @@ extern "C" qbx_status qbx_direct_qbx_eval_noalloc(
   if (n_src > 0)
     strengths_kernel<<<nblk(n_src, 256), 256, 0, s>>>(
         n_src, src_weight, mk(cS_re, cS_im), (const cd*)sigma_S, mk(cD_re, cD_im),
-        (const cd*)sigma_D, q, d);
+        (const cd*)sigma_D, q, d, 0, nullptr);
   if (n_ctr > 0)
     p2qbxl_direct(n_ctr, nullptr, ctr_xy, n_src, src_xy, src_normal_xy, q, d, sigma_S != nullptr,
                   sigma_D != nullptr, k, p, alpha, s);

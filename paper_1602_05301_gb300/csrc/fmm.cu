@@ -76,6 +76,7 @@ struct Fmm {
   const float4* ab32;    // FP32 dipole factors (A, B) (mixed path)
   const float4* dn32;    // FP32 (d k/2, nu) (mixed path)
   const float4 *qf, *df, *nf;  // float-float charges, d k and normals (mixed P2P)
+  const int* sexp;       // e: the strengths carry 2^-e (mixed path)
   const double2* cxy;
   const double* crad;    // sorted centre radii
   const int* cid;
@@ -107,6 +108,8 @@ struct Fmm {
 };
 
 __device__ __forceinline__ const double* pw_row(const Fmm& F, int l) { return F.pw + (size_t)l * (2 * F.pbmax + 3); }
+// 2^e, with which every FP64 result of the mixed path is multiplied
+__device__ __forceinline__ double out_scale(const Fmm& F) { return pow2d(__ldg(F.sexp)); }
 __device__ __forceinline__ const double* ipw_row(const Fmm& F, int l) { return F.ipw + (size_t)l * (F.pbmax + 2); }
 
 // Unnormalised Miller recurrence for J_0..J_M of x into row[0..M]; returns the
@@ -233,8 +236,10 @@ __global__ void powers_kernel(int n_levels, int pbmax, const int* __restrict__ l
 }
 
 // ---------------------------------------------------------------- strengths
-// Sorted strengths; for the mixed path also their FP32 forms, with the dipole
-// factors A = d (k/2) nu and B = d (k/2) conj(nu) (nu = n_x + i n_y) formed
+// Sorted strengths; for the mixed path (str_exp set) times 2^-e, e the exponent of the
+// largest of them, so that a density of any size keeps the FP32 stages in range
+// (out_scale puts 2^e back where FP64 results are formed; every step is the same to
+// the bit for 2^n times a density), and their FP32 forms, with the dipole factors A = d (k/2) nu and B = d (k/2) conj(nu) (nu = n_x + i n_y) formed
 // once per source instead of once per (source, centre) pair.
 __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
                                         const cd* __restrict__ q, const cd* __restrict__ d,
@@ -242,10 +247,22 @@ __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
                                         cd* __restrict__ qs, cd* __restrict__ ds,
                                         float2* __restrict__ q32, float4* __restrict__ ab32,
                                         float4* __restrict__ dn32, float4* __restrict__ qf,
-                                        float4* __restrict__ df, float4* __restrict__ nf) {
+                                        float4* __restrict__ df, float4* __restrict__ nf,
+                                        const int* __restrict__ str_exp, int n_exp,
+                                        int* __restrict__ sexp) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int at = i < n ? perm[i] : 0;
+  cd qi = q[at], di = d[at];
+  if (str_exp) {
+    int e = 0;
+    for (int j = threadIdx.x; j < n_exp; j += 256) e = max(e, str_exp[j]);
+    e = block_exponent(e);
+    e = e == 0 ? 0 : min(e - 1023, 1022);  // 2^e and 2^-e are normal
+    if (i == 0) *sexp = e;
+    qi = cscale(qi, pow2d(-e));
+    di = cscale(di, pow2d(-e));
+  }
   if (i >= n) return;
-  const cd qi = q[perm[i]], di = d[perm[i]];
   qs[i] = qi;
   ds[i] = di;
   if (q32) {
@@ -1140,7 +1157,8 @@ __global__ void __launch_bounds__(kThreads) m2qbxl_pair_kernel(Fmm F, const int*
 // (centres clist[0..n), pairs of position t at cpo[t]..cpo[t+1]).
 __global__ void m2qbxl_sum_kernel(int n, int P, const int* __restrict__ cpo,
                                   const cd* __restrict__ partial, const int* __restrict__ cid,
-                                  const int* __restrict__ clist, cd* __restrict__ alpha) {
+                                  const int* __restrict__ clist, const int* __restrict__ sexp,
+                                  cd* __restrict__ alpha) {
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= (int64_t)n * P) return;
   const int t = (int)(g / P), l = (int)(g % P);
@@ -1148,6 +1166,7 @@ __global__ void m2qbxl_sum_kernel(int n, int P, const int* __restrict__ cpo,
   if (t1 == t0) return;
   cd sum = mk(0.0, 0.0);
   for (int e = t0; e < t1; ++e) sum = cadd(sum, partial[(size_t)e * P + l]);
+  if (sexp) sum = cscale(sum, pow2d(*sexp));  // mixed path (out_scale)
   cd* dst = alpha + (size_t)cid[clist[t]] * P + l;
   *dst = cadd(*dst, sum);
 }
@@ -1477,7 +1496,8 @@ __global__ void __launch_bounds__(32) l2qbxl_mixed_kernel(Fmm F, const int* __re
     }
     const double sc = pow2d(emax);
     cd* dst = alpha + (size_t)F.cid[i] * P + p + so;
-    *dst = cadd(*dst, mk(((double)S.x - (double)C.x) * sc, ((double)S.y - (double)C.y) * sc));
+    *dst = cadd(*dst, cscale(mk(((double)S.x - (double)C.x) * sc, ((double)S.y - (double)C.y) * sc),
+                             out_scale(F)));
   }
 }
 
@@ -1571,8 +1591,9 @@ __global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restr
     }
     const double f1 = pow2d(s * a), f2 = pow2d(-s * a);
     cd* dst = alpha + (size_t)F.cid[i] * P + p + so;
-    *dst = cadd(*dst, mk(((double)S1.x - (double)C1.x) * f1 + ((double)S2.x - (double)C2.x) * f2,
-                         ((double)S1.y - (double)C1.y) * f1 + ((double)S2.y - (double)C2.y) * f2));
+    const cd v = mk(((double)S1.x - (double)C1.x) * f1 + ((double)S2.x - (double)C2.x) * f2,
+                    ((double)S1.y - (double)C1.y) * f1 + ((double)S2.y - (double)C2.y) * f2);
+    *dst = cadd(*dst, cscale(v, out_scale(F)));
   }
 }
 
@@ -1729,7 +1750,7 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_mixed_kernel(Fmm F, const i
   }
   if (lane == 0) {
     cd* dst = out + F.tid[i];
-    *dst = cadd(*dst, sum);
+    *dst = cadd(*dst, cscale(sum, out_scale(F)));
   }
 }
 
@@ -1737,8 +1758,9 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_mixed_kernel(Fmm F, const i
 // l2p_kernel's Miller and Clenshaw recurrences in float-float, on 2^{-s m} J_m
 // and the coefficients scaled by 2^{s m} (s = ffs of the level):
 //   f_{n-1} = (2 n 2^s / x) f_n - 4^s f_{n+1},  norm = f_0 + 2 4^s (f_2 + 4^s (f_4 + ...)),
-// everything kept rescaled by 2^-60 when |f| passes 2^20 (with the coefficients
-// below 2^60 no product leaves FP32's range). About 110 FP32 instructions per
+// everything kept rescaled by 2^-60 when |f| passes 2^20: the coefficients are sums of
+// strengths below 2 times Hankel values below 2^60 (float_float_scale), which leaves
+// 2^47 for the number of sources. About 110 FP32 instructions per
 // order instead of 11 on the FP64 pipe, which bound it (86 % of its rate): 0.9 M
 // targets of 200 ellipses 1.75 -> 0.32 ms.
 // Levels without a scale and targets within x = 1e-8 of the centre take the
@@ -1764,7 +1786,7 @@ __global__ void __launch_bounds__(kThreads) l2p_mixed_kernel(Fmm F, const int* _
   if (!in) {
     cd v;
     l2p_value_outside(F, i, b, &v);
-    *dst = cadd(*dst, v);
+    *dst = cadd(*dst, cscale(v, out_scale(F)));
     return;
   }
   const float4* pq = reinterpret_cast<const float4*>(F.lpq + F.eoff[b]);
@@ -1829,7 +1851,7 @@ __global__ void __launch_bounds__(kThreads) l2p_mixed_kernel(Fmm F, const int* _
   auto finish = [&](ff u1, ff u2, ff v1) {
     return ff_add(ff_add(u1, ff_mul(mkff(-co.h, -co.l), u2)), ff_mul(si, v1));
   };
-  const double in64 = 1.0 / ff_f64(norm);
+  const double in64 = out_scale(F) / ff_f64(norm);
   const ff ax = finish(ux1, ux2, vx1), ay = finish(uy1, uy2, vy1);
   *dst = cadd(*dst, mk(ff_f64(ax) * in64, ff_f64(ay) * in64));
 }
@@ -1977,7 +1999,7 @@ __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
 // out[target] += sum of its pairs' float-float terms, in pair order.
 __global__ void m2p_sum_mixed_kernel(int n, const int* __restrict__ wtgt, const int* __restrict__ off,
                                      const float4* __restrict__ partial, const int* __restrict__ tid,
-                                     cd* __restrict__ out) {
+                                     const int* __restrict__ sexp, cd* __restrict__ out) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   ff x = mkff(0.f, 0.f), y = x;
@@ -1987,7 +2009,7 @@ __global__ void m2p_sum_mixed_kernel(int n, const int* __restrict__ wtgt, const 
     y = ff_add(y, mkff(v.z, v.w));
   }
   cd* dst = out + tid[wtgt[t]];
-  *dst = cadd(*dst, mk(ff_f64(x), ff_f64(y)));
+  *dst = cadd(*dst, cscale(mk(ff_f64(x), ff_f64(y)), pow2d(*sexp)));
 }
 
 // ---------------------------------------------------------------- P2M in mixed precision
@@ -2433,9 +2455,10 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
   const cd a0 = f64(acc[0]), a1 = W == 16 ? f64(acc[1]) : a0;
   const cd x32 = PM == 16 ? f64(y32) : a0, x33 = PM == 16 ? f64(y33) : a0;
   cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
+  const double os = out_scale(F);
   pair_coefficients<W, PM>(a0, a1, x32, x33, lane, p, [&](int l, cd a) {
     // the sums carry sigma^{|l|+1}
-    if (live) dst[l] = cadd(dst[l], cscale(a, pow2d(-s * (abs(l) + 1))));
+    if (live) dst[l] = cadd(dst[l], cscale(cscale(a, pow2d(-s * (abs(l) + 1))), os));
   });
 }
 
@@ -2572,6 +2595,8 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
   QBX_CUDA_TRY(f->ab32.alloc(std::max<int64_t>(1, h->n_src)));
   for (DevBuf<float4>* v : {&f->dn32, &f->qf, &f->df, &f->nf})
     QBX_CUDA_TRY(v->alloc(std::max<int64_t>(1, h->n_src)));
+  QBX_CUDA_TRY(f->sexp.alloc(1));
+  QBX_CUDA_TRY(cudaMemset(f->sexp.ptr, 0, sizeof(int)));
   // leaves holding sources (P2M)
   QBX_CUDA_TRY(cudaDeviceSynchronize());
   // stats
@@ -2947,7 +2972,7 @@ Fmm make_view(qbx_handle* h, FmmPlan* f, bool S, bool D) {
   F.xoff = f->X.off.ptr; F.xidx = f->X.idx.ptr;
   F.sxy = f->s_xy.ptr; F.snrm = f->s_nrm.ptr; F.qs = f->qs.ptr; F.ds = f->ds.ptr;
   F.q32 = f->q32.ptr; F.ab32 = f->ab32.ptr; F.dn32 = f->dn32.ptr;
-  F.qf = f->qf.ptr; F.df = f->df.ptr; F.nf = f->nf.ptr;
+  F.qf = f->qf.ptr; F.df = f->df.ptr; F.nf = f->nf.ptr; F.sexp = f->sexp.ptr;
   F.cxy = f->c_xy.ptr; F.crad = f->c_r.ptr; F.cid = f->perm[PT_CTR].ptr;
   F.txy = f->t_xy.ptr; F.tid = f->perm[PT_TGT].ptr; F.tassoc = f->t_assoc.ptr;
   F.lpb = f->lpb.ptr; F.eoff = f->eoff.ptr;
@@ -3047,6 +3072,7 @@ qbx_status launch_m2qbxl(const Fmm& F, FmmPlan* f, qbx_handle* h, bool S, bool D
     const int P = 2 * h->p + 1;
     m2qbxl_sum_kernel<<<nblk((int64_t)C.n * P, 256), 256, 0, s>>>(C.n, P, C.wp_off.ptr, part,
                                                                  f->perm[PT_CTR].ptr, C.clist.ptr,
+                                                                 mixed ? f->sexp.ptr : nullptr,
                                                                  alpha);
     QBX_KCHECK("m2qbxl_sum", s);
     h->launches += 2;
@@ -3127,7 +3153,8 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
     gather_strengths_kernel<<<nblk(h->n_src, 256), 256, 0, s>>>(
         h->n_src, f->perm[PT_SRC].ptr, h->q_str.ptr, h->d_str.ptr, f->s_nrm.ptr, h->k,
         f->qs.ptr, f->ds.ptr, mixed ? f->q32.ptr : nullptr, mixed ? f->ab32.ptr : nullptr,
-        f->dn32.ptr, f->qf.ptr, f->df.ptr, f->nf.ptr);
+        f->dn32.ptr, f->qf.ptr, f->df.ptr, f->nf.ptr, mixed ? h->str_exp.ptr : nullptr,
+        (int)strength_blocks(h->n_src), f->sexp.ptr);
     QBX_KCHECK("gather_strengths", s);
     h->launches += 1;
   }
@@ -3253,7 +3280,7 @@ qbx_status fmm_eval(qbx_handle* h, bool S, bool D, cd* out, int precision, bool 
       QBX_KCHECK("m2p", s2);
       m2p_sum_mixed_kernel<<<nblk(f->n_wtgt, kThreads), kThreads, 0, s2>>>(
           f->n_wtgt, f->wtgt.ptr, f->m2p_off.ptr, reinterpret_cast<float4*>(f->m2p_part.ptr),
-          f->perm[PT_TGT].ptr, out);
+          f->perm[PT_TGT].ptr, f->sexp.ptr, out);
     } else {
       mpole_pq_kernel<<<f->n_m2p_wbox, kThreads, 0, s2>>>(F, f->m2p_wbox.ptr, f->m2p_big.ptr,
                                                          f->m2p_pq.ptr);

@@ -127,6 +127,7 @@ struct qbx_handle {
   bool has_avg = false;
   // evaluation scratch
   DevBuf<cd> q_str, d_str;                  // per-source charge / dipole strengths
+  DevBuf<int> str_exp;                      // [kStrengthBlocks] (see strength_exponent)
   DevBuf<cd> sigS_dev, sigD_dev, out_dev;   // staging for host buffers
   DevBuf<cd> alpha;                         // [n_ctr][2p+1]
   DevBuf<int32_t> counters;                 // small device counters
@@ -143,6 +144,34 @@ struct qbx_handle {
 };
 
 // ---------------------------------------------------------------- kernels entry points
+// The kernels that make the strengths leave the largest binary exponent of each of
+// their blocks (FP64's field, of a finite charge or dipole times k; 0: none) in str_exp,
+// for the mixed path (gather_strengths_kernel). At most this many blocks, each taking
+// several sources.
+constexpr int kStrengthBlocks = 1024;
+inline unsigned strength_blocks(int64_t n) {
+  const int64_t b = (n + 255) / 256;
+  return (unsigned)(b < kStrengthBlocks ? b : kStrengthBlocks);
+}
+// of the strengths q, d; lk = ilogb(k)
+__device__ __forceinline__ int strength_exponent(cd q, cd d, int lk) {
+  auto field = [](cd v) {
+    const int x = (__double2hiint(v.x) >> 20) & 0x7FF, y = (__double2hiint(v.y) >> 20) & 0x7FF;
+    return max(x == 0x7FF ? 0 : x, y == 0x7FF ? 0 : y);
+  };
+  const int f = field(d);
+  return max(field(q), f ? min(max(f + lk, 1), 0x7FE) : 0);
+}
+// the block's largest e (blocks of 256 threads)
+__device__ __forceinline__ int block_exponent(int e) {
+  __shared__ int w[8];
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = e;
+  __syncthreads();
+  for (int i = 0; i < 8; ++i) e = max(e, w[i]);
+  return e;
+}
+
 // direct.cu
 qbx_status launch_strengths(qbx_handle* h, cd cS, const cd* sigS, cd cD, const cd* sigD,
                             cudaStream_t s);

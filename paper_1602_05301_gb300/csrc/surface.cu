@@ -118,26 +118,35 @@ __global__ void upsample_geometry_kernel(int64_t n_panels, int q, int qs,
 // Strengths on the library-made source grid: the densities (given on the
 // density grid) interpolated to source node i of panel k, times the weight and
 // the kernel's factor i/4 (as for a caller's grid):
-// q_i = (i/4) w_i cS sigma_S(s_i), d_i = (i/4) w_i cD sigma_D(s_i).
-__global__ void strengths_upsampled_kernel(int64_t n_panels, int q, int qs,
+// q_i = (i/4) w_i cS sigma_S(s_i), d_i = (i/4) w_i cD sigma_D(s_i); each block's
+// largest exponent in str_exp.
+__global__ void __launch_bounds__(256) strengths_upsampled_kernel(int64_t n_panels, int q, int qs,
                                            const double* __restrict__ L,
                                            const double* __restrict__ w, cd cS,
                                            const cd* __restrict__ sS, cd cD,
                                            const cd* __restrict__ sD, cd* __restrict__ qo,
-                                           cd* __restrict__ dout) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n_panels * qs) return;
-  const int64_t k = i / qs;
-  const int j = (int)(i % qs);
-  const double* Lj = L + (size_t)j * q;
-  cd a = mk(0.0, 0.0), b = mk(0.0, 0.0);
-  for (int r = 0; r < q; ++r) {
-    if (sS) a = mk(fma(Lj[r], sS[k * q + r].x, a.x), fma(Lj[r], sS[k * q + r].y, a.y));
-    if (sD) b = mk(fma(Lj[r], sD[k * q + r].x, b.x), fma(Lj[r], sD[k * q + r].y, b.y));
+                                           cd* __restrict__ dout, int lk,
+                                           int* __restrict__ str_exp) {
+  int e = 0;
+  for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n_panels * qs;
+       i += (int64_t)256 * gridDim.x) {
+    const int64_t k = i / qs;
+    const int j = (int)(i % qs);
+    const double* Lj = L + (size_t)j * q;
+    cd a = mk(0.0, 0.0), b = mk(0.0, 0.0);
+    for (int r = 0; r < q; ++r) {
+      if (sS) a = mk(fma(Lj[r], sS[k * q + r].x, a.x), fma(Lj[r], sS[k * q + r].y, a.y));
+      if (sD) b = mk(fma(Lj[r], sD[k * q + r].x, b.x), fma(Lj[r], sD[k * q + r].y, b.y));
+    }
+    const cd i4 = mk(0.0, 0.25 * w[i]);
+    a = sS ? cmul(i4, cmul(cS, a)) : mk(0.0, 0.0);
+    b = sD ? cmul(i4, cmul(cD, b)) : mk(0.0, 0.0);
+    qo[i] = a;
+    dout[i] = b;
+    e = max(e, strength_exponent(a, b, lk));
   }
-  const cd i4 = mk(0.0, 0.25 * w[i]);
-  qo[i] = sS ? cmul(i4, cmul(cS, a)) : mk(0.0, 0.0);
-  dout[i] = sD ? cmul(i4, cmul(cD, b)) : mk(0.0, 0.0);
+  e = block_exponent(e);
+  if (threadIdx.x == 0) str_exp[blockIdx.x] = e;
 }
 
 }  // namespace
@@ -172,9 +181,9 @@ qbx_status upsample_geometry(qbx_handle* h) {
 qbx_status launch_strengths_upsampled(qbx_handle* h, cd cS, const cd* sigS, cd cD,
                                       const cd* sigD, cudaStream_t s) {
   if (h->n_src == 0) return QBX_OK;
-  strengths_upsampled_kernel<<<nblk(h->n_src, 256), 256, 0, s>>>(
+  strengths_upsampled_kernel<<<strength_blocks(h->n_src), 256, 0, s>>>(
       h->n_panels, h->q, h->q_src, h->up_L.ptr, h->src_w.ptr, cS, sigS, cD, sigD, h->q_str.ptr,
-      h->d_str.ptr);
+      h->d_str.ptr, std::ilogb(h->k), h->str_exp.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
   h->launches += 1;
   return QBX_OK;

@@ -178,6 +178,7 @@ struct FmmPlan {
   DevBuf<float2> q32;                   // their FP32 charges and dipole factors (mixed path)
   DevBuf<float4> ab32;
   DevBuf<float4> dn32, qf, df, nf;      // FP32 (d k/2, nu); float-float charges, d k, normals
+  DevBuf<int> sexp;                     // e: the mixed path's strengths carry 2^-e
   DevBuf<int> err;                      // device error flags
   // mixed precision (sigma-normalised FP32 M2L)
   DevBuf<double> lsig, conv, iconv;     // [n_levels][pb_max+1] log sig_j, s^j / sig_j, its inverse
