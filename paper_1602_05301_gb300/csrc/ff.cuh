@@ -211,19 +211,28 @@ inline FfUnits make_ff_units(double k) {
   return U;
 }
 
-// (x, y) = a displacement in those units; x = k r, ir = 1 / r and the direction
-// e^{i th} in FP32. False at r = 0.
+// (x, y) = a displacement in those units; z = k r, ir = 1 / r and the direction
+// e^{i th} in FP32. False at r = 0 (both components below FP32's normal range).
+// Where r^2 or its second part would leave that range, r is formed at 2^100 times
+// the size (rsqrt.approx.ftz is infinite at a subnormal square).
 struct FfPolar {
   ff x, y, ir, z;  // z = k r
   float c, s;
   __device__ __forceinline__ bool set(double dx, double dy, const FfUnits& U) {
     x = ff_from_f64(dx, U.off);
     y = ff_from_f64(dy, U.off);
-    const ff xx = ff_mul_raw(x, x), yy = ff_mul_raw(y, y);
-    const ff d2 = ff_add(xx, yy);
-    if (d2.h == 0.f) return false;
-    ir = ff_rsqrt(d2);
-    z = ff_mul(ff_mul_raw(d2, ir), U.kk);
+    ff d2 = ff_add(ff_mul_raw(x, x), ff_mul_raw(y, y));
+    if (d2.h < 0x1p-76f) {
+      if (x.h == 0.f && y.h == 0.f) return false;
+      const ff xs = ff_scale(x, 0x1p100f), ys = ff_scale(y, 0x1p100f);
+      d2 = ff_add(ff_mul_raw(xs, xs), ff_mul_raw(ys, ys));
+      ir = ff_rsqrt(d2);
+      z = ff_scale(ff_mul(ff_mul_raw(d2, ir), U.kk), 0x1p-100f);
+      ir = ff_scale(ir, 0x1p100f);
+    } else {
+      ir = ff_rsqrt(d2);
+      z = ff_mul(ff_mul_raw(d2, ir), U.kk);
+    }
     const float irf = ff_f32(ir);
     c = ff_f32(x) * irf;
     s = ff_f32(y) * irf;
