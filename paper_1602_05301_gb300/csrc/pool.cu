@@ -4,7 +4,8 @@
 // nodes: 14.2 -> 11.2 ms). Blocks given back are therefore kept for later buffers of
 // the same size class:
 //  * at most kPoolBytes are kept per device; what exceeds that, and everything
-//    when an allocation fails, goes back to the driver;
+//    when an allocation fails, goes back to the driver (an allocation that fails
+//    is tried again without the rounding to its class);
 //  * a block is kept only after a device synchronisation on its device, as
 //    cudaFree has it, so that it may serve any stream and thread at once
 //    (DeviceQuiet makes one synchronisation serve many blocks);
@@ -37,12 +38,17 @@ Pool& pool() {
 }
 thread_local int t_quiet = 0;
 
-// Size classes: multiples of 512 bytes to 4 KB, then four steps per power of two.
+size_t multiple(size_t n, size_t step) { return (n + step - 1) / step * step; }
+// Size classes: multiples of 512 bytes to 4 KB, four steps per power of two to 2 MB,
+// then multiples of 2 MB, which cudaMalloc hands out anyway: a plan's large buffers
+// take no more memory than without the pool.
+constexpr size_t kGranule = 2u << 20;
 size_t size_class(size_t n) {
-  if (n <= 4096) return (n + 511) / 512 * 512;
+  if (n <= 4096) return multiple(n, 512);
+  if (n > kGranule) return multiple(n, kGranule);
   size_t step = 1024;
   while (step * 8 < n) step *= 2;
-  return (n + step - 1) / step * step;
+  return multiple(n, step);
 }
 
 void drop_kept(Pool& P, int dev) {
@@ -61,7 +67,7 @@ cudaError_t dev_alloc(void** out, size_t bytes) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const size_t n = size_class(bytes);
+  size_t n = size_class(bytes);
   Pool& P = pool();
   std::lock_guard<std::mutex> lock(P.mu);
   auto it = P.kept.find({dev, n});
@@ -74,6 +80,11 @@ cudaError_t dev_alloc(void** out, size_t bytes) {
     if (e == cudaErrorMemoryAllocation && P.kept_bytes[dev] > 0) {
       cudaGetLastError();
       drop_kept(P, dev);
+      e = cudaMalloc(out, n);
+    }
+    if (e == cudaErrorMemoryAllocation) {  // what the buffer needs may still be there
+      cudaGetLastError();
+      n = multiple(bytes, 512);
       e = cudaMalloc(out, n);
     }
     if (e != cudaSuccess) {
@@ -108,7 +119,7 @@ void dev_free(void* p) {
     }
   }
   std::lock_guard<std::mutex> lock(P.mu);
-  if (P.kept_bytes[b.dev] + b.size > kPoolBytes) {
+  if (P.kept_bytes[b.dev] + b.size > kPoolBytes || b.size != size_class(b.size)) {
     cudaFree(p);
     return;
   }

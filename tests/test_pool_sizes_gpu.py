@@ -1,0 +1,36 @@
+"""How much device memory the pool takes and gives back."""
+import numpy as np
+import pytest
+
+from qbx_workloads import circle, discretise_curve
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def qbxmod():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1602_05301_gb300 import build as b
+    b.build()
+    from paper_1602_05301_gb300 import qbx
+    return qbx
+
+
+def test_large_buffers_are_not_rounded_up(qbxmod):
+    """Plans of 2^25 and 2^25 + 1024 targets (buffers of 128 and 512 MB and one step
+    above): 48 bytes per target apart, and at most a granule of 2 MB per buffer."""
+    import torch
+    g = discretise_curve(*circle(0.01), 2, 4, k=1.0)
+    used = []
+    for n in (1 << 25, (1 << 25) + 1024):
+        tgt = np.full((n, 2), 3.0)
+        lp = qbxmod.LayerPotential(g.as_dict(), 2, sides=1)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        lp.build(tgt, mode=qbxmod.QBX_DIRECT)
+        used.append(free - torch.cuda.mem_get_info()[0])
+        lp.close()
+    assert used[0] > (1 << 30)
+    assert abs(used[1] - used[0]) < 16 * (2 << 20)
