@@ -3,17 +3,17 @@
 // device), which was a fifth of the time of building and dropping a plan (8192
 // nodes: 14.2 -> 11.2 ms). Blocks given back are therefore kept for later buffers of
 // the same size class:
-//  * at most kPoolBytes are kept per device; what exceeds that, and everything
-//    when an allocation fails, goes back to the driver (an allocation that fails
-//    is tried again without the rounding to its class);
+//  * at most kPoolBytes are kept per device; the oldest blocks beyond that, and all
+//    when an allocation fails, go back to the driver (an allocation that fails is
+//    tried again without the rounding to its class);
 //  * a block is kept only after a device synchronisation on its device, as
 //    cudaFree has it, so that it may serve any stream and thread at once
 //    (DeviceQuiet makes one synchronisation serve many blocks);
 //  * all under one mutex.
+#include <deque>
 #include <map>
 #include <mutex>
 #include <unordered_map>
-#include <vector>
 
 #include "qbx_internal.h"
 
@@ -27,9 +27,19 @@ struct Pool {
     int dev;
   };
   std::mutex mu;
+  struct Kept {
+    void* p;
+    unsigned long long age;  // smaller: kept for longer
+  };
   std::unordered_map<void*, Block> live;
-  std::map<std::pair<int, size_t>, std::vector<void*>> kept;
-  std::map<int, size_t> kept_bytes;
+  // per device: the blocks kept by size, oldest first, and their sizes by age
+  struct Device {
+    std::map<size_t, std::deque<Kept>> of_size;
+    std::map<unsigned long long, size_t> by_age;
+    size_t bytes = 0;
+  };
+  std::map<int, Device> devs;
+  unsigned long long clock = 0;
 };
 // never destroyed: the driver may be gone when static destructors run
 Pool& pool() {
@@ -51,13 +61,17 @@ size_t size_class(size_t n) {
   return multiple(n, step);
 }
 
-void drop_kept(Pool& P, int dev) {
-  for (auto& e : P.kept)
-    if (e.first.first == dev) {
-      for (void* p : e.second) cudaFree(p);
-      e.second.clear();
-    }
-  P.kept_bytes[dev] = 0;
+// Gives the oldest kept blocks of D back to the driver until at most `most` bytes stay.
+void trim(Pool::Device& D, size_t most) {
+  while (D.bytes > most) {
+    const auto oldest = D.by_age.begin();
+    auto it = D.of_size.find(oldest->second);
+    cudaFree(it->second.front().p);
+    D.bytes -= it->first;
+    it->second.pop_front();
+    if (it->second.empty()) D.of_size.erase(it);
+    D.by_age.erase(oldest);
+  }
 }
 
 }  // namespace
@@ -70,16 +84,19 @@ cudaError_t dev_alloc(void** out, size_t bytes) {
   size_t n = size_class(bytes);
   Pool& P = pool();
   std::lock_guard<std::mutex> lock(P.mu);
-  auto it = P.kept.find({dev, n});
-  if (it != P.kept.end() && !it->second.empty()) {
-    *out = it->second.back();
+  Pool::Device& D = P.devs[dev];
+  auto it = D.of_size.find(n);
+  if (it != D.of_size.end()) {
+    *out = it->second.back().p;
+    D.by_age.erase(it->second.back().age);
     it->second.pop_back();
-    P.kept_bytes[dev] -= n;
+    if (it->second.empty()) D.of_size.erase(it);
+    D.bytes -= n;
   } else {
     e = cudaMalloc(out, n);
-    if (e == cudaErrorMemoryAllocation && P.kept_bytes[dev] > 0) {
+    if (e == cudaErrorMemoryAllocation && D.bytes > 0) {
       cudaGetLastError();
-      drop_kept(P, dev);
+      trim(D, 0);
       e = cudaMalloc(out, n);
     }
     if (e == cudaErrorMemoryAllocation) {  // what the buffer needs may still be there
@@ -119,12 +136,15 @@ void dev_free(void* p) {
     }
   }
   std::lock_guard<std::mutex> lock(P.mu);
-  if (P.kept_bytes[b.dev] + b.size > kPoolBytes || b.size != size_class(b.size)) {
+  if (b.size > kPoolBytes || b.size != size_class(b.size)) {
     cudaFree(p);
     return;
   }
-  P.kept[{b.dev, b.size}].push_back(p);
-  P.kept_bytes[b.dev] += b.size;
+  Pool::Device& D = P.devs[b.dev];
+  trim(D, kPoolBytes - b.size);
+  D.of_size[b.size].push_back({p, P.clock});
+  D.by_age[P.clock++] = b.size;
+  D.bytes += b.size;
 }
 
 // (where it cannot synchronise, each block tries for itself)

@@ -34,3 +34,21 @@ def test_large_buffers_are_not_rounded_up(qbxmod):
         lp.close()
     assert used[0] > (1 << 30)
     assert abs(used[1] - used[0]) < 16 * (2 << 20)
+
+
+def _direct_plan(qbxmod, n):
+    lp = qbxmod.LayerPotential(discretise_curve(*circle(0.01), 2, 4, k=1.0).as_dict(), 2, sides=1)
+    lp.build(np.full((n, 2), 3.0), mode=qbxmod.QBX_DIRECT)
+    return lp
+
+
+def test_old_blocks_make_room(qbxmod):
+    """Blocks of an earlier plan that fill the pool (240 MB) give way to those of later
+    plans (132 MB): a plan like the last one takes no new device memory."""
+    import torch
+    _direct_plan(qbxmod, 6_000_000).close()
+    _direct_plan(qbxmod, 3_300_000).close()
+    free = torch.cuda.mem_get_info()[0]
+    lp = _direct_plan(qbxmod, 3_300_000)
+    assert free - torch.cuda.mem_get_info()[0] < (16 << 20)
+    lp.close()
