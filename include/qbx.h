@@ -24,7 +24,7 @@
  *  - The caller owns every buffer it passes; the library copies what it keeps
  *    and never frees caller memory. The handle owns all memory it allocates;
  *    when it is destroyed the library may keep up to 256 MiB of it per device
- *    for later handles.
+ *    for later handles (qbx_release_memory gives it back).
  *  - No C++ exception crosses this boundary. Every call returns a status; on a
  *    non-OK status qbx_last_error() holds a message (thread-local).
  *  - One handle must not be used from two threads at once; distinct handles
@@ -182,6 +182,11 @@ qbx_status qbx_layer_potential_eval(qbx_handle *h, double cS_re, double cS_im,
 /* Frees every resource of the handle. NULL-safe. Synchronises the device work
  * of the handle first. */
 void qbx_destroy(qbx_handle *h);
+
+/* Gives the device memory that the library keeps for later handles back to the
+ * driver, on every device, and returns the number of bytes. Live handles keep
+ * theirs. */
+int64_t qbx_release_memory(void);
 
 /* Message of the last non-OK status on this thread ("" if none). */
 const char *qbx_last_error(void);

@@ -6,6 +6,7 @@
 //  * at most kPoolBytes are kept per device; the oldest blocks beyond that, and all
 //    when an allocation fails, go back to the driver (an allocation that fails is
 //    tried again without the rounding to its class);
+//  * qbx_release_memory gives all of them back;
 //  * a block is kept only after a device synchronisation on its device, as
 //    cudaFree has it, so that it may serve any stream and thread at once
 //    (DeviceQuiet makes one synchronisation serve many blocks);
@@ -153,4 +154,15 @@ DeviceQuiet::DeviceQuiet() : quiet(t_quiet > 0 || cudaDeviceSynchronize() == cud
 }
 DeviceQuiet::~DeviceQuiet() {
   if (quiet) --t_quiet;
+}
+
+extern "C" int64_t qbx_release_memory(void) {
+  Pool& P = pool();
+  std::lock_guard<std::mutex> lock(P.mu);
+  size_t n = 0;
+  for (auto& d : P.devs) {
+    n += d.second.bytes;
+    trim(d.second, 0);
+  }
+  return (int64_t)n;
 }

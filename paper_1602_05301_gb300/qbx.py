@@ -78,6 +78,8 @@ def library() -> ctypes.CDLL:
                 _vp, _vp, _vp, ctypes.c_int32, _vp]
             lib.qbx_destroy.restype = None
             lib.qbx_destroy.argtypes = [_vp]
+            lib.qbx_release_memory.restype = ctypes.c_int64
+            lib.qbx_release_memory.argtypes = []
             lib.qbx_last_error.restype = ctypes.c_char_p
             lib.qbx_last_error.argtypes = []
             lib.qbx_get_stats.restype = ctypes.c_int
@@ -176,6 +178,11 @@ def qbx_layer_potential_eval(handle, cS, sigma_S, cD, sigma_D, out, alpha_out=No
 def qbx_destroy(handle):
     if handle:
         library().qbx_destroy(handle)
+
+
+def qbx_release_memory() -> int:
+    """Gives the device memory kept for later handles back; the number of bytes."""
+    return int(library().qbx_release_memory())
 
 
 def qbx_get_stats(handle):

@@ -52,3 +52,21 @@ def test_old_blocks_make_room(qbxmod):
     lp = _direct_plan(qbxmod, 3_300_000)
     assert free - torch.cuda.mem_get_info()[0] < (16 << 20)
     lp.close()
+
+
+def test_release_memory(qbxmod):
+    """What the pool keeps after the last handle (here over 100 MB) can be had back, a
+    live handle is not affected, and later plans work."""
+    import torch
+    kept = _direct_plan(qbxmod, 1000)
+    _direct_plan(qbxmod, 3_300_000).close()
+    free = torch.cuda.mem_get_info()[0]
+    n = qbxmod.qbx_release_memory()
+    assert n > (100 << 20) and torch.cuda.mem_get_info()[0] - free >= n // 2
+    assert qbxmod.qbx_release_memory() == 0
+    sig = np.ones(8, complex)
+    u = kept.eval(sigma_S=sig, cS=1.0)
+    kept.close()
+    lp = _direct_plan(qbxmod, 1000)
+    assert np.isfinite(u).all() and np.array_equal(u, lp.eval(sigma_S=sig, cS=1.0))
+    lp.close()
