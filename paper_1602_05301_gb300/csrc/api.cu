@@ -212,7 +212,7 @@ extern "C" qbx_status qbx_geometry_create(const qbx_geometry_desc* d, qbx_handle
     return fail(QBX_ERR_OOM);
   }
   if ((st = launch_place_centres(h, 0)) != QBX_OK) return fail(st);
-  if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
+  if ((e = dev_sync()) != cudaSuccess) {
     set_error("geometry set-up failed: %s", cudaGetErrorString(e));
     return fail(QBX_ERR_CUDA);
   }
@@ -288,7 +288,7 @@ extern "C" qbx_status qbx_tree_build(qbx_handle* h, const qbx_tree_desc* d) {
   } else {
     QBX_TRY(launch_associate_direct(h, dn.ptr, ds.ptr, eps, 0));
   }
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   int32_t ctr[2];
   QBX_CUDA_TRY(cudaMemcpy(ctr, h->counters.ptr, sizeof(ctr), cudaMemcpyDeviceToHost));
   std::vector<int32_t> assoc = to_host(h->assoc.ptr, (size_t)h->n_tgt);
@@ -423,7 +423,7 @@ extern "C" qbx_status qbx_layer_potential_eval(qbx_handle* h, double cS_re, doub
 extern "C" qbx_status qbx_sync(qbx_handle* h) {
   set_error("%s", "");
   if (!h) { set_error("qbx_sync: NULL handle"); return QBX_ERR_ARG; }
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   return read_wait_flag(h);
 }
 
@@ -441,7 +441,7 @@ void take(DevBuf<T>& dst, DevBuf<T>& src) {
 qbx_status replace_geometry(qbx_handle* h, int64_t n_panels, DevBuf<double>& node_xy,
                             DevBuf<double>& node_nrm, DevBuf<double>& node_w,
                             const std::vector<double>& panel_h) {
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   if (h->fmm) fmm_plan_free(h->fmm);
   h->fmm = nullptr;
   h->planned = false;
@@ -477,7 +477,7 @@ qbx_status replace_geometry(qbx_handle* h, int64_t n_panels, DevBuf<double>& nod
     return QBX_ERR_OOM;
   }
   QBX_TRY(launch_place_centres(h, 0));
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   h->stats[0] = h->n_src;
   h->stats[1] = h->n_ctr;
   return QBX_OK;

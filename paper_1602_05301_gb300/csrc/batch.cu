@@ -120,27 +120,31 @@ qbx_status capture(qbx_batch* b, const double* cS, bool S, const double* cD, boo
     b->graph = nullptr;
   }
   const int n = (int)b->h.size(), ns = (int)b->streams.size();
-  QBX_CUDA_TRY(cudaStreamBeginCapture(b->main, cudaStreamCaptureModeRelaxed));
   qbx_status st = QBX_OK;
-  cudaEventRecord(b->ev_fork, b->main);
-  for (int j = 0; j < ns; ++j) cudaStreamWaitEvent(b->streams[j], b->ev_fork, 0);
-  for (int i = 0; i < n && st == QBX_OK; ++i) {
-    qbx_handle* h = b->h[i];
-    const bool timing = h->timing;
-    h->timing = false;
-    st = qbx_layer_potential_eval(
-        h, S ? cS[2 * i] : 0.0, S ? cS[2 * i + 1] : 0.0,
-        S ? (const double*)(b->sS.ptr + b->soff[i]) : nullptr, D ? cD[2 * i] : 0.0,
-        D ? cD[2 * i + 1] : 0.0, D ? (const double*)(b->sD.ptr + b->soff[i]) : nullptr,
-        (double*)(b->out.ptr + b->toff[i]), nullptr, prec, b->streams[i % ns]);
-    h->timing = timing;
-  }
-  for (int j = 0; j < ns; ++j) {
-    cudaEventRecord(b->evs[j], b->streams[j]);
-    cudaStreamWaitEvent(b->main, b->evs[j], 0);
-  }
   cudaGraph_t g = nullptr;
-  const cudaError_t e = cudaStreamEndCapture(b->main, &g);
+  cudaError_t e;
+  {
+    CaptureScope alone;
+    QBX_CUDA_TRY(cudaStreamBeginCapture(b->main, cudaStreamCaptureModeRelaxed));
+    cudaEventRecord(b->ev_fork, b->main);
+    for (int j = 0; j < ns; ++j) cudaStreamWaitEvent(b->streams[j], b->ev_fork, 0);
+    for (int i = 0; i < n && st == QBX_OK; ++i) {
+      qbx_handle* h = b->h[i];
+      const bool timing = h->timing;
+      h->timing = false;
+      st = qbx_layer_potential_eval(
+          h, S ? cS[2 * i] : 0.0, S ? cS[2 * i + 1] : 0.0,
+          S ? (const double*)(b->sS.ptr + b->soff[i]) : nullptr, D ? cD[2 * i] : 0.0,
+          D ? cD[2 * i + 1] : 0.0, D ? (const double*)(b->sD.ptr + b->soff[i]) : nullptr,
+          (double*)(b->out.ptr + b->toff[i]), nullptr, prec, b->streams[i % ns]);
+      h->timing = timing;
+    }
+    for (int j = 0; j < ns; ++j) {
+      cudaEventRecord(b->evs[j], b->streams[j]);
+      cudaStreamWaitEvent(b->main, b->evs[j], 0);
+    }
+    e = cudaStreamEndCapture(b->main, &g);
+  }
   if (st != QBX_OK) {
     if (g) cudaGraphDestroy(g);
     return st;

@@ -384,7 +384,7 @@ qbx_status prepare(qbx_handle* h, PanelData& D) {
   QBX_CUDA_TRY(D.coff.alloc(h->curve_off.size()));
   QBX_CUDA_TRY(cudaMemcpy(D.coff.ptr, h->curve_off.data(), h->curve_off.size() * 8,
                           cudaMemcpyHostToDevice));
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   return QBX_OK;
 }
 
@@ -409,7 +409,7 @@ qbx_status expansion_weights(qbx_handle* h, PanelData& D, DevBuf<double>& wn) {
     new_nodes_kernel<<<nblk(np * q, kT), kT>>>(np, q, par.ptr, ab.ptr, D.cx.ptr, D.cn.ptr,
                                                D.gl.ptr, D.gw.ptr, tmp_xy.ptr, tmp_n.ptr, wn.ptr);
     QBX_CUDA_TRY(cudaGetLastError());
-    QBX_CUDA_TRY(cudaDeviceSynchronize());
+    QBX_CUDA_TRY(dev_sync());
   }
   return QBX_OK;
 }

@@ -2598,7 +2598,7 @@ qbx_status fmm_plan_build(qbx_handle* h, const qbx_tree_desc* d, const int64_t* 
   QBX_CUDA_TRY(f->sexp.alloc(1));
   QBX_CUDA_TRY(cudaMemset(f->sexp.ptr, 0, sizeof(int)));
   // leaves holding sources (P2M)
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   // stats
   std::vector<int> uoff(f->n_boxes + 1), woff(f->n_boxes + 1), xoff(f->n_boxes + 1);
   std::vector<int2> rs(f->n_boxes), rc(f->n_boxes), rt(f->n_boxes);

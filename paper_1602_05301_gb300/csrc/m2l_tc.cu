@@ -1288,7 +1288,7 @@ qbx_status tc_plan_build(qbx_handle* h, FmmPlan* f) {
                                      reinterpret_cast<__nv_bfloat16*>(f->tc_A.ptr),
                                      f->tc_fexp.ptr);
     QBX_CUDA_TRY(cudaGetLastError());
-    QBX_CUDA_TRY(cudaDeviceSynchronize());
+    QBX_CUDA_TRY(dev_sync());
   }
   // vector-slice room per V-list source on a tensor-core level
   std::vector<int> vsrc(std::max(1, f->n_vsrc)), blev(f->n_boxes);
@@ -1453,9 +1453,9 @@ extern "C" qbx_status qbx_selftest_wait_timeout(qbx_handle* h, int32_t limit_us)
     set_error("qbx_selftest_wait_timeout: needs a handle with an FMM plan");
     return QBX_ERR_STATE;
   }
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   wait_selftest_kernel<<<1, 32>>>(h->fmm->err.ptr + 1, 1000ull * (unsigned long long)limit_us);
   QBX_CUDA_TRY(cudaGetLastError());
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   return QBX_OK;
 }

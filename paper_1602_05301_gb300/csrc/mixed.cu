@@ -1160,7 +1160,7 @@ qbx_status mixed_plan_build(qbx_handle* h, FmmPlan* f) {
       gather_offsets_kernel<<<nblk((int64_t)row_src.size(), 256), 256>>>(rs.ptr, f->eoff.ptr,
                                                                           f->m2l_rowoff.ptr, (int64_t)row_src.size());
       QBX_CUDA_TRY(cudaGetLastError());
-      QBX_CUDA_TRY(cudaDeviceSynchronize());  // before rs is freed
+      QBX_CUDA_TRY(dev_sync());  // before rs is freed
     }
     QBX_CUDA_TRY(cudaMemcpy(f->m2l_yoff.ptr, yoff.data(), yoff.size() * sizeof(long long), cudaMemcpyHostToDevice));
   }

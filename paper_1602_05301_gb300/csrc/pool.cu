@@ -14,6 +14,7 @@
 #include <deque>
 #include <map>
 #include <mutex>
+#include <shared_mutex>
 #include <unordered_map>
 
 #include "qbx_internal.h"
@@ -48,6 +49,8 @@ Pool& pool() {
   return *p;
 }
 thread_local int t_quiet = 0;
+std::shared_mutex g_capture;  // held alone by a capture, shared by synchronisations
+thread_local bool t_capturing = false;
 
 size_t multiple(size_t n, size_t step) { return (n + step - 1) / step * step; }
 // Size classes: multiples of 512 bytes to 4 KB, four steps per power of two to 2 MB,
@@ -76,6 +79,20 @@ void trim(Pool::Device& D, size_t most) {
 }
 
 }  // namespace
+
+cudaError_t dev_sync() {
+  if (t_capturing) return cudaErrorStreamCaptureUnsupported;
+  std::shared_lock<std::shared_mutex> lock(g_capture);
+  return cudaDeviceSynchronize();
+}
+CaptureScope::CaptureScope() {
+  g_capture.lock();
+  t_capturing = true;
+}
+CaptureScope::~CaptureScope() {
+  t_capturing = false;
+  g_capture.unlock();
+}
 
 cudaError_t dev_alloc(void** out, size_t bytes) {
   *out = nullptr;
@@ -129,9 +146,9 @@ void dev_free(void* p) {
   cudaGetDevice(&dev);
   if (t_quiet == 0 || dev != b.dev) {
     if (dev != b.dev) cudaSetDevice(b.dev);
-    const cudaError_t e = cudaDeviceSynchronize();
+    const cudaError_t e = dev_sync();
     if (dev != b.dev) cudaSetDevice(dev);
-    if (e != cudaSuccess) {  // a broken context: nothing to keep
+    if (e != cudaSuccess) {  // a broken context or this thread's capture: not kept
       cudaFree(p);
       return;
     }
@@ -149,7 +166,7 @@ void dev_free(void* p) {
 }
 
 // (where it cannot synchronise, each block tries for itself)
-DeviceQuiet::DeviceQuiet() : quiet(t_quiet > 0 || cudaDeviceSynchronize() == cudaSuccess) {
+DeviceQuiet::DeviceQuiet() : quiet(t_quiet > 0 || dev_sync() == cudaSuccess) {
   if (quiet) ++t_quiet;
 }
 DeviceQuiet::~DeviceQuiet() {

@@ -44,6 +44,17 @@ void set_error(const char* fmt, ...);
 // pool.cu: device memory for DevBuf, kept in size classes between buffers
 cudaError_t dev_alloc(void** p, size_t bytes);
 void dev_free(void* p);
+// The library's only device synchronisation. CUDA forbids one while any stream of the
+// device is being captured (it fails and spoils the capture), so it waits for the
+// captures of other threads, which a CaptureScope marks; in the capturing thread it
+// fails.
+cudaError_t dev_sync();
+struct CaptureScope {
+  CaptureScope();
+  ~CaptureScope();
+  CaptureScope(const CaptureScope&) = delete;
+  CaptureScope& operator=(const CaptureScope&) = delete;
+};
 // Buffers released while one is alive share its device synchronisation: for
 // scopes that release many and launch nothing meanwhile.
 struct DeviceQuiet {

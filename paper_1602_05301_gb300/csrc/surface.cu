@@ -174,7 +174,7 @@ qbx_status upsample_geometry(qbx_handle* h) {
                                                          h->src_xy.ptr, h->src_nrm.ptr,
                                                          h->src_w.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
-  QBX_CUDA_TRY(cudaDeviceSynchronize());  // before the temporaries are freed
+  QBX_CUDA_TRY(dev_sync());  // before the temporaries are freed
   return QBX_OK;
 }
 

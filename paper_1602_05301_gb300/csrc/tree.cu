@@ -765,7 +765,7 @@ qbx_status tree_associate(qbx_handle* h, FmmPlan* f, const int64_t* on_node, con
       f->box.rng[PT_CTR].ptr, f->box.rng[PT_NODE].ptr, f->perm[PT_CTR].ptr, f->perm[PT_NODE].ptr,
       h->assoc.ptr, h->counters.ptr, f->err.ptr);
   QBX_CUDA_TRY(cudaGetLastError());
-  QBX_CUDA_TRY(cudaDeviceSynchronize());
+  QBX_CUDA_TRY(dev_sync());
   int herr = 0;
   QBX_CUDA_TRY(cudaMemcpy(&herr, f->err.ptr, sizeof(int), cudaMemcpyDeviceToHost));
   if (herr & 2) {
