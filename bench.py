@@ -291,7 +291,9 @@ def flop_model(lp, stats, p, has_S, has_D, assoc, fmm, mixed=False, active_frac=
     precision all but QBXL2P is FP32: values and recurrences are float-float,
     whose splitting is charged nothing.
     active_frac scales the centre stages to the centres whose coefficients are
-    formed (those some target uses)."""
+    formed (those some target uses). Direct mode (fmm false) is FP64 in either
+    precision."""
+    mixed = mixed and fmm
     P = 2 * p + 1
     lay = (1 if has_S else 0) + (1 if has_D else 0)
     acc = (18 * P if has_S else 0) + (10 * P if has_D else 0)

@@ -169,7 +169,10 @@ qbx_status qbx_tree_build(qbx_handle *h, const qbx_tree_desc *desc);
  * some target is associated with (the only ones the evaluation reads); with
  * it, at every centre. The potential at the targets is the same either way (in
  * direct mode up to rounding).
- * precision: QBX_FP64 or QBX_MIXED. cuda_stream: a cudaStream_t (NULL: the
+ * precision: QBX_FP64 or QBX_MIXED (direct mode is FP64 with either).
+ * In QBX_MIXED the translations, near-field sums and special functions of FMM
+ * mode are evaluated in FP32 with compensation or in pairs of FP32 numbers (46
+ * bits); results stay within 1e-6, at densities of any size. cuda_stream: a cudaStream_t (NULL: the
  * legacy default stream). With device buffers the call is asynchronous on the
  * stream; with any host buffer it copies through the stream and returns after
  * the result is in host memory.
