@@ -213,8 +213,9 @@ inline FfUnits make_ff_units(double k) {
 
 // (x, y) = a displacement in those units; z = k r, ir = 1 / r and the direction
 // e^{i th} in FP32. False at r = 0 (both components below FP32's normal range).
-// Where r^2 or its second part would leave that range, r is formed at 2^100 times
-// the size (rsqrt.approx.ftz is infinite at a subnormal square).
+// Where r^2 or its second part would leave that range, r is formed at 2^64 times
+// the size (rsqrt.approx.ftz is infinite at a subnormal square). Components below
+// 2^-102 have no second part.
 struct FfPolar {
   ff x, y, ir, z;  // z = k r
   float c, s;
@@ -224,11 +225,11 @@ struct FfPolar {
     ff d2 = ff_add(ff_mul_raw(x, x), ff_mul_raw(y, y));
     if (d2.h < 0x1p-76f) {
       if (x.h == 0.f && y.h == 0.f) return false;
-      const ff xs = ff_scale(x, 0x1p100f), ys = ff_scale(y, 0x1p100f);
+      const ff xs = ff_scale(x, 0x1p64f), ys = ff_scale(y, 0x1p64f);
       d2 = ff_add(ff_mul_raw(xs, xs), ff_mul_raw(ys, ys));
       ir = ff_rsqrt(d2);
-      z = ff_scale(ff_mul(ff_mul_raw(d2, ir), U.kk), 0x1p-100f);
-      ir = ff_scale(ir, 0x1p100f);
+      z = ff_scale(ff_mul(ff_mul_raw(d2, ir), U.kk), 0x1p-64f);
+      ir = ff_scale(ir, 0x1p64f);
     } else {
       ir = ff_rsqrt(d2);
       z = ff_mul(ff_mul_raw(d2, ir), U.kk);
