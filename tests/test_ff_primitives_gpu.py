@@ -52,6 +52,23 @@ def _pair(x):
     return h + (x - h).astype(np.float32)
 
 
+@pytest.mark.parametrize("op,near,far", [(0, 2.6e-11, 3.3e-10), (1, 5.3e-15, 4.3e-14)])
+def test_hankel(probe, op, near, far):
+    import mpmath as mp
+    mp.mp.dps = 40
+    rng = np.random.default_rng(op)
+    # interval ends and random points of both tables, and arguments outside them
+    ends = np.concatenate([2.0 ** np.arange(-16, 4), 8.0 + 0.5 * np.arange(48)])
+    x = _pair(np.concatenate([ends, ends * (1 - 2.0 ** -24), np.geomspace(2.0 ** -16, 8, 300),
+                              rng.uniform(8, 31.98, 300), [2.0 ** -20, 1e-12, 32.0, 40.5, 300.0]]))
+    h = probe(op, x, 4)
+    h = h[:, 0::2] + 1j * h[:, 1::2]
+    ref = np.array([[complex(mp.hankel1(n, mp.mpf(v))) for n in (0, 1)] for v in x])
+    err = np.max(np.abs(h - ref) / np.abs(ref), axis=1)
+    # (outside the tables the value is FP64's rounded to a pair)
+    assert np.all(err < np.where(x < 1, near, far) + 10 * U)
+
+
 def test_rounding_of_fp64(probe):
     rng = np.random.default_rng(1)
     v = np.concatenate([rng.uniform(-2, 2, 500), np.ldexp(rng.uniform(-1, 1, 500),
