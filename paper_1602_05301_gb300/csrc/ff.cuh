@@ -77,7 +77,8 @@ __device__ __forceinline__ ff ff_from_f64(double v, int off) {
 }
 // ff_from_f64 that keeps a NaN (which it makes infinite): coefficients, once each
 __device__ __forceinline__ ff ff_from_f64_nan(double v, int off) {
-  return v == v ? ff_from_f64(v, off) : mkff(__int_as_float(0x7FC00000), 0.f);
+  return ((unsigned)__double2hiint(v) & 0x7FF00000u) != 0x7FF00000u ? ff_from_f64(v, off)
+                                                                    : mkff(f32_from_f64(v), 0.f);
 }
 // FP64 constant (any magnitude FP32 holds) as float-float, for kernel arguments
 // and per-thread set-up

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "f32x2.cuh"
+#include "ff.cuh"
 #include "tree.cuh"
 #include "m2l_entry.cuh"
 
@@ -609,14 +610,16 @@ __global__ void __launch_bounds__(kT) m2l_f64_reduce_kernel(
 //   L2L  lambda'_{rho,s} = e^{i s pi/4} sum_k i^{rho k} t_k,
 //        t_k = sum over n = s - k mod 4 of J_{n-s} e^{-i n pi/4} lambda_n:
 // one real matrix product and a four-point transform in place of four complex matrix
-// products, an eighth of the multiplications (200 ellipses: M2M 0.69 -> 0.38 ms, L2L with
-// the leaves' unscaling 0.97 -> 0.50; starfish at k = 50 0.18 -> 0.11 and 0.20 -> 0.11).
-// What is left is the FP64 conversion of the coefficients. Coefficients sigma-normalised (mu_n =
+// products, an eighth of the multiplications (200 ellipses: M2M 0.69 -> 0.37 ms, L2L with
+// the leaves' unscaling 0.97 -> 0.45; starfish at k = 50 0.18 -> 0.11 and 0.20 -> 0.11).
+// What is left is the FP64 scaling of the coefficients. Coefficients sigma-normalised (mu_n =
 // mh_n conv_n, lambda_n = lh_n / conv_n); the matrices T[n][s] hold the ratio of sigmas
 // and 1/sqrt 2 for each odd order of the eighth turns (turn8 leaves it out).
 constexpr int child_at(int rho) { return (0x4B >> (2 * rho)) & 3; }  // quadrant at pi/4 + rho pi/2
-// Their sums carry the rounding errors along (fe: value and error, fec: complex), so
-// that a coefficient is rounded to FP32 once before and once after the product.
+// Their sums carry the rounding errors along (fe: value and error, fec: complex), and a
+// coefficient comes from FP64 and goes back with its error, so that it is rounded to FP32
+// once, before the product: with two more roundings per level (a turned coefficient, L2L's
+// result) a starfish of 11 levels at k = 4.35 was 1.39e-7 from FP64 instead of 1.23e-7.
 struct fe {
   float h, l;
 };
@@ -648,6 +651,16 @@ __device__ __forceinline__ void dft4(fec (&v)[4]) {  // v_j <- sum_rho i^{rho j}
   v[3] = sub(b, d);
 }
 __device__ __forceinline__ float2 f32(fec v) { return make_float2(v.x.h + v.x.l, v.y.h + v.y.l); }
+// v f as values and errors, and (value + error) f added to v, with integer instructions
+// for the conversions (those of the FP64 pipe would take as long as the products)
+__device__ __forceinline__ fec pair_of(cd v, double f) {
+  const ff x = ff_from_f64_nan(v.x * f, 896), y = ff_from_f64_nan(v.y * f, 896);
+  return {{x.h, x.l}, {y.h, y.l}};
+}
+__device__ __forceinline__ cd add_pair(cd v, fec a, double f) {
+  return mk(fma(f64_from_f32(a.x.l), f, fma(f64_from_f32(a.x.h), f, v.x)),
+            fma(f64_from_f32(a.y.l), f, fma(f64_from_f32(a.y.h), f, v.y)));
+}
 
 // The matrix of parent level l (M2M: from child order n to parent order s; L2L: from
 // parent to child), from the tables of the quadrant at pi/4 (row stride 4 pbmax + 1,
@@ -789,7 +802,7 @@ __global__ void __launch_bounds__(kT, 4) m2m_fold_kernel(
             v[c] = {{0.f, 0.f}, {0.f, 0.f}};
             if (coff[c][r] >= 0) {
               const cd a = mpole[coff[c][r] + n0 + n];
-              v[c] = turn8({{(float)(a.x * f), 0.f}, {(float)(a.y * f), 0.f}}, m);
+              v[c] = turn8(pair_of(a, f), m);
             }
           }
           dft4(v);
@@ -814,8 +827,7 @@ __global__ void __launch_bounds__(kT, 4) m2m_fold_kernel(
 #pragma unroll
         for (int w = 0; w < 4; ++w) v[w] = red[(w * R + r) * 32 + lane];
         const fec u = turn8(add(add(v[0], v[1]), add(v[2], v[3])), -s);
-        mpole[poff[r] + at] =
-            mk(((double)u.x.h + (double)u.x.l) * f, ((double)u.y.h + (double)u.y.l) * f);
+        mpole[poff[r] + at] = add_pair(mk(0.0, 0.0), u, f);
       }
     }
   }
@@ -863,8 +875,7 @@ __global__ void __launch_bounds__(kT, 4) l2l_fold_kernel(
           if (r < nr) {
             const cd g = local[poff[r] + n0 + n];
             const double f = icp[abs(m)];
-            const fec u = turn8({{(float)(g.x * f), 0.f}, {(float)(g.y * f), 0.f}}, -m);
-            v = f32(u);
+            v = f32(turn8(pair_of(g, f), -m));
           }
           stage_put(fx, n, r, RS, v);
         }
@@ -889,10 +900,8 @@ __global__ void __launch_bounds__(kT, 4) l2l_fold_kernel(
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           if (coff[c][r] < 0) continue;
-          const float2 u = f32(turn8(v[c], s));
           cd* dst = local + coff[c][r] + at;
-          dst->x += (double)u.x * f;
-          dst->y += (double)u.y * f;
+          *dst = add_pair(*dst, turn8(v[c], s), f);
         }
       }
     }

@@ -207,6 +207,13 @@ __device__ __forceinline__ float f32_from_f64(double v) {
   return __uint_as_float(bits | (hi & 0x80000000u));
 }
 
+// an FP32 value as FP64, exact, by the bit fields (subnormals become zero)
+__device__ __forceinline__ double f64_from_f32(float v) {
+  const unsigned b = __float_as_uint(v), e = b & 0x7F800000u;
+  unsigned hi = ((b & 0x7FFFFFFFu) >> 3) + (e == 0x7F800000u ? 1792u << 20 : 896u << 20);
+  return __hiloint2double((int)((b & 0x80000000u) | (e == 0u ? 0u : hi)), (int)(e == 0u ? 0u : b << 29));
+}
+
 // f32_from_f64(v * 2^sh) without the multiplication: the exponent field is
 // offset before the rounding (zero stays zero)
 __device__ __forceinline__ float f32_from_f64_sh(double v, int sh) {

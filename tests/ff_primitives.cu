@@ -34,6 +34,8 @@ __global__ void probe(int op, int n, const double* __restrict__ a, const double*
     o[2] = off ? ff_f64(D.ir) : 0.0;
     o[3] = off ? D.c : 0.0;
     o[4] = off ? D.s : 0.0;
+  } else if (op == 5) {  // FP32 back to FP64
+    out[i] = f64_from_f32((float)a[i]);
   } else {  // J_0 .. J_M of |a|, M = op - 100, scaled by 2^{-iarg j}
     const int M = op - 100;
     float2 row[128];
@@ -48,7 +50,7 @@ __global__ void probe(int op, int n, const double* __restrict__ a, const double*
 
 extern "C" int ff_probe(int op, int n, const double* a, const double* b, int iarg, double k,
                         int width, double* out) {
-  if (n < 1 || op < 0 || (op > 4 && (op < 101 || op > 227))) return -1;
+  if (n < 1 || op < 0 || (op > 5 && (op < 101 || op > 227))) return -1;
   double *da = nullptr, *db = nullptr, *dout = nullptr;
   cudaMalloc(&da, n * sizeof(double));
   cudaMalloc(&db, n * sizeof(double));

@@ -82,6 +82,16 @@ def test_rounding_of_fp64(probe):
     assert got[0] == 0 and got[1] == 0 and got[2] == 2.0 ** -126 and np.isinf(got[3])
 
 
+def test_fp32_to_fp64(probe):
+    rng = np.random.default_rng(4)
+    v = np.concatenate([rng.standard_normal(500), np.ldexp(rng.uniform(-1, 1, 500),
+                        rng.integers(-125, 128, 500)), [0.0, -0.0, 1.0, np.inf, -np.inf, np.nan,
+                        2.0 ** -126, -2.0 ** -126, np.finfo(np.float32).max]])
+    v = v.astype(np.float32)
+    v[np.abs(v) < 2.0 ** -126] = 0  # subnormals become zero
+    assert np.array_equal(probe(5, v, 1)[:, 0], v.astype(float), equal_nan=True)
+
+
 def test_reciprocal_root(probe):
     x = _pair(np.random.default_rng(2).uniform(1, 4, 2000) * 4.0 ** np.repeat(np.arange(-35, 45), 25))
     got = probe(3, x, 1)[:, 0]
