@@ -108,8 +108,8 @@ struct Fmm {
 };
 
 __device__ __forceinline__ const double* pw_row(const Fmm& F, int l) { return F.pw + (size_t)l * (2 * F.pbmax + 3); }
-// 2^e, with which every FP64 result of the mixed path is multiplied
-__device__ __forceinline__ double out_scale(const Fmm& F) { return pow2d(__ldg(F.sexp)); }
+// e: every FP64 result of the mixed path is multiplied by 2^e
+__device__ __forceinline__ int out_exp(const Fmm& F) { return __ldg(F.sexp); }
 __device__ __forceinline__ const double* ipw_row(const Fmm& F, int l) { return F.ipw + (size_t)l * (F.pbmax + 2); }
 
 // Unnormalised Miller recurrence for J_0..J_M of x into row[0..M]; returns the
@@ -238,9 +238,10 @@ __global__ void powers_kernel(int n_levels, int pbmax, const int* __restrict__ l
 // ---------------------------------------------------------------- strengths
 // Sorted strengths; for the mixed path (str_exp set) times 2^-e, e the exponent of the
 // largest of them, so that a density of any size keeps the FP32 stages in range
-// (out_scale puts 2^e back where FP64 results are formed; every step is the same to
-// the bit for 2^n times a density), and their FP32 forms, with the dipole factors A = d (k/2) nu and B = d (k/2) conj(nu) (nu = n_x + i n_y) formed
-// once per source instead of once per (source, centre) pair.
+// (out_exp: 2^e is put back where FP64 results are formed; every step is the same to
+// the bit for 2^n times a density), and their FP32 forms, with the dipole factors
+// A = d (k/2) nu and B = d (k/2) conj(nu) (nu = n_x + i n_y) formed once per source
+// instead of once per (source, centre) pair.
 __global__ void gather_strengths_kernel(int64_t n, const int* __restrict__ perm,
                                         const cd* __restrict__ q, const cd* __restrict__ d,
                                         const double2* __restrict__ snrm, double k,
@@ -1166,7 +1167,7 @@ __global__ void m2qbxl_sum_kernel(int n, int P, const int* __restrict__ cpo,
   if (t1 == t0) return;
   cd sum = mk(0.0, 0.0);
   for (int e = t0; e < t1; ++e) sum = cadd(sum, partial[(size_t)e * P + l]);
-  if (sexp) sum = cscale(sum, pow2d(*sexp));  // mixed path (out_scale)
+  if (sexp) sum = cscale2(sum, *sexp);  // mixed path (out_exp)
   cd* dst = alpha + (size_t)cid[clist[t]] * P + l;
   *dst = cadd(*dst, sum);
 }
@@ -1496,8 +1497,8 @@ __global__ void __launch_bounds__(32) l2qbxl_mixed_kernel(Fmm F, const int* __re
     }
     const double sc = pow2d(emax);
     cd* dst = alpha + (size_t)F.cid[i] * P + p + so;
-    *dst = cadd(*dst, cscale(mk(((double)S.x - (double)C.x) * sc, ((double)S.y - (double)C.y) * sc),
-                             out_scale(F)));
+    *dst = cadd(*dst, cscale2(mk(((double)S.x - (double)C.x) * sc, ((double)S.y - (double)C.y) * sc),
+                              out_exp(F)));
   }
 }
 
@@ -1593,7 +1594,7 @@ __global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restr
     cd* dst = alpha + (size_t)F.cid[i] * P + p + so;
     const cd v = mk(((double)S1.x - (double)C1.x) * f1 + ((double)S2.x - (double)C2.x) * f2,
                     ((double)S1.y - (double)C1.y) * f1 + ((double)S2.y - (double)C2.y) * f2);
-    *dst = cadd(*dst, cscale(v, out_scale(F)));
+    *dst = cadd(*dst, cscale2(v, out_exp(F)));
   }
 }
 
@@ -1750,7 +1751,7 @@ __global__ void __launch_bounds__(kThreads) p2p_warp_mixed_kernel(Fmm F, const i
   }
   if (lane == 0) {
     cd* dst = out + F.tid[i];
-    *dst = cadd(*dst, cscale(sum, out_scale(F)));
+    *dst = cadd(*dst, cscale2(sum, out_exp(F)));
   }
 }
 
@@ -1786,7 +1787,7 @@ __global__ void __launch_bounds__(kThreads) l2p_mixed_kernel(Fmm F, const int* _
   if (!in) {
     cd v;
     l2p_value_outside(F, i, b, &v);
-    *dst = cadd(*dst, cscale(v, out_scale(F)));
+    *dst = cadd(*dst, cscale2(v, out_exp(F)));
     return;
   }
   const float4* pq = reinterpret_cast<const float4*>(F.lpq + F.eoff[b]);
@@ -1851,7 +1852,7 @@ __global__ void __launch_bounds__(kThreads) l2p_mixed_kernel(Fmm F, const int* _
   auto finish = [&](ff u1, ff u2, ff v1) {
     return ff_add(ff_add(u1, ff_mul(mkff(-co.h, -co.l), u2)), ff_mul(si, v1));
   };
-  const double in64 = out_scale(F) / ff_f64(norm);
+  const double in64 = scale2(1.0 / ff_f64(norm), out_exp(F));
   const ff ax = finish(ux1, ux2, vx1), ay = finish(uy1, uy2, vy1);
   *dst = cadd(*dst, mk(ff_f64(ax) * in64, ff_f64(ay) * in64));
 }
@@ -2009,7 +2010,7 @@ __global__ void m2p_sum_mixed_kernel(int n, const int* __restrict__ wtgt, const 
     y = ff_add(y, mkff(v.z, v.w));
   }
   cd* dst = out + tid[wtgt[t]];
-  *dst = cadd(*dst, cscale(mk(ff_f64(x), ff_f64(y)), pow2d(*sexp)));
+  *dst = cadd(*dst, cscale2(mk(ff_f64(x), ff_f64(y)), *sexp));
 }
 
 // ---------------------------------------------------------------- P2M in mixed precision
@@ -2455,7 +2456,7 @@ __global__ void __launch_bounds__(kThreads) p2qbxl_warp_mixed_kernel(Fmm F, cons
   const cd a0 = f64(acc[0]), a1 = W == 16 ? f64(acc[1]) : a0;
   const cd x32 = PM == 16 ? f64(y32) : a0, x33 = PM == 16 ? f64(y33) : a0;
   cd* dst = alpha + (size_t)F.cid[i] * (2 * p + 1) + p;
-  const double os = out_scale(F);
+  const double os = pow2d(out_exp(F));
   pair_coefficients<W, PM>(a0, a1, x32, x33, lane, p, [&](int l, cd a) {
     // the sums carry sigma^{|l|+1}
     if (live) dst[l] = cadd(dst[l], cscale(cscale(a, pow2d(-s * (abs(l) + 1))), os));

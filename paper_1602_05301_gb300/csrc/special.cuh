@@ -270,6 +270,16 @@ __device__ __forceinline__ double pow2d(int d) {
   return __hiloint2double((d + 1023) << 20, 0);
 }
 
+// v 2^d by an addition to the exponent field (a product would take the FP64 pipe);
+// zero, subnormal and non-finite values and results by the product
+__device__ __forceinline__ double scale2(double v, int d) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const unsigned f = ((unsigned)hi >> 20) & 0x7FFu, g = f + (unsigned)d;
+  if (f - 1u < 2046u && g - 1u < 2046u) return __hiloint2double(hi + (int)((unsigned)d << 20), lo);
+  return ((hi & 0x7FFFFFFF) | lo) == 0 ? v : v * pow2d(d / 2) * pow2d(d - d / 2);
+}
+__device__ __forceinline__ cd cscale2(cd v, int d) { return mk(scale2(v.x, d), scale2(v.y, d)); }
+
 // Start index of the backward recurrence for orders 0..pmax at argument x.
 // Started at N, the recurrence returns J_m contaminated by the dominant
 // solution with relative weight about (J_{N+1} Y_m) / (Y_{N+1} J_m); above the
