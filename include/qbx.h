@@ -397,14 +397,17 @@ qbx_status qbx_sync(qbx_handle *h);
 qbx_status qbx_selftest_wait_timeout(qbx_handle *h, int32_t limit_us);
 
 /*
- * H_0(x) and H_1(x) of the first kind, as every kernel of the library
- * evaluates them on the device (the Hankel values that start the recurrences
- * of Sec. 7.2's translations and the kernel G = (i/4) H_0(k|x - y|) of Sec. 1):
- * below x = 8 piecewise polynomials (Chebyshev fits on eight intervals per
- * octave from 2^-9; below that the ascending series, DLMF 10.2.2 and 10.8.1,
- * economised), the CUDA math library's j0/y0/j1/y1 above. variant 0: the FP64
- * path (degree 10, relative error below 1e-15 of |H_0|, |H_1|); 1: the
- * mixed-precision path (degree 8, below 1e-13). x: host [n], positive and
+ * H_0(x) and H_1(x) of the first kind, as the kernels evaluate them on the
+ * device in FP64 (the Hankel values that start the recurrences of Sec. 7.2's
+ * translations and the kernel G = (i/4) H_0(k|x - y|) of Sec. 1): below x = 8 piecewise polynomials (Chebyshev fits on eight intervals
+ * per octave from 2^-9; below that the ascending series, DLMF 10.2.2 and 10.8.1,
+ * economised), on intervals of width 1/2 below x = 32, Hankel's expansion (DLMF
+ * 10.17.5) above. variant 0: the FP64 path (degree 10, relative error below 1e-15
+ * of |H_0|, |H_1|, 4e-15 beyond x = 8); 1: degree 8 below x = 8 (below 1e-13),
+ * which the mixed-precision path takes where its arguments leave the tables in
+ * pairs of FP32 numbers that it uses otherwise (2^-16 <= x < 32: 2.7e-14 of |H|
+ * in the near field, 1.5e-11, 1.9e-10 beyond x = 1, where the terms are rounded
+ * to FP32). x: host [n], positive and
  * finite; out: host [n][4] =
  * (Re H_0, Im H_0, Re H_1, Im H_1). Synchronous. Errors: QBX_ERR_ARG (NULL
  * pointer with n > 0, n < 0, x[i] <= 0 or not finite, unknown variant),
@@ -414,7 +417,8 @@ qbx_status qbx_hankel01(const double *x, int64_t n, int32_t variant, double *out
 
 /*
  * The FP64 -> FP32 rounding of the mixed-precision kernels (Sec. 7.2 Stages
- * 3, 5 in mixed precision: Hankel values from the FP64 recurrences), done
+ * 3, 5 in mixed precision: coefficients, and rows of levels beyond the FP32 pairs'
+ * range), done
  * with integer instructions: round to nearest (ties away from zero), results
  * below 2^-126 in magnitude flushed to zero, overflow to infinity, NaN kept.
  * x: host [n]; out: host float [n]. Synchronous. Errors: QBX_ERR_ARG (NULL

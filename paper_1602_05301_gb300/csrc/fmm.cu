@@ -1175,11 +1175,11 @@ __global__ void m2qbxl_sum_kernel(int n, int P, const int* __restrict__ cpo,
 // ---------------------------------------------------------------- mixed precision P2QBXL
 // H_0, H_1 and the Hankel recurrence in float-float (ff.cuh); the terms are
 // rounded to FP32, multiplied by the FP32 strengths and added with Kahan
-// compensation; the lanes' sums are added and unscaled in FP64 at the end.
+// compensation; the lanes' sums are added in float-float and unscaled in FP64.
 // With the recurrence in FP64 the kernel was bound by the FP64 pipe (82 % of
 // its rate, 95 FP64 instructions per pair); now two FP64 subtractions per pair
 // are left and FP32 issue bounds it: 104 459 centres of 200 ellipses, p = 16, 5.83
-// -> 3.45 ms; 32 curves as a batch, p = 12, both layers, 14.0 -> 10.0 ms in all.
+// -> 1.24 ms with what p2qbxl_pair_mixed and the half warps add.
 __device__ __forceinline__ void kahan2(float2& s, float2& c, float2 v) {
   float y = v.x - c.x, t = s.x + y;
   c.x = (t - s.x) - y;
@@ -1516,7 +1516,7 @@ __global__ void __launch_bounds__(32) l2qbxl_mixed_kernel(Fmm F, const int* __re
 __global__ void __launch_bounds__(32) l2qbxl_ff_kernel(Fmm F, const int* __restrict__ cleaf,
                                                        const int* __restrict__ clist, int n_ctr,
                                                        int G, int TW, cd* __restrict__ alpha) {
-  extern __shared__ __align__(16) float2 frow[];  // [G][TW], TW > max M + 1
+  extern __shared__ __align__(16) float2 frow[];  // [G][TW], TW = max M + 1
   const int lane = threadIdx.x;
   const int c0 = blockIdx.x * G;
   const int p = F.p, P = 2 * p + 1;
@@ -1704,7 +1704,7 @@ __global__ void __launch_bounds__(32) m2qbxl_ff_kernel(
 // float-float (strengths, normals, tables to degree-6 second parts, the lanes'
 // sums; the warp's sum is FP64): about 300 FP32 instructions per source and
 // layer in place of 45 on the FP64 pipe, which bound it (82 % of its rate): 11 M
-// pairs of 200 ellipses 1.22 -> 0.29 ms, the starfish grid 0.19 -> 0.05 ms.
+// pairs of 200 ellipses 1.22 -> 0.26 ms, the starfish grid 0.19 -> 0.05 ms.
 struct FfSum {
   ff x, y;
   __device__ __forceinline__ FfSum() : x(mkff(0.f, 0.f)), y(mkff(0.f, 0.f)) {}
@@ -1909,7 +1909,7 @@ __global__ void __launch_bounds__(kThreads) mpole_f32_list_kernel(
 // Angular factors, products and the compensated (Kahan) sum are FP32. With the
 // recurrence in FP64 on every level the kernel ran at 87 % of the FP64 pipe (4.8 M
 // pairs of 200 ellipses: 2.11 -> 0.76 ms; with packed pairs and the pairs' sums joined
-// in float-float 0.62).
+// in float-float 0.62; with the multipoles rounded by integer instructions 0.57).
 __global__ void __launch_bounds__(kThreads) m2p_pair_mixed_kernel(
     Fmm F, const int* __restrict__ pt, const int* __restrict__ pbx, const int* __restrict__ slot,
     int n, const float2* __restrict__ mu, const double2* __restrict__ rec,
@@ -2358,6 +2358,8 @@ qbx_status configure_kernels() {
 // coefficient is the same sum whichever are formed. Measured with a warp and half a
 // warp each: 200 ellipses, mixed, 2.37 and 2.03 ms; 32 curves of 512 to 32768 centres in
 // a batch 5.99 and 5.34 ms in all; the GMRES solve with 3072 centres 38.3 and 42.6 ms.
+// A handle of many centres that forms few of them loses by it (the starfish at k = 50,
+// mixed, few targets near the curve: 0.037 and 0.066 ms, beside the main stream).
 constexpr int kHalfWarpCentres = 6144;
 // Launches of fewer centres than this run one-warp blocks, which spread over the SMs
 // more evenly.

@@ -180,8 +180,11 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
 constexpr int kGemmRows = 16;
 constexpr int kGemmBlock = 8;
 // Complex products of M2L between Kahan steps: with eight the rotated form's error
-// against FP64 (18 cases, geometric mean) is 1.71e-7, with four 1.62e-7 (1.75e-7 with
-// one matrix per offset class), at 2.32 ms instead of 2.21 on 200 ellipses.
+// against FP64 was 1.71e-7, with four 1.62e-7 (1.75e-7 with one matrix per offset class;
+// now, with M2M and L2L rounded once per level, 1.51e-7), at 2.32 ms instead of 2.21 on
+// 200 ellipses. (Relative l2, geometric mean over the four mixed cases that
+// perf/cases.py lists and the first fourteen FMM evaluations that it draws from
+// random.Random(77), in mixed precision, inputs of seed 5.)
 constexpr int kKahanBlock = 4;
 // Staged rows: order n of the row pair (r, r + 1), r even, is the float4 (re r,
 // re r+1, im r, im r+1) at x + n * stage_stride(R) + r, so that each half is an

@@ -1,6 +1,6 @@
-// qbx_hankel01: the device evaluation of H_0 and H_1 of the first kind that
-// every kernel of the library uses (piecewise polynomials below x = 32,
-// Hankel's expansion above), exposed so that it can be checked on its own.
+// qbx_hankel01: the device evaluation of H_0 and H_1 of the first kind in FP64
+// (piecewise polynomials below x = 32, Hankel's expansion above), exposed so that it
+// can be checked on its own. The mixed path's tables of FP32 pairs are in ff.cuh.
 #include <cmath>
 
 #include "special.cuh"
