@@ -244,7 +244,8 @@ __device__ __forceinline__ void store16(const float (&hi)[16], const float (&lo)
 // most significant first, as bf16 (exact: |d| <= 2^(beta - 1) <= 128): the
 // lower S - 1 digits in [-2^(beta-1), 2^(beta-1)), the top one whatever is left,
 // which is at most 2^(beta - 1) in magnitude since |rint(x 2^(beta S - e))| <=
-// 2^(beta S - 1).
+// 2^(beta S - 1). A value that is not finite has a NaN there, which makes its rows'
+// products NaN (as an integer it would vanish).
 __device__ __forceinline__ void split_digits(double x, int e, int beta, int S,
                                              __nv_bfloat16* __restrict__ out, size_t stride) {
   long long Z = __double2ll_rn(ldexp(x, beta * S - e));
@@ -256,7 +257,8 @@ __device__ __forceinline__ void split_digits(double x, int e, int beta, int S,
     out[(size_t)i * stride] = __float2bfloat16_rn((float)d);
   }
   // the top digit takes the rest, |Z| <= 2^(beta - 1) (no carry is dropped)
-  out[0] = __float2bfloat16_rn((float)Z);
+  const bool finite = (__double2hiint(x) & 0x7FF00000) != 0x7FF00000;
+  out[0] = __float2bfloat16_rn(finite ? (float)Z : __int_as_float(0x7FC00000));
 }
 // exponent e with max_abs 2^-e in [1/4, 1/2) (0 for max_abs == 0)
 __device__ __forceinline__ int scale_exponent(double max_abs) {
